@@ -105,15 +105,17 @@ static eas_status make_a_tmap_deep(CUtensorMap* m, const void* a, int64_t run, i
 }
 
 // output [rows, ld] as a store / reduce target: 32-row boxes whose rows are 128 bytes (64 bf16 or 32 fp32)
-static eas_status make_out_tmap(CUtensorMap* m, const void* out, bool fp32, int64_t cols, int64_t ld, int64_t rows) {
+// (bf16_cols: 64, or 32 for narrow tiles, whose staging rows are then 64 bytes with the 64-byte swizzle)
+static eas_status make_out_tmap(CUtensorMap* m, const void* out, bool fp32, int64_t cols, int64_t ld, int64_t rows, int bf16_cols = 64) {
   PFN_cuTensorMapEncodeTiled_v12000 fn = get_encode_fn();
   if (fn == nullptr) return fail(EAS_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
   const cuuint64_t gdim[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
   const cuuint64_t gstr[1] = {static_cast<cuuint64_t>(ld) * (fp32 ? 4 : 2)};
-  const cuuint32_t box[2] = {fp32 ? 32u : 64u, 32u};
+  const cuuint32_t box[2] = {fp32 ? 32u : static_cast<cuuint32_t>(bf16_cols), 32u};
   const cuuint32_t es[2] = {1, 1};
   CUresult r = fn(m, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(out),
-                  gdim, gstr, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  gdim, gstr, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  !fp32 && bf16_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                   CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(EAS_ERR_CUDA, "cuTensorMapEncodeTiled (output) failed with code %d", static_cast<int>(r));
   return EAS_OK;
@@ -126,7 +128,8 @@ struct Linear {
   int N = 0, K = 0;
   CUtensorMap tmap;        // box of 256 weight rows
   CUtensorMap tmap_half;   // box of 128 weight rows (CTA-pair kernel)
-  CUtensorMap tmap_deep, tmap_half_deep;   // the same for the deep kernels (two k-blocks per box)
+  CUtensorMap tmap_quarter;  // box of 64 weight rows (128x64 tiles)
+  CUtensorMap tmap_half_deep, tmap_quarter_deep;   // the same for the deep kernels (two k-blocks per box)
 };
 struct Layer {
   const bf16 *n1g = nullptr, *n1b = nullptr, *n2g = nullptr, *n2b = nullptr;
@@ -310,60 +313,54 @@ struct OncePerDevice {
 static eas_status finish_linear(Linear& L) {
   EAS_TRY(make_w_tmap(&L.tmap, L.w, L.N, L.K, kBN));
   EAS_TRY(make_w_tmap(&L.tmap_half, L.w, L.N, L.K, kBN / 2));
-  EAS_TRY(make_w_tmap_deep(&L.tmap_deep, L.w, L.N, L.K, kBN));
+  EAS_TRY(make_w_tmap(&L.tmap_quarter, L.w, L.N, L.K, kBN / 4));
+  EAS_TRY(make_w_tmap_deep(&L.tmap_quarter_deep, L.w, L.N, L.K, kBN / 4));
   return make_w_tmap_deep(&L.tmap_half_deep, L.w, L.N, L.K, kBN / 2);
 }
 
 typedef void (*GemmKernel)(GemmParams);
-// ctas: 1 = one CTA per 128x256 tile; 2 = CTA pair per 256x256 tile; 3 = CTA pair per 256x512 tile ("wide");
-// deep (pair tiles only): two 64-wide k-blocks per stage and TMA operation
-// out_fp32: 0 bf16, 1 fp32 (reduce-add when a residual is given), 2 the folding residual epilogue (OUT_F32_FOLD)
-static GemmKernel gemm_kernel_for(int act, int out_fp32, int ctas, bool deep = false, bool split = false) {
-  if (out_fp32 == 2) {
-    if (act != ACT_NONE || split) return nullptr;
-    if (ctas == 3) return gemm_kernel<ACT_NONE, OUT_F32_FOLD, 2, 2>;
-    if (ctas == 2) return deep ? gemm_kernel<ACT_NONE, OUT_F32_FOLD, 2, 1, 2> : gemm_kernel<ACT_NONE, OUT_F32_FOLD, 2, 1>;
-    return gemm_kernel<ACT_NONE, OUT_F32_FOLD, 1, 1>;
-  }
-  if (split) {             // split K: the fp32 residual GEMMs only
-    if (act != ACT_NONE || !out_fp32) return nullptr;
-    if (ctas == 3) return gemm_kernel<ACT_NONE, OUT_F32, 2, 2, 1, true>;
-    if (ctas == 2) return deep ? gemm_kernel<ACT_NONE, OUT_F32, 2, 1, 2, true> : gemm_kernel<ACT_NONE, OUT_F32, 2, 1, 1, true>;
-    return gemm_kernel<ACT_NONE, OUT_F32, 1, 1, 1, true>;
-  }
-  if (ctas == 3) {
-    if (act == ACT_NONE && !out_fp32) return gemm_kernel<ACT_NONE, OUT_BF16, 2, 2>;
-    if (act == ACT_GELU && !out_fp32) return gemm_kernel<ACT_GELU, OUT_BF16, 2, 2>;
-    if (act == ACT_NONE && out_fp32) return gemm_kernel<ACT_NONE, OUT_F32, 2, 2>;
-  } else if (ctas == 2 && deep) {
-    if (act == ACT_NONE && !out_fp32) return gemm_kernel<ACT_NONE, OUT_BF16, 2, 1, 2>;
-    if (act == ACT_GELU && !out_fp32) return gemm_kernel<ACT_GELU, OUT_BF16, 2, 1, 2>;
-    if (act == ACT_SWIGLU && !out_fp32) return gemm_kernel<ACT_SWIGLU, OUT_BF16, 2, 1, 2>;
-    if (act == ACT_NONE && out_fp32) return gemm_kernel<ACT_NONE, OUT_F32, 2, 1, 2>;
-    if (act == ACT_GELU && out_fp32) return gemm_kernel<ACT_GELU, OUT_F32, 2, 1, 2>;
-  } else if (ctas == 2) {
-    if (act == ACT_NONE && !out_fp32) return gemm_kernel<ACT_NONE, OUT_BF16, 2, 1>;
-    if (act == ACT_GELU && !out_fp32) return gemm_kernel<ACT_GELU, OUT_BF16, 2, 1>;
-    if (act == ACT_SWIGLU && !out_fp32) return gemm_kernel<ACT_SWIGLU, OUT_BF16, 2, 1>;
-    if (act == ACT_NONE && out_fp32) return gemm_kernel<ACT_NONE, OUT_F32, 2, 1>;
-    if (act == ACT_GELU && out_fp32) return gemm_kernel<ACT_GELU, OUT_F32, 2, 1>;
+// Tile shapes of the GEMM.  All accumulate every output element over K in the same order: bit-identical results.
+enum { TILE_AUTO = 0, TILE_SINGLE = 1, TILE_PAIR = 2, TILE_WIDE = 3, TILE_N128 = 4, TILE_N64 = 5, TILE_COUNT = 6 };
+struct TileShape { int ctas, rows, cols; };
+static const TileShape kTiles[TILE_COUNT] = {{0, 0, 0}, {1, 128, 256}, {2, 256, 256}, {2, 256, 512}, {1, 128, 128}, {1, 128, 64}};
+// deep (pair and narrow tiles): two 64-wide k-blocks per stage and TMA operation (convolutions walk their taps as 64-wide
+// k-blocks and use the shallow kernels).  nullptr: no such kernel.
+template <int ACT, int OUT, bool SPLIT = false>
+static GemmKernel gemm_kernel_of(int tile, bool deep) {
+  if constexpr (OUT == OUT_F32_FOLD) {
+    if (tile == TILE_WIDE) return gemm_kernel<ACT, OUT, 2, 512>;
+    if (tile == TILE_PAIR) return deep ? gemm_kernel<ACT, OUT, 2, 256, 2> : gemm_kernel<ACT, OUT, 2, 256>;
+    if (tile == TILE_SINGLE) return gemm_kernel<ACT, OUT, 1, 256>;
+    return nullptr;
   } else {
-    if (act == ACT_NONE && !out_fp32) return gemm_kernel<ACT_NONE, OUT_BF16, 1, 1>;
-    if (act == ACT_GELU && !out_fp32) return gemm_kernel<ACT_GELU, OUT_BF16, 1, 1>;
-    if (act == ACT_SWIGLU && !out_fp32) return gemm_kernel<ACT_SWIGLU, OUT_BF16, 1, 1>;
-    if (act == ACT_NONE && out_fp32) return gemm_kernel<ACT_NONE, OUT_F32, 1, 1>;
-    if (act == ACT_GELU && out_fp32) return gemm_kernel<ACT_GELU, OUT_F32, 1, 1>;
+    if (tile == TILE_SINGLE) return gemm_kernel<ACT, OUT, 1, 256, 1, SPLIT>;
+    if (tile == TILE_PAIR) return deep ? gemm_kernel<ACT, OUT, 2, 256, 2, SPLIT> : gemm_kernel<ACT, OUT, 2, 256, 1, SPLIT>;
+    if (tile == TILE_N128) return deep ? gemm_kernel<ACT, OUT, 1, 128, 2, SPLIT> : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 1, 128, 1>);
+    if constexpr (ACT != ACT_SWIGLU) {
+      if (tile == TILE_N64) return deep ? gemm_kernel<ACT, OUT, 1, 64, 2, SPLIT> : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 1, 64, 1>);
+      if constexpr (!(ACT == ACT_GELU && OUT == OUT_F32))
+        if (tile == TILE_WIDE) return gemm_kernel<ACT, OUT, 2, 512, 1, SPLIT>;
+    }
+    return nullptr;
   }
+}
+// out_fp32: 0 bf16, 1 fp32 (reduce-add when a residual is given), 2 the folding residual epilogue (OUT_F32_FOLD)
+static GemmKernel gemm_kernel_for(int act, int out_fp32, int tile, bool deep = false, bool split = false) {
+  if (out_fp32 == 2) return act == ACT_NONE && !split ? gemm_kernel_of<ACT_NONE, OUT_F32_FOLD>(tile, deep) : nullptr;
+  if (split) return act == ACT_NONE && out_fp32 ? gemm_kernel_of<ACT_NONE, OUT_F32, true>(tile, deep) : nullptr;   // the fp32 residual GEMMs only
+  if (act == ACT_NONE) return out_fp32 ? gemm_kernel_of<ACT_NONE, OUT_F32>(tile, deep) : gemm_kernel_of<ACT_NONE, OUT_BF16>(tile, deep);
+  if (act == ACT_GELU) return out_fp32 ? gemm_kernel_of<ACT_GELU, OUT_F32>(tile, deep) : gemm_kernel_of<ACT_GELU, OUT_BF16>(tile, deep);
+  if (act == ACT_SWIGLU && !out_fp32) return gemm_kernel_of<ACT_SWIGLU, OUT_BF16>(tile, deep);
   return nullptr;
 }
 static eas_status set_kernel_attributes() {
   for (int deep = 0; deep < 2; ++deep)
-    for (int ctas = 1; ctas <= 3; ++ctas)
+    for (int tile = TILE_SINGLE; tile < TILE_COUNT; ++tile)
       for (int act = 0; act < 3; ++act)
         for (int f32 = 0; f32 < 3; ++f32) {
-          GemmKernel ks = gemm_kernel_for(act, f32, ctas, deep != 0, true);
+          GemmKernel ks = gemm_kernel_for(act, f32, tile, deep != 0, true);
           if (ks != nullptr) CUDA_TRY(cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemBytes));
-          GemmKernel k = gemm_kernel_for(act, f32, ctas, deep != 0);
+          GemmKernel k = gemm_kernel_for(act, f32, tile, deep != 0);
           if (k != nullptr)
             CUDA_TRY(cudaFuncSetAttribute(reinterpret_cast<const void*>(k), cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmemBytes));
         }
@@ -698,7 +695,7 @@ struct GemmCall {
   const float2* rope_cs = nullptr;
   int reverse = 0;             // walk the tiles last to first
   int w_const = 1;             // the weights are constant (set at create time): their loads may start before the stream's earlier work ends
-  int force_tile = 0;          // 0: the launcher picks; 1 one CTA per 128x256 tile, 2 CTA pair per 256x256, 3 pair per 256x512 (tests)
+  int force_tile = TILE_AUTO;  // others: tests
   int splits = 1;              // split K (see GemmParams::splits); the partial sums of splits 1.. go to `part`
   float* part = nullptr;       // [(splits - 1) * part_rows, N] fp32
   int64_t part_rows = 0;
@@ -717,62 +714,76 @@ struct GemmCall {
 };
 }  // namespace
 
+// Tile shape: a pure speed choice (the results are bit-identical): the smallest estimated time,
+//     base + waves * (kb * per_kb + per_wave)      kb: 64-wide k-blocks of a work item,
+// where a last wave that fills a fraction f of the slots counts `partial` + (1 - partial) * f (fewer SMs share the path to L2).
+// Fitted to 480 measurements on B200: every shape forced over the encoder's GEMMs, 100 <= M <= 18464 tokens, d 256, 1024 and
+// 1280, on 37, 74, 111 and 148 SMs.  The choice is on average 0.2 % and at most 6 % slower than the best shape; without the
+// narrow shapes it was 10 % on average: M = 577 on 148 SMs (N, K): (1024, 4096) 25.3 us as 256x256, 15.1 as 128x64; (1024, 1024)
+// 11.3, 6.4; (3072, 1024) 9.9, 7.5 as 128x128; M = 1500 (1280, 5120) 30.8, 22.5 as 128x128; from a few full waves of pair
+// tiles on those win (M = 18464 (4096, 1024): 115 us, single CTAs 138).
+template <typename Usable>
+static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bool plain, Usable usable) {
+  struct Cost { int tile; double base, per_kb, per_wave, partial; };    // us
+  static const Cost costs[] = {{TILE_SINGLE, 5.5, 0.406, 0.04, 0.80}, {TILE_PAIR, 6.4, 0.336, 0.14, 0.85}, {TILE_WIDE, 5.5, 0.661, 4.5, 0.84},
+                               {TILE_N128, 4.1, 0.241, 0.45, 0.94}, {TILE_N64, 3.4, 0.174, 0.22, 1.0}};
+  int tile = TILE_SINGLE;
+  double best = 0.0;
+  for (const Cost& c : costs) {
+    const TileShape& t = kTiles[c.tile];
+    if (t.ctas > budget || !usable(c.tile)) continue;
+    const int64_t slots = budget / t.ctas;
+    const int64_t tiles = ((M + t.rows - 1) / t.rows) * ((N + t.cols - 1) / t.cols) * splits;
+    const int64_t rem = tiles % slots;
+    const double waves = static_cast<double>(tiles / slots) + (rem != 0 ? c.partial + (1.0 - c.partial) * static_cast<double>(rem) / static_cast<double>(slots) : 0.0);
+    const double shallow = c.tile == TILE_PAIR && !plain ? 1.075 : 1.0;       // convolutions: pair tiles without deep stages
+    const double cost = c.base + waves * (kb * c.per_kb * shallow + c.per_wave);
+    if (best == 0.0 || cost < best) { best = cost; tile = c.tile; }
+  }
+  return tile;
+}
+
 static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream, uint32_t* status) {
   const Linear& L = *g.lin;
   if (g.M <= 0) return EAS_OK;
   if (L.N % 32 != 0 || g.a_run % kBK != 0) return fail(EAS_ERR_UNSUPPORTED, "GEMM needs N %% 32 == 0 and K %% 64 == 0 (N=%d, K=%lld)", L.N, static_cast<long long>(g.a_run));
-  // Tile shape: one CTA per 128x256 tile, a CTA pair per 256x256 tile, or a pair per wide 256x512 tile.  All three
-  // accumulate every output element over K in the same order, so the results are bit-identical and this is a pure
-  // speed choice: estimated time = waves x time of one tile.  The per-k-block times are measured on B200 with each
-  // shape forced over the encoder's GEMM shapes (M = 1154 ... 24000): a 64-wide k-block takes 0.47 us (single CTA),
-  // 0.40 us (pair, deep stages; 0.43 for the convolutions' shallow ones) or 0.75 us for twice the columns (wide
-  // pair); the wide tile's epilogue (about 4 us) does not overlap the next main loop.  What decides in practice is
-  // the wave count: at M = 4616 (c1, micro-batch 8) the out-projection is 2 half-empty waves of
-  // pair tiles but exactly 1 wave of single-CTA tiles.
   const bool tma_out = g.row_map == nullptr && g.pos == nullptr && (g.resid == nullptr || g.resid == g.out);
-  const int64_t k_total = g.a_run * g.taps;
-  const double kb = static_cast<double>(k_total / kBK);
-  auto waves = [](long long tiles, long long slots) { return static_cast<double>((tiles + slots - 1) / slots); };
-  const long long n256 = (L.N + kBN - 1) / kBN;
-  int ctas = 1;
-  bool wide = false;
-  if (budget >= 2) {
-    const long long pairs = budget / 2;
-    const long long m128 = (g.M + kBM - 1) / kBM, m256 = (g.M + 2 * kBM - 1) / (2 * kBM);
-    const double cost_single = waves(m128 * n256 * g.splits, budget) * kb / g.splits * 0.47;
-    const double cost_pair = waves(m256 * n256 * g.splits, pairs) * kb / g.splits * (g.conv_stride == 1 && g.taps == 1 ? 0.40 : 0.43);
-    ctas = cost_single < cost_pair ? 1 : 2;
-    // wide tiles: long reductions whose output splits evenly into 512-column blocks, plain TMA-stored epilogue
-    if (tma_out && g.act != ACT_SWIGLU && k_total >= 2048 && L.N % 512 == 0 && gemm_kernel_for(g.act, g.out_fp32, 3) != nullptr) {
-      const double cost_wide = waves(m256 * (L.N / (2 * kBN)) * g.splits, pairs) * (kb / g.splits * 0.75 + 4.0);
-      if (cost_wide < std::min(cost_single, cost_pair)) { ctas = 2; wide = true; }
-    }
-    if (g.force_tile != 0) {
-      const bool wide_ok = tma_out && g.act != ACT_SWIGLU && L.N % 512 == 0 && gemm_kernel_for(g.act, g.out_fp32, 3) != nullptr;
-      if (g.force_tile == 3 && !wide_ok) return fail(EAS_ERR_UNSUPPORTED, "no wide (256x512) tile for this GEMM: it needs N %% 512 == 0, a plain or GELU epilogue and row-aligned output");
-      ctas = g.force_tile == 1 ? 1 : 2;
-      wide = g.force_tile == 3;
-    }
-#ifdef EAS_GEMM_FORCE_TILE   // calibration builds only: 1 single CTA, 2 pair, 3 wide pair (where a wide kernel exists)
-    ctas = EAS_GEMM_FORCE_TILE == 1 ? 1 : 2;
-    wide = EAS_GEMM_FORCE_TILE == 3 && tma_out && g.act != ACT_SWIGLU && L.N % 512 == 0 && gemm_kernel_for(g.act, g.out_fp32, 3) != nullptr;
-#endif
-  }
   const bool fold_out = g.fold_stats_out != nullptr;
   if (fold_out && (!tma_out || !g.out_fp32 || g.resid != g.out || g.splits != 1 || g.act != ACT_NONE || g.fold_xb == nullptr || g.fold_gamma == nullptr || L.N % kFoldGroup != 0))
     return fail(EAS_ERR_UNSUPPORTED, "the folding epilogue needs an in-place fp32 residual GEMM with N %% %d == 0", kFoldGroup);
   if (g.fold_stats != nullptr && (!tma_out || g.fold_c0 == nullptr || g.a_run % kFoldGroup != 0 || g.taps != 1))
     return fail(EAS_ERR_UNSUPPORTED, "a folded normalisation needs a plain GEMM with row-aligned output and K %% %d == 0", kFoldGroup);
   const int out_mode = fold_out ? 2 : (g.out_fp32 ? 1 : 0);
-  const int tile_n = wide ? 2 * kBN : kBN;
-  // pair tiles of plain GEMMs run the deep kernel (two k-blocks per stage and TMA operation: 8 % faster at K = 1024);
-  // single-CTA and wide tiles would be left with two 96 KB stages and measured no better, and convolutions walk their
-  // taps as 64-wide k-blocks
-  const bool deep = g.conv_stride == 1 && g.taps == 1 && ctas == 2 && !wide;
+  const bool plain = g.conv_stride == 1 && g.taps == 1;
+  // pair and narrow tiles of plain GEMMs run the deep kernels (two k-blocks per stage and TMA operation: 8 % faster at
+  // K = 1024); the 128x256 and wide tiles would be left with two 96 KB stages and measured no better
+  auto is_deep = [&](int t) { return plain && (t == TILE_PAIR || t == TILE_N128 || t == TILE_N64); };
+  auto kernel_of = [&](int t) -> GemmKernel {       // nullptr: this GEMM has no kernel of that shape
+    // wide tiles: the output splits evenly into 512-column blocks, plain TMA-stored epilogue
+    if (t == TILE_WIDE && (!tma_out || L.N % 512 != 0)) return nullptr;
+    return gemm_kernel_for(g.act, out_mode, t, is_deep(t), g.splits > 1);
+  };
+  const int64_t k_total = g.a_run * g.taps;
+  const double kb = static_cast<double>(k_total / kBK) / g.splits;
+  int tile = TILE_SINGLE;
+  if (g.force_tile != TILE_AUTO && (kTiles[g.force_tile].ctas == 1 || budget >= 2)) {
+    tile = g.force_tile;
+    if (kernel_of(tile) == nullptr)
+      return fail(EAS_ERR_UNSUPPORTED, "no %dx%d tile for this GEMM (512 columns: N %% 512 == 0, a plain or GELU epilogue and row-aligned output; 64: no gated epilogue)", kTiles[tile].rows, kTiles[tile].cols);
+  } else if (g.force_tile == TILE_AUTO) {
+    tile = pick_tile(g.M, L.N, kb, g.splits, budget, plain, [&](int t) { return kernel_of(t) != nullptr && (t != TILE_WIDE || k_total >= 2048); });
+#ifdef EAS_GEMM_FORCE_TILE   // calibration builds only: this shape wherever it exists
+    if (budget >= 2 && kernel_of(EAS_GEMM_FORCE_TILE) != nullptr) tile = EAS_GEMM_FORCE_TILE;
+#endif
+  }
+  const int ctas = kTiles[tile].ctas, tile_n = kTiles[tile].cols;
+  const bool deep = is_deep(tile);
   GemmParams p{};
   if (deep) EAS_TRY(make_a_tmap_deep(&p.tma_a, g.A, g.a_run, g.a_row_elems, g.a_rows));
   else EAS_TRY(make_a_tmap(&p.tma_a, g.A, g.a_run, g.a_row_elems, g.conv_stride, g.a_rows));
-  p.tma_b = deep ? (ctas == 2 ? L.tmap_half_deep : L.tmap_deep) : (ctas == 2 ? L.tmap_half : L.tmap);
+  // weight rows per TMA box: the CTA's share of a 256-column accumulator, or the narrow tile's columns
+  const int w_rows = std::min(tile_n, static_cast<int>(kBN)) / ctas;
+  p.tma_b = w_rows == 256 ? L.tmap : w_rows == 128 ? (deep ? L.tmap_half_deep : L.tmap_half) : (deep ? L.tmap_quarter_deep : L.tmap_quarter);
   p.M = g.M; p.N = L.N;
   p.kb_per_tap = static_cast<int>(g.a_run / kBK);
   p.k_blocks = deep ? (p.kb_per_tap + 1) / 2 : p.kb_per_tap * g.taps;
@@ -804,10 +815,10 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
   p.use_tma_out = tma_out ? 1 : 0;
   if (p.use_tma_out) {
     const int64_t out_cols = g.act == ACT_SWIGLU ? L.N / 2 : L.N;
-    EAS_TRY(make_out_tmap(&p.tma_out, g.out, g.out_fp32 != 0, out_cols, g.ldo, g.M));
+    EAS_TRY(make_out_tmap(&p.tma_out, g.out, g.out_fp32 != 0, out_cols, g.ldo, g.M, gemm_out_row(g.act, tile_n)));
   }
   const int tiles = p.m_blocks * p.n_blocks * p.splits;
-  GemmKernel kern = gemm_kernel_for(g.act, out_mode, wide ? 3 : ctas, deep, p.splits > 1);
+  GemmKernel kern = kernel_of(tile);
   if (kern == nullptr) return fail(EAS_ERR_UNSUPPORTED, "no GEMM epilogue for act=%d out_fp32=%d", g.act, g.out_fp32);
   return launch_kernel(kern, std::min(budget / ctas, tiles) * ctas, kGemmThreads, kGemmSmemBytes, stream, p, ctas);
 }
@@ -1557,7 +1568,7 @@ extern "C" eas_status eas_kernel_gemm(const void* A, const void* W, const void* 
 extern "C" eas_status eas_kernel_gemm_tile(const void* A, const void* W, const void* bias, void* out, const float* resid,
                                            int32_t M, int32_t N, int32_t K, int32_t act, int32_t out_fp32, int32_t sm_budget,
                                            void* stream, uint32_t* status_dev, int32_t tile_shape) {
-  if (tile_shape < 0 || tile_shape > 3) return fail(EAS_ERR_INVALID_ARG, "tile_shape %d outside 0..3", tile_shape);
+  if (tile_shape < 0 || tile_shape >= TILE_COUNT) return fail(EAS_ERR_INVALID_ARG, "tile_shape %d outside 0..%d", tile_shape, TILE_COUNT - 1);
   if (A == nullptr || W == nullptr || bias == nullptr || out == nullptr || status_dev == nullptr)
     return fail(EAS_ERR_INVALID_ARG, "a required pointer is null");
   if (M <= 0 || N <= 0 || K <= 0 || K % 64 != 0 || N % 32 != 0) return fail(EAS_ERR_INVALID_ARG, "need M,N,K > 0, K %% 64 == 0, N %% 32 == 0");

@@ -6,8 +6,9 @@
 //   warps 2..9  epilogue: tcgen05.ld -> bias / activation / rotary -> swizzled shared-memory staging -> TMA store
 //               (TMA reduce-add into the fp32 residual stream); scatter epilogues (row maps) store directly
 //
-// Three tile shapes (template arguments CTAS, NW, KD; the launcher picks by estimated time): one CTA per 128x256 tile,
-// a CTA pair (cta_group::2) per 256x256 tile with "deep" stages, a pair per "wide" 256x512 tile.
+// Five tile shapes (template arguments CTAS, TN, KD; the launcher picks by estimated time): one CTA per 128x256 tile,
+// a CTA pair (cta_group::2) per 256x256 tile with "deep" stages, a pair per "wide" 256x512 tile, and, for few tokens, one CTA
+// per "narrow" 128x128 or 128x64 tile.
 //
 // The grid is `sm_budget` CTAs (one per SM: the shared-memory request excludes a second resident
 // CTA) and each CTA walks tiles  blockIdx.x, blockIdx.x + gridDim.x, ...  in a fixed order; every output element is
@@ -27,7 +28,7 @@ constexpr int kProducerBWarp = 2 + kEpiWarps;
 constexpr int kABytes = kBM * kBK * 2;            // 16 KB: 128 rows of A
 // one CTA per tile: a stage holds A (16 KB) + the whole 256-row weight tile (32 KB), 4 stages;
 // CTA pair per 256x256 tile: a stage holds A (16 KB) + this CTA's 128 weight rows (16 KB), 6 stages
-// NW = 2 ("wide", CTA pairs only): the pair owns a 256x512 tile, i.e. two 256-column accumulators fed by the same
+// TN = 512 ("wide", CTA pairs only): the pair owns a 256x512 tile, i.e. two 256-column accumulators fed by the same
 // A tile (three TMA operations for twice the columns) at the price of a single accumulator set: the epilogue no longer
 // overlaps the next main loop, so it pays for large K only.
 // KD = 2 ("deep"): a stage holds TWO 64-wide k-blocks of each operand, fetched by ONE TMA operation per operand
@@ -35,19 +36,24 @@ constexpr int kABytes = kBM * kBK * 2;            // 16 KB: 128 rows of A
 // what a CTA can pull from L2 is set by the number of TMA operations in flight, not by their bytes (two 16 KB
 // boxes per 0.46 us, but also two 32 KB boxes per 0.47 us), so deep stages double the operand rate and move the main
 // loop from the load path to the tensor pipe.  Half as many, twice as large stages: same shared memory.
-template <int CTAS, int NW, int KD = 1> struct GemmCfg {
-  static constexpr int kBBytes = (kBN / CTAS) * kBK * 2 * NW;      // per 64-wide k-block
+// TN = 128 or 64 ("narrow", one CTA): with few tokens a launch has fewer 128x256 tiles than the device has SMs and the K loop
+// of ONE tile is the kernel's time, at the rate one SM pulls operands from L2 (48 KB per 64-wide k-block of a 128x256 tile,
+// 24 KB of a 128x64 one): more, narrower tiles shorten that loop and use the idle SMs.  Measured back to back, M = 577:
+// N = 1024, K = 4096 25.8 (256x256) -> 17.7 us (128x64), K = 1024 11.4 -> 7.1; N = 3072, K = 1024 9.6 -> 7.5 (128x128).
+template <int CTAS, int TN, int KD = 1> struct GemmCfg {
+  static constexpr int kBBytes = (TN / CTAS) * kBK * 2;            // per 64-wide k-block
   static constexpr int kStageBytes = (kABytes + kBBytes) * KD;
-  static constexpr int kStages = (CTAS == 2 ? (NW == 2 ? 4 : 6) : 4) / KD;
-  static constexpr int kAccBuffers = NW == 2 ? 1 : 2;
+  static constexpr int kStages = 4 * 49152 / kStageBytes;          // the ring's 192 KB
+  static constexpr int kAccBuffers = TN == 512 ? 1 : 2;
+  static constexpr int kAccCols = TN < kBN ? TN : kBN;             // tensor-memory columns of one accumulator
+  static constexpr int kTmemCols = TN < kBN ? 2 * TN : 512;
 };
-constexpr int kMaxStages = 6;
+constexpr int kMaxStages = 8;
 constexpr int kStagingOff = 4 * 49152;                         // == 6 * 32768; 8 epilogue warps x 4 KB output staging (TMA store source)
 constexpr int kBiasOff = kStagingOff + kEpiWarps * 4096;       // 2 x 256 fp32 bias values of the current tiles
 constexpr int kBarOff = kBiasOff + 2 * 256 * 4;
 constexpr int kGemmSmemBytes = kBarOff + 192 /*barriers*/ + 832 /*alignment slack*/;
 static_assert(kGemmSmemBytes <= 232448, "exceeds the 227 KB shared memory of an SM");
-constexpr int kTmemCols = 512;
 constexpr int kPanelM = 8;                        // m-blocks per rasterisation panel (L2 reuse of W tiles)
 
 enum { ACT_NONE = 0, ACT_GELU = 1, ACT_SWIGLU = 2 };
@@ -148,17 +154,34 @@ __device__ __noinline__ float2 fold_row_factors(const float2* stats, long long r
   return make_float2(a, -a * mu);
 }
 
+// bf16 outputs of an epilogue warp's row: the columns of one output box (64, or 32 where a warp has no more)
+__host__ __device__ constexpr int gemm_out_row(int act, int tn) {
+  const int per_warp = act == ACT_SWIGLU ? tn / 4 : tn / 2;
+  return per_warp >= 64 ? 64 : 32;
+}
+
 // SPLIT: the launch splits K (GemmParams::splits > 1); the ordinary instantiations keep their code free of it.
-template <int ACT, int OUT, int CTAS, int NW, int KD = 1, bool SPLIT = false>
+template <int ACT, int OUT, int CTAS, int TN, int KD = 1, bool SPLIT = false>
 __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_constant__ GemmParams p) {
-  static_assert(NW == 1 || (CTAS == 2 && ACT != ACT_SWIGLU), "wide tiles: CTA pairs, no gated epilogue");
+  static_assert(TN == 64 || TN == 128 || TN == 256 || TN == 512, "tile width");
+  static_assert(TN < 512 || (CTAS == 2 && ACT != ACT_SWIGLU), "wide tiles: CTA pairs, no gated epilogue");
+  static_assert(TN >= 256 || (CTAS == 1 && OUT != OUT_F32_FOLD), "narrow tiles: one CTA, no folding epilogue");
+  static_assert(TN >= 128 || ACT != ACT_SWIGLU, "a gated epilogue halves the columns: 128 at least");
   static_assert(KD == 1 || KD == 2, "one or two 64-wide k-blocks per stage");
-  constexpr int kStages = GemmCfg<CTAS, NW, KD>::kStages;
-  constexpr int kStageBytes = GemmCfg<CTAS, NW, KD>::kStageBytes;
-  constexpr int kAccBuffers = GemmCfg<CTAS, NW, KD>::kAccBuffers;
-  constexpr int kBRows = kBN / CTAS;               // weight rows per CTA and 256-column accumulator
+  using Cfg = GemmCfg<CTAS, TN, KD>;
+  constexpr int kStages = Cfg::kStages;
+  static_assert(kStages <= kMaxStages, "barrier area");
+  constexpr int kStageBytes = Cfg::kStageBytes;
+  constexpr int kAccBuffers = Cfg::kAccBuffers;
+  constexpr int kAccCols = Cfg::kAccCols;
+  constexpr int kTmemCols = Cfg::kTmemCols;
+  constexpr int NW = TN / kAccCols;                // accumulators of a tile
+  constexpr int kBRows = kAccCols / CTAS;          // weight rows per CTA and accumulator
   constexpr int kBAtom = kBRows * kBK * 2;         // bytes of one 64-wide k-block of those rows
-  constexpr int kTileN = kBN * NW;                 // output columns of a tile
+  constexpr int kTileN = TN;                       // output columns of a tile
+  constexpr int kHalfN = TN / 2;                   // ... of which an epilogue warp's four-warp group takes half
+  // bf16 output: columns of one staging row (and of the output map's box): 64, 128-byte swizzle; 32, 64-byte swizzle
+  constexpr int kOutRow = gemm_out_row(ACT, TN);
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // 1024-byte alignment: the 128-byte swizzle pattern repeats every 8 rows of 128 bytes
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -247,7 +270,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
               }
             } else {
               if (do_a) tma_load_3d(sa, &p.tma_a, &full_bar[s], 0, mb * kBM, kb * KD);
-              if (do_b) tma_load_3d(sb, &p.tma_b, &full_bar[s], 0, nb * kBN, kb * KD);
+              if (do_b) tma_load_3d(sb, &p.tma_b, &full_bar[s], 0, nb * kTileN, kb * KD);
             }
             continue;
           }
@@ -262,7 +285,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
             }
           } else {
             if (do_a) tma_load_3d(sa, &p.tma_a, &full_bar[s], kx, tap % p.conv_stride, mb * kBM + tap / p.conv_stride);
-            if (do_b) tma_load_2d(sb, &p.tma_b, &full_bar[s], kb * kBK, nb * kBN);
+            if (do_b) tma_load_2d(sb, &p.tma_b, &full_bar[s], kb * kBK, nb * kTileN);
           }
         }
       }
@@ -277,7 +300,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   } else if (warp == 1) {
     // ------------------------------------------------------------------ UMMA issuer
     if (lane == 0 && cta_rank == 0) {
-      constexpr uint32_t idesc = make_idesc_bf16(kBM * CTAS, kBN, 0, 0);
+      constexpr uint32_t idesc = make_idesc_bf16(kBM * CTAS, kAccCols, 0, 0);
       uint32_t it = 0, tcount = 0;
       bool ok = true;
       for (int work = first_tile; work < num_work && ok; work += tile_step, ++tcount) {
@@ -285,7 +308,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         const uint32_t acc_ph = (tcount / kAccBuffers) & 1u;
         if (!mbar_wait(&acc_empty[acc], acc_ph ^ 1u, abort_flag)) { ok = false; break; }
         tc_fence_after_sync();
-        const uint32_t tmem_d = tmem_base + acc * kBN;
+        const uint32_t tmem_d = tmem_base + acc * kAccCols;
         const int split = SPLIT ? work % n_splits : 0;
         const int kb0 = split * kb_per_split, kb1 = SPLIT ? min(p.k_blocks, kb0 + kb_per_split) : p.k_blocks;
         for (int kb = kb0; kb < kb1; ++kb, ++it) {
@@ -355,6 +378,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         {
 #pragma unroll
           for (int h = 0; h < NW; ++h) {
+            if (TN < 256 && ew * 32 >= TN) break;
             const int col = nb * kTileN + h * 256 + ew * 32 + lane;
             sbias[h * 256 + ew * 32 + lane] = (col < p.N && split == 0) ? (p.fold_stats != nullptr ? p.fold_c0[col] : __bfloat162float(p.bias[col])) : 0.f;
           }
@@ -373,10 +397,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           // the rows this tile updates, towards L2 while the main loop runs (the epilogue reads them with plain loads)
           const int r = mb * kBM + quarter * 32 + lane;
           if (r < p.M) {
-            const char* base = reinterpret_cast<const char*>(p.resid + static_cast<long long>(r) * p.ldo + nb * kTileN + half * (128 * NW));
+            const char* base = reinterpret_cast<const char*>(p.resid + static_cast<long long>(r) * p.ldo + nb * kTileN + half * kHalfN);
 #pragma unroll
             for (int i = 0; i < 4 * NW; ++i)
-              if (nb * kTileN + half * (128 * NW) + i * 32 < p.N) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + i * 128));
+              if (nb * kTileN + half * kHalfN + i * 32 < p.N) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + i * 128));
           }
         }
         GEMM_STAMP(0);
@@ -387,15 +411,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         tc_fence_after_sync();
         GEMM_STAMP(2);
         uint8_t* stage = smem + kStagingOff + ew * 4096;
-        uint8_t* srow = stage + lane * 128;
-        const int sw = lane & 7;
+        constexpr int kRowBytes = OUT == OUT_BF16 ? kOutRow * 2 : 128;     // 128: 128-byte swizzle; 64: 64-byte swizzle
+        uint8_t* srow = stage + lane * kRowBytes;
+        const int sw = kRowBytes == 128 ? (lane & 7) : ((lane >> 1) & 3);
         const int arow = mb * kBM + quarter * 32 + lane;
-        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * kBN + half * (128 * NW);
+        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * kAccCols + half * kHalfN;
         const int ycoord = mb * kBM + quarter * 32;
 
         auto finish_chunk = [&](float (&v)[32], int c) {   // bias, rotary, activation on 32 accumulator columns
-          const int col0 = nb * kTileN + half * (128 * NW) + c * 32;
-          const float4* b4 = reinterpret_cast<const float4*>(sbias + half * (128 * NW) + c * 32);
+          const int col0 = nb * kTileN + half * kHalfN + c * 32;
+          const float4* b4 = reinterpret_cast<const float4*>(sbias + half * kHalfN + c * 32);
           if (p.fold_stats != nullptr) {
             // out = rstd * acc + (c0 - rstd * mean * c1): the staged "bias" is c0
             const bool centred = p.fold_c1 != nullptr && col0 < p.N;
@@ -469,11 +494,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           static_assert(OUT != OUT_F32_FOLD || ACT == ACT_NONE, "the folding residual epilogue has no activation");
           constexpr int kChunks = 4 * NW;
           const bool row_ok = arow < p.M;
-          const int tcol0 = nb * kTileN + half * (128 * NW);
+          const int tcol0 = nb * kTileN + half * kHalfN;
           const long long roff = static_cast<long long>(row_ok ? arow : 0) * p.ldo + tcol0;
           const float4* xin = reinterpret_cast<const float4*>(p.resid + roff);
           uint4* xb = reinterpret_cast<uint4*>(p.fold_xb + roff);
-          const float4* b4 = reinterpret_cast<const float4*>(sbias + half * (128 * NW));
+          const float4* b4 = reinterpret_cast<const float4*>(sbias + half * kHalfN);
           uint32_t r[32];
           float4 xo[8];
           __syncwarp();
@@ -544,7 +569,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           // fp32 output: 32 columns = one 128-byte staging row, so every 32-column chunk is a sub-tile (and a TMA
           // operation) of its own.  One chunk per round, the next chunk's TMEM load in flight meanwhile, so that the
           // wait for the previous operation to release the staging buffer falls behind a load and the chunk's math.
-          constexpr int kChunks = 4 * NW;
+          constexpr int kChunks = kHalfN / 32;
           uint32_t r[32];
           __syncwarp();
           tmem_ld_32x32(taddr, r);
@@ -559,7 +584,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
               tmem_ld_32x32(taddr + (c + 1) * 32, r);
             }
             finish_chunk(v, c);
-            const int col0 = nb * kTileN + half * (128 * NW) + c * 32;
+            const int col0 = nb * kTileN + half * kHalfN + c * 32;
             staging_free();
 #pragma unroll
             for (int q = 0; q < 8; ++q)
@@ -568,32 +593,22 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           }
         } else {
 #pragma unroll 1
-        for (int pr = 0; pr < 2 * NW; ++pr) {       // two chunks (64 accumulator columns) per round
+        for (int pr = 0; pr < (kHalfN + 63) / 64; ++pr) {       // two chunks (64 accumulator columns) per round
+          constexpr int kPerRound = kHalfN >= 64 ? 2 : 1;
           uint32_t r0[32], r1[32];
           __syncwarp();
           tmem_ld_32x32(taddr + pr * 64, r0);
-          tmem_ld_32x32(taddr + pr * 64 + 32, r1);
+          if (kPerRound == 2) tmem_ld_32x32(taddr + pr * 64 + 32, r1);
           tmem_ld_wait();
           GEMM_STAMP(3 + pr * 4);
           float v0[32], v1[32];
 #pragma unroll
-          for (int i = 0; i < 32; ++i) { v0[i] = __uint_as_float(r0[i]); v1[i] = __uint_as_float(r1[i]); }
+          for (int i = 0; i < 32; ++i) { v0[i] = __uint_as_float(r0[i]); v1[i] = kPerRound == 2 ? __uint_as_float(r1[i]) : 0.f; }
           finish_chunk(v0, pr * 2);
-          finish_chunk(v1, pr * 2 + 1);
+          if (kPerRound == 2) finish_chunk(v1, pr * 2 + 1);
           GEMM_STAMP(4 + pr * 4);
-          const int col0 = nb * kTileN + half * (128 * NW) + pr * 64;
-          if (OUT == OUT_F32) {
-            // 32 fp32 columns = one 128-byte staging row; two sub-tiles per round
-#pragma unroll
-            for (int h2 = 0; h2 < 2; ++h2) {
-              float (&v)[32] = h2 ? v1 : v0;
-              staging_free();
-#pragma unroll
-              for (int q = 0; q < 8; ++q)
-                *reinterpret_cast<float4*>(srow + ((q ^ sw) << 4)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-              if (col0 + h2 * 32 < p.N) store_subtile(col0 + h2 * 32);
-            }
-          } else if (ACT == ACT_SWIGLU) {
+          const int col0 = nb * kTileN + half * kHalfN + pr * 64;
+          if (ACT == ACT_SWIGLU) {
             // (gate, up) pairs -> 32 outputs per round; the 64 outputs of both rounds form one staging row
             if (pr == 0) staging_free();
 #pragma unroll
@@ -607,13 +622,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
               *reinterpret_cast<uint4*>(srow + (((q0) ^ sw) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
               *reinterpret_cast<uint4*>(srow + (((q0 + 1) ^ sw) << 4)) = make_uint4(w[4], w[5], w[6], w[7]);
             }
-            if (pr == 1 && nb * kBN + half * 128 < p.N) store_subtile((nb * kBN + half * 128) >> 1);
+            if (pr + 1 == (kHalfN + 63) / 64 && nb * kTileN + half * kHalfN < p.N) store_subtile((nb * kTileN + half * kHalfN) >> 1);
           } else {
-            // 64 bf16 columns = one 128-byte staging row
+            // 64 bf16 columns = one 128-byte staging row (128x64 tiles: 32 columns, 64 bytes)
             staging_free();
             GEMM_STAMP(5 + pr * 4);
 #pragma unroll
-            for (int h2 = 0; h2 < 2; ++h2) {
+            for (int h2 = 0; h2 < kPerRound; ++h2) {
               float (&v)[32] = h2 ? v1 : v0;
 #pragma unroll
               for (int q = 0; q < 4; ++q)
@@ -647,12 +662,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
       const int posrow = (row_ok && p.pos_idx != nullptr) ? p.pos_idx[arow] : 0;
 
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
-        const int col_in_tile = half * 128 + c * 32;
-        const int col0 = nb * kBN + col_in_tile;                  // first of 32 output-space accumulator columns
+      for (int c = 0; c < kHalfN / 32; ++c) {
+        const int col_in_tile = half * kHalfN + c * 32;
+        const int col0 = nb * kTileN + col_in_tile;                  // first of 32 output-space accumulator columns
         uint32_t raw[32];
         __syncwarp();   // the TMEM load is warp-collective: reconverge after the per-row branches below
-        tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * kBN + col_in_tile, raw);
+        tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * kAccCols + col_in_tile, raw);
         tmem_ld_wait();
         if (!row_ok || col0 >= p.N) continue;
         float v[32];
