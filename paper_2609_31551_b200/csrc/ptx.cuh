@@ -66,6 +66,32 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 
+// The wait of a whole warp: the outcome is the same for all lanes, so the warp leaves a loop together (and is converged
+// afterwards, as warp-collective instructions want it).  `ready` is the result of an earlier mbar_try_wait on the same
+// phase: testing ahead hides the test's latency.
+__device__ __forceinline__ bool warp_mbar_wait_tested(uint32_t ready, uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag) {
+  if (__builtin_expect(__all_sync(0xffffffffu, ready), 1)) return true;
+  const long long t0 = clock64();
+  uint32_t it = 0;
+  while (true) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if ((++it & 63u) == 0u) {
+      if (clock64() - t0 > kWaitCycleLimit) *abort_flag = 1u;
+      if (__any_sync(0xffffffffu, *abort_flag != 0u)) return false;
+    }
+  }
+}
+__device__ __forceinline__ bool warp_mbar_wait(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag) {
+  return warp_mbar_wait_tested(mbar_try_wait(bar, parity), bar, parity, abort_flag);
+}
+// true in one lane of a converged warp.  The control flow around it stays warp-uniform, so that operands computed outside
+// (UMMA descriptors) live in uniform registers instead of being moved there for every instruction.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t pred;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
+  return pred != 0u;
+}
+
 // Programmatic dependent launch: a kernel launched with the stream-serialization attribute may start while its
 // predecessor drains; it must not touch the predecessor's results before pdl_wait().  Both are no-ops otherwise.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
