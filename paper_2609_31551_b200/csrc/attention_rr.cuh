@@ -1,0 +1,495 @@
+// Block-diagonal (variable-length) softmax attention on tcgen05 tensor cores: the default kernel.
+//
+// A query tile is 128 rows of one head of one item.  A work unit is up to three consecutive query tiles of one item, counted
+// head by head; a softmax warpgroup (one thread per query row) works on each.  The key loop walks the item's keys 80 at a
+// time; keys past the item's end are masked to probability exactly 0, keys of other items are never multiplied in.  The
+// tiles of a unit may belong to several heads (an item of 577 tokens has 5 query tiles a head): each head of the unit is a
+// "stream" of K/V tiles of its own, shared by its tiles.
+//
+//   warp 0       TMA producer of K and V tiles (ring)
+//   warps 1..3   UMMA issuers, one per warpgroup: S = Q K^T (128 x 80) into TMEM, O += P V (128 x head_dim) in TMEM; they also
+//                load the warpgroup's Q tiles (one buffer each, refilled as soon as its last scores are complete)
+//   warps 4..15  three softmax warpgroups
+//
+// What bounds it, and why three tiles: a tile's chain (scores -> row maximum -> exponentials -> P to tensor memory -> P V and
+// the next scores -> back) takes 1750 cycles a step of 80 keys when a tile is alone, of which the exponentials need 480 (a
+// quarter of them on the FMA pipe) and the tensor pipe 320-400: mostly latency, so what counts is the number of tiles in
+// flight.  Three take 2450 cycles a step together; two with 128 (112) keys a step and P in columns of its own, the former
+// kernel, 3100 (2780).  Tensor memory holds three because P takes S's own columns (dead once the row is in registers):
+// 3 x (80 + head_dim) columns.  The scores of a tile's next step then have to wait for its P V, but the other warpgroups'
+// exponentials fill that time; UMMAs complete in order, so "scores ready" also says that the warpgroup's previous P V is
+// complete, and a step has one wait.  Each warpgroup has an issuer of its own: one issuer for all (about 900 cycles of waits,
+// issues and commits a step) was what the warpgroups waited for (1.37 times the time).
+// Measured, same session, former kernel -> this one: 4 x 8192 tokens, 16 heads of 64: 1493 -> 1275 us; 2 x 8192, heads of 80:
+// 784 -> 735 us; 32768, heads of 80: 6.2 -> 5.7 ms; ragged 256 ... 4900, heads of 80: 316 -> 272 us; 32 x 577, heads of 64:
+// 108 -> 87 us.  Not better: four warpgroups (64 keys at head_dim 64, 48 at 80), P in columns of its own with 64 or 48 keys
+// (the next scores early), no row maximum while a safe reference stands, other shares of the FMA-pipe exponentials.
+//
+// The reference maximum only moves when the row maximum grows by more than 2^8 in the exponent; then the thread rescales
+// its O row in TMEM.  Final O / l is written as bf16.  A row's arithmetic does not depend on its unit.
+// Persistent: gridDim.x = sm_budget CTAs; the units are dealt to them in rounds of gridDim.x, alternate rounds in
+// opposite directions (the host sorts the units by decreasing cost: a fixed direction would hand CTA 0 the costliest
+// unit of every round).
+#pragma once
+#include "attention_tc.cuh"
+#include "ptx.cuh"
+
+namespace eas {
+
+struct AttnRrParams {
+  CUtensorMap map_q_lo;   // qkv [T, 3d], box {64 columns, 128 rows}, 128-byte swizzle
+  CUtensorMap map_q_hi;   // box {16 columns, 128 rows}, 32-byte swizzle (head_dim 80: columns 64..79)
+  CUtensorMap map_k_lo;   // box {64 columns, KEYS rows}, 128-byte swizzle (K and V tiles)
+  CUtensorMap map_k_hi;   // box {16 columns, KEYS rows}, 32-byte swizzle
+  bf16* out;
+  long long ldo;
+  int d_model, n_heads;
+  float scale_log2;       // log2(e) / sqrt(head_dim)
+  int n_items, total_units;
+  int item_start[128];
+  int item_len[128];
+  int unit_prefix[129];
+  // an item's units: item_full of them with kWg query tiles, the others with small_tiles (<= kWg): see attention_plan
+  int item_full[128];
+  int small_tiles;
+  uint32_t* status;
+};
+
+template <int HD> struct AttnRrCfg;
+template <> struct AttnRrCfg<64> { static constexpr int kStages = 6; };
+template <> struct AttnRrCfg<80> { static constexpr int kStages = 4; };
+
+template <int HD>
+struct AttnRrSmem : AttnRrCfg<HD> {
+  using C = AttnRrCfg<HD>;
+  static constexpr int kWg = 3, kKeys = 80;
+  static constexpr int kRegsLight = 104, kRegsSoftmax = 136, kRegsLaunch = 128;
+  static constexpr int HI = HD - 64;                       // 0 or 16 extra columns
+  static constexpr int kThreads = 128 * (1 + kWg);
+  static constexpr int kLoBytes = 128 * 128;               // Q tile: 128 rows x 64 bf16
+  static constexpr int kHiBytes = 128 * HI * 2;            // 128 rows x 16 bf16, 32-byte swizzle
+  static constexpr int kQBytes = kLoBytes + kHiBytes;
+  static constexpr int kAtomBytes = kKeys * 128;        // keys x 64 bf16
+  static constexpr int kKHiBytes = kKeys * HI * 2;
+  static constexpr int kKTxBytes = kAtomBytes + kKHiBytes;
+  static constexpr int kKBytes = (kKTxBytes + 1023) / 1024 * 1024;
+  // head_dim 80: V is loaded 128 columns wide (two 64-column boxes; the extra 48 columns belong to the next head, or are
+  // zero past the last one) so that P V is ONE UMMA per 16 keys, N = 80 across the two swizzle atoms.
+  static constexpr int kVBytes = kAtomBytes * (HI ? 2 : 1);
+  static constexpr int kStageBytes = kKBytes + kVBytes;
+  static constexpr int kKvOff = kWg * kQBytes;
+  static constexpr int kBarOff = kKvOff + C::kStages * kStageBytes;
+  static constexpr int kBytes = kBarOff + 512 + 1024;      // barriers + alignment slack
+  static_assert(kBytes <= 232448, "exceeds the shared memory of an SM");
+  static_assert(kBytes > 116224, "a second CTA must not fit beside this one");
+  static_assert(kQBytes % 1024 == 0 && kStageBytes % 1024 == 0 && kAtomBytes % 1024 == 0, "tiles start on swizzle-atom boundaries");
+  // TMEM columns of warpgroup w: S (and P in its first half) at w * kColStride, O behind it
+  static constexpr int kColStride = kKeys + HD;
+  static_assert(kWg * kColStride <= 512, "tensor memory columns");
+  static_assert(kKeys == 80, "five UMMA k-steps; a row of scores is 32 + 32 + 16 registers");
+  static_assert(C::kStages > kWg, "an issuer looks at most kWg ring positions ahead of the stage it holds");
+  // setmaxnreg: the pool is the CTA's launch allocation
+  static_assert(128 * kRegsLight + 128 * kWg * kRegsSoftmax <= kThreads * kRegsLaunch, "setmaxnreg budget exceeds the CTA's register allocation");
+  static_assert(kThreads * kRegsLaunch <= 65536, "registers");
+};
+
+#ifndef EAS_RR_POLY_OF_8
+#define EAS_RR_POLY_OF_8 2      // of every 8 pairs of probabilities, this many take the polynomial path
+#endif
+
+// Wait for this thread's tensor-memory loads, tied to registers they fill so that no use can move ahead of it.
+template <int OFF, int N>
+__device__ __forceinline__ void tmem_ld_wait_16(uint32_t (&r)[N]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[OFF]), "+r"(r[OFF + 1]), "+r"(r[OFF + 2]), "+r"(r[OFF + 3]), "+r"(r[OFF + 4]), "+r"(r[OFF + 5]), "+r"(r[OFF + 6]), "+r"(r[OFF + 7]),
+                 "+r"(r[OFF + 8]), "+r"(r[OFF + 9]), "+r"(r[OFF + 10]), "+r"(r[OFF + 11]), "+r"(r[OFF + 12]), "+r"(r[OFF + 13]), "+r"(r[OFF + 14]), "+r"(r[OFF + 15])
+               ::"memory");
+}
+// ties 16 more registers behind the wait above (no instruction)
+template <int OFF, int N>
+__device__ __forceinline__ void tmem_ld_tie_16(uint32_t (&r)[N]) {
+  asm volatile("" : "+r"(r[OFF]), "+r"(r[OFF + 1]), "+r"(r[OFF + 2]), "+r"(r[OFF + 3]), "+r"(r[OFF + 4]), "+r"(r[OFF + 5]), "+r"(r[OFF + 6]), "+r"(r[OFF + 7]),
+                    "+r"(r[OFF + 8]), "+r"(r[OFF + 9]), "+r"(r[OFF + 10]), "+r"(r[OFF + 11]), "+r"(r[OFF + 12]), "+r"(r[OFF + 13]), "+r"(r[OFF + 14]), "+r"(r[OFF + 15])
+               ::"memory");
+}
+
+struct RrUnit {
+  int r0, nt, n_q, head0, n_streams, S, n_kv, row0;
+};
+
+template <int HD>
+__global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(const __grid_constant__ AttnRrParams p) {
+  using L = AttnRrSmem<HD>;
+  constexpr int HI = L::HI, NST = L::kStages, NWG = L::kWg, KEYS = L::kKeys;
+  extern __shared__ uint8_t smem_raw_attn[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_attn) + 1023) & ~uintptr_t(1023));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::kBarOff);
+  uint64_t* q_full = bars;                 // [NWG]
+  uint64_t* s_full = q_full + NWG;         // [NWG] scores of a step complete (and everything issued before them)
+  uint64_t* p_ready = s_full + NWG;        // [NWG] P stored, O rescaled if it had to be
+  uint64_t* k_full = p_ready + NWG;        // [NST]
+  uint64_t* v_full = k_full + NST;         // [NST]
+  uint64_t* kv_empty = v_full + NST;       // [NST] every issuer hands every stage back
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(kv_empty + NST);
+  volatile uint32_t* abort_flag = tmem_slot + 1;
+  static_assert((3 * NWG + 3 * NST) * 8 + 8 <= 512, "barrier area");
+
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < NWG; ++i) { mbar_init(&q_full[i], 1); mbar_init(&s_full[i], 1); mbar_init(&p_ready[i], 4); }
+    for (int i = 0; i < NST; ++i) { mbar_init(&k_full[i], 1); mbar_init(&v_full[i], 1); mbar_init(&kv_empty[i], NWG); }
+    *abort_flag = 0;
+    mbar_fence_init();
+    tma_prefetch_desc(&p.map_q_lo);
+    tma_prefetch_desc(&p.map_k_lo);
+    if (HI) { tma_prefetch_desc(&p.map_q_hi); tma_prefetch_desc(&p.map_k_hi); }
+  }
+  if (warp == 1) {
+    tmem_alloc(tmem_slot, 512);
+    tmem_relinquish();
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_launch_dependents();
+  pdl_wait();
+
+  // this CTA's unit of a round; increasing in `round`
+  auto unit_at = [&](uint32_t round) -> int {
+    const int g = static_cast<int>(gridDim.x), b = static_cast<int>(blockIdx.x);
+    return static_cast<int>(round) * g + ((round & 1u) ? g - 1 - b : b);
+  };
+  // units are visited in increasing order: the item is found by stepping forward from the previous unit's (`cursor`)
+  auto decode = [&](int unit, int& cursor) -> RrUnit {
+    int lo = cursor;
+    while (lo + 1 < p.n_items && p.unit_prefix[lo + 1] <= unit) ++lo;
+    cursor = lo;
+    RrUnit u;
+    u.S = p.item_len[lo];
+    u.row0 = p.item_start[lo];
+    u.nt = (u.S + kTcTile - 1) / kTcTile;
+    u.n_kv = (u.S + KEYS - 1) / KEYS;
+    const int k = unit - p.unit_prefix[lo], full = p.item_full[lo];
+    u.r0 = k < full ? k * NWG : full * NWG + (k - full) * p.small_tiles;
+    u.n_q = min(k < full ? NWG : p.small_tiles, p.n_heads * u.nt - u.r0);
+    u.head0 = u.r0 / u.nt;
+    u.n_streams = (u.r0 + u.n_q - 1) / u.nt - u.head0 + 1;
+    return u;
+  };
+  auto stream_of = [](const RrUnit& u, int w) { return (u.r0 + w) / u.nt - u.head0; };
+  auto q_tile = [&](int w) { return smem + w * L::kQBytes; };
+  auto k_tile = [&](int s) { return smem + L::kKvOff + s * L::kStageBytes; };
+  auto v_tile = [&](int s) { return smem + L::kKvOff + s * L::kStageBytes + L::kKBytes; };
+
+  if (warp == 0) {
+    // ------------------------------------------------------------------ K / V producer
+    setmaxnreg_dec<L::kRegsLight>();
+    if (lane == 0) {
+      uint32_t g = 0, round = 0;
+      bool ok = true;
+      int cursor = 0;
+      for (int unit = unit_at(0); unit < p.total_units && ok; unit = unit_at(++round)) {
+        const RrUnit u = decode(unit, cursor);
+        for (int j = 0; j < u.n_kv && ok; ++j)
+          for (int st = 0; st < u.n_streams; ++st, ++g) {
+            const int s = g % NST;
+            if (!mbar_wait(&kv_empty[s], ((g / NST) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+            const int x = (u.head0 + st) * HD, y = u.row0 + j * KEYS;
+            mbar_expect_tx(&k_full[s], L::kKTxBytes);
+            tma_load_2d(k_tile(s), &p.map_k_lo, &k_full[s], p.d_model + x, y);
+            if (HI) tma_load_2d(k_tile(s) + L::kAtomBytes, &p.map_k_hi, &k_full[s], p.d_model + x + 64, y);
+            mbar_expect_tx(&v_full[s], L::kVBytes);
+            tma_load_2d(v_tile(s), &p.map_k_lo, &v_full[s], 2 * p.d_model + x, y);
+            if (HI) tma_load_2d(v_tile(s) + L::kAtomBytes, &p.map_k_lo, &v_full[s], 2 * p.d_model + x + 64, y);
+          }
+      }
+      if (!ok) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < 4000000) {}     // let loads in flight land before the CTA retires
+      }
+    }
+  } else if (warp <= NWG) {
+    // ------------------------------------------------------------------ UMMA issuers, one warp per warpgroup
+    // The whole warp walks the steps (uniform control flow: see elect_one) and one elected lane issues.  A step: P V of
+    // this step and the scores of the next as soon as P is there.  What they need beside P (V, the next K, the next tile's
+    // Q) is waited for before P, so that the path from P to the next scores holds one wait.
+    // An issuer sees every K/V stage of the CTA land, in order, also those of streams its tile has no part in (it hands those
+    // back with a plain arrival), so that it never mistakes a barrier's phase for an earlier one.  Holding its own stage g it
+    // waits for no stage past g + kWg < g + kStages (warpgroup w belongs at most to stream w, and at most kWg - 1 - w streams
+    // follow its own), so the waits of the issuers have no cycle.
+    setmaxnreg_dec<L::kRegsLight>();
+    const int w = warp - 1;
+    constexpr uint32_t idesc_s = make_idesc_bf16(128, KEYS, 0, 0);         // S = Q K^T, both K-major
+    constexpr uint32_t idesc_o = make_idesc_bf16(128, HD, 0, 1);           // O += P V, V is MN-major
+    const uint32_t tm = tmem_base + w * L::kColStride;
+    uint32_t n_q = 0, n_s = 0, n_p = 0;          // Q tiles waited for, s_full phases committed, p_ready phases waited for
+    bool started = false;                        // the first scores of this unit's tile are issued already
+    bool owed = false;                           // the warpgroup still has to say that it has seen a bare commit
+    uint32_t base = 0, round = 0;                // base: ring position of the unit's first K/V tile
+    bool ok = true;
+    int cursor = 0;
+    RrUnit un{};
+    if (unit_at(0) < p.total_units) un = decode(unit_at(0), cursor);
+
+    auto load_q = [&](const RrUnit& u) {
+      const int head = (u.r0 + w) / u.nt, y = u.row0 + ((u.r0 + w) - head * u.nt) * kTcTile;
+      if (elect_one()) {
+        mbar_expect_tx(&q_full[w], L::kQBytes);
+        tma_load_2d(q_tile(w), &p.map_q_lo, &q_full[w], head * HD, y);
+        if (HI) tma_load_2d(q_tile(w) + L::kLoBytes, &p.map_q_hi, &q_full[w], head * HD + 64, y);
+      }
+      __syncwarp();
+    };
+    auto q_landed = [&]() -> bool {
+      if (!warp_mbar_wait(&q_full[w], n_q & 1u, abort_flag)) return false;
+      ++n_q;
+      return true;
+    };
+    auto k_landed = [&](uint32_t g) -> bool { return warp_mbar_wait(&k_full[g % NST], (g / NST) & 1u, abort_flag); };
+    auto hand_back = [&](uint32_t from, uint32_t to) -> bool {   // stages of other streams
+      for (uint32_t g = from; g < to; ++g) {
+        if (!k_landed(g)) return false;
+        if (elect_one()) mbar_arrive(&kv_empty[g % NST]);
+        __syncwarp();
+      }
+      return true;
+    };
+    // by the elected lane: scores against the K tile at ring position g
+    auto mma_s = [&](uint32_t g) {
+      const uint32_t qa = smem_u32(q_tile(w)), ka = smem_u32(k_tile(g % NST));
+      const uint64_t ad = make_smem_desc(qa, 16, 1024, kSwizzle128B);
+      const uint64_t bd = make_smem_desc(ka, 16, 1024, kSwizzle128B);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) umma_bf16_ss(tm, ad + 2 * k, bd + 2 * k, idesc_s, k != 0);
+      if (HI) {
+        const uint64_t ah = make_smem_desc(qa + L::kLoBytes, 16, 256, kSwizzle32B);
+        const uint64_t bh = make_smem_desc(ka + L::kAtomBytes, 16, 256, kSwizzle32B);
+        umma_bf16_ss(tm, ah, bh, idesc_s, 1);
+      }
+      umma_commit(&s_full[w]);
+    };
+
+    for (int unit = unit_at(0); unit < p.total_units && ok; unit = unit_at(++round)) {
+      const RrUnit u = un;
+      const bool has_next = unit_at(round + 1) < p.total_units;
+      if (has_next) un = decode(unit_at(round + 1), cursor);
+      const uint32_t ns = static_cast<uint32_t>(u.n_streams);
+      const uint32_t next_base = base + static_cast<uint32_t>(u.n_kv) * ns;
+      if (w >= u.n_q) {
+        ok = hand_back(base, next_base);
+        base = next_base;
+        continue;
+      }
+      const bool chain = has_next && w < un.n_q;      // the next unit's first scores follow this unit's last P V
+      const uint32_t st = static_cast<uint32_t>(stream_of(u, w)), st_next = chain ? static_cast<uint32_t>(stream_of(un, w)) : 0u;
+      if (!started) {
+        if (owed) {                              // the warpgroup has seen the bare commit, so s_full may be used again
+          if (!warp_mbar_wait(&p_ready[w], n_p & 1u, abort_flag)) { ok = false; break; }
+          ++n_p;
+        }
+        load_q(u);
+        if (!hand_back(base, base + st) || !q_landed() || !k_landed(base + st)) { ok = false; break; }
+        tc_fence_after_sync();
+        if (elect_one()) mma_s(base + st);
+        __syncwarp();
+        ++n_s;
+      }
+      for (int j = 0; j < u.n_kv; ++j) {
+        const bool last = j + 1 == u.n_kv;
+        const bool more = !last || chain;
+        const uint32_t row = base + static_cast<uint32_t>(j) * ns, g = row + st;
+        const uint32_t gn = last ? next_base + st_next : g + ns;      // the K tile of the scores to come
+        if (last && chain) {
+          // the last scores are complete: the Q buffer is free
+          if (!warp_mbar_wait(&s_full[w], (n_s - 1u) & 1u, abort_flag)) { ok = false; break; }
+          load_q(un);
+        }
+        if (!hand_back(g + 1, row + ns)) { ok = false; break; }
+        if (!warp_mbar_wait(&v_full[g % NST], (g / NST) & 1u, abort_flag)) { ok = false; break; }
+        if (more && (!hand_back(last ? next_base : row + ns, gn) || !k_landed(gn))) { ok = false; break; }
+        if (last && chain && !q_landed()) { ok = false; break; }
+        if (!warp_mbar_wait(&p_ready[w], n_p & 1u, abort_flag)) { ok = false; break; }
+        ++n_p;
+        tc_fence_after_sync();
+        // 64-column swizzle atoms kAtomBytes apart (leading byte offset; head_dim 64 has one), 8-key groups 1 KB apart
+        const uint64_t bd = make_smem_desc(smem_u32(v_tile(g % NST)), L::kAtomBytes, 1024, kSwizzle128B);
+        if (elect_one()) {
+#pragma unroll
+          for (int ks = 0; ks < KEYS / 16; ++ks)                 // 16 keys: 8 columns of P, 2 KB of V
+            umma_bf16_ts(tm + KEYS, tm + ks * 8, bd + ks * (2048 >> 4), idesc_o, (j != 0 || ks != 0) ? 1u : 0u);
+          if (more) mma_s(gn);
+          else umma_commit(&s_full[w]);                          // bare: tells the warpgroup that its O is final
+          umma_commit(&kv_empty[g % NST]);
+        }
+        __syncwarp();
+        ++n_s;
+      }
+      started = chain;
+      owed = !chain;
+      base = next_base;
+    }
+  } else {
+    // ------------------------------------------------------------------ softmax warpgroups
+    setmaxnreg_inc<L::kRegsSoftmax>();
+    const int w = (warp - 4) >> 2;
+    const int quarter = warp & 3;                  // TMEM lane quarter of this warp
+    const uint32_t s_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + w * L::kColStride;
+    const uint32_t o_addr = s_addr + KEYS;
+    const uint64_t scale2 = pack2(p.scale_log2, p.scale_log2);
+    uint32_t n = 0;                                // s_full phases waited for
+    bool ok = true;
+    // the finished tile whose output is still in tensor memory
+    bool pend = false;
+    bf16* pend_dst = nullptr;                      // nullptr: the row is past the item's end
+    float pend_l = 1.f;
+    auto flush_output = [&]() {
+      const float inv = 1.0f / pend_l;
+      uint4* dst = reinterpret_cast<uint4*>(pend_dst);
+#pragma unroll 1
+      for (int c = 0; c < HD / 16; ++c) {
+        uint32_t o[16];
+        __syncwarp();
+        tmem_ld_32x16(o_addr + c * 16, o);
+        tmem_ld_wait_16<0>(o);
+        uint32_t pkd[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) pkd[i] = pack_bf16x2(__uint_as_float(o[2 * i]) * inv, __uint_as_float(o[2 * i + 1]) * inv);
+        if (dst != nullptr) {
+          dst[2 * c] = make_uint4(pkd[0], pkd[1], pkd[2], pkd[3]);
+          dst[2 * c + 1] = make_uint4(pkd[4], pkd[5], pkd[6], pkd[7]);
+        }
+      }
+      __syncwarp();
+      pend = false;
+    };
+
+    int cursor = 0;
+    uint32_t round = 0;
+    for (int unit = unit_at(0); unit < p.total_units && ok; unit = unit_at(++round)) {
+      const RrUnit u = decode(unit, cursor);
+      if (w >= u.n_q) {                             // no tile in this unit
+        if (pend) {
+          if (!warp_mbar_wait(&s_full[w], n & 1u, abort_flag)) { ok = false; break; }
+          ++n;
+          tc_fence_after_sync();
+          flush_output();
+          tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&p_ready[w]);       // the issuer may use s_full[w] again
+        }
+        continue;
+      }
+      float m_used = 0.f;
+      uint64_t l2[2] = {0, 0};                      // row sum, two packed accumulators
+      int left = u.S;                               // keys from this step on
+#pragma unroll 1
+      for (int j = 0; j < u.n_kv; ++j, left -= KEYS) {
+        if (!warp_mbar_wait(&s_full[w], n & 1u, abort_flag)) { ok = false; break; }
+        ++n;
+        tc_fence_after_sync();
+        if (__builtin_expect(pend, 0)) flush_output();       // the previous tile's P V is complete
+        uint32_t s[KEYS];
+        tmem_ld_32x32_at<0>(s_addr, s);
+        tmem_ld_32x32_at<32>(s_addr, s);
+        tmem_ld_32x16_at<64>(s_addr, s);
+        tmem_ld_wait_16<0>(s); tmem_ld_tie_16<16>(s); tmem_ld_tie_16<32>(s); tmem_ld_tie_16<48>(s); tmem_ld_tie_16<64>(s);
+        if (__builtin_expect(left < KEYS, 0)) {              // keys past the item's end
+#pragma unroll
+          for (int i = 0; i < KEYS; ++i) if (i >= left) s[i] = 0xff800000u;   // -inf
+        }
+        float mx;
+        {
+          float c0 = -INFINITY, c1 = -INFINITY, c2 = -INFINITY, c3 = -INFINITY;
+#pragma unroll
+          for (int i = 0; i < KEYS; i += 8) {
+            c0 = fmax3(c0, __uint_as_float(s[i]), __uint_as_float(s[i + 1]));
+            c1 = fmax3(c1, __uint_as_float(s[i + 2]), __uint_as_float(s[i + 3]));
+            c2 = fmax3(c2, __uint_as_float(s[i + 4]), __uint_as_float(s[i + 5]));
+            c3 = fmax3(c3, __uint_as_float(s[i + 6]), __uint_as_float(s[i + 7]));
+          }
+          mx = fmax3(fmaxf(c0, c1), c2, c3);
+        }
+        // the reference maximum moves only when the row maximum grew by more than the threshold (the first step: always)
+        const float m_old = m_used;
+        const bool moved = j == 0 || (mx - m_used) * p.scale_log2 > kRescaleThreshold;
+        m_used = moved ? mx : m_used;
+        const uint32_t rescale = __ballot_sync(0xffffffffu, moved && j != 0);
+        const float mb = m_used * p.scale_log2;
+        const uint64_t nmb2 = pack2(-mb, -mb);
+        const uint64_t l_old[2] = {l2[0], l2[1]};
+        l2[0] = l2[1] = 0;
+        uint32_t pk[KEYS / 2];
+#pragma unroll
+        for (int i = 0; i < KEYS / 2; ++i) {
+          const uint64_t t = ffma2(pack2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), scale2, nmb2);
+          float p0, p1;
+          if ((i * EAS_RR_POLY_OF_8) % 8 < EAS_RR_POLY_OF_8) {
+            exp2_poly_pair(t, p0, p1);
+          } else {
+            float t0, t1;
+            unpack2(t, t0, t1);
+            p0 = fast_ex2(t0);
+            p1 = fast_ex2(t1);
+          }
+          l2[i & 1] = fadd2(l2[i & 1], pack2(p0, p1));
+          pk[i] = pack_bf16x2(p0, p1);
+        }
+        if (__builtin_expect(rescale != 0u, 0)) {
+          // (the sum of this step is in l2 already and was taken against the new reference: the correction is applied to
+          // what was there before, kept in l_old)
+          const float corr = moved ? fast_ex2((m_old - m_used) * p.scale_log2) : 1.0f;
+          const uint64_t corr2 = pack2(corr, corr);
+          l2[0] = fadd2(fmul2(l_old[0], corr2), l2[0]);
+          l2[1] = fadd2(fmul2(l_old[1], corr2), l2[1]);
+#pragma unroll 1
+          for (int c = 0; c < HD / 8; ++c) {
+            uint32_t o[8];
+            asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=r"(o[0]), "=r"(o[1]), "=r"(o[2]), "=r"(o[3]), "=r"(o[4]), "=r"(o[5]), "=r"(o[6]), "=r"(o[7]) : "r"(o_addr + c * 8) : "memory");
+            asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(o[0]), "+r"(o[1]), "+r"(o[2]), "+r"(o[3]), "+r"(o[4]), "+r"(o[5]), "+r"(o[6]), "+r"(o[7])::"memory");
+#pragma unroll
+            for (int i = 0; i < 8; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * corr);
+            tmem_st_32x8_from(o_addr + c * 8, o);
+          }
+        } else {
+          l2[0] = fadd2(l_old[0], l2[0]);
+          l2[1] = fadd2(l_old[1], l2[1]);
+        }
+        // P row into S's columns: two bf16 per column of this thread's lane
+        __syncwarp();
+        tmem_st_32x32_from(s_addr, pk);
+        tmem_st_32x8_from(s_addr + 32, pk + 32);
+        tmem_st_wait();
+        tc_fence_before_sync();
+        __syncwarp();
+        mbar_arrive_if(&p_ready[w], lane == 0);
+      }
+      if (!ok) break;
+      pend = true;
+      float l0, l1, l3, l4;
+      unpack2(l2[0], l0, l1);
+      unpack2(l2[1], l3, l4);
+      pend_l = (l0 + l1) + (l3 + l4);
+      const int head = (u.r0 + w) / u.nt, qrow = ((u.r0 + w) - head * u.nt) * kTcTile + quarter * 32 + lane;
+      pend_dst = qrow < u.S ? p.out + static_cast<long long>(u.row0 + qrow) * p.ldo + head * HD : nullptr;
+    }
+    if (ok && pend) {
+      if (warp_mbar_wait(&s_full[w], n & 1u, abort_flag)) {
+        tc_fence_after_sync();
+        flush_output();
+      }
+    }
+  }
+
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after_sync();
+    tmem_dealloc(tmem_base, 512);
+  }
+  if (threadIdx.x == 0 && *abort_flag) atomicCAS(p.status, DEV_OK, DEV_ERR_WAIT_TIMEOUT);
+}
+
+}  // namespace eas

@@ -11,6 +11,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -18,6 +19,7 @@
 #include <vector>
 
 #include "attention_mma.cuh"
+#include "attention_rr.cuh"
 #include "attention_tc.cuh"
 #include "elementwise.cuh"
 #include "embed_gemm.cuh"
@@ -931,9 +933,9 @@ static eas_status launch_attention_mma(const bf16* qkv, bf16* out, const int32_t
   return fail(EAS_ERR_UNSUPPORTED, "head_dim %d", hd);
 }
 
-template <bool PT>
 static eas_status launch_attention_tc(const bf16* qkv, bf16* out, const int32_t* cu, int n_items, int H, int hd, int budget,
                                       cudaStream_t stream, uint32_t* status, bool reverse) {
+  constexpr bool PT = false;
   AttnTcParams ap{};
   const int d = H * hd;
   const int64_t T = cu[n_items];
@@ -970,7 +972,7 @@ static eas_status launch_attention_tc(const bf16* qkv, bf16* out, const int32_t*
   if (once.first()) {
     CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<64, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnTcSmem<64, PT>::kBytes));
     CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<80, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnTcSmem<80, PT>::kBytes));
-    if (AttnTcSmem<64, PT>::kDualHeadOk)
+    if constexpr (AttnTcSmem<64, PT>::kDualHeadOk)
       CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<64, PT, AttnTcSmem<64, PT>::kDualHeadOk>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnTcSmem<64, PT>::kBytes));
     once.settled();
   }
@@ -981,11 +983,118 @@ static eas_status launch_attention_tc(const bf16* qkv, bf16* out, const int32_t*
   return fail(EAS_ERR_UNSUPPORTED, "head_dim %d", hd);
 }
 
+// How attn_rr_kernel's work is cut into units: the query tiles of all items, longest item first, in units of kWg tiles up to
+// the tile `full_tiles` and of `small` tiles from there on.
+struct AttnPlan { int full_tiles = 1 << 30, small = 1; };
+// the units of an item of n tiles that follows `before` tiles: units of kWg tiles, then smaller ones
+static void attention_item_units(int n, int before, const AttnPlan& plan, int* full, int* rest) {
+  constexpr int kWg = AttnRrSmem<64>::kWg;
+  const int in_full = std::max(0, std::min(n, plan.full_tiles - before));
+  *full = in_full == n ? (n + kWg - 1) / kWg : in_full / kWg;
+  *rest = (std::max(0, n - *full * kWg) + plan.small - 1) / plan.small;
+}
+
+// Units of three tiles use an SM best but are coarse: one clip of 8192 tokens and 16 heads is 342 of them, 2.3 rounds on 148
+// SMs, and one of 1500 tokens and 20 heads is 80.  The plan takes the cut and the small unit with the shortest estimated
+// time over the CTAs, from the measured time of an 80-key step with one, two and three tiles (relative to three: 0.69, 0.82, 1)
+// and 1.5 steps per unit.  Past eight rounds the last one does not matter and everything is cut into threes.
+static AttnPlan attention_plan(const int32_t* cu, int n_items, int H, int budget) {
+  constexpr int kWg = AttnRrSmem<64>::kWg, kKeys = AttnRrSmem<64>::kKeys;
+  static const double step[kWg + 1] = {0.0, 0.69, 0.82, 1.0};
+  std::vector<int> len(n_items);
+  int64_t tiles = 0;
+  for (int i = 0; i < n_items; ++i) {
+    len[i] = cu[i + 1] - cu[i];
+    tiles += static_cast<int64_t>(H) * ((len[i] + kTcTile - 1) / kTcTile);
+  }
+  AttnPlan best;
+  if (tiles > static_cast<int64_t>(8) * kWg * budget) return best;
+  std::sort(len.begin(), len.end(), std::greater<int>());
+  std::vector<double> load(budget);
+  double best_time = 0.0;
+  auto consider = [&](int full_tiles, int small) {
+    std::fill(load.begin(), load.end(), 0.0);
+    int unit = 0, before = 0;
+    double time = 0.0;
+    for (int S : len) {
+      const int n = H * ((S + kTcTile - 1) / kTcTile);
+      int full, rest;
+      attention_item_units(n, before, {full_tiles, small}, &full, &rest);
+      const double steps = (S + kKeys - 1) / kKeys + 1.5;
+      for (int k = 0; k < full + rest; ++k, ++unit) {
+        const int t = k < full ? std::min(kWg, n - k * kWg) : std::min(small, n - full * kWg - (k - full) * small);
+        const int round = unit / budget, pos = unit - round * budget;
+        double& l = load[(round & 1) ? budget - 1 - pos : pos];
+        l += steps * step[t];
+        time = std::max(time, l);
+      }
+      before += n;
+    }
+    if (best_time == 0.0 || time < 0.999 * best_time) { best_time = time; best = {full_tiles, small}; }
+  };
+  consider(1 << 30, 1);
+  const int rounds = static_cast<int>(tiles / (static_cast<int64_t>(kWg) * budget));     // whole rounds of full units
+  for (int small = 1; small < kWg; ++small)
+    for (int q = std::max(0, 4 * (rounds - 2)); q <= 4 * (rounds + 1); ++q) consider(kWg * (q * budget / 4), small);
+  return best;
+}
+
+template <int HD>
+static eas_status launch_attention_rr(const bf16* qkv, bf16* out, const int32_t* cu, int n_items, int H, int budget,
+                                      cudaStream_t stream, uint32_t* status, bool reverse, const AttnPlan& plan) {
+  using L = AttnRrSmem<HD>;
+  AttnRrParams ap{};
+  const int d = H * HD;
+  const int64_t T = cu[n_items];
+  {
+    const uint64_t dims[2] = {static_cast<uint64_t>(3 * d), static_cast<uint64_t>(T)};
+    const uint64_t strides[1] = {static_cast<uint64_t>(3 * d) * 2};
+    const uint32_t box_q_lo[2] = {64, kTcTile}, box_q_hi[2] = {16, kTcTile}, box_k_lo[2] = {64, L::kKeys}, box_k_hi[2] = {16, L::kKeys};
+    EAS_TRY(make_tmap(&ap.map_q_lo, qkv, 2, dims, strides, box_q_lo, CU_TENSOR_MAP_SWIZZLE_128B));
+    EAS_TRY(make_tmap(&ap.map_k_lo, qkv, 2, dims, strides, box_k_lo, CU_TENSOR_MAP_SWIZZLE_128B));
+    if (L::HI) {
+      EAS_TRY(make_tmap(&ap.map_q_hi, qkv, 2, dims, strides, box_q_hi, CU_TENSOR_MAP_SWIZZLE_32B));
+      EAS_TRY(make_tmap(&ap.map_k_hi, qkv, 2, dims, strides, box_k_hi, CU_TENSOR_MAP_SWIZZLE_32B));
+    }
+  }
+  ap.out = out; ap.ldo = d; ap.d_model = d; ap.n_heads = H;
+  ap.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(HD)));
+  ap.n_items = n_items;
+  ap.status = status;
+  std::vector<int> order(n_items);      // longest items first (stable), so the tail of the static round-robin is short work
+  for (int i = 0; i < n_items; ++i) order[i] = reverse ? n_items - 1 - i : i;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return (cu[a + 1] - cu[a]) > (cu[b + 1] - cu[b]); });
+  int units = 0, before = 0;            // units and tiles of the items before
+  for (int k = 0; k < n_items; ++k) {
+    const int i = order[k];
+    ap.item_start[k] = cu[i];
+    ap.item_len[k] = cu[i + 1] - cu[i];
+    ap.unit_prefix[k] = units;
+    const int tiles = H * ((ap.item_len[k] + kTcTile - 1) / kTcTile);
+    int rest;
+    attention_item_units(tiles, before, plan, &ap.item_full[k], &rest);
+    units += ap.item_full[k] + rest;
+    before += tiles;
+  }
+  ap.small_tiles = plan.small;
+  ap.unit_prefix[n_items] = units;
+  ap.total_units = units;
+  if (units == 0) return EAS_OK;
+  static OncePerDevice once;
+  if (once.first()) {
+    CUDA_TRY(cudaFuncSetAttribute(attn_rr_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kBytes));
+    once.settled();
+  }
+  return launch_kernel(attn_rr_kernel<HD>, std::min(budget, units), L::kThreads, L::kBytes, stream, ap);
+}
+
 static eas_status launch_attention(const bf16* qkv, bf16* out, const int32_t* cu, int n_items, int H, int hd, int budget,
-                                   cudaStream_t stream, int impl, uint32_t* status, bool reverse = false) {
+                                   cudaStream_t stream, int impl, uint32_t* status, const AttnPlan& plan, bool reverse = false) {
   if (impl == 1) return launch_attention_mma(qkv, out, cu, n_items, H, hd, budget, stream);
-  if (impl == 2) return launch_attention_tc<false>(qkv, out, cu, n_items, H, hd, budget, stream, status, reverse);
-  return launch_attention_tc<true>(qkv, out, cu, n_items, H, hd, budget, stream, status, reverse);
+  if (impl == 2) return launch_attention_tc(qkv, out, cu, n_items, H, hd, budget, stream, status, reverse);
+  if (hd == 64) return launch_attention_rr<64>(qkv, out, cu, n_items, H, budget, stream, status, reverse, plan);
+  if (hd == 80) return launch_attention_rr<80>(qkv, out, cu, n_items, H, budget, stream, status, reverse, plan);
+  return fail(EAS_ERR_UNSUPPORTED, "head_dim %d", hd);
 }
 
 // ------------------------------------------------------------------------------------ the forward pass
@@ -1171,6 +1280,7 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
     EAS_TRY(mark(e, EAS_KC_NORM, stream));
     EAS_TRY(launch_fold_stats(fp, budget, stream)); ++launches;
   }
+  const AttnPlan attn_plan = attention_plan(cu, n, c.n_heads, budget);      // the same for every block
   auto fold_in = [&](GemmCall& g, const float* c0, const float* c1) {    // a GEMM on rows scaled by gamma only
     g.fold_stats = stats; g.fold_c0 = c0; g.fold_c1 = ln_kind == NORM_LN ? c1 : nullptr;
     g.fold_rms = ln_kind == NORM_RMS ? 1 : 0; g.fold_eps = c.norm_eps; g.fold_rows = T;
@@ -1195,7 +1305,7 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
       EAS_TRY(launch_gemm(g, budget, stream, status)); ++launches;
     }
     EAS_TRY(mark(e, EAS_KC_ATTENTION, stream));
-    EAS_TRY(launch_attention(qkv, obuf, cu, n, c.n_heads, e->hd, budget, stream, e->attn_impl, status, dir != 0)); ++launches;
+    EAS_TRY(launch_attention(qkv, obuf, cu, n, c.n_heads, e->hd, budget, stream, e->attn_impl, status, attn_plan, dir != 0)); ++launches;
     dir ^= 1;
     {
       GemmCall g;
@@ -1608,7 +1718,7 @@ extern "C" eas_status eas_kernel_attention(const void* qkv, void* out, const int
   int budget = 0;
   EAS_TRY(resolve_budget(sm_budget, &budget));
   return launch_attention(static_cast<const bf16*>(qkv), static_cast<bf16*>(out), cu, n_items, n_heads, head_dim, budget,
-                          static_cast<cudaStream_t>(stream), impl, status_dev);
+                          static_cast<cudaStream_t>(stream), impl, status_dev, attention_plan(cu, n_items, n_heads, budget));
 }
 
 #ifdef EAS_GEMM_PROFILE

@@ -196,6 +196,32 @@ def test_attention_block_diagonal(hd, H, lens, impl):
     assert torch.equal(out, out2)
 
 
+@pytest.mark.parametrize("hd", [64, 80])
+@pytest.mark.parametrize("H,lens", [(1, [79]), (1, [80, 81]), (5, [160, 161, 1]), (7, [129, 240, 400]), (2, [513, 128, 385])])
+def test_attention_units_at_key_tile_and_head_edges(hd, H, lens):
+    """Items at the edges of the 80-key steps, units of up to three query tiles that span one to three heads, and budgets
+    from one CTA (every unit in a row, warpgroups idle in some) to all (units of one tile): the oracle's values, and the same
+    bits whatever the units are."""
+    import paper_2609_31551_b200 as P
+    rng = np.random.Generator(np.random.PCG64(hd + H + sum(lens)))
+    T, d = sum(lens), H * hd
+    qkv = _bf16_exact(rng, (T, 3 * d))
+    qkv[:, : 2 * d] *= 1.5
+    qkv = S.round_to_bf16(qkv)
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    q = O._t(qkv)
+    ref = torch.cat([O.attention_one_item(q[a:b, :d].reshape(-1, H, hd), q[a:b, d:2 * d].reshape(-1, H, hd),
+                                          q[a:b, 2 * d:].reshape(-1, H, hd)) for a, b in zip(cu[:-1], cu[1:])])
+    first = None
+    for budget in (0, 1, 2, 3, 5, 11):
+        out, status = P.kernel_attention(_dev(qkv), cu, H, hd, sm_budget=budget)
+        torch.cuda.synchronize()
+        assert int(status[0]) == 0
+        first = out if first is None else first
+        assert torch.equal(out, first), budget
+    assert (first.double().cpu() - ref).abs().max() <= 2e-2      # as in test_attention_block_diagonal
+
+
 @pytest.mark.parametrize("H", [1, 2, 5, 16])
 def test_attention_dual_head_units(H):
     """head_dim 64, items with an odd number of 128-row query tiles: their last tiles of two adjacent heads share a
