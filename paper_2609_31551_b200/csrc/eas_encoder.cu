@@ -1097,6 +1097,39 @@ static eas_status launch_attention(const bf16* qkv, bf16* out, const int32_t* cu
   return fail(EAS_ERR_UNSUPPORTED, "head_dim %d", hd);
 }
 
+// Patch embedding: rows R of a patch block and column groups by estimated time (the result does not depend on them).
+// A unit gathers its k-blocks (G) and works off its column blocks (E: mostly the scattered fp32 stores; a later pass over K
+// adds to them), and units of a CTA overlap: G + E + (waves - 1) max(G, E), us.  Fitted to every (R, groups) forced over one
+// image to three 1344 x 1344 ones, one clip of 4 to 64 frames.  Kernel time, one 336 x 336 image (d 1024): 77 us as 5 units of
+// R = 128, 19 as 72 of R = 32; 8 images 72 -> 37; 32 images stay at R = 128, one group (74; 76 with R = 64); one 224 x 224 image
+// (d 256) 41 -> 18; a 16-frame clip 182 -> 117; three 1344 x 1344 images 154 -> 122 (R = 64).
+static eas_status launch_embed_gemm(EmbedGemmParams& gp, int budget, cudaStream_t stream) {
+  static OncePerDevice once;
+  if (once.first()) {
+    CUDA_TRY(cudaFuncSetAttribute(embed_gemm_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgSmemBytes));
+    CUDA_TRY(cudaFuncSetAttribute(embed_gemm_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgSmemBytes));
+    CUDA_TRY(cudaFuncSetAttribute(embed_gemm_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgSmemBytes));
+    once.settled();
+  }
+  const int k_blocks = gp.k_pad / 64, n_blocks = (gp.N + 255) / 256;
+  int rows = 128, groups = 1;
+  double best = 0.0;
+  const int passes = (k_blocks + kEgMaxResident - 1) / kEgMaxResident;
+  static const struct { int rows; double gather, block, again; } kShapes[] = {{128, 2.1, 13.0, 20.0}, {64, 1.9, 7.0, 8.0}, {32, 1.15, 6.0, 6.0}};
+  for (const auto& sh : kShapes)
+    for (int g = 1; g <= n_blocks; ++g) {
+      const int64_t units = static_cast<int64_t>((gp.n_patches + sh.rows - 1) / sh.rows) * g;
+      const double waves = static_cast<double>((units + budget - 1) / budget);
+      const double G = k_blocks * sh.gather, E = (n_blocks + g - 1) / g * (sh.block + (passes - 1) * sh.again);
+      const double cost = G + E + (waves - 1.0) * std::max(G, E);
+      if (best == 0.0 || cost < best) { best = cost; rows = sh.rows; groups = g; }
+    }
+  gp.col_groups = groups;
+  const int units = (gp.n_patches + rows - 1) / rows * groups;
+  void (*kern)(EmbedGemmParams) = rows == 128 ? embed_gemm_kernel<128> : rows == 64 ? embed_gemm_kernel<64> : embed_gemm_kernel<32>;
+  return launch_kernel(kern, std::min(budget, units), kEgThreads, kEgSmemBytes, stream, gp);
+}
+
 // ------------------------------------------------------------------------------------ the forward pass
 // The forward pass.  `workspace` / `workspace_bytes` override the fields of `in` (the entry points differ only in
 // where the scratch comes from).
@@ -1254,14 +1287,8 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
     gp.table = e->embed_table;
     gp.status = status;
     gp.items = items;
-    static OncePerDevice once;
-    if (once.first()) {
-      CUDA_TRY(cudaFuncSetAttribute(embed_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgSmemBytes));
-      once.settled();
-    }
-    const int tiles = static_cast<int>((pl.embed_rows + 127) / 128);     // a CTA owns whole blocks of 128 patches
     EAS_TRY(mark(e, EAS_KC_GEMM_EMBED, stream));
-    EAS_TRY(launch_kernel(embed_gemm_kernel, std::min(budget, tiles), kEgThreads, kEgSmemBytes, stream, gp));
+    EAS_TRY(launch_embed_gemm(gp, budget, stream));
     ++launches;
   }
   if (c.embed_norm) {

@@ -8,21 +8,27 @@
 // reads them through the same UMMA descriptors as any other A tile.  (TMA itself cannot fetch them: a run of a
 // 14-pixel patch row is 28 bytes long and starts on a 28-byte grid, neither a multiple of 16.)
 //
-// Gathering is the expensive part (small scattered loads), so it is done ONCE per patch: a CTA owns a block of 128
-// patches, keeps up to kEgMaxResident 64-wide k-blocks of their rows resident in shared memory and runs ALL column
-// blocks of the output against them while the weight tiles stream through a small TMA ring.  A patch vector longer
-// than the resident part is processed in passes over K: the first pass stores bias + position + partial sum, every
-// later pass adds its partial sum to the stored row (one fixed order, so the result is deterministic).
+// Gathering is the expensive part (small scattered loads): a CTA takes a block of R patches, keeps up to kEgMaxResident
+// 64-wide k-blocks of their rows resident in shared memory and runs a group of column blocks of the output against them
+// while the weight tiles stream through a small TMA ring.  With many patches R is 128 and the group is all columns, so every
+// patch is gathered once.  With few patches that leaves most SMs idle and one CTA's gather and column loop is the kernel's
+// time (38-76 us for one image): the columns are dealt to several CTAs, which gather the same patches again, and R shrinks
+// to 64 or 32 (the other rows of the 128-row UMMA tile are whatever lies in shared memory; their results are not stored), so
+// that a row has 4 or 8 gather threads.  The host picks both by estimated time.
+// A patch vector longer than the resident part is processed in passes over K: the first pass stores bias + position +
+// partial sum, every later pass adds its partial sum to the stored row.  The passes do not depend on R or the column groups,
+// so the result does not either.
 //
 //   warp 0        TMA producer of the weight tiles (256 rows x 64 columns per stage), lane 0
 //   warp 1        UMMA issuer (128 x 256 x 16, fp32 accumulators in TMEM, two accumulator buffers), lane 0
-//   warps 2..9    gather: two threads per patch row, each loads 16 pixel pairs of a k-block (4-byte loads; a pair
-//                 never straddles a run because patch edges are even) and stores four swizzled 16-byte chunks; the
-//                 loads of the next k-block are issued before the current one is stored
-//   warps 10..13  epilogue: tcgen05.ld -> + bias (+ position row) or + stored row -> fp32 rows of the residual stream,
-//                 scattered by the row map (CLS rows and item boundaries make output rows differ from patch rows)
+//   warps 2..9    gather: 256 / R threads per patch row, each loads pixel pairs of a k-block (4-byte loads; a pair never
+//                 straddles a run because patch edges are even) and stores swizzled 16-byte chunks; the loads of several
+//                 k-blocks are in flight
+//   warps 10..17  epilogue, two warps per TMEM lane quarter (half of the columns each): tcgen05.ld -> + bias (+ position row)
+//                 or + stored row -> fp32 rows of the residual stream, scattered by the row map (CLS rows and item boundaries
+//                 make output rows differ from patch rows)
 //
-// The grid is at most `sm_budget` CTAs, one per SM, walking the patch blocks blockIdx.x, + gridDim.x, ...; every output
+// The grid is at most `sm_budget` CTAs, one per SM, walking the units (patch block, column group) blockIdx.x, + gridDim.x, ...; every output
 // element is accumulated over K in one fixed order, so results do not depend on the budget.
 #pragma once
 #include "elementwise.cuh"
@@ -30,13 +36,14 @@
 
 namespace eas {
 
-constexpr int kEgThreads = 14 * 32;
+constexpr int kEgThreads = 18 * 32;
 constexpr int kEgGatherWarps = 8;
 constexpr int kEgMaxResident = 10;                      // k-blocks of the A rows kept in shared memory per pass, at most
 constexpr int kEgWStages = 2;
 constexpr int kEgABytes = 128 * 64 * 2;                 // 16 KB: 128 patch rows x 64 elements
 constexpr int kEgBBytes = 256 * 64 * 2;                 // 32 KB: 256 weight rows x 64 elements
-// shared memory: [resident A: R x 16 KB][weight ring: 2 x 32 KB][barriers]; R = 10 fills an SM's 227 KB
+// shared memory: [resident A: 10 x 16 KB, or 10 x R x 128 bytes][weight ring: 2 x 32 KB][barriers]: fills an SM's 227 KB at R = 128
+// (smaller R: the last slot's tile reads past the slots, into the ring: rows of no patch)
 constexpr int kEgSmemBytes = kEgMaxResident * kEgABytes + kEgWStages * kEgBBytes + 512 + 1024;   // + barriers + alignment slack
 static_assert(kEgSmemBytes <= 232448, "exceeds the shared memory of an SM");
 
@@ -52,6 +59,7 @@ struct EmbedGemmParams {
   int k, k_pad;            // patch elements C * pt * P * P, and the same padded to a multiple of 64
   int channels, patch, tpatch;
   int merge_order;         // 0: patches in raster order; 1: merge-group-major (the four patches of a 2x2 group adjacent)
+  int col_groups;          // the column blocks are dealt to this many units per patch block
   int pairs_ok;            // 1: patch edge, image widths and item offsets are even, so pixel pairs are 4-byte aligned
   const uint32_t* table;   // [k_pad / 2] where each pixel pair of the patch vector comes from (built once per encoder)
   uint32_t* status;
@@ -78,31 +86,36 @@ __global__ void embed_table_kernel(uint32_t* table, int k, int k_pad, int patch,
   }
 }
 
+template <int R>
 __global__ void __launch_bounds__(kEgThreads, 1) embed_gemm_kernel(const __grid_constant__ EmbedGemmParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw_eg[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_eg) + 1023) & ~uintptr_t(1023));
   const int k_blocks = p.k_pad / 64;
   const int resident = min(k_blocks, kEgMaxResident);
-  uint8_t* wring = smem + resident * kEgABytes;
+  constexpr int kSlot = R * 128;                       // R patch rows x 64 elements
+  static_assert(R == 32 || R == 64 || R == 128, "rows of a patch block");
+  uint8_t* wring = smem + kEgMaxResident * kSlot;
   uint64_t* bars = reinterpret_cast<uint64_t*>(wring + kEgWStages * kEgBBytes);
   uint64_t* a_full = bars;                             // [resident] the gather warps have written the slot
   uint64_t* a_free = bars + kEgMaxResident;            // [resident] the last UMMA that reads the slot has completed
   uint64_t* w_full = bars + 2 * kEgMaxResident;        // [kEgWStages]
   uint64_t* w_empty = w_full + kEgWStages;             // [kEgWStages]
   uint64_t* acc_full = w_empty + kEgWStages;           // [2]
-  uint64_t* acc_empty = acc_full + 2;                  // [2] 4 epilogue warps
+  uint64_t* acc_empty = acc_full + 2;                  // [2] 8 epilogue warps
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m_blocks = (p.n_patches + 127) / 128;
+  const int m_blocks = (p.n_patches + R - 1) / R;
   const int n_blocks = (p.N + 255) / 256;
+  const int n_units = m_blocks * p.col_groups;         // unit: patch block unit / col_groups, column group unit % col_groups
+  auto first_col = [&](int group) { return group * n_blocks / p.col_groups; };     // a group's column blocks, as even as possible
   const int passes = (k_blocks + resident - 1) / resident;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < resident; ++s) { mbar_init(&a_full[s], kEgGatherWarps); mbar_init(&a_free[s], 1); }
     for (int s = 0; s < kEgWStages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(&acc_full[a], 1); mbar_init(&acc_empty[a], 4); }
+    for (int a = 0; a < 2; ++a) { mbar_init(&acc_full[a], 1); mbar_init(&acc_empty[a], 8); }
     *abort_flag = 0;
     mbar_fence_init();
     tma_prefetch_desc(&p.tma_w);
@@ -131,9 +144,9 @@ __global__ void __launch_bounds__(kEgThreads, 1) embed_gemm_kernel(const __grid_
     if (lane == 0) {
       uint32_t it = 0;
       bool ok = true;
-      for (int mb = blockIdx.x; mb < m_blocks && ok; mb += gridDim.x)
+      for (int unit = blockIdx.x; unit < n_units && ok; unit += gridDim.x)
         for (int pass = 0; pass < passes && ok; ++pass)
-          for (int nb = 0; nb < n_blocks && ok; ++nb)
+          for (int nb = first_col(unit % p.col_groups); nb < first_col(unit % p.col_groups + 1) && ok; ++nb)
             for (int j = 0; j < pass_blocks(pass); ++j, ++it) {
               const int s = it % kEgWStages;
               if (it == kEgWStages) pdl_wait();      // the next wait needs the consumer, hence the earlier kernels
@@ -153,10 +166,11 @@ __global__ void __launch_bounds__(kEgThreads, 1) embed_gemm_kernel(const __grid_
       uint32_t it = 0, tcount = 0;                   // weight stages used, accumulators used
       uint32_t full_par = 0;                         // bit j: parity of slot j's next fill (slots are not all used in every pass)
       bool ok = true;
-      for (int mb = blockIdx.x; mb < m_blocks && ok; mb += gridDim.x)
+      for (int unit = blockIdx.x; unit < n_units && ok; unit += gridDim.x)
         for (int pass = 0; pass < passes && ok; ++pass) {
           const int nj = pass_blocks(pass);
-          for (int nb = 0; nb < n_blocks && ok; ++nb, ++tcount) {
+          const int nb0 = first_col(unit % p.col_groups), nb1 = first_col(unit % p.col_groups + 1);
+          for (int nb = nb0; nb < nb1 && ok; ++nb, ++tcount) {
             const uint32_t acc = tcount & 1u;
             if (!mbar_wait(&acc_empty[acc], ((tcount >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
             tc_fence_after_sync();
@@ -164,32 +178,34 @@ __global__ void __launch_bounds__(kEgThreads, 1) embed_gemm_kernel(const __grid_
             for (int j = 0; j < nj; ++j, ++it) {
               const int s = it % kEgWStages;
               // the first column block runs behind the gather; the others find every slot filled
-              if (nb == 0) {
+              if (nb == nb0) {
                 if (!mbar_wait(&a_full[j], (full_par >> j) & 1u, abort_flag)) { ok = false; break; }
                 full_par ^= 1u << j;
               }
               if (!mbar_wait(&w_full[s], (it / kEgWStages) & 1u, abort_flag)) { ok = false; break; }
               tc_fence_after_sync();
-              const uint64_t adesc = make_smem_desc(smem_u32(smem + j * kEgABytes), 16, 1024, kSwizzle128B);
+              const uint64_t adesc = make_smem_desc(smem_u32(smem + j * kSlot), 16, 1024, kSwizzle128B);
               const uint64_t bdesc = make_smem_desc(smem_u32(wring + s * kEgBBytes), 16, 1024, kSwizzle128B);
 #pragma unroll
               for (int k = 0; k < 4; ++k) umma_bf16_ss(tmem_d, adesc + 2 * k, bdesc + 2 * k, idesc, (j | k) != 0);
               umma_commit(&w_empty[s]);
-              if (nb == n_blocks - 1) umma_commit(&a_free[j]);   // the slot's last reader: the gather may refill it
+              if (nb == nb1 - 1) umma_commit(&a_free[j]);   // the slot's last reader: the gather may refill it
             }
             if (ok) umma_commit(&acc_full[acc]);
           }
         }
     }
   } else if (warp < 2 + kEgGatherWarps) {
-    // ------------------------------------------------------------------ gather: two threads per patch row
+    // ------------------------------------------------------------------ gather: kThreadsPerRow threads per patch row
+    constexpr int kThreadsPerRow = 32 * kEgGatherWarps / R, kChunks = 8 / kThreadsPerRow;   // 16-byte chunks per thread and k-block
+    constexpr int kDepth = R == 128 ? 3 : 6;        // k-blocks whose loads are in flight
     const int t = threadIdx.x - 64;                 // 0..255
-    const int row = t >> 1, half = t & 1;           // this thread writes 16-byte chunks 4 * half .. 4 * half + 3 of the row
+    const int row = t / kThreadsPerRow, sub = t % kThreadsPerRow;   // this thread writes chunks kChunks * sub ... of the row
     const int sw = row & 7;
     uint32_t used = 0, free_par = 0;                // bit j: slot j has been filled before; parity of its next hand-back
     bool ok = true;
-    for (int mb = blockIdx.x; mb < m_blocks && ok; mb += gridDim.x) {
-      const int m = mb * 128 + row;
+    for (int unit = blockIdx.x; unit < n_units && ok; unit += gridDim.x) {
+      const int m = unit / p.col_groups * R + row;
       // this patch: first pixel of its top-left corner in frame-in-patch 0 of channel 0, and the strides
       const bf16* base = p.data;
       int plane_stride = 0, frame_stride = 0;       // elements between channels, and between frames of a clip (an item
@@ -219,11 +235,11 @@ __global__ void __launch_bounds__(kEgThreads, 1) embed_gemm_kernel(const __grid_
         base = p.data + p.items.offset[item] + static_cast<long long>(tt) * p.tpatch * frame_stride +
                static_cast<long long>(r) * p.patch * W + c * p.patch;
       }
-      // the 16 pairs of this thread in k-block kb (registers only)
-      auto load_block = [&](int kb, uint32_t (&v)[16]) {
-        const uint4* tab4 = reinterpret_cast<const uint4*>(p.table + kb * 32 + half * 16);
+      // the pairs of this thread in k-block kb (registers only)
+      auto load_block = [&](int kb, uint32_t (&v)[4 * kChunks]) {
+        const uint4* tab4 = reinterpret_cast<const uint4*>(p.table + kb * 32 + sub * (4 * kChunks));
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < kChunks; ++q) {
           const uint4 e4 = __ldg(tab4 + q);
           const uint32_t e[4] = {e4.x, e4.y, e4.z, e4.w};
 #pragma unroll
@@ -242,7 +258,7 @@ __global__ void __launch_bounds__(kEgThreads, 1) embed_gemm_kernel(const __grid_
                 int px1 = px + 1, py1 = py, f1 = f, ch1 = ch;
                 if (px1 == p.patch) { px1 = 0; if (++py1 == p.patch) { py1 = 0; if (++f1 == p.tpatch) { f1 = 0; ++ch1; } } }
                 unsigned short hi = 0;
-                if (2 * (kb * 32 + half * 16 + q * 4 + j) + 1 < p.k)
+                if (2 * (kb * 32 + (sub * kChunks + q) * 4 + j) + 1 < p.k)
                   hi = *reinterpret_cast<const unsigned short*>(base + (f1 * frame_stride + ch1 * plane_stride + py1 * W + px1));
                 val = static_cast<uint32_t>(lo) | (static_cast<uint32_t>(hi) << 16);
               }
@@ -253,36 +269,42 @@ __global__ void __launch_bounds__(kEgThreads, 1) embed_gemm_kernel(const __grid_
       };
       for (int pass = 0; pass < passes && ok; ++pass) {
         const int nj = pass_blocks(pass), kb0 = pass_first(pass);
-        uint32_t cur[16], nxt[16];
-        load_block(kb0, cur);
-        for (int j = 0; j < nj; ++j) {
-          if (j + 1 < nj) load_block(kb0 + j + 1, nxt);     // in flight while this one is stored
-          // the slot's previous contents (an earlier pass or patch block) have been read by their last UMMA
-          if ((used >> j) & 1u) {
-            if (!warp_wait(&a_free[j], (free_par >> j) & 1u)) { ok = false; break; }
-            free_par ^= 1u << j;
+        uint32_t buf[kDepth][4 * kChunks];
+#pragma unroll
+        for (int d = 0; d < kDepth; ++d)
+          if (d < nj) load_block(kb0 + d, buf[d]);
+        for (int j0 = 0; j0 < nj && ok; j0 += kDepth) {
+#pragma unroll
+          for (int d = 0; d < kDepth; ++d) {
+            const int j = j0 + d;
+            if (j >= nj) break;
+            // the slot's previous contents (an earlier pass or unit) have been read by their last UMMA
+            if ((used >> j) & 1u) {
+              if (!warp_wait(&a_free[j], (free_par >> j) & 1u)) { ok = false; break; }
+              free_par ^= 1u << j;
+            }
+            used |= 1u << j;
+            uint8_t* srow = smem + j * kSlot + row * 128;
+#pragma unroll
+            for (int q = 0; q < kChunks; ++q)
+              *reinterpret_cast<uint4*>(srow + (((sub * kChunks + q) ^ sw) << 4)) = make_uint4(buf[d][4 * q], buf[d][4 * q + 1], buf[d][4 * q + 2], buf[d][4 * q + 3]);
+            fence_proxy_async_smem();               // generic-proxy stores -> visible to the tensor core's operand reads
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&a_full[j]);
+            if (j + kDepth < nj) load_block(kb0 + j + kDepth, buf[d]);
           }
-          used |= 1u << j;
-          uint8_t* srow = smem + j * kEgABytes + row * 128;
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<uint4*>(srow + (((half * 4 + q) ^ sw) << 4)) = make_uint4(cur[4 * q], cur[4 * q + 1], cur[4 * q + 2], cur[4 * q + 3]);
-          fence_proxy_async_smem();               // generic-proxy stores -> visible to the tensor core's operand reads
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&a_full[j]);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) cur[i] = nxt[i];
         }
       }
     }
   } else {
     // ------------------------------------------------------------------ epilogue
-    const int quarter = warp & 3;                 // TMEM lane quarter this warp may read (warps 10..13 -> 2, 3, 0, 1)
+    const int quarter = warp & 3;                 // TMEM lane quarter this warp may read (warps 10..17 -> 2, 3, 0, 1, 2, 3, 0, 1)
+    const int half = (warp - 2 - kEgGatherWarps) >> 2;       // which 128 of the 256 columns
     uint32_t tcount = 0;
     bool ok = true;
-    for (int mb = blockIdx.x; mb < m_blocks && ok; mb += gridDim.x) {
-      const int m = mb * 128 + quarter * 32 + lane;
-      bool row_ok = m < p.n_patches;
+    for (int unit = blockIdx.x; unit < n_units && ok; unit += gridDim.x) {
+      const int m = unit / p.col_groups * R + quarter * 32 + lane;
+      bool row_ok = quarter * 32 < R && m < p.n_patches;
       long long orow = 0;
       int posrow = 0;
       if (row_ok) {
@@ -292,12 +314,12 @@ __global__ void __launch_bounds__(kEgThreads, 1) embed_gemm_kernel(const __grid_
         if (p.pos != nullptr) posrow = p.pos_idx[m];
       }
       for (int pass = 0; pass < passes && ok; ++pass)
-        for (int nb = 0; nb < n_blocks && ok; ++nb, ++tcount) {
+        for (int nb = first_col(unit % p.col_groups); nb < first_col(unit % p.col_groups + 1) && ok; ++nb, ++tcount) {
           const uint32_t acc = tcount & 1u;
           if (!warp_wait(&acc_full[acc], (tcount >> 1) & 1u)) { ok = false; break; }
           tc_fence_after_sync();
 #pragma unroll 1
-          for (int c = 0; c < 8; ++c) {
+          for (int c = half * 4; c < half * 4 + 4 && quarter * 32 < R; ++c) {
             const int col0 = nb * 256 + c * 32;
             uint32_t raw[32];
             __syncwarp();

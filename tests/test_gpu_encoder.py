@@ -191,6 +191,25 @@ def test_fused_patch_embedding_alone(name):
         assert torch.equal(b, dev), budget
 
 
+@pytest.mark.parametrize("name", ["c0", "c1", "c2", "c3"])
+def test_fused_patch_embedding_same_bits_for_every_block_shape(name):
+    """The embedding's patch blocks (32, 64 or 128 rows) and column groups follow the micro-batch size and the budget: an
+    item's rows must have the same bits alone, packed, and at budgets that take every shape."""
+    cfg = S.get_config(name, n_layers=0)
+    w, enc = _make(cfg)
+    shapes = {"c0": [(1, 224, 224)] * 9, "c1": [(1, 336, 336), (1, 14, 28), (1, 336, 322)] * 2, "c2": [(1, 28, 28), (1, 560, 588), (1, 252, 364)],
+              "c3": [(2, 28, 56), (6, 224, 252), (2, 364, 364)]}[name]
+    items = S.make_items(cfg, shapes, seed=2070)
+    first, rows = None, [S.out_tokens_per_item(cfg, s) for s in shapes]
+    for budget in (0, 1, 2, 5, 9, 17, 40):
+        _, dev = G.run_gpu(enc, cfg, items, sm_budget=budget)
+        first = dev.clone() if first is None else first
+        assert torch.equal(dev, first), budget
+    for k in range(len(items)):
+        _, dev = G.run_gpu(enc, cfg, items[k:k + 1])
+        assert torch.equal(dev, first[sum(rows[:k]):sum(rows[:k + 1])]), k
+
+
 def test_fused_patch_embedding_with_odd_item_offsets():
     """Item offsets that are odd element counts break the 4-byte alignment of pixel pairs: the gather then loads
     single elements.  Same values, same accumulation order: the result must be the same bytes."""
