@@ -1224,7 +1224,6 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
   int launches = 0;
   e->last_status = status;
 
-  CUDA_TRY(cudaMemsetAsync(status, 0, 16, stream));
   e->tcls.clear();
   EAS_TRY(mark(e, EAS_KC_PREP, stream));
 

@@ -237,9 +237,13 @@ __global__ void __launch_bounds__(256) prep_kernel(const __grid_constant__ PrepP
   const int n = p.items.n_items;
   pdl_launch_dependents();
   pdl_wait();
-  if (p.cu_seqlens_dev != nullptr) {
-    for (int i = gtid; i <= n; i += gsz)
-      if (p.cu_seqlens_dev[i] != p.items.tok_start[i]) atomicCAS(p.status, DEV_OK, DEV_ERR_CU_SEQLENS_MISMATCH);
+  // The call's first kernel sets its status word (every later kernel only raises it): a memset in front of it would cut the
+  // chain of overlapped launches from one forward pass to the next.
+  if (blockIdx.x == 0) {
+    bool bad = false;
+    for (int i = threadIdx.x; i <= n; i += blockDim.x) bad = bad || p.cu_seqlens_dev[i] != p.items.tok_start[i];
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x == 0) *p.status = bad ? DEV_ERR_CU_SEQLENS_MISMATCH : DEV_OK;
   }
   if (p.family == 0 || p.family == 1) {
     for (int m = gtid; m < p.n_embed_rows; m += gsz) {
