@@ -25,6 +25,13 @@
 // 108 -> 87 us.  Not better: four warpgroups (64 keys at head_dim 64, 48 at 80), P in columns of its own with 64 or 48 keys
 // (the next scores early), no row maximum while a safe reference stands, other shares of the FMA-pipe exponentials.
 //
+// OWN_P, the variant for little work (the host's plan decides): two tiles at most, P in columns of its own
+// (2 x (80 + 40 + head_dim) columns) and two Q buffers a tile, so that the next scores are issued as soon as the row has
+// been read and are there when the exponentials are done: a step of a tile alone takes 1480 instead of 1750 cycles.  Same
+// 80-key steps in the same order: the same bits.  One item, kernel time: 577 tokens, 16 heads of 64: 12.1 -> 10.3 us; 1500 tokens, 20
+// heads of 64: 27.5 -> 25.7; 468 tokens, 16 heads of 80: 11.5 -> 10.1; 2304 tokens: 39.9 -> 37.6.  With three tiles' worth of work the
+// third tile is worth more (4 x 8192 tokens: 1275 us against 1500).
+//
 // The reference maximum only moves when the row maximum grows by more than 2^8 in the exponent; then the thread rescales
 // its O row in TMEM.  Final O / l is written as bf16.  A row's arithmetic does not depend on its unit.
 // Persistent: gridDim.x = sm_budget CTAs; the units are dealt to them in rounds of gridDim.x, alternate rounds in
@@ -55,21 +62,19 @@ struct AttnRrParams {
   uint32_t* status;
 };
 
-template <int HD> struct AttnRrCfg;
-template <> struct AttnRrCfg<64> { static constexpr int kStages = 6; };
-template <> struct AttnRrCfg<80> { static constexpr int kStages = 4; };
-
-template <int HD>
-struct AttnRrSmem : AttnRrCfg<HD> {
-  using C = AttnRrCfg<HD>;
-  static constexpr int kWg = 3, kKeys = 80;
-  static constexpr int kRegsLight = 104, kRegsSoftmax = 136, kRegsLaunch = 128;
+template <int HD, bool OWN_P>
+struct AttnRrSmem {
+  static constexpr int kKeys = 80;
+  static constexpr int kWg = OWN_P ? 2 : 3;                // softmax warpgroups, tiles per unit
+  static constexpr int kQBufs = OWN_P ? 2 : 1;             // Q tiles per warpgroup
+  static constexpr int kStages = HD == 64 ? 6 : 4;
+  static constexpr int kRegsLight = OWN_P ? 112 : 80, kRegsSoftmax = OWN_P ? 192 : 144, kRegsLaunch = OWN_P ? 168 : 128;
   static constexpr int HI = HD - 64;                       // 0 or 16 extra columns
   static constexpr int kThreads = 128 * (1 + kWg);
   static constexpr int kLoBytes = 128 * 128;               // Q tile: 128 rows x 64 bf16
   static constexpr int kHiBytes = 128 * HI * 2;            // 128 rows x 16 bf16, 32-byte swizzle
   static constexpr int kQBytes = kLoBytes + kHiBytes;
-  static constexpr int kAtomBytes = kKeys * 128;        // keys x 64 bf16
+  static constexpr int kAtomBytes = kKeys * 128;           // keys x 64 bf16
   static constexpr int kKHiBytes = kKeys * HI * 2;
   static constexpr int kKTxBytes = kAtomBytes + kKHiBytes;
   static constexpr int kKBytes = (kKTxBytes + 1023) / 1024 * 1024;
@@ -77,17 +82,18 @@ struct AttnRrSmem : AttnRrCfg<HD> {
   // zero past the last one) so that P V is ONE UMMA per 16 keys, N = 80 across the two swizzle atoms.
   static constexpr int kVBytes = kAtomBytes * (HI ? 2 : 1);
   static constexpr int kStageBytes = kKBytes + kVBytes;
-  static constexpr int kKvOff = kWg * kQBytes;
-  static constexpr int kBarOff = kKvOff + C::kStages * kStageBytes;
+  static constexpr int kKvOff = kWg * kQBufs * kQBytes;
+  static constexpr int kBarOff = kKvOff + kStages * kStageBytes;
   static constexpr int kBytes = kBarOff + 512 + 1024;      // barriers + alignment slack
   static_assert(kBytes <= 232448, "exceeds the shared memory of an SM");
   static_assert(kBytes > 116224, "a second CTA must not fit beside this one");
   static_assert(kQBytes % 1024 == 0 && kStageBytes % 1024 == 0 && kAtomBytes % 1024 == 0, "tiles start on swizzle-atom boundaries");
-  // TMEM columns of warpgroup w: S (and P in its first half) at w * kColStride, O behind it
-  static constexpr int kColStride = kKeys + HD;
+  // TMEM columns of warpgroup w from w * kColStride: S, (own) P: two bf16 per column, O.  P otherwise takes S's first columns.
+  static constexpr int kPCol = OWN_P ? kKeys : 0, kOCol = kKeys + (OWN_P ? kKeys / 2 : 0), kColStride = kOCol + HD;
   static_assert(kWg * kColStride <= 512, "tensor memory columns");
   static_assert(kKeys == 80, "five UMMA k-steps; a row of scores is 32 + 32 + 16 registers");
-  static_assert(C::kStages > kWg, "an issuer looks at most kWg ring positions ahead of the stage it holds");
+  static_assert(kWg <= 3, "the issuers are warps 1 .. kWg of the first warpgroup");
+  static_assert(kStages > kWg, "an issuer looks at most kWg ring positions ahead of the stage it holds");
   // setmaxnreg: the pool is the CTA's launch allocation
   static_assert(128 * kRegsLight + 128 * kWg * kRegsSoftmax <= kThreads * kRegsLaunch, "setmaxnreg budget exceeds the CTA's register allocation");
   static_assert(kThreads * kRegsLaunch <= 65536, "registers");
@@ -117,27 +123,30 @@ struct RrUnit {
   int r0, nt, n_q, head0, n_streams, S, n_kv, row0;
 };
 
-template <int HD>
-__global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(const __grid_constant__ AttnRrParams p) {
-  using L = AttnRrSmem<HD>;
+template <int HD, bool OWN_P>
+__global__ void __launch_bounds__(AttnRrSmem<HD, OWN_P>::kThreads, 1) attn_rr_kernel(const __grid_constant__ AttnRrParams p) {
+  using L = AttnRrSmem<HD, OWN_P>;
   constexpr int HI = L::HI, NST = L::kStages, NWG = L::kWg, KEYS = L::kKeys;
   extern __shared__ uint8_t smem_raw_attn[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_attn) + 1023) & ~uintptr_t(1023));
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::kBarOff);
-  uint64_t* q_full = bars;                 // [NWG]
-  uint64_t* s_full = q_full + NWG;         // [NWG] scores of a step complete (and everything issued before them)
+  uint64_t* q_full = bars;                 // [NWG][kQBufs]
+  uint64_t* s_full = q_full + 2 * NWG;     // [NWG] scores of a step complete (and everything issued before them)
   uint64_t* p_ready = s_full + NWG;        // [NWG] P stored, O rescaled if it had to be
-  uint64_t* k_full = p_ready + NWG;        // [NST]
+  uint64_t* s_free = p_ready + NWG;        // [NWG] own P: the warpgroup has read the scores out of tensor memory
+  uint64_t* pv_done = s_free + NWG;        // [NWG] own P: P V of a step complete
+  uint64_t* k_full = pv_done + NWG;        // [NST]
   uint64_t* v_full = k_full + NST;         // [NST]
   uint64_t* kv_empty = v_full + NST;       // [NST] every issuer hands every stage back
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(kv_empty + NST);
   volatile uint32_t* abort_flag = tmem_slot + 1;
-  static_assert((3 * NWG + 3 * NST) * 8 + 8 <= 512, "barrier area");
+  static_assert((6 * NWG + 3 * NST) * 8 + 8 <= 512, "barrier area");
 
   const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < NWG; ++i) { mbar_init(&q_full[i], 1); mbar_init(&s_full[i], 1); mbar_init(&p_ready[i], 4); }
+    for (int i = 0; i < NWG * L::kQBufs; ++i) mbar_init(&q_full[i], 1);
+    for (int i = 0; i < NWG; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_ready[i], 4); mbar_init(&s_free[i], 4); mbar_init(&pv_done[i], 1); }
     for (int i = 0; i < NST; ++i) { mbar_init(&k_full[i], 1); mbar_init(&v_full[i], 1); mbar_init(&kv_empty[i], NWG); }
     *abort_flag = 0;
     mbar_fence_init();
@@ -179,7 +188,7 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
     return u;
   };
   auto stream_of = [](const RrUnit& u, int w) { return (u.r0 + w) / u.nt - u.head0; };
-  auto q_tile = [&](int w) { return smem + w * L::kQBytes; };
+  auto q_tile = [&](int w, uint32_t b) { return smem + (w * L::kQBufs + b) * L::kQBytes; };
   auto k_tile = [&](int s) { return smem + L::kKvOff + s * L::kStageBytes; };
   auto v_tile = [&](int s) { return smem + L::kKvOff + s * L::kStageBytes + L::kKBytes; };
 
@@ -213,14 +222,16 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
   } else if (warp <= NWG) {
     // ------------------------------------------------------------------ UMMA issuers, one warp per warpgroup
     // The whole warp walks the steps (uniform control flow: see elect_one) and one elected lane issues.  A step: P V of
-    // this step and the scores of the next as soon as P is there.  What they need beside P (V, the next K, the next tile's
-    // Q) is waited for before P, so that the path from P to the next scores holds one wait.
+    // this step and the scores of the next as soon as P is there; what they need beside P (V, the next K, the next tile's
+    // Q) is waited for before P, so that the path from P to the next scores holds one wait.  With P in columns of its own the
+    // next scores come first, as soon as the warpgroup has read the previous ones.
     // An issuer sees every K/V stage of the CTA land, in order, also those of streams its tile has no part in (it hands those
     // back with a plain arrival), so that it never mistakes a barrier's phase for an earlier one.  Holding its own stage g it
     // waits for no stage past g + kWg < g + kStages (warpgroup w belongs at most to stream w, and at most kWg - 1 - w streams
     // follow its own), so the waits of the issuers have no cycle.
     setmaxnreg_dec<L::kRegsLight>();
     const int w = warp - 1;
+    constexpr uint32_t QB = L::kQBufs;
     constexpr uint32_t idesc_s = make_idesc_bf16(128, KEYS, 0, 0);         // S = Q K^T, both K-major
     constexpr uint32_t idesc_o = make_idesc_bf16(128, HD, 0, 1);           // O += P V, V is MN-major
     const uint32_t tm = tmem_base + w * L::kColStride;
@@ -233,17 +244,18 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
     RrUnit un{};
     if (unit_at(0) < p.total_units) un = decode(unit_at(0), cursor);
 
-    auto load_q = [&](const RrUnit& u) {
+    auto load_q = [&](const RrUnit& u) {         // into the buffer of the next tile to be waited for
       const int head = (u.r0 + w) / u.nt, y = u.row0 + ((u.r0 + w) - head * u.nt) * kTcTile;
       if (elect_one()) {
-        mbar_expect_tx(&q_full[w], L::kQBytes);
-        tma_load_2d(q_tile(w), &p.map_q_lo, &q_full[w], head * HD, y);
-        if (HI) tma_load_2d(q_tile(w) + L::kLoBytes, &p.map_q_hi, &q_full[w], head * HD + 64, y);
+        const uint32_t b = n_q % QB;
+        mbar_expect_tx(&q_full[w * QB + b], L::kQBytes);
+        tma_load_2d(q_tile(w, b), &p.map_q_lo, &q_full[w * QB + b], head * HD, y);
+        if (HI) tma_load_2d(q_tile(w, b) + L::kLoBytes, &p.map_q_hi, &q_full[w * QB + b], head * HD + 64, y);
       }
       __syncwarp();
     };
     auto q_landed = [&]() -> bool {
-      if (!warp_mbar_wait(&q_full[w], n_q & 1u, abort_flag)) return false;
+      if (!warp_mbar_wait(&q_full[w * QB + n_q % QB], (n_q / QB) & 1u, abort_flag)) return false;
       ++n_q;
       return true;
     };
@@ -256,9 +268,9 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
       }
       return true;
     };
-    // by the elected lane: scores against the K tile at ring position g
+    // by the elected lane: scores of the current tile (the last one waited for) against the K tile at ring position g
     auto mma_s = [&](uint32_t g) {
-      const uint32_t qa = smem_u32(q_tile(w)), ka = smem_u32(k_tile(g % NST));
+      const uint32_t qa = smem_u32(q_tile(w, (n_q - 1u) % QB)), ka = smem_u32(k_tile(g % NST));
       const uint64_t ad = make_smem_desc(qa, 16, 1024, kSwizzle128B);
       const uint64_t bd = make_smem_desc(ka, 16, 1024, kSwizzle128B);
 #pragma unroll
@@ -282,7 +294,7 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
         base = next_base;
         continue;
       }
-      const bool chain = has_next && w < un.n_q;      // the next unit's first scores follow this unit's last P V
+      const bool chain = has_next && w < un.n_q;      // the next unit's first scores follow this unit's last ones
       const uint32_t st = static_cast<uint32_t>(stream_of(u, w)), st_next = chain ? static_cast<uint32_t>(stream_of(un, w)) : 0u;
       if (!started) {
         if (owed) {                              // the warpgroup has seen the bare commit, so s_full may be used again
@@ -291,25 +303,36 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
         }
         load_q(u);
         if (!hand_back(base, base + st) || !q_landed() || !k_landed(base + st)) { ok = false; break; }
+        if (OWN_P && n_s > 0 && !warp_mbar_wait(&s_free[w], (n_s - 1u) & 1u, abort_flag)) { ok = false; break; }
         tc_fence_after_sync();
         if (elect_one()) mma_s(base + st);
         __syncwarp();
         ++n_s;
       }
+      // two Q buffers: the last scores against the other one are read (s_free was waited for before this tile's first)
+      if (OWN_P && chain) load_q(un);
       for (int j = 0; j < u.n_kv; ++j) {
         const bool last = j + 1 == u.n_kv;
         const bool more = !last || chain;
         const uint32_t row = base + static_cast<uint32_t>(j) * ns, g = row + st;
         const uint32_t gn = last ? next_base + st_next : g + ns;      // the K tile of the scores to come
-        if (last && chain) {
-          // the last scores are complete: the Q buffer is free
+        if (!OWN_P && last && chain) {
+          // one Q buffer: free when the last scores are complete
           if (!warp_mbar_wait(&s_full[w], (n_s - 1u) & 1u, abort_flag)) { ok = false; break; }
           load_q(un);
         }
         if (!hand_back(g + 1, row + ns)) { ok = false; break; }
-        if (!warp_mbar_wait(&v_full[g % NST], (g / NST) & 1u, abort_flag)) { ok = false; break; }
+        if (!OWN_P && !warp_mbar_wait(&v_full[g % NST], (g / NST) & 1u, abort_flag)) { ok = false; break; }
         if (more && (!hand_back(last ? next_base : row + ns, gn) || !k_landed(gn))) { ok = false; break; }
         if (last && chain && !q_landed()) { ok = false; break; }
+        if (OWN_P && more) {
+          if (!warp_mbar_wait(&s_free[w], (n_s - 1u) & 1u, abort_flag)) { ok = false; break; }
+          tc_fence_after_sync();
+          if (elect_one()) mma_s(gn);
+          __syncwarp();
+          ++n_s;
+        }
+        if (OWN_P && !warp_mbar_wait(&v_full[g % NST], (g / NST) & 1u, abort_flag)) { ok = false; break; }
         if (!warp_mbar_wait(&p_ready[w], n_p & 1u, abort_flag)) { ok = false; break; }
         ++n_p;
         tc_fence_after_sync();
@@ -318,27 +341,30 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
         if (elect_one()) {
 #pragma unroll
           for (int ks = 0; ks < KEYS / 16; ++ks)                 // 16 keys: 8 columns of P, 2 KB of V
-            umma_bf16_ts(tm + KEYS, tm + ks * 8, bd + ks * (2048 >> 4), idesc_o, (j != 0 || ks != 0) ? 1u : 0u);
-          if (more) mma_s(gn);
+            umma_bf16_ts(tm + L::kOCol, tm + L::kPCol + ks * 8, bd + ks * (2048 >> 4), idesc_o, (j != 0 || ks != 0) ? 1u : 0u);
+          if (OWN_P) umma_commit(&pv_done[w]);
+          else if (more) mma_s(gn);
           else umma_commit(&s_full[w]);                          // bare: tells the warpgroup that its O is final
           umma_commit(&kv_empty[g % NST]);
         }
         __syncwarp();
-        ++n_s;
+        if (!OWN_P) ++n_s;
       }
       started = chain;
-      owed = !chain;
+      owed = !OWN_P && !chain;
       base = next_base;
     }
+  } else if (warp < 4) {
+    setmaxnreg_dec<L::kRegsLight>();
   } else {
     // ------------------------------------------------------------------ softmax warpgroups
     setmaxnreg_inc<L::kRegsSoftmax>();
     const int w = (warp - 4) >> 2;
     const int quarter = warp & 3;                  // TMEM lane quarter of this warp
     const uint32_t s_addr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + w * L::kColStride;
-    const uint32_t o_addr = s_addr + KEYS;
+    const uint32_t p_addr = s_addr + L::kPCol, o_addr = s_addr + L::kOCol;
     const uint64_t scale2 = pack2(p.scale_log2, p.scale_log2);
-    uint32_t n = 0;                                // s_full phases waited for
+    uint32_t n = 0;                                // s_full phases waited for (own P: steps done)
     bool ok = true;
     // the finished tile whose output is still in tensor memory
     bool pend = false;
@@ -371,13 +397,15 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
       const RrUnit u = decode(unit, cursor);
       if (w >= u.n_q) {                             // no tile in this unit
         if (pend) {
-          if (!warp_mbar_wait(&s_full[w], n & 1u, abort_flag)) { ok = false; break; }
-          ++n;
+          if (!warp_mbar_wait(OWN_P ? &pv_done[w] : &s_full[w], (OWN_P ? n - 1u : n) & 1u, abort_flag)) { ok = false; break; }
           tc_fence_after_sync();
           flush_output();
-          tc_fence_before_sync();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&p_ready[w]);       // the issuer may use s_full[w] again
+          if (!OWN_P) {
+            ++n;
+            tc_fence_before_sync();
+            __syncwarp();
+            mbar_arrive_if(&p_ready[w], lane == 0);        // the issuer may use s_full[w] again
+          }
         }
         continue;
       }
@@ -389,12 +417,17 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
         if (!warp_mbar_wait(&s_full[w], n & 1u, abort_flag)) { ok = false; break; }
         ++n;
         tc_fence_after_sync();
-        if (__builtin_expect(pend, 0)) flush_output();       // the previous tile's P V is complete
+        if (!OWN_P && __builtin_expect(pend, 0)) flush_output();       // the previous tile's P V is complete
         uint32_t s[KEYS];
         tmem_ld_32x32_at<0>(s_addr, s);
         tmem_ld_32x32_at<32>(s_addr, s);
         tmem_ld_32x16_at<64>(s_addr, s);
         tmem_ld_wait_16<0>(s); tmem_ld_tie_16<16>(s); tmem_ld_tie_16<32>(s); tmem_ld_tie_16<48>(s); tmem_ld_tie_16<64>(s);
+        if (OWN_P) {
+          tc_fence_before_sync();
+          __syncwarp();
+          mbar_arrive_if(&s_free[w], lane == 0);
+        }
         if (__builtin_expect(left < KEYS, 0)) {              // keys past the item's end
 #pragma unroll
           for (int i = 0; i < KEYS; ++i) if (i >= left) s[i] = 0xff800000u;   // -inf
@@ -420,6 +453,7 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
         const uint64_t nmb2 = pack2(-mb, -mb);
         const uint64_t l_old[2] = {l2[0], l2[1]};
         l2[0] = l2[1] = 0;
+        const uint32_t pv_ok = OWN_P ? mbar_try_wait(&pv_done[w], n & 1u) : 1u;      // the previous step's, tested ahead
         uint32_t pk[KEYS / 2];
 #pragma unroll
         for (int i = 0; i < KEYS / 2; ++i) {
@@ -435,6 +469,12 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
           }
           l2[i & 1] = fadd2(l2[i & 1], pack2(p0, p1));
           pk[i] = pack_bf16x2(p0, p1);
+        }
+        if (OWN_P) {
+          // P goes where the previous step's was, and O may change: that step's P V has to be complete
+          if (n > 1u && !warp_mbar_wait_tested(pv_ok, &pv_done[w], n & 1u, abort_flag)) { ok = false; break; }
+          tc_fence_after_sync();
+          if (__builtin_expect(pend, 0)) flush_output();
         }
         if (__builtin_expect(rescale != 0u, 0)) {
           // (the sum of this step is in l2 already and was taken against the new reference: the correction is applied to
@@ -457,10 +497,10 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
           l2[0] = fadd2(l_old[0], l2[0]);
           l2[1] = fadd2(l_old[1], l2[1]);
         }
-        // P row into S's columns: two bf16 per column of this thread's lane
+        // P row: two bf16 per column of this thread's lane
         __syncwarp();
-        tmem_st_32x32_from(s_addr, pk);
-        tmem_st_32x8_from(s_addr + 32, pk + 32);
+        tmem_st_32x32_from(p_addr, pk);
+        tmem_st_32x8_from(p_addr + 32, pk + 32);
         tmem_st_wait();
         tc_fence_before_sync();
         __syncwarp();
@@ -476,7 +516,7 @@ __global__ void __launch_bounds__(AttnRrSmem<HD>::kThreads, 1) attn_rr_kernel(co
       pend_dst = qrow < u.S ? p.out + static_cast<long long>(u.row0 + qrow) * p.ldo + head * HD : nullptr;
     }
     if (ok && pend) {
-      if (warp_mbar_wait(&s_full[w], n & 1u, abort_flag)) {
+      if (warp_mbar_wait(OWN_P ? &pv_done[w] : &s_full[w], (OWN_P ? n - 1u : n) & 1u, abort_flag)) {
         tc_fence_after_sync();
         flush_output();
       }

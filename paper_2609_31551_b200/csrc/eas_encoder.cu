@@ -985,22 +985,25 @@ static eas_status launch_attention_tc(const bf16* qkv, bf16* out, const int32_t*
 
 // How attn_rr_kernel's work is cut into units: the query tiles of all items, longest item first, in units of kWg tiles up to
 // the tile `full_tiles` and of `small` tiles from there on.
-struct AttnPlan { int full_tiles = 1 << 30, small = 1; };
+// own_p: the kernel's variant for little work (kWg = 2).
+struct AttnPlan { int full_tiles = 1 << 30, small = 1; bool own_p = false; };
 // the units of an item of n tiles that follows `before` tiles: units of kWg tiles, then smaller ones
 static void attention_item_units(int n, int before, const AttnPlan& plan, int* full, int* rest) {
-  constexpr int kWg = AttnRrSmem<64>::kWg;
+  const int kWg = plan.own_p ? AttnRrSmem<64, true>::kWg : AttnRrSmem<64, false>::kWg;
   const int in_full = std::max(0, std::min(n, plan.full_tiles - before));
   *full = in_full == n ? (n + kWg - 1) / kWg : in_full / kWg;
   *rest = (std::max(0, n - *full * kWg) + plan.small - 1) / plan.small;
 }
 
 // Units of three tiles use an SM best but are coarse: one clip of 8192 tokens and 16 heads is 342 of them, 2.3 rounds on 148
-// SMs, and one of 1500 tokens and 20 heads is 80.  The plan takes the cut and the small unit with the shortest estimated
-// time over the CTAs, from the measured time of an 80-key step with one, two and three tiles (relative to three: 0.69, 0.82, 1)
-// and 1.5 steps per unit.  Past eight rounds the last one does not matter and everything is cut into threes.
+// SMs, and one of 1500 tokens and 20 heads is 80.  The plan takes the variant, the cut and the small unit with the shortest
+// estimated time over the CTAs, from the measured time of an 80-key step with one, two and three tiles (relative to three)
+// and 1.5 steps per unit.  Past eight rounds the last one matters little and everything is cut into threes (the search is host work: at
+// most 0.05 ms, once per forward pass).  (Rows do not
+// depend on the plan: it may follow the micro-batch and the budget.)
 static AttnPlan attention_plan(const int32_t* cu, int n_items, int H, int budget) {
-  constexpr int kWg = AttnRrSmem<64>::kWg, kKeys = AttnRrSmem<64>::kKeys;
-  static const double step[kWg + 1] = {0.0, 0.69, 0.82, 1.0};
+  constexpr int kKeys = AttnRrSmem<64, false>::kKeys;
+  static const double step[2][4] = {{0.0, 0.69, 0.82, 1.0}, {0.0, 0.58, 0.77, 0.0}};
   std::vector<int> len(n_items);
   int64_t tiles = 0;
   for (int i = 0; i < n_items; ++i) {
@@ -1008,41 +1011,46 @@ static AttnPlan attention_plan(const int32_t* cu, int n_items, int H, int budget
     tiles += static_cast<int64_t>(H) * ((len[i] + kTcTile - 1) / kTcTile);
   }
   AttnPlan best;
-  if (tiles > static_cast<int64_t>(8) * kWg * budget) return best;
+  if (tiles > static_cast<int64_t>(8 * 3) * budget) return best;
   std::sort(len.begin(), len.end(), std::greater<int>());
   std::vector<double> load(budget);
   double best_time = 0.0;
-  auto consider = [&](int full_tiles, int small) {
+  auto consider = [&](const AttnPlan& plan) {
+    const int kWg = plan.own_p ? 2 : 3;
     std::fill(load.begin(), load.end(), 0.0);
     int unit = 0, before = 0;
     double time = 0.0;
     for (int S : len) {
       const int n = H * ((S + kTcTile - 1) / kTcTile);
       int full, rest;
-      attention_item_units(n, before, {full_tiles, small}, &full, &rest);
+      attention_item_units(n, before, plan, &full, &rest);
       const double steps = (S + kKeys - 1) / kKeys + 1.5;
       for (int k = 0; k < full + rest; ++k, ++unit) {
-        const int t = k < full ? std::min(kWg, n - k * kWg) : std::min(small, n - full * kWg - (k - full) * small);
+        const int t = k < full ? std::min(kWg, n - k * kWg) : std::min(plan.small, n - full * kWg - (k - full) * plan.small);
         const int round = unit / budget, pos = unit - round * budget;
         double& l = load[(round & 1) ? budget - 1 - pos : pos];
-        l += steps * step[t];
+        l += steps * step[plan.own_p][t];
         time = std::max(time, l);
       }
       before += n;
     }
-    if (best_time == 0.0 || time < 0.999 * best_time) { best_time = time; best = {full_tiles, small}; }
+    if (best_time == 0.0 || time < 0.999 * best_time) { best_time = time; best = plan; }
   };
-  consider(1 << 30, 1);
-  const int rounds = static_cast<int>(tiles / (static_cast<int64_t>(kWg) * budget));     // whole rounds of full units
-  for (int small = 1; small < kWg; ++small)
-    for (int q = std::max(0, 4 * (rounds - 2)); q <= 4 * (rounds + 1); ++q) consider(kWg * (q * budget / 4), small);
+  consider(AttnPlan{});
+  for (int own = 0; own < (tiles <= static_cast<int64_t>(4) * budget ? 2 : 1); ++own) {
+    const int kWg = own ? 2 : 3;
+    if (own) consider({1 << 30, 1, true});
+    const int rounds = static_cast<int>(tiles / (static_cast<int64_t>(kWg) * budget));     // whole rounds of full units
+    for (int small = 1; small < kWg; ++small)
+      for (int q = std::max(0, 4 * (rounds - 1)); q <= 4 * (rounds + 1); q += rounds > 2 ? 2 : 1) consider({kWg * (q * budget / 4), small, own != 0});
+  }
   return best;
 }
 
-template <int HD>
+template <int HD, bool OWN_P>
 static eas_status launch_attention_rr(const bf16* qkv, bf16* out, const int32_t* cu, int n_items, int H, int budget,
                                       cudaStream_t stream, uint32_t* status, bool reverse, const AttnPlan& plan) {
-  using L = AttnRrSmem<HD>;
+  using L = AttnRrSmem<HD, OWN_P>;
   AttnRrParams ap{};
   const int d = H * HD;
   const int64_t T = cu[n_items];
@@ -1082,18 +1090,19 @@ static eas_status launch_attention_rr(const bf16* qkv, bf16* out, const int32_t*
   if (units == 0) return EAS_OK;
   static OncePerDevice once;
   if (once.first()) {
-    CUDA_TRY(cudaFuncSetAttribute(attn_rr_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kBytes));
+    CUDA_TRY(cudaFuncSetAttribute(attn_rr_kernel<HD, OWN_P>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kBytes));
     once.settled();
   }
-  return launch_kernel(attn_rr_kernel<HD>, std::min(budget, units), L::kThreads, L::kBytes, stream, ap);
+  return launch_kernel(attn_rr_kernel<HD, OWN_P>, std::min(budget, units), L::kThreads, L::kBytes, stream, ap);
 }
 
 static eas_status launch_attention(const bf16* qkv, bf16* out, const int32_t* cu, int n_items, int H, int hd, int budget,
                                    cudaStream_t stream, int impl, uint32_t* status, const AttnPlan& plan, bool reverse = false) {
   if (impl == 1) return launch_attention_mma(qkv, out, cu, n_items, H, hd, budget, stream);
   if (impl == 2) return launch_attention_tc(qkv, out, cu, n_items, H, hd, budget, stream, status, reverse);
-  if (hd == 64) return launch_attention_rr<64>(qkv, out, cu, n_items, H, budget, stream, status, reverse, plan);
-  if (hd == 80) return launch_attention_rr<80>(qkv, out, cu, n_items, H, budget, stream, status, reverse, plan);
+  auto launch = plan.own_p ? (hd == 64 ? launch_attention_rr<64, true> : launch_attention_rr<80, true>)
+                           : (hd == 64 ? launch_attention_rr<64, false> : launch_attention_rr<80, false>);
+  if (hd == 64 || hd == 80) return launch(qkv, out, cu, n_items, H, budget, stream, status, reverse, plan);
   return fail(EAS_ERR_UNSUPPORTED, "head_dim %d", hd);
 }
 
