@@ -23,6 +23,7 @@ struct AttnParams {
   int item_start[kMaxItems];     // first token row of the item (in schedule order)
   int item_len[kMaxItems];
   int unit_prefix[kMaxItems + 1];  // units before item i (schedule order: longest items first)
+  int early_launch;       // see pdl_launch_dependents
 };
 
 __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc, bool valid) {
@@ -61,7 +62,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_mma_kernel(const __grid_
   bf16* sV = sK + 2 * kAttnBKV * LDS;      // [2][64][LDS]
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  pdl_launch_dependents();
+  if (p.early_launch) pdl_launch_dependents();
   pdl_wait();
 
   for (int unit = blockIdx.x; unit < p.total_units; unit += gridDim.x) {

@@ -60,6 +60,7 @@ struct AttnRrParams {
   int item_full[128];
   int small_tiles;
   uint32_t* status;
+  int early_launch;       // see pdl_launch_dependents
 };
 
 template <int HD, bool OWN_P>
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(AttnRrSmem<HD, OWN_P>::kThreads, 1) attn_rr_ke
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_launch_dependents();
+  if (p.early_launch) pdl_launch_dependents();
   pdl_wait();
 
   // this CTA's unit of a round; increasing in `round`

@@ -47,6 +47,7 @@ struct AttnTcParams {
   int item_len[128];
   int unit_prefix[129];
   uint32_t* status;
+  int early_launch;       // see pdl_launch_dependents
 };
 
 // PT: the probabilities P live in tensor memory (the A operand of P V is read from there); otherwise they are
@@ -326,7 +327,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_launch_dependents();
+  if (p.early_launch) pdl_launch_dependents();
   pdl_wait();
 
   // this CTA's unit of a round; increasing in `round`

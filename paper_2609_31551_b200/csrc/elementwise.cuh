@@ -47,6 +47,7 @@ struct NormParams {
   long long part_stride; // elements between consecutive partial matrices
   int n_part;
   float* x_rw;
+  int early_launch;       // see pdl_launch_dependents
 };
 
 // One warp per row, the row held in registers (NV float4 per lane), two-pass statistics in fp32.
@@ -69,7 +70,7 @@ __global__ void __launch_bounds__(512, 1) norm_kernel(const NormParams p) {
     }
   }
   const float inv_d = 1.0f / static_cast<float>(p.d);
-  pdl_launch_dependents();
+  if (p.early_launch) pdl_launch_dependents();
   pdl_wait();
   // The forward pass alternates the direction in which consecutive kernels walk the token rows: a kernel starts with
   // the rows its producer wrote last, which are the ones still in L2.  (Rows are independent: the order does not change
@@ -144,6 +145,7 @@ struct FoldStatsParams {
   float2* stats;         // [d / 128][rows]
   const bf16* gamma;     // [d]
   int rows, d;
+  int early_launch;       // see pdl_launch_dependents
 };
 template <int NV>
 __global__ void __launch_bounds__(512, 1) fold_stats_kernel(const FoldStatsParams p) {
@@ -155,7 +157,7 @@ __global__ void __launch_bounds__(512, 1) fold_stats_kernel(const FoldStatsParam
     const uint2 gv = __ldg(reinterpret_cast<const uint2*>(p.gamma + i * 128 + lane * 4));
     g[i] = make_float4(bf16_lo(gv.x), bf16_hi(gv.x), bf16_lo(gv.y), bf16_hi(gv.y));
   }
-  pdl_launch_dependents();
+  if (p.early_launch) pdl_launch_dependents();
   pdl_wait();
   for (int row = blockIdx.x * warps_per_cta + warp; row < p.rows; row += gridDim.x * warps_per_cta) {
     const float4* xr = reinterpret_cast<const float4*>(p.x + static_cast<long long>(row) * p.d);
@@ -229,13 +231,14 @@ struct PrepParams {
   int* conv1_row_map;     // audio: [padded frames] -> padded h1 row or -1
   int n_conv1_rows;
   uint32_t* status;
+  int early_launch;       // see pdl_launch_dependents
 };
 
 __global__ void __launch_bounds__(256) prep_kernel(const __grid_constant__ PrepParams p) {
   const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
   const int gsz = gridDim.x * blockDim.x;
   const int n = p.items.n_items;
-  pdl_launch_dependents();
+  if (p.early_launch) pdl_launch_dependents();
   pdl_wait();
   // The call's first kernel sets its status word (every later kernel only raises it): a memset in front of it would cut the
   // chain of overlapped launches from one forward pass to the next.
@@ -322,12 +325,13 @@ struct AudioStageParams {
   bf16* h1_pad;        // [padded rows, d]
   int n_mel, d_model, padded_rows;
   ItemTable items;     // aux_start = padded-row prefix
+  int early_launch;       // see pdl_launch_dependents
 };
 
 __global__ void __launch_bounds__(512, 1) audio_stage_kernel(const __grid_constant__ AudioStageParams p) {
   const long long total = static_cast<long long>(p.padded_rows) * p.n_mel;
   const long long gsz = static_cast<long long>(gridDim.x) * blockDim.x;
-  pdl_launch_dependents();
+  if (p.early_launch) pdl_launch_dependents();
   pdl_wait();
   for (long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; idx < total; idx += gsz) {
     const int m = static_cast<int>(idx / p.n_mel);

@@ -64,6 +64,7 @@ struct EmbedGemmParams {
   const uint32_t* table;   // [k_pad / 2] where each pixel pair of the patch vector comes from (built once per encoder)
   uint32_t* status;
   ItemTable items;         // aux_start = patch-row prefix per item
+  int early_launch;       // see pdl_launch_dependents
 };
 
 // Table entry of a pixel pair (elements k, k + 1 of the patch vector): channel << 24 | frame-in-patch << 16 | py << 8 | px.
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(kEgThreads, 1) embed_gemm_kernel(const __grid_
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_launch_dependents();
+  if (p.early_launch) pdl_launch_dependents();
   if (warp != 0) pdl_wait();     // the weights are constant: their loads need not wait for the stream's earlier work
 
   // a whole warp waits on a barrier: lane 0 polls, the outcome is the same for all lanes (so the warp leaves a loop together)

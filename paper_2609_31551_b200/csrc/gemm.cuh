@@ -114,6 +114,7 @@ struct alignas(64) GemmParams {
   bf16* fold_xb;              // producer: bf16(gamma .* updated rows), [*, ldo]
   const bf16* fold_gamma;     // producer: [N], the gamma of the normalisation the rows go through next
   uint32_t* status;       // device status word
+  int early_launch;       // see pdl_launch_dependents
 };
 
 #ifdef EAS_GEMM_PROFILE
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   if (threadIdx.x == 0) GEMM_TL(1);
-  pdl_launch_dependents();   // the next kernel may set itself up while this one runs
+  if (p.early_launch) pdl_launch_dependents();   // the next kernel may set itself up while this one runs
   // everything before this kernel in the stream is complete and visible; the W producer of a GEMM on constant
   // weights goes ahead and fills the ring's W halves meanwhile (the stages complete once A has arrived too)
   if (!(p.w_const && warp == kProducerBWarp)) pdl_wait();

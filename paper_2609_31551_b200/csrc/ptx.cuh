@@ -97,8 +97,10 @@ __device__ __forceinline__ bool elect_one() {
   return pred != 0u;
 }
 
-// Programmatic dependent launch: a kernel launched with the stream-serialization attribute may start while its
-// predecessor drains; it must not touch the predecessor's results before pdl_wait().  Both are no-ops otherwise.
+// Programmatic dependent launch: a kernel launched with the stream-serialization attribute may start before its predecessor
+// is complete; it must not touch the predecessor's results before pdl_wait().  It may start once every CTA of the predecessor
+// has called pdl_launch_dependents() or has exited.  Kernels call it at their start when the call owns the whole device
+// (Params::early_launch); on a share of the SMs they do not, so that a successor's CTAs never hold SMs beside theirs.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
