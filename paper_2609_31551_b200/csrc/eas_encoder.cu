@@ -722,14 +722,16 @@ struct GemmCall {
 //     base + waves * (kb * per_kb + per_wave)      kb: 64-wide k-blocks of a work item,
 // where a last wave that fills a fraction f of the slots counts `partial` + (1 - partial) * f (fewer SMs share the path to L2).
 // Fitted to 480 measurements on B200: every shape forced over the encoder's GEMMs, 100 <= M <= 18464 tokens, d 256, 1024 and
-// 1280, on 37, 74, 111 and 148 SMs.  The choice is on average 0.2 % and at most 6 % slower than the best shape; without the
+// 1280, on 37, 74, 111 and 148 SMs.  The wide
+// shape's figures also follow 0.25 s runs back to back at the power cap, where it is the best one for K >= 4096 (M = 4096, N = K = 8192
+// on 134 SMs: 430 us, pairs 446).  The choice is on average 0.2 % and at most 6 % slower than the best shape; without the
 // narrow shapes it was 10 % on average: M = 577 on 148 SMs (N, K): (1024, 4096) 25.3 us as 256x256, 15.1 as 128x64; (1024, 1024)
 // 11.3, 6.4; (3072, 1024) 9.9, 7.5 as 128x128; M = 1500 (1280, 5120) 30.8, 22.5 as 128x128; from a few full waves of pair
 // tiles on those win (M = 18464 (4096, 1024): 115 us, single CTAs 138).
 template <typename Usable>
 static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bool plain, Usable usable) {
   struct Cost { int tile; double base, per_kb, per_wave, partial; };    // us
-  static const Cost costs[] = {{TILE_SINGLE, 5.5, 0.406, 0.04, 0.80}, {TILE_PAIR, 6.4, 0.336, 0.14, 0.85}, {TILE_WIDE, 5.5, 0.661, 4.5, 0.84},
+  static const Cost costs[] = {{TILE_SINGLE, 5.5, 0.406, 0.04, 0.80}, {TILE_PAIR, 6.4, 0.336, 0.14, 0.85}, {TILE_WIDE, 5.5, 0.65, 2.0, 0.84},
                                {TILE_N128, 4.1, 0.241, 0.45, 0.94}, {TILE_N64, 3.4, 0.174, 0.22, 1.0}};
   int tile = TILE_SINGLE;
   double best = 0.0;
