@@ -12,18 +12,21 @@
 //   warps 4..15  three softmax warpgroups
 //
 // What bounds it, and why three tiles: a tile's chain (scores -> row maximum -> exponentials -> P to tensor memory -> P V and
-// the next scores -> back) takes 1750 cycles a step of 80 keys when a tile is alone, of which the exponentials need 480 (a
-// quarter of them on the FMA pipe) and the tensor pipe 320-400: mostly latency, so what counts is the number of tiles in
-// flight.  Three take 2450 cycles a step together; two with 128 (112) keys a step and P in columns of its own, the former
+// the next scores -> back) takes 1750 cycles a step of 80 keys when a tile is alone, of which the exponentials need 640 and the
+// tensor pipe 320-400: mostly latency, so what counts is the number of tiles in flight.  Three take 2450 cycles a step
+// together (the special-function unit 1920 of them); two with 128 (112) keys a step and P in columns of its own, the former
 // kernel, 3100 (2780).  Tensor memory holds three because P takes S's own columns (dead once the row is in registers):
 // 3 x (80 + head_dim) columns.  The scores of a tile's next step then have to wait for its P V, but the other warpgroups'
 // exponentials fill that time; UMMAs complete in order, so "scores ready" also says that the warpgroup's previous P V is
 // complete, and a step has one wait.  Each warpgroup has an issuer of its own: one issuer for all (about 900 cycles of waits,
 // issues and commits a step) was what the warpgroups waited for (1.37 times the time).
-// Measured, same session, former kernel -> this one: 4 x 8192 tokens, 16 heads of 64: 1493 -> 1275 us; 2 x 8192, heads of 80:
-// 784 -> 735 us; 32768, heads of 80: 6.2 -> 5.7 ms; ragged 256 ... 4900, heads of 80: 316 -> 272 us; 32 x 577, heads of 64:
-// 108 -> 87 us.  Not better: four warpgroups (64 keys at head_dim 64, 48 at 80), P in columns of its own with 64 or 48 keys
-// (the next scores early), no row maximum while a safe reference stands, other shares of the FMA-pipe exponentials.
+// Measured, same session, former kernel -> this one: 4 x 8192 tokens, 16 heads of 64: 1493 -> 1265 us; 2 x 8192, heads of 80:
+// 803 -> 735 us; ragged 256 ... 4900, heads of 80: 338 -> 272 us; 32 x 577, heads of 64: 106 -> 89 us.
+// In forward passes the board sits at its power cap, where instructions cost time even if their pipe has room: taking a
+// quarter of the exponentials to the FMA pipe (a cubic), which is neutral in short runs, is 2-3 % slower in 0.3 s runs
+// (32768 tokens, heads of 80: 6.03 ms without, 6.22 with), so all of them are on the special-function unit.
+// Not better: four warpgroups (64 keys at head_dim 64, 48 at 80), P in columns of its own with 64 or 48 keys and three tiles,
+// no row maximum while the standing reference is safe.
 //
 // OWN_P, the variant for little work (the host's plan decides): two tiles at most, P in columns of its own
 // (2 x (80 + 40 + head_dim) columns) and two Q buffers a tile, so that the next scores are issued as soon as the row has
@@ -38,10 +41,12 @@
 // opposite directions (the host sorts the units by decreasing cost: a fixed direction would hand CTA 0 the costliest
 // unit of every round).
 #pragma once
-#include "attention_tc.cuh"
 #include "ptx.cuh"
 
 namespace eas {
+
+constexpr int kTcTile = 128;            // query rows per tile
+constexpr float kRescaleThreshold = 8.0f;
 
 struct AttnRrParams {
   CUtensorMap map_q_lo;   // qkv [T, 3d], box {64 columns, 128 rows}, 128-byte swizzle
@@ -99,10 +104,6 @@ struct AttnRrSmem {
   static_assert(128 * kRegsLight + 128 * kWg * kRegsSoftmax <= kThreads * kRegsLaunch, "setmaxnreg budget exceeds the CTA's register allocation");
   static_assert(kThreads * kRegsLaunch <= 65536, "registers");
 };
-
-#ifndef EAS_RR_POLY_OF_8
-#define EAS_RR_POLY_OF_8 2      // of every 8 pairs of probabilities, this many take the polynomial path
-#endif
 
 // Wait for this thread's tensor-memory loads, tied to registers they fill so that no use can move ahead of it.
 template <int OFF, int N>
@@ -460,14 +461,9 @@ __global__ void __launch_bounds__(AttnRrSmem<HD, OWN_P>::kThreads, 1) attn_rr_ke
         for (int i = 0; i < KEYS / 2; ++i) {
           const uint64_t t = ffma2(pack2(__uint_as_float(s[2 * i]), __uint_as_float(s[2 * i + 1])), scale2, nmb2);
           float p0, p1;
-          if ((i * EAS_RR_POLY_OF_8) % 8 < EAS_RR_POLY_OF_8) {
-            exp2_poly_pair(t, p0, p1);
-          } else {
-            float t0, t1;
-            unpack2(t, t0, t1);
-            p0 = fast_ex2(t0);
-            p1 = fast_ex2(t1);
-          }
+          unpack2(t, p0, p1);
+          p0 = fast_ex2(p0);
+          p1 = fast_ex2(p1);
           l2[i & 1] = fadd2(l2[i & 1], pack2(p0, p1));
           pk[i] = pack_bf16x2(p0, p1);
         }

@@ -889,14 +889,11 @@ static eas_status launch_norm(int kind, bool out_fp32, const NormParams& p, int 
   return fail(EAS_ERR_INVALID_ARG, "unknown norm kind %d", kind);
 }
 
-// schedule order: longest items first (stable), so the tail of the static round-robin is short work
-// dual_head: the tcgen05 kernel's unit order for head_dim 64 (see decode_unit): per item H x (full pairs of query
-// tiles), then one unit per two heads for an odd last tile.
-// reverse: items of equal length are taken last to first (the producer of qkv wrote the last rows most recently: L2).
+// schedule order of the cross-check kernels: longest items first (stable), so the tail of the static round-robin is short work
 static void attention_schedule(const int32_t* cu, int n_items, int rows_per_unit, int H, int* item_start, int* item_len,
-                               int* unit_prefix, int* total_units, bool dual_head = false, bool reverse = false) {
+                               int* unit_prefix, int* total_units) {
   std::vector<int> order(n_items);
-  for (int i = 0; i < n_items; ++i) order[i] = reverse ? n_items - 1 - i : i;
+  for (int i = 0; i < n_items; ++i) order[i] = i;
   std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return (cu[a + 1] - cu[a]) > (cu[b + 1] - cu[b]); });
   int units = 0;
   for (int k = 0; k < n_items; ++k) {
@@ -904,12 +901,7 @@ static void attention_schedule(const int32_t* cu, int n_items, int rows_per_unit
     item_start[k] = cu[i];
     item_len[k] = cu[i + 1] - cu[i];
     unit_prefix[k] = units;
-    if (dual_head) {
-      const int tiles = (item_len[k] + rows_per_unit / 2 - 1) / (rows_per_unit / 2);
-      units += (tiles / 2) * H + (tiles % 2) * ((H + 1) / 2);
-    } else {
-      units += ((item_len[k] + rows_per_unit - 1) / rows_per_unit) * H;
-    }
+    units += ((item_len[k] + rows_per_unit - 1) / rows_per_unit) * H;
   }
   unit_prefix[n_items] = units;
   *total_units = units;
@@ -938,52 +930,32 @@ static eas_status launch_attention_mma(const bf16* qkv, bf16* out, const int32_t
 }
 
 static eas_status launch_attention_tc(const bf16* qkv, bf16* out, const int32_t* cu, int n_items, int H, int hd, int budget,
-                                      cudaStream_t stream, uint32_t* status, bool reverse) {
-  constexpr bool PT = false;
+                                      cudaStream_t stream, uint32_t* status) {
   AttnTcParams ap{};
   const int d = H * hd;
   const int64_t T = cu[n_items];
   {
     const uint64_t dims[2] = {static_cast<uint64_t>(3 * d), static_cast<uint64_t>(T)};
     const uint64_t strides[1] = {static_cast<uint64_t>(3 * d) * 2};
-    const uint32_t box_lo[2] = {64, kTcTile};
+    const uint32_t box_lo[2] = {64, kTcTile}, box_hi[2] = {16, kTcTile};
     EAS_TRY(make_tmap(&ap.map_lo, qkv, 2, dims, strides, box_lo, CU_TENSOR_MAP_SWIZZLE_128B));
-    const uint32_t box_hi[2] = {16, kTcTile};
     EAS_TRY(make_tmap(&ap.map_hi, qkv, 2, dims, strides, box_hi, CU_TENSOR_MAP_SWIZZLE_32B));
-    // K and V tiles: the kernel's keys per tile (head_dim 80 with P in tensor memory: 112)
-    const uint32_t keys = hd == 64 ? AttnTcSmem<64, PT>::kKeys : AttnTcSmem<80, PT>::kKeys;
-    const uint32_t box_klo[2] = {64, keys};
-    EAS_TRY(make_tmap(&ap.map_klo, qkv, 2, dims, strides, box_klo, CU_TENSOR_MAP_SWIZZLE_128B));
-    const uint32_t box_khi[2] = {16, keys};
-    EAS_TRY(make_tmap(&ap.map_khi, qkv, 2, dims, strides, box_khi, CU_TENSOR_MAP_SWIZZLE_32B));
-    const uint64_t odims[2] = {static_cast<uint64_t>(d), static_cast<uint64_t>(T)};
-    const uint64_t ostrides[1] = {static_cast<uint64_t>(d) * 2};
-    const uint32_t obox[2] = {64, 32};
-    EAS_TRY(make_tmap(&ap.map_out, out, 2, odims, ostrides, obox, CU_TENSOR_MAP_SWIZZLE_128B));
   }
   ap.out = out; ap.ldo = d; ap.d_model = d; ap.n_heads = H;
   ap.scale_log2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(hd)));
   ap.n_items = n_items;
   ap.status = status;
-  // dual-head units (two heads' odd last query tiles in one unit) when some item has an odd number of 128-row tiles
-  bool dual = false;
-  if (hd == 64 && AttnTcSmem<64, PT>::kDualHeadOk && H >= 2)
-    for (int i = 0; i < n_items; ++i) dual = dual || (((cu[i + 1] - cu[i] + kTcTile - 1) / kTcTile) & 1) != 0;
-  attention_schedule(cu, n_items, 2 * kTcTile, H, ap.item_start, ap.item_len, ap.unit_prefix, &ap.total_units, dual, reverse);
+  attention_schedule(cu, n_items, 2 * kTcTile, H, ap.item_start, ap.item_len, ap.unit_prefix, &ap.total_units);
   if (ap.total_units == 0) return EAS_OK;
   const int grid = std::min(budget, ap.total_units);
   static OncePerDevice once;
   if (once.first()) {
-    CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<64, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnTcSmem<64, PT>::kBytes));
-    CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<80, PT>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnTcSmem<80, PT>::kBytes));
-    if constexpr (AttnTcSmem<64, PT>::kDualHeadOk)
-      CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<64, PT, AttnTcSmem<64, PT>::kDualHeadOk>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnTcSmem<64, PT>::kBytes));
+    CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnTcSmem<64>::kBytes));
+    CUDA_TRY(cudaFuncSetAttribute(attn_tc_kernel<80>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnTcSmem<80>::kBytes));
     once.settled();
   }
-  if (hd == 64 && dual)
-    return launch_kernel(attn_tc_kernel<64, PT, AttnTcSmem<64, PT>::kDualHeadOk>, grid, kTcThreads, AttnTcSmem<64, PT>::kBytes, stream, ap);
-  if (hd == 64) return launch_kernel(attn_tc_kernel<64, PT>, grid, kTcThreads, AttnTcSmem<64, PT>::kBytes, stream, ap);
-  if (hd == 80) return launch_kernel(attn_tc_kernel<80, PT>, grid, kTcThreads, AttnTcSmem<80, PT>::kBytes, stream, ap);
+  if (hd == 64) return launch_kernel(attn_tc_kernel<64>, grid, kTcThreads, AttnTcSmem<64>::kBytes, stream, ap);
+  if (hd == 80) return launch_kernel(attn_tc_kernel<80>, grid, kTcThreads, AttnTcSmem<80>::kBytes, stream, ap);
   return fail(EAS_ERR_UNSUPPORTED, "head_dim %d", hd);
 }
 
@@ -1103,7 +1075,7 @@ static eas_status launch_attention_rr(const bf16* qkv, bf16* out, const int32_t*
 static eas_status launch_attention(const bf16* qkv, bf16* out, const int32_t* cu, int n_items, int H, int hd, int budget,
                                    cudaStream_t stream, int impl, uint32_t* status, const AttnPlan& plan, bool reverse = false) {
   if (impl == 1) return launch_attention_mma(qkv, out, cu, n_items, H, hd, budget, stream);
-  if (impl == 2) return launch_attention_tc(qkv, out, cu, n_items, H, hd, budget, stream, status, reverse);
+  if (impl == 2) return launch_attention_tc(qkv, out, cu, n_items, H, hd, budget, stream, status);
   auto launch = plan.own_p ? (hd == 64 ? launch_attention_rr<64, true> : launch_attention_rr<80, true>)
                            : (hd == 64 ? launch_attention_rr<64, false> : launch_attention_rr<80, false>);
   if (hd == 64 || hd == 80) return launch(qkv, out, cu, n_items, H, budget, stream, status, reverse, plan);
@@ -1763,10 +1735,5 @@ extern "C" eas_status eas_kernel_attention(const void* qkv, void* out, const int
 #ifdef EAS_GEMM_PROFILE
 extern "C" int eas_debug_gemm_stamps(unsigned long long* host_out /* [32*16] */) {
   return cudaMemcpyFromSymbol(host_out, eas::g_gemm_dbg, sizeof(unsigned long long) * 32 * 16) == cudaSuccess ? 0 : 1;
-}
-#endif
-#ifdef EAS_ATTN_PROFILE
-extern "C" int eas_debug_attn_stamps(unsigned long long* host_out /* [2*64*12] */) {
-  return cudaMemcpyFromSymbol(host_out, eas::g_attn_dbg, sizeof(unsigned long long) * 2 * 64 * 12) == cudaSuccess ? 0 : 1;
 }
 #endif
