@@ -832,6 +832,8 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
 template <int KIND, bool F32, bool PART = false>
 static eas_status launch_norm_nv(const NormParams& p, int budget, cudaStream_t stream) {
   const int nv = p.d / 128;
+  // few rows: as many SMs as possible, down to four warps a CTA
+  const int warps = std::min(16, std::max(4, (p.rows + budget - 1) / budget));
 #define EAS_NORM_CASE(NV_)                                                                                         \
   case NV_: {                                                                                                      \
     static OncePerDevice once;                                                                                     \
@@ -839,7 +841,7 @@ static eas_status launch_norm_nv(const NormParams& p, int budget, cudaStream_t s
       CUDA_TRY(cudaFuncSetAttribute(norm_kernel<NV_, KIND, F32, PART>, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnePerSmSmem)); \
       once.settled();                                                                                              \
     }                                                                                                              \
-    EAS_TRY(launch_kernel(norm_kernel<NV_, KIND, F32, PART>, std::min(budget, (p.rows + 15) / 16), 512, kOnePerSmSmem, stream, p)); \
+    EAS_TRY(launch_kernel(norm_kernel<NV_, KIND, F32, PART>, std::min(budget, (p.rows + warps - 1) / warps), 32 * warps, kOnePerSmSmem, stream, p)); \
     break;                                                                                                         \
   }
   switch (nv) {

@@ -765,8 +765,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
       // all TMEM reads of this warp are complete (wait::ld above): hand the accumulator back
       release_accumulator(acc);
     }
-    // bulk stores still reading the staging buffer must finish before the CTA's shared memory is released
-    if (p.use_tma_out && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    // bulk stores still READING the staging buffer must finish before the CTA's shared memory is released; that they are
+    // performed is the grid's completion, which the next kernel waits for: the tear-down overlaps it (one 252 x 364 image: 2304 -> 2214 us a pass, with the norm rows
+    // spread over more SMs)
+    if (p.use_tma_out && lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
     if (ew == 0 && lane == 0) GEMM_TL(6);
   }
 
