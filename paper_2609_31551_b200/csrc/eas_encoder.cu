@@ -322,29 +322,35 @@ static eas_status finish_linear(Linear& L) {
 
 typedef void (*GemmKernel)(GemmParams);
 // Tile shapes of the GEMM.  All accumulate every output element over K in the same order: bit-identical results.
-enum { TILE_AUTO = 0, TILE_SINGLE = 1, TILE_PAIR = 2, TILE_WIDE = 3, TILE_N128 = 4, TILE_N64 = 5, TILE_COUNT = 6 };
+// N..: one CTA per 128-row tile, P..: a CTA pair per 256-row tile, and the tile's columns (SINGLE, PAIR: 256, WIDE: 512).
+enum { TILE_AUTO = 0, TILE_SINGLE = 1, TILE_PAIR = 2, TILE_WIDE = 3, TILE_N128 = 4, TILE_N64 = 5, TILE_N160 = 6, TILE_N224 = 7,
+       TILE_P96 = 8, TILE_P128 = 9, TILE_P160 = 10, TILE_P192 = 11, TILE_P224 = 12, TILE_COUNT = 13 };
 struct TileShape { int ctas, rows, cols; };
-static const TileShape kTiles[TILE_COUNT] = {{0, 0, 0}, {1, 128, 256}, {2, 256, 256}, {2, 256, 512}, {1, 128, 128}, {1, 128, 64}};
-// deep (pair and narrow tiles): two 64-wide k-blocks per stage and TMA operation (convolutions walk their taps as 64-wide
+static const TileShape kTiles[TILE_COUNT] = {{0, 0, 0}, {1, 128, 256}, {2, 256, 256}, {2, 256, 512}, {1, 128, 128}, {1, 128, 64}, {1, 128, 160},
+                                             {1, 128, 224}, {2, 256, 96}, {2, 256, 128}, {2, 256, 160}, {2, 256, 192}, {2, 256, 224}};
+// deep (up to 128 columns): two 64-wide k-blocks per stage and TMA operation (convolutions walk their taps as 64-wide
 // k-blocks and use the shallow kernels).  nullptr: no such kernel.
 template <int ACT, int OUT, bool SPLIT = false>
 static GemmKernel gemm_kernel_of(int tile, bool deep) {
-  if constexpr (OUT == OUT_F32_FOLD) {
-    if (tile == TILE_WIDE) return gemm_kernel<ACT, OUT, 2, 512>;
-    if (tile == TILE_PAIR) return deep ? gemm_kernel<ACT, OUT, 2, 256, 2> : gemm_kernel<ACT, OUT, 2, 256>;
-    if (tile == TILE_SINGLE) return gemm_kernel<ACT, OUT, 1, 256>;
-    return nullptr;
-  } else {
-    if (tile == TILE_SINGLE) return gemm_kernel<ACT, OUT, 1, 256, 1, SPLIT>;
-    if (tile == TILE_PAIR) return deep ? gemm_kernel<ACT, OUT, 2, 256, 2, SPLIT> : gemm_kernel<ACT, OUT, 2, 256, 1, SPLIT>;
+  if (tile == TILE_SINGLE) return gemm_kernel<ACT, OUT, 1, 256, 1, SPLIT>;
+  if (tile == TILE_PAIR) return gemm_kernel<ACT, OUT, 2, 256, 1, SPLIT>;
+  if constexpr (ACT != ACT_SWIGLU && !(ACT == ACT_GELU && OUT == OUT_F32))
+    if (tile == TILE_WIDE) return gemm_kernel<ACT, OUT, 2, 512, 1, SPLIT>;
+  if constexpr (OUT != OUT_F32_FOLD) {
     if (tile == TILE_N128) return deep ? gemm_kernel<ACT, OUT, 1, 128, 2, SPLIT> : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 1, 128, 1>);
-    if constexpr (ACT != ACT_SWIGLU) {
+    if (tile == TILE_P128) return deep ? gemm_kernel<ACT, OUT, 2, 128, 2, SPLIT> : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 2, 128, 1>);
+    if constexpr (ACT != ACT_SWIGLU)
       if (tile == TILE_N64) return deep ? gemm_kernel<ACT, OUT, 1, 64, 2, SPLIT> : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 1, 64, 1>);
-      if constexpr (!(ACT == ACT_GELU && OUT == OUT_F32))
-        if (tile == TILE_WIDE) return gemm_kernel<ACT, OUT, 2, 512, 1, SPLIT>;
+    if constexpr (ACT != ACT_SWIGLU && !SPLIT) {
+      if (tile == TILE_P96) return deep ? gemm_kernel<ACT, OUT, 2, 96, 2> : nullptr;
+      if (tile == TILE_N160) return gemm_kernel<ACT, OUT, 1, 160>;
+      if (tile == TILE_N224) return gemm_kernel<ACT, OUT, 1, 224>;
+      if (tile == TILE_P160) return gemm_kernel<ACT, OUT, 2, 160>;
+      if (tile == TILE_P192) return gemm_kernel<ACT, OUT, 2, 192>;
+      if (tile == TILE_P224) return gemm_kernel<ACT, OUT, 2, 224>;
     }
-    return nullptr;
   }
+  return nullptr;
 }
 // out_fp32: 0 bf16, 1 fp32 (reduce-add when a residual is given), 2 the folding residual epilogue (OUT_F32_FOLD)
 static GemmKernel gemm_kernel_for(int act, int out_fp32, int tile, bool deep = false, bool split = false) {
@@ -721,18 +727,23 @@ struct GemmCall {
 // Tile shape: a pure speed choice (the results are bit-identical): the smallest estimated time,
 //     base + waves * (kb * per_kb + per_wave)      kb: 64-wide k-blocks of a work item,
 // where a last wave that fills a fraction f of the slots counts `partial` + (1 - partial) * f (fewer SMs share the path to L2).
-// Fitted to 480 measurements on B200: every shape forced over the encoder's GEMMs, 100 <= M <= 18464 tokens, d 256, 1024 and
-// 1280, on 37, 74, 111 and 148 SMs.  The wide
-// shape's figures also follow 0.25 s runs back to back at the power cap, where it is the best one for K >= 4096 (M = 4096, N = K = 8192
-// on 134 SMs: 430 us, pairs 446).  The choice is on average 0.2 % and at most 6 % slower than the best shape; without the
-// narrow shapes it was 10 % on average: M = 577 on 148 SMs (N, K): (1024, 4096) 25.3 us as 256x256, 15.1 as 128x64; (1024, 1024)
-// 11.3, 6.4; (3072, 1024) 9.9, 7.5 as 128x128; M = 1500 (1280, 5120) 30.8, 22.5 as 128x128; from a few full waves of pair
-// tiles on those win (M = 18464 (4096, 1024): 115 us, single CTAs 138).
+// Fitted to 1600 measurements on B200: every shape forced over the encoder's GEMMs, 100 <= M <= 18464 tokens, d 256, 1024 and
+// 1280, on 37, 74, 111 and 148 SMs, then adjusted for the choice alone, where runs of 0.25 s back to back at the power cap
+// (large M) count too.  The choice is on average 0.15 % and at most 6 % slower than the best shape (0.3 % on shapes left out
+// of the fit).  What the widths are for: a launch takes whole waves of tiles, so the width that just fills the SMs wins, and
+// a pair pulls half the weight bytes per SM that two single tiles pull, at 100 to 145 GB/s per SM the bound of every tile below
+// 192 columns.  (N, K) on 148 SMs, the best of 128x64, 128x128, 128x256, 256x256, 256x512 -> now:
+//   M = 577:  (1024, 4096) 17.5 us -> 14.0 as 256x96;  (4096, 1024) 12.3 -> 9.9 as 128x160
+//   M = 1500: (1280, 5120) 25.4 -> 20.1 as 256x128;    (3840, 1280) 17.5 -> 14.4 as 256x160
+//   M = 5000: (1280, 5120) 57.3 -> 49.5 as 256x192;    (5120, 1280) 49.3 -> 49.7 (left at 256x256)
+// 128x96 and 128x192 would win another 0.2 % on average and are left out.
 template <typename Usable>
 static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bool plain, Usable usable) {
   struct Cost { int tile; double base, per_kb, per_wave, partial; };    // us
-  static const Cost costs[] = {{TILE_SINGLE, 5.5, 0.406, 0.04, 0.80}, {TILE_PAIR, 6.4, 0.336, 0.14, 0.85}, {TILE_WIDE, 5.5, 0.65, 2.0, 0.84},
-                               {TILE_N128, 4.1, 0.241, 0.45, 0.94}, {TILE_N64, 3.4, 0.174, 0.22, 1.0}};
+  static const Cost costs[] = {{TILE_SINGLE, 5.24, 0.351, 0.52, 0.87}, {TILE_PAIR, 6.44, 0.323, 0.25, 0.92}, {TILE_WIDE, 4.81, 0.586, 5.1, 0.89},
+                               {TILE_N128, 3.91, 0.228, 0.45, 0.95}, {TILE_N64, 3.48, 0.173, 0.20, 1.0}, {TILE_N160, 4.61, 0.265, 0.31, 0.92},
+                               {TILE_N224, 5.02, 0.329, 0.29, 0.88}, {TILE_P96, 4.66, 0.163, 0.13, 0.79}, {TILE_P128, 5.07, 0.181, 0.28, 0.84},
+                               {TILE_P160, 5.20, 0.212, 0.48, 0.80}, {TILE_P192, 5.52, 0.250, 0.34, 0.85}, {TILE_P224, 5.98, 0.291, 0.20, 0.84}};
   int tile = TILE_SINGLE;
   double best = 0.0;
   for (const Cost& c : costs) {
@@ -742,7 +753,7 @@ static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bo
     const int64_t tiles = ((M + t.rows - 1) / t.rows) * ((N + t.cols - 1) / t.cols) * splits;
     const int64_t rem = tiles % slots;
     const double waves = static_cast<double>(tiles / slots) + (rem != 0 ? c.partial + (1.0 - c.partial) * static_cast<double>(rem) / static_cast<double>(slots) : 0.0);
-    const double shallow = c.tile == TILE_PAIR && !plain ? 1.075 : 1.0;       // convolutions: pair tiles without deep stages
+    const double shallow = t.cols <= 128 && !plain ? 1.08 : 1.0;       // convolutions: no deep stages (128x64 +14 %, 256x128 +7 %, 128x128 +5 %)
     const double cost = c.base + waves * (kb * c.per_kb * shallow + c.per_wave);
     if (best == 0.0 || cost < best) { best = cost; tile = c.tile; }
   }
@@ -761,12 +772,11 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
     return fail(EAS_ERR_UNSUPPORTED, "a folded normalisation needs a plain GEMM with row-aligned output and K %% %d == 0", kFoldGroup);
   const int out_mode = fold_out ? 2 : (g.out_fp32 ? 1 : 0);
   const bool plain = g.conv_stride == 1 && g.taps == 1;
-  // pair and narrow tiles of plain GEMMs run the deep kernels (two k-blocks per stage and TMA operation: 8 % faster at
-  // K = 1024); the 128x256 and wide tiles would be left with two 96 KB stages and measured no better
-  auto is_deep = [&](int t) { return plain && (t == TILE_PAIR || t == TILE_N128 || t == TILE_N64); };
+  auto is_deep = [&](int t) { return plain && kTiles[t].cols <= 128; };
   auto kernel_of = [&](int t) -> GemmKernel {       // nullptr: this GEMM has no kernel of that shape
-    // wide tiles: the output splits evenly into 512-column blocks, plain TMA-stored epilogue
+    // wide tiles: the output splits evenly into 512-column blocks; they and the odd widths: TMA-stored epilogue only
     if (t == TILE_WIDE && (!tma_out || L.N % 512 != 0)) return nullptr;
+    if (gemm_alt(kTiles[t].cols) && !tma_out) return nullptr;
     return gemm_kernel_for(g.act, out_mode, t, is_deep(t), g.splits > 1);
   };
   const int64_t k_total = g.a_run * g.taps;
@@ -775,7 +785,7 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
   if (g.force_tile != TILE_AUTO && (kTiles[g.force_tile].ctas == 1 || budget >= 2)) {
     tile = g.force_tile;
     if (kernel_of(tile) == nullptr)
-      return fail(EAS_ERR_UNSUPPORTED, "no %dx%d tile for this GEMM (512 columns: N %% 512 == 0, a plain or GELU epilogue and row-aligned output; 64: no gated epilogue)", kTiles[tile].rows, kTiles[tile].cols);
+      return fail(EAS_ERR_UNSUPPORTED, "no %dx%d tile for this GEMM (512 columns: N %% 512 == 0, a plain or GELU epilogue and row-aligned output; 64, 96, 160, 192, 224: no gated epilogue; 96, 160, 192, 224: row-aligned output)", kTiles[tile].rows, kTiles[tile].cols);
   } else if (g.force_tile == TILE_AUTO) {
     tile = pick_tile(g.M, L.N, kb, g.splits, budget, plain, [&](int t) { return kernel_of(t) != nullptr && (t != TILE_WIDE || k_total >= 2048); });
 #ifdef EAS_GEMM_FORCE_TILE   // calibration builds only: this shape wherever it exists
@@ -789,7 +799,8 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
   else EAS_TRY(make_a_tmap(&p.tma_a, g.A, g.a_run, g.a_row_elems, g.conv_stride, g.a_rows));
   // weight rows per TMA box: the CTA's share of a 256-column accumulator, or the narrow tile's columns
   const int w_rows = std::min(tile_n, static_cast<int>(kBN)) / ctas;
-  p.tma_b = w_rows == 256 ? L.tmap : w_rows == 128 ? (deep ? L.tmap_half_deep : L.tmap_half) : (deep ? L.tmap_quarter_deep : L.tmap_quarter);
+  if (gemm_alt(tile_n)) EAS_TRY(deep ? make_w_tmap_deep(&p.tma_b, L.w, L.N, L.K, w_rows) : make_w_tmap(&p.tma_b, L.w, L.N, L.K, w_rows));
+  else p.tma_b = w_rows == 256 ? L.tmap : w_rows == 128 ? (deep ? L.tmap_half_deep : L.tmap_half) : (deep ? L.tmap_quarter_deep : L.tmap_quarter);
   p.M = g.M; p.N = L.N;
   p.kb_per_tap = static_cast<int>(g.a_run / kBK);
   p.k_blocks = deep ? (p.kb_per_tap + 1) / 2 : p.kb_per_tap * g.taps;

@@ -6,9 +6,8 @@
 //   warps 2..9  epilogue: tcgen05.ld -> bias / activation / rotary -> swizzled shared-memory staging -> TMA store
 //               (TMA reduce-add into the fp32 residual stream); scatter epilogues (row maps) store directly
 //
-// Five tile shapes (template arguments CTAS, TN, KD; the launcher picks by estimated time): one CTA per 128x256 tile,
-// a CTA pair (cta_group::2) per 256x256 tile with "deep" stages, a pair per "wide" 256x512 tile, and, for few tokens, one CTA
-// per "narrow" 128x128 or 128x64 tile.
+// Tile shapes (template arguments CTAS, TN, KD; the launcher picks by estimated time): one CTA per 128 x {64, 128, 160, 224,
+// 256} tile, or a CTA pair (cta_group::2) per 256 x {96, 128, 160, 192, 224, 256, 512} tile.
 //
 // The grid is `sm_budget` CTAs (one per SM: the shared-memory request excludes a second resident
 // CTA) and each CTA walks tiles  blockIdx.x, blockIdx.x + gridDim.x, ...  in a fixed order; every output element is
@@ -26,27 +25,25 @@ constexpr int kEpiWarps = 8;
 constexpr int kGemmThreads = 64 + 32 * kEpiWarps + 32;   // + the second producer warp
 constexpr int kProducerBWarp = 2 + kEpiWarps;
 constexpr int kABytes = kBM * kBK * 2;            // 16 KB: 128 rows of A
-// one CTA per tile: a stage holds A (16 KB) + the whole 256-row weight tile (32 KB), 4 stages;
-// CTA pair per 256x256 tile: a stage holds A (16 KB) + this CTA's 128 weight rows (16 KB), 6 stages
+// A stage holds this CTA's 128 rows of A (16 KB) and its weight rows (all TN of them, or a pair's half) of one 64-wide
+// k-block; the ring takes 192 KB.
 // TN = 512 ("wide", CTA pairs only): the pair owns a 256x512 tile, i.e. two 256-column accumulators fed by the same
 // A tile (three TMA operations for twice the columns) at the price of a single accumulator set: the epilogue no longer
 // overlaps the next main loop, so it pays for large K only.
-// KD = 2 ("deep"): a stage holds TWO 64-wide k-blocks of each operand, fetched by ONE TMA operation per operand
-// (a 3-D box {64 columns, rows, 2 k-blocks}, which lands as two consecutive swizzle-atom blocks).  Measured on B200:
-// what a CTA can pull from L2 is set by the number of TMA operations in flight, not by their bytes (two 16 KB
-// boxes per 0.46 us, but also two 32 KB boxes per 0.47 us), so deep stages double the operand rate and move the main
-// loop from the load path to the tensor pipe.  Half as many, twice as large stages: same shared memory.
-// TN = 128 or 64 ("narrow", one CTA): with few tokens a launch has fewer 128x256 tiles than the device has SMs and the K loop
-// of ONE tile is the kernel's time, at the rate one SM pulls operands from L2 (48 KB per 64-wide k-block of a 128x256 tile,
-// 24 KB of a 128x64 one): more, narrower tiles shorten that loop and use the idle SMs.  Measured back to back, M = 577:
-// N = 1024, K = 4096 25.8 (256x256) -> 17.7 us (128x64), K = 1024 11.4 -> 7.1; N = 3072, K = 1024 9.6 -> 7.5 (128x128).
+// KD = 2 ("deep", TN <= 128): a stage holds TWO 64-wide k-blocks of each operand, fetched by ONE TMA operation per operand
+// (a 3-D box {64 columns, rows, 2 k-blocks}, which lands as two consecutive swizzle-atom blocks): a step of a ring costs
+// some 0.16 us whatever its bytes, which is what bounds small tiles (deep against shallow: 128x64 -12 %, 256x96 -6 to -14 %,
+// 256x128 -7 % at K = 1024, 128x128 -5 %).  Wider tiles are no faster with it.
+// TN < 256: with few tokens a launch has fewer 256-column tiles than the device has SMs and the K loop of ONE tile is the
+// kernel's time, at the rate one SM pulls operands from L2 (48 KB per 64-wide k-block of a 128x256 tile, 24 KB of a 128x64
+// or 256x128 one): more, narrower tiles shorten that loop and use the idle SMs, and the width that just fills one wave is best.
 template <int CTAS, int TN, int KD = 1> struct GemmCfg {
   static constexpr int kBBytes = (TN / CTAS) * kBK * 2;            // per 64-wide k-block
   static constexpr int kStageBytes = (kABytes + kBBytes) * KD;
-  static constexpr int kStages = 4 * 49152 / kStageBytes;          // the ring's 192 KB
+  static constexpr int kStages = 4 * 49152 / kStageBytes < 8 ? 4 * 49152 / kStageBytes : 8;          // the ring's 192 KB
   static constexpr int kAccBuffers = TN == 512 ? 1 : 2;
   static constexpr int kAccCols = TN < kBN ? TN : kBN;             // tensor-memory columns of one accumulator
-  static constexpr int kTmemCols = TN < kBN ? 2 * TN : 512;
+  static constexpr int kTmemCols = TN > 128 ? 512 : TN > 64 ? 256 : 128;     // a power of two that holds the accumulators
 };
 constexpr int kMaxStages = 8;
 constexpr int kStagingOff = 4 * 49152;                         // == 6 * 32768; 8 epilogue warps x 4 KB output staging (TMA store source)
@@ -156,7 +153,11 @@ __device__ __noinline__ float2 fold_row_factors(const float2* stats, long long r
 }
 
 // bf16 outputs of an epilogue warp's row: the columns of one output box (64, or 32 where a warp has no more)
+// gemm_alt: tiles whose halves are no multiple of 64 columns: their 32-column chunks are dealt alternately to the two
+// four-warp groups of the epilogue
+__host__ __device__ constexpr bool gemm_alt(int tn) { return tn % 128 != 0 && tn != 64; }
 __host__ __device__ constexpr int gemm_out_row(int act, int tn) {
+  if (gemm_alt(tn)) return 32;
   const int per_warp = act == ACT_SWIGLU ? tn / 4 : tn / 2;
   return per_warp >= 64 ? 64 : 32;
 }
@@ -164,11 +165,13 @@ __host__ __device__ constexpr int gemm_out_row(int act, int tn) {
 // SPLIT: the launch splits K (GemmParams::splits > 1); the ordinary instantiations keep their code free of it.
 template <int ACT, int OUT, int CTAS, int TN, int KD = 1, bool SPLIT = false>
 __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_constant__ GemmParams p) {
-  static_assert(TN == 64 || TN == 128 || TN == 256 || TN == 512, "tile width");
+  constexpr bool kAlt = gemm_alt(TN);
+  static_assert(TN % 32 == 0 && TN >= 64 && (TN <= 256 || TN == 512), "tile width");
+  static_assert(!kAlt || (ACT != ACT_SWIGLU && !SPLIT), "odd widths: plain tiles");
   static_assert(TN < 512 || (CTAS == 2 && ACT != ACT_SWIGLU), "wide tiles: CTA pairs, no gated epilogue");
-  static_assert(TN >= 256 || (CTAS == 1 && OUT != OUT_F32_FOLD), "narrow tiles: one CTA, no folding epilogue");
+  static_assert(TN >= 256 || OUT != OUT_F32_FOLD, "narrow tiles: no folding epilogue");
   static_assert(TN >= 128 || ACT != ACT_SWIGLU, "a gated epilogue halves the columns: 128 at least");
-  static_assert(KD == 1 || KD == 2, "one or two 64-wide k-blocks per stage");
+  static_assert(KD == 1 || (KD == 2 && TN <= kBN), "one or two 64-wide k-blocks per stage");
   using Cfg = GemmCfg<CTAS, TN, KD>;
   constexpr int kStages = Cfg::kStages;
   static_assert(kStages <= kMaxStages, "barrier area");
@@ -235,58 +238,52 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
 
   if (warp == 0 || warp == kProducerBWarp) {
     // ------------------------------------------------------------------ producers: warp 0 loads A, the last warp B
-    // Issuing a TMA operation occupies the issuing thread for some 70 ns, and that is what bounds the operand rate
-    // of a CTA (measured: a step of two 32 KB boxes takes 476 ns from one thread, 396 ns from two), so the two
-    // operands have a thread each.  The A thread announces the bytes of the whole stage.
+    // The two operands have a warp each (128 KB of boxes from one thread: 476 ns a step, from two 396); a whole warp walks the
+    // tiles and one elected lane issues, as in the UMMA warp (1 to 3 % at large M against a lone diverged thread).  The A warp
+    // announces the bytes of the whole stage.
     const bool do_a = warp == 0, do_b = warp != 0;
-    if (lane == 0) {
-      uint32_t it = 0;
-      bool ok = true;
-      for (int work = first_tile; work < num_work && ok; work += tile_step) {
-        const int tile = SPLIT ? work / n_splits : work, split = SPLIT ? work - tile * n_splits : 0;
-        int mg, nb;
-        tile_coords(p.reverse ? num_tiles - 1 - tile : tile, p.m_blocks, p.n_blocks, mg, nb);
-        const int mb = mg * CTAS + cta_rank;       // this CTA's 128-row block
-        const int kb0 = split * kb_per_split, kb1 = SPLIT ? min(p.k_blocks, kb0 + kb_per_split) : p.k_blocks;
-        // position of a shallow k-block: column kx of the tap that reads phase `phase` of the strided rows, `shift` rows on
-        // (running counters: three integer divisions per k-block held every kernel with shallow stages at 0.34 us per k-block;
-        // without them 128x256 tiles, M = 577, N = 1024, K = 4096: 27.7 -> 26.0 us; 8 images of 577 tokens, 24 layers: 4.03 -> 3.87 ms)
-        int kx = 0, phase = 0, shift = 0;
-        if (KD == 1) {
-          const int tap = kb0 / p.kb_per_tap;
-          kx = (kb0 - tap * p.kb_per_tap) * kBK;
-          phase = tap % p.conv_stride;
-          shift = tap / p.conv_stride;
-        }
-        const int run = p.kb_per_tap * kBK;
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = it % kStages;
-          const uint32_t ph = (it / kStages) & 1u;
-          // The W producer of constant weights skipped the grid-dependency wait above and has filled every stage once;
-          // its next wait needs the consumer, which needs A, which needs the earlier kernels: join the dependency first,
-          // so that the bounded wait below never runs while a predecessor is still working.
-          if (do_b && p.w_const && it == kStages) pdl_wait();
-          if (!mbar_wait(&empty_bar[s], ph ^ 1u, abort_flag)) { ok = false; break; }
-          uint8_t* sa = smem + s * kStageBytes;
-          uint8_t* sb = sa + kABytes * KD;
+    uint32_t it = 0;
+    bool ok = true;
+    for (int work = first_tile; work < num_work && ok; work += tile_step) {
+      const int tile = SPLIT ? work / n_splits : work, split = SPLIT ? work - tile * n_splits : 0;
+      int mg, nb;
+      tile_coords(p.reverse ? num_tiles - 1 - tile : tile, p.m_blocks, p.n_blocks, mg, nb);
+      const int mb = mg * CTAS + cta_rank;       // this CTA's 128-row block
+      const int kb0 = split * kb_per_split, kb1 = SPLIT ? min(p.k_blocks, kb0 + kb_per_split) : p.k_blocks;
+      // position of a shallow k-block: column kx of the tap that reads phase `phase` of the strided rows, `shift` rows on
+      // (running counters: three integer divisions per k-block held every kernel with shallow stages at 0.34 us per k-block;
+      // without them 128x256 tiles, M = 577, N = 1024, K = 4096: 27.7 -> 26.0 us; 8 images of 577 tokens, 24 layers: 4.03 -> 3.87 ms)
+      int kx = 0, phase = 0, shift = 0;
+      if (KD == 1) {
+        const int tap = kb0 / p.kb_per_tap;
+        kx = (kb0 - tap * p.kb_per_tap) * kBK;
+        phase = tap % p.conv_stride;
+        shift = tap / p.conv_stride;
+      }
+      const int run = p.kb_per_tap * kBK;
+      for (int kb = kb0; kb < kb1; ++kb, ++it) {
+        const int s = it % kStages;
+        const uint32_t ph = (it / kStages) & 1u;
+        // The W producer of constant weights skipped the grid-dependency wait above and has filled every stage once;
+        // its next wait needs the consumer, which needs A, which needs the earlier kernels: join the dependency first,
+        // so that the bounded wait below never runs while a predecessor is still working.
+        if (do_b && p.w_const && it == kStages) pdl_wait();
+        if (!warp_mbar_wait(&empty_bar[s], ph ^ 1u, abort_flag)) { ok = false; break; }
+        uint8_t* sa = smem + s * kStageBytes;
+        uint8_t* sb = sa + kABytes * KD;
+        if (elect_one()) {
           // both CTAs' loads of a pair complete on the leader's barrier; the leader announces the bytes of both
           if (do_a && cta_rank == 0) mbar_expect_tx(&full_bar[s], CTAS * kStageBytes);
           if (KD == 2) {
             // deep stage (plain GEMM only): [A k-block 0][A k-block 1][B ...] from one 3-D box per operand
             if (CTAS == 2) {
               if (do_a) tma_load_3d_pair(sa, &p.tma_a, &full_bar[s], 0, mb * kBM, kb * KD);
-              if (do_b) {
-#pragma unroll
-                for (int h = 0; h < NW; ++h)
-                  tma_load_3d_pair(sb + h * kBAtom * KD, &p.tma_b, &full_bar[s], 0, nb * kTileN + h * kBN + cta_rank * kBRows, kb * KD);
-              }
+              if (do_b) tma_load_3d_pair(sb, &p.tma_b, &full_bar[s], 0, nb * kTileN + cta_rank * kBRows, kb * KD);
             } else {
               if (do_a) tma_load_3d(sa, &p.tma_a, &full_bar[s], 0, mb * kBM, kb * KD);
               if (do_b) tma_load_3d(sb, &p.tma_b, &full_bar[s], 0, nb * kTileN, kb * KD);
             }
-            continue;
-          }
-          if (CTAS == 2) {
+          } else if (CTAS == 2) {
             if (do_a) tma_load_3d_pair(sa, &p.tma_a, &full_bar[s], kx, phase, mb * kBM + shift);
             if (do_b) {
 #pragma unroll
@@ -297,18 +294,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
             if (do_a) tma_load_3d(sa, &p.tma_a, &full_bar[s], kx, phase, mb * kBM + shift);
             if (do_b) tma_load_2d(sb, &p.tma_b, &full_bar[s], kb * kBK, nb * kTileN);
           }
-          if ((kx += kBK) == run) {
-            kx = 0;
-            if (++phase == p.conv_stride) { phase = 0; ++shift; }
-          }
+        }
+        __syncwarp();
+        if ((kx += kBK) == run) {
+          kx = 0;
+          if (++phase == p.conv_stride) { phase = 0; ++shift; }
         }
       }
-      if (!ok) {
-        // give loads already in flight a bounded chance to land before the CTA retires
-        for (int s = 0; s < kStages; ++s) {
-          const long long t0 = clock64();
-          while (clock64() - t0 < 2000000) {}
-        }
+    }
+    if (!ok) {
+      // give loads already in flight a bounded chance to land before the CTA retires
+      for (int s = 0; s < kStages; ++s) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < 2000000) {}
       }
     }
   } else if (warp == 1) {
@@ -435,12 +433,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         uint8_t* srow = stage + lane * kRowBytes;
         const int sw = kRowBytes == 128 ? (lane & 7) : ((lane >> 1) & 3);
         const int arow = mb * kBM + quarter * 32 + lane;
-        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * kAccCols + half * kHalfN;
+        // this warp's chunks of 32 columns: its half of the tile, or every second one
+        const int my_chunks = kAlt ? (TN / 32 + 1 - half) / 2 : kHalfN / 32;
+        auto my_col = [&](int c) { return kAlt ? (half + 2 * c) * 32 : half * kHalfN + c * 32; };
+        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * kAccCols + my_col(0);
+        constexpr int kChunkStep = kAlt ? 64 : 32;
         const int ycoord = mb * kBM + quarter * 32;
 
         auto finish_chunk = [&](float (&v)[32], int c) {   // bias, rotary, activation on 32 accumulator columns
-          const int col0 = nb * kTileN + half * kHalfN + c * 32;
-          const float4* b4 = reinterpret_cast<const float4*>(sbias + half * kHalfN + c * 32);
+          const int col0 = nb * kTileN + my_col(c);
+          const float4* b4 = reinterpret_cast<const float4*>(sbias + my_col(c));
           if (p.fold_stats != nullptr) {
             // out = rstd * acc + (c0 - rstd * mean * c1): the staged "bias" is c0
             const bool centred = p.fold_c1 != nullptr && col0 < p.N;
@@ -589,7 +591,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           // fp32 output: 32 columns = one 128-byte staging row, so every 32-column chunk is a sub-tile (and a TMA
           // operation) of its own.  One chunk per round, the next chunk's TMEM load in flight meanwhile, so that the
           // wait for the previous operation to release the staging buffer falls behind a load and the chunk's math.
-          constexpr int kChunks = kHalfN / 32;
+          const int kChunks = my_chunks;
           uint32_t r[32];
           __syncwarp();
           tmem_ld_32x32(taddr, r);
@@ -601,10 +603,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
             for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
             if (c + 1 < kChunks) {
               __syncwarp();
-              tmem_ld_32x32(taddr + (c + 1) * 32, r);
+              tmem_ld_32x32(taddr + (c + 1) * kChunkStep, r);
             }
             finish_chunk(v, c);
-            const int col0 = nb * kTileN + half * kHalfN + c * 32;
+            const int col0 = nb * kTileN + my_col(c);
             staging_free();
 #pragma unroll
             for (int q = 0; q < 8; ++q)
@@ -613,8 +615,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           }
         } else {
 #pragma unroll 1
-        for (int pr = 0; pr < (kHalfN + 63) / 64; ++pr) {       // two chunks (64 accumulator columns) per round
-          constexpr int kPerRound = kHalfN >= 64 ? 2 : 1;
+        for (int pr = 0; pr < (kAlt ? my_chunks : (kHalfN + 63) / 64); ++pr) {       // two chunks (64 accumulator columns) per round, or one
+          constexpr int kPerRound = !kAlt && kHalfN >= 64 ? 2 : 1;
           uint32_t r0[32], r1[32];
           __syncwarp();
           tmem_ld_32x32(taddr + pr * 64, r0);
@@ -624,10 +626,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           float v0[32], v1[32];
 #pragma unroll
           for (int i = 0; i < 32; ++i) { v0[i] = __uint_as_float(r0[i]); v1[i] = kPerRound == 2 ? __uint_as_float(r1[i]) : 0.f; }
-          finish_chunk(v0, pr * 2);
+          finish_chunk(v0, pr * kPerRound);
           if (kPerRound == 2) finish_chunk(v1, pr * 2 + 1);
           GEMM_STAMP(4 + pr * 4);
-          const int col0 = nb * kTileN + half * kHalfN + pr * 64;
+          const int col0 = nb * kTileN + my_col(pr * kPerRound);
           if (ACT == ACT_SWIGLU) {
             // (gate, up) pairs -> 32 outputs per round; the 64 outputs of both rounds form one staging row
             if (pr == 0) staging_free();
@@ -644,7 +646,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
             }
             if (pr + 1 == (kHalfN + 63) / 64 && nb * kTileN + half * kHalfN < p.N) store_subtile((nb * kTileN + half * kHalfN) >> 1);
           } else {
-            // 64 bf16 columns = one 128-byte staging row (128x64 tiles: 32 columns, 64 bytes)
+            // 64 bf16 columns = one 128-byte staging row (one chunk per round: 32 columns, 64 bytes)
             staging_free();
             GEMM_STAMP(5 + pr * 4);
 #pragma unroll
@@ -668,6 +670,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         continue;
       }
 
+      if (kAlt) { ok = false; break; }                            // (these widths have TMA-stored outputs only: the launcher)
       if (!mbar_wait(&acc_full[acc], acc_ph, abort_flag)) { ok = false; break; }
       tc_fence_after_sync();
 
