@@ -735,7 +735,7 @@ struct GemmCall {
 // 192 columns.  (N, K) on 148 SMs, the best of 128x64, 128x128, 128x256, 256x256, 256x512 -> now:
 //   M = 577:  (1024, 4096) 17.5 us -> 14.0 as 256x96;  (4096, 1024) 12.3 -> 9.9 as 128x160
 //   M = 1500: (1280, 5120) 25.4 -> 20.1 as 256x128;    (3840, 1280) 17.5 -> 14.4 as 256x160
-//   M = 5000: (1280, 5120) 57.3 -> 49.5 as 256x192;    (5120, 1280) 49.3 -> 49.7 (left at 256x256)
+//   M = 5000: (1280, 5120) 57.3 -> 49.5 as 256x192
 // 128x96 and 128x192 would win another 0.2 % on average and are left out.
 template <typename Usable>
 static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bool plain, Usable usable) {

@@ -152,10 +152,10 @@ __device__ __noinline__ float2 fold_row_factors(const float2* stats, long long r
   return make_float2(a, -a * mu);
 }
 
-// bf16 outputs of an epilogue warp's row: the columns of one output box (64, or 32 where a warp has no more)
 // gemm_alt: tiles whose halves are no multiple of 64 columns: their 32-column chunks are dealt alternately to the two
 // four-warp groups of the epilogue
 __host__ __device__ constexpr bool gemm_alt(int tn) { return tn % 128 != 0 && tn != 64; }
+// bf16 outputs of an epilogue warp's row: the columns of one output box (64, or 32 where a warp has no more)
 __host__ __device__ constexpr int gemm_out_row(int act, int tn) {
   if (gemm_alt(tn)) return 32;
   const int per_warp = act == ACT_SWIGLU ? tn / 4 : tn / 2;
