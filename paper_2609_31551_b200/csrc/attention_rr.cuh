@@ -2,7 +2,8 @@
 //
 // A query tile is 128 rows of one head of one item.  A work unit is up to three consecutive query tiles of one item, counted
 // head by head; a softmax warpgroup (one thread per query row) works on each.  The key loop walks the item's keys 80 at a
-// time; keys past the item's end are masked to probability exactly 0, keys of other items are never multiplied in.  The
+// time; keys past the item's end are masked to probability exactly 0 and their value rows (the next item's) are cleared, since
+// 0 x Inf or NaN is not 0: an item's output does not depend on what is packed behind it.  The
 // tiles of a unit may belong to several heads (an item of 577 tokens has 5 query tiles a head): each head of the unit is a
 // "stream" of K/V tiles of its own, shared by its tiles.
 //
@@ -270,6 +271,23 @@ __global__ void __launch_bounds__(AttnRrSmem<HD, OWN_P>::kThreads, 1) attn_rr_ke
       }
       return true;
     };
+    // Only the first `rows` value rows of the V tile at ring position g belong to the item: clears the others (their probabilities
+    // are 0, but 0 x Inf or NaN is not).  Every issuer of the stream does so before its own P V; later ones store the zeros that
+    // are there already.  Once a tile, beside the softmax of its last step and before the next tile's Q is waited for.  (P V of
+    // the last step over fewer keys would have less to clear, but the branch costs every step: +1 % at 8192 keys.)
+    auto clear_behind = [&](uint32_t g, int rows) {
+      uint8_t* v = v_tile(g % NST);
+#pragma unroll 4
+      for (int c = rows * 8 + lane; c < KEYS * 8; c += 32)      // 16-byte chunks, 8 a row
+        *reinterpret_cast<uint4*>(v + c * 16) = make_uint4(0u, 0u, 0u, 0u);
+      if (HI) {                                                // columns 64..79: two swizzled chunks a row of the second atom
+#pragma unroll 2
+        for (int c = rows * 2 + lane; c < KEYS * 2; c += 32)
+          *reinterpret_cast<uint4*>(v + L::kAtomBytes + (c >> 1) * 128 + (((c & 1) ^ ((c >> 1) & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+      }
+      fence_proxy_async_smem();                                // generic-proxy stores -> visible to the tensor core's operand reads
+      __syncwarp();
+    };
     // by the elected lane: scores of the current tile (the last one waited for) against the K tile at ring position g
     auto mma_s = [&](uint32_t g) {
       const uint32_t qa = smem_u32(q_tile(w, (n_q - 1u) % QB)), ka = smem_u32(k_tile(g % NST));
@@ -325,6 +343,7 @@ __global__ void __launch_bounds__(AttnRrSmem<HD, OWN_P>::kThreads, 1) attn_rr_ke
         }
         if (!hand_back(g + 1, row + ns)) { ok = false; break; }
         if (!OWN_P && !warp_mbar_wait(&v_full[g % NST], (g / NST) & 1u, abort_flag)) { ok = false; break; }
+        if (!OWN_P && last && u.S % KEYS != 0) clear_behind(g, u.S - j * KEYS);
         if (more && (!hand_back(last ? next_base : row + ns, gn) || !k_landed(gn))) { ok = false; break; }
         if (last && chain && !q_landed()) { ok = false; break; }
         if (OWN_P && more) {
@@ -335,6 +354,7 @@ __global__ void __launch_bounds__(AttnRrSmem<HD, OWN_P>::kThreads, 1) attn_rr_ke
           ++n_s;
         }
         if (OWN_P && !warp_mbar_wait(&v_full[g % NST], (g / NST) & 1u, abort_flag)) { ok = false; break; }
+        if (OWN_P && last && u.S % KEYS != 0) clear_behind(g, u.S - j * KEYS);
         if (!warp_mbar_wait(&p_ready[w], n_p & 1u, abort_flag)) { ok = false; break; }
         ++n_p;
         tc_fence_after_sync();

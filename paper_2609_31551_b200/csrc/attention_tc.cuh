@@ -3,7 +3,8 @@
 //
 // One work unit = (item, head, 256 query rows) = two 128-row query tiles A and B that share every
 // K/V tile.  Keys and values come from the same item only: the key loop stops at the item's last
-// 128-key tile and the keys past the item's end are masked to -inf (probability exactly 0).
+// 128-key tile, the keys past the item's end are masked to -inf (probability exactly 0) and their value rows are cleared or
+// left out of P V (0 x Inf or NaN is not 0).
 //
 //   warp 0       TMA producer: Q tiles (double buffered across units), K/V tiles through a ring
 //   warp 1       UMMA issuer:  S = Q K^T (128 x 128 x {64|80}) into TMEM, O += P V (128 x {64|80} x 128) in TMEM
@@ -196,11 +197,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
         }
         umma_commit(&s_full[w]);
       };
-      auto issue_pv = [&](int w, int s, bool accumulate) {
+      // rows of the V tile that belong to the item; the rest of the last 16 that P V multiplies in is cleared (by this thread,
+      // once a tile: before tile A's P V)
+      auto clear_behind = [&](int s, int rows) {
+        for (int c = rows * 8; c < (rows + 15) / 16 * 16 * 8; ++c) *reinterpret_cast<uint4*>(v_tile(s) + c * 16) = make_uint4(0u, 0u, 0u, 0u);
+        if (HI)
+          for (int c = rows * 2; c < (rows + 15) / 16 * 16 * 2; ++c) *reinterpret_cast<uint4*>(v_tile(s) + L::kLoBytes + c * 16) = make_uint4(0u, 0u, 0u, 0u);
+        fence_proxy_async_smem();
+      };
+      auto issue_pv = [&](int w, int s, bool accumulate, int rows) {
         const uint32_t va = smem_u32(v_tile(s));
         const uint32_t d = tmem_base + L::kOCol0 + w * L::kOStride;
 #pragma unroll
         for (int ks = 0; ks < kTcTile / 16; ++ks) {        // 16 keys per step
+          if (ks * 16 >= rows) break;
           const uint64_t bd = make_smem_desc(va + ks * 2048, 1024, 1024, kSwizzle128B);
           const uint32_t acc = (accumulate || ks != 0) ? 1u : 0u;
           const uint32_t pa = smem_u32(p_tile(w));
@@ -236,7 +246,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
             }
             if (!mbar_wait(&v_full[s], (kv_it / NST) & 1u, abort_flag)) { ok = false; break; }
             tc_fence_after_sync();
-            issue_pv(w, s, j != 0);
+            const int rows = min(kTcTile, u.S - j * kTcTile);
+            if (w == 0 && rows % 16 != 0) clear_behind(s, rows);
+            issue_pv(w, s, j != 0, rows);
           }
           if (ok) umma_commit(&kv_empty[s]);
         }

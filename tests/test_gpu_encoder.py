@@ -228,3 +228,19 @@ def test_fused_patch_embedding_with_odd_item_offsets():
     out = enc.encode_microbatch(buf.cuda(), shapes, offsets, cu)
     enc.status()
     assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("case", list(CASES))
+def test_item_is_untouched_by_a_non_finite_neighbour(case):
+    """Items do not interact: with one item of the micro-batch all NaN, the others keep their bits."""
+    import paper_2609_31551_b200 as P
+    name, over, shapes = CASES[case]
+    cfg = S.get_config(name, **over)
+    w, enc = _make(cfg)
+    items = S.make_items(cfg, shapes, seed=2050)
+    _, want = G.run_gpu(enc, cfg, items)
+    items[1] = np.full_like(items[1], np.nan)
+    _, got = G.run_gpu(enc, cfg, items)
+    rows = np.concatenate([[0], np.cumsum([S.out_tokens_per_item(cfg, s) for s in shapes])])
+    assert torch.isnan(got[rows[1]:rows[2]].float()).all()
+    assert torch.equal(got[:rows[1]], want[:rows[1]]) and torch.equal(got[rows[2]:], want[rows[2]:])

@@ -223,6 +223,28 @@ def test_attention_units_at_key_tile_and_head_edges(hd, H, lens):
     assert (first.double().cpu() - ref).abs().max() <= 2e-2      # as in test_attention_block_diagonal
 
 
+@pytest.mark.parametrize("hd", [64, 80])
+@pytest.mark.parametrize("impl", [0, 1, 2])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_attention_is_untouched_by_non_finite_neighbours(hd, impl, value):
+    """An item's rows do not depend on what is packed around it, NaN and infinities included: items whose last key step holds
+    1 to 80 (128) keys, followed by one item that is not finite.  Their output has the bits that it has with a finite one there."""
+    import paper_2609_31551_b200 as P
+    for n in (1, 15, 16, 17, 79, 80, 81, 96, 128, 129, 200, 255, 256, 577):
+        lens, H = [n, 300, n], 3
+        cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        qkv = _dev(_bf16_exact(np.random.Generator(np.random.PCG64(n)), (sum(lens), 3 * H * hd)))
+        broken = qkv.clone()
+        broken[n:n + 300] = value
+        for budget in (0, 1):
+            want, _ = P.kernel_attention(qkv, cu, H, hd, impl=impl, sm_budget=budget)
+            got, status = P.kernel_attention(broken, cu, H, hd, impl=impl, sm_budget=budget)
+            torch.cuda.synchronize()
+            assert int(status[0]) == 0
+            for a, b in ((0, n), (n + 300, 2 * n + 300)):
+                assert torch.equal(got[a:b], want[a:b]), (n, budget, a)
+
+
 @pytest.mark.parametrize("H", [1, 2, 5, 16])
 def test_attention_dual_head_units(H):
     """head_dim 64, items with an odd number of 128-row query tiles: their last tiles of two adjacent heads share a
