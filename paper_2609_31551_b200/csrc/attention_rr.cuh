@@ -217,6 +217,9 @@ __global__ void __launch_bounds__(AttnRrSmem<HD, OWN_P>::kThreads, 1) attn_rr_ke
             if (HI) tma_load_2d(v_tile(s) + L::kAtomBytes, &p.map_k_lo, &v_full[s], 2 * p.d_model + x + 64, y);
           }
       }
+      // The last hand-backs of the stages are asynchronous arrivals (UMMA commits) that nothing else waits for: they have to be
+      // in before the CTA's shared memory passes to another one.  (Never used stages pass at once.)
+      for (uint32_t e = g; e < g + NST && ok; ++e) ok = mbar_wait(&kv_empty[e % NST], ((e / NST) & 1u) ^ 1u, abort_flag);
       if (!ok) {
         const long long t0 = clock64();
         while (clock64() - t0 < 4000000) {}     // let loads in flight land before the CTA retires

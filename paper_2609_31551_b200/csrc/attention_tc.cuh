@@ -167,6 +167,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(const __grid_con
           if (HI) tma_load_2d(v_tile(s) + L::kLoBytes, &p.map_hi, &v_full[s], x + p.d_model + 64, y);
         }
       }
+      // the last hand-backs of the K/V stages and Q buffers: asynchronous arrivals, in before the CTA's shared memory passes on
+      for (uint32_t e = kv_it; e < kv_it + NST && ok; ++e) ok = mbar_wait(&kv_empty[e % NST], ((e / NST) & 1u) ^ 1u, abort_flag);
+      for (uint32_t e = u_cnt; e < u_cnt + 2 && ok; ++e) ok = mbar_wait(&q_empty[e & 1], ((e >> 1) & 1u) ^ 1u, abort_flag);
       if (!ok) {
         const long long t0 = clock64();
         while (clock64() - t0 < 4000000) {}     // let loads in flight land before the CTA retires

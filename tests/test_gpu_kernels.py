@@ -245,6 +245,32 @@ def test_attention_is_untouched_by_non_finite_neighbours(hd, impl, value):
                 assert torch.equal(got[a:b], want[a:b]), (n, budget, a)
 
 
+@pytest.mark.parametrize("hd", [64, 80])
+@pytest.mark.parametrize("impl", [0, 2])
+def test_attention_ctas_leave_nothing_behind_for_their_successors(hd, impl):
+    """Launches back to back, each CTA of one following at once on an SM whose barriers lay elsewhere: an arrival still under
+    way when a CTA retires would land in its successor's shared memory.  Short units (one key step, so that a CTA ends right
+    behind its last UMMA), alternating with a kernel of another barrier layout; every result has the bits of a lone call."""
+    import paper_2609_31551_b200 as P
+    H = 2
+    rng = np.random.Generator(np.random.PCG64(hd + impl))
+    calls = []
+    for lens in ([60] * 74, [16, 80, 200] * 20, [600]):
+        cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        qkv = _dev(_bf16_exact(rng, (sum(lens), 3 * H * hd)))
+        calls.append((qkv, cu, P.kernel_attention(qkv, cu, H, hd, impl=impl)[0]))
+    A, W, b = _dev(_bf16_exact(rng, (500, 256))), _dev(_bf16_exact(rng, (512, 256), 0.05)), _dev(_bf16_exact(rng, (512,)))
+    want, _ = P.kernel_gemm(A, W, b)
+    torch.cuda.synchronize()
+    got = []
+    for _ in range(40):
+        got += [P.kernel_attention(qkv, cu, H, hd, impl=impl) + (ref,) for qkv, cu, ref in calls]
+        got.append(P.kernel_gemm(A, W, b) + (want,))
+    torch.cuda.synchronize()
+    for out, status, ref in got:
+        assert int(status[0]) == 0 and torch.equal(out, ref)
+
+
 @pytest.mark.parametrize("H", [1, 2, 5, 16])
 def test_attention_dual_head_units(H):
     """head_dim 64, items with an odd number of 128-row query tiles: their last tiles of two adjacent heads share a
