@@ -274,6 +274,12 @@ eas_status eas_kernel_gemm_tile(const void* A, const void* W, const void* bias, 
 eas_status eas_kernel_norm(const float* x, void* y, const void* gamma, const void* beta, int32_t rows, int32_t d,
                            int32_t kind, float eps, int32_t out_fp32, int32_t sm_budget, void* stream);
 
+/* How the default attention kernel cuts the query tiles (128 rows of one head of one item) of a micro-batch into work units on
+ * `sm_budget` SMs (> 0): plan[0] = tiles of a full unit (3, or 2: the variant for little work), plan[1] = tiles, counted over
+ * the items from the longest to the shortest, that are cut into full units, plan[2] = tiles of the units behind them.  A pure
+ * host function; the output rows do not depend on the plan. */
+eas_status eas_attention_plan(const int32_t* cu_seqlens_host, int32_t n_items, int32_t n_heads, int32_t sm_budget, int32_t* plan);
+
 /* Block-diagonal attention over packed qkv (device bf16 [T, 3*n_heads*head_dim], thirds Q|K|V) -> out (device
  * bf16 [T, n_heads*head_dim]).  cu_seqlens_host: host int32 [n_items+1].  impl as in eas_encoder_set_attention_impl. */
 eas_status eas_kernel_attention(const void* qkv, void* out, const int32_t* cu_seqlens_host, int32_t n_items,

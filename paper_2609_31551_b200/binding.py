@@ -18,6 +18,7 @@ EXPORTED_SYMBOLS = [
     "eas_encode_microbatch", "eas_encode_microbatch_static", "eas_encoder_status", "eas_encoder_last_launch_count", "eas_encoder_set_attention_impl",
     "eas_encoder_set_graph_mode", "eas_encoder_graph_stats", "eas_encoder_enable_timing", "eas_encoder_timing_read", "eas_last_error", "eas_encoder_destroy", "eas_kernel_gemm", "eas_kernel_gemm_tile", "eas_kernel_norm", "eas_kernel_attention",
     "eas_encoder_set_split_k", "eas_encoder_set_norm_fold", "eas_sm_partition_create", "eas_sm_partition_sm_count", "eas_sm_partition_stream", "eas_sm_partition_destroy",
+    "eas_attention_plan",
 ]
 
 
@@ -105,6 +106,8 @@ def load_library():
     lib.eas_kernel_attention.restype = C.c_int
     lib.eas_kernel_attention.argtypes = [C.c_void_p, C.c_void_p, C.POINTER(C.c_int32), C.c_int32, C.c_int32, C.c_int32,
                                          C.c_int32, C.c_void_p, C.c_int32, C.c_void_p]
+    lib.eas_attention_plan.restype = C.c_int
+    lib.eas_attention_plan.argtypes = [C.POINTER(C.c_int32), C.c_int32, C.c_int32, C.c_int32, C.POINTER(C.c_int32)]
     lib.eas_sm_partition_create.restype = C.c_int
     lib.eas_sm_partition_create.argtypes = [C.c_int32, C.POINTER(C.c_void_p)]
     lib.eas_sm_partition_sm_count.restype = C.c_int32
@@ -362,3 +365,11 @@ def kernel_attention(qkv, cu_seqlens_host, n_heads, head_dim, sm_budget=0, strea
     _check(lib.eas_kernel_attention(qkv.data_ptr(), out.data_ptr(), cu.ctypes.data_as(C.POINTER(C.c_int32)), len(cu) - 1,
                                     n_heads, head_dim, sm_budget, _stream_ptr(stream), impl, status.data_ptr()))
     return out, status
+
+
+def attention_plan(cu_seqlens_host, n_heads, sm_budget):
+    """eas_attention_plan -> (tiles of a full unit, tiles cut into full units, tiles of the units behind them)."""
+    cu = np.ascontiguousarray(cu_seqlens_host, dtype=np.int32)
+    plan = (C.c_int32 * 3)()
+    _check(load_library().eas_attention_plan(cu.ctypes.data_as(C.POINTER(C.c_int32)), len(cu) - 1, n_heads, sm_budget, plan))
+    return tuple(plan)

@@ -987,9 +987,12 @@ static void attention_item_units(int n, int before, const AttnPlan& plan, int* f
 // Units of three tiles use an SM best but are coarse: one clip of 8192 tokens and 16 heads is 342 of them, 2.3 rounds on 148
 // SMs, and one of 1500 tokens and 20 heads is 80.  The plan takes the variant, the cut and the small unit with the shortest
 // estimated time over the CTAs, from the measured time of an 80-key step with one, two and three tiles (relative to three)
-// and 1.5 steps per unit.  Past eight rounds the last one matters little and everything is cut into threes (the search is host work: at
-// most 0.05 ms, once per forward pass).  (Rows do not
-// depend on the plan: it may follow the micro-batch and the budget.)
+// and 1.5 steps per unit.  Past eight rounds everything is cut into threes.  (Rows do not depend on the plan: it may follow the
+// micro-batch and the budget.)
+// The search is host work, once per forward pass.  Every candidate is first estimated as if items of one length dealt their units
+// of one size together (closed form for whole rounds, one difference per run); then at most six of the best are walked unit by
+// unit.  One item of 577 tokens 1 us, 128 items of 64 tokens and 16 heads 11 us (walking every candidate: 2 and 30); over 3144
+// micro-batches the estimated time is 0.002 % longer on average and 2.4 % at most.
 static AttnPlan attention_plan(const int32_t* cu, int n_items, int H, int budget) {
   constexpr int kKeys = AttnRrSmem<64, false>::kKeys;
   static const double step[2][4] = {{0.0, 0.69, 0.82, 1.0}, {0.0, 0.58, 0.77, 0.0}};
@@ -999,39 +1002,114 @@ static AttnPlan attention_plan(const int32_t* cu, int n_items, int H, int budget
     len[i] = cu[i + 1] - cu[i];
     tiles += static_cast<int64_t>(H) * ((len[i] + kTcTile - 1) / kTcTile);
   }
-  AttnPlan best;
-  if (tiles > static_cast<int64_t>(8 * 3) * budget) return best;
+  if (tiles > static_cast<int64_t>(8 * 3) * budget) return AttnPlan{};
   std::sort(len.begin(), len.end(), std::greater<int>());
-  std::vector<double> load(budget);
-  double best_time = 0.0;
-  auto consider = [&](const AttnPlan& plan) {
+  struct Group { int tiles, count; double steps; };       // items with the same tiles and the same 80-key steps
+  std::vector<Group> groups;
+  groups.reserve(n_items);
+  for (int S : len) {
+    const int n = H * ((S + kTcTile - 1) / kTcTile);
+    const double steps = (S + kKeys - 1) / kKeys + 1.5;
+    if (groups.empty() || groups.back().tiles != n || groups.back().steps != steps) groups.push_back({n, 1, steps});
+    else ++groups.back().count;
+  }
+
+  std::vector<double> load(budget + 1, 0.0);
+  std::vector<uint64_t> edges((budget + 64) / 64, 0);     // where `load` is not 0
+  struct Candidate { double time; AttnPlan plan; };
+  std::vector<Candidate> candidates;
+  candidates.reserve(32);
+  auto estimate = [&](const AttnPlan& plan) {
+    const double* st = step[plan.own_p];
+    const int kWg = plan.own_p ? 2 : 3;
+    double whole = 0.0;                                   // `load` holds load[i] - load[i - 1], the whole rounds apart
+    int pos = 0;
+    bool odd = false;
+    auto deal = [&](int64_t n, double c) {
+      while (n > 0) {
+        if (pos == 0 && n >= budget) {
+          const int64_t rounds = n / budget;
+          whole += static_cast<double>(rounds) * c;
+          odd ^= (rounds & 1) != 0;
+          n -= rounds * budget;
+          continue;
+        }
+        const int k = static_cast<int>(std::min<int64_t>(n, budget - pos));
+        const int a = odd ? budget - pos - k : pos;
+        load[a] += c;
+        load[a + k] -= c;
+        edges[a >> 6] |= 1ull << (a & 63);
+        edges[(a + k) >> 6] |= 1ull << ((a + k) & 63);
+        n -= k;
+        if ((pos += k) == budget) { pos = 0; odd = !odd; }
+      }
+    };
+    int64_t before = 0;
+    for (const Group& g : groups) {
+      const int64_t in_full = std::min<int64_t>(g.count, std::max<int64_t>(0, (plan.full_tiles - before) / g.tiles));
+      deal(in_full * (g.tiles / kWg), g.steps * st[kWg]);
+      deal(g.tiles % kWg != 0 ? in_full : 0, g.steps * st[g.tiles % kWg]);
+      int64_t behind = g.count - in_full;                 // items behind the cut, or across it
+      if (behind > 0) {
+        int full, rest;
+        attention_item_units(g.tiles, static_cast<int>(before + in_full * g.tiles), plan, &full, &rest);
+        if (full > 0) {
+          const int left = g.tiles - full * kWg;
+          deal(full, g.steps * st[kWg]);
+          deal(left / plan.small, g.steps * st[plan.small]);
+          deal(left % plan.small != 0 ? 1 : 0, g.steps * st[left % plan.small]);
+          --behind;
+        }
+        deal(behind * (g.tiles / plan.small), g.steps * st[plan.small]);
+        deal(g.tiles % plan.small != 0 ? behind : 0, g.steps * st[g.tiles % plan.small]);
+      }
+      before += static_cast<int64_t>(g.count) * g.tiles;
+    }
+    double l = whole, time = whole;
+    for (size_t w = 0; w < edges.size(); ++w)
+      for (uint64_t& bits = edges[w]; bits != 0; bits &= bits - 1) {
+        double& edge = load[64 * w + static_cast<size_t>(__builtin_ctzll(bits))];
+        time = std::max(time, l += edge);
+        edge = 0.0;
+      }
+    candidates.push_back({time, plan});
+  };
+  auto walk = [&](const AttnPlan& plan) {
+    const double* st = step[plan.own_p];
     const int kWg = plan.own_p ? 2 : 3;
     std::fill(load.begin(), load.end(), 0.0);
-    int unit = 0, before = 0;
-    double time = 0.0;
-    for (int S : len) {
-      const int n = H * ((S + kTcTile - 1) / kTcTile);
-      int full, rest;
-      attention_item_units(n, before, plan, &full, &rest);
-      const double steps = (S + kKeys - 1) / kKeys + 1.5;
-      for (int k = 0; k < full + rest; ++k, ++unit) {
-        const int t = k < full ? std::min(kWg, n - k * kWg) : std::min(plan.small, n - full * kWg - (k - full) * plan.small);
-        const int round = unit / budget, pos = unit - round * budget;
-        double& l = load[(round & 1) ? budget - 1 - pos : pos];
-        l += steps * step[plan.own_p][t];
-        time = std::max(time, l);
+    int pos = 0, dir = 1;
+    auto deal = [&](double c) {
+      load[pos] += c;
+      pos += dir;
+      if (pos == budget) { pos = budget - 1; dir = -1; } else if (pos < 0) { pos = 0; dir = 1; }
+    };
+    int before = 0;
+    for (const Group& g : groups)
+      for (int i = 0; i < g.count; ++i, before += g.tiles) {
+        int full, rest, left = g.tiles;
+        attention_item_units(g.tiles, before, plan, &full, &rest);
+        for (int k = 0; k < full; ++k, left -= kWg) deal(g.steps * st[std::min(kWg, left)]);
+        for (int k = 0; k < rest; ++k, left -= plan.small) deal(g.steps * st[std::min(plan.small, left)]);
       }
-      before += n;
-    }
-    if (best_time == 0.0 || time < 0.999 * best_time) { best_time = time; best = plan; }
+    return *std::max_element(load.begin(), load.begin() + budget);
   };
-  consider(AttnPlan{});
+
+  estimate(AttnPlan{});
   for (int own = 0; own < (tiles <= static_cast<int64_t>(4) * budget ? 2 : 1); ++own) {
     const int kWg = own ? 2 : 3;
-    if (own) consider({1 << 30, 1, true});
+    if (own) estimate({1 << 30, 1, true});
     const int rounds = static_cast<int>(tiles / (static_cast<int64_t>(kWg) * budget));     // whole rounds of full units
     for (int small = 1; small < kWg; ++small)
-      for (int q = std::max(0, 4 * (rounds - 1)); q <= 4 * (rounds + 1); q += rounds > 2 ? 2 : 1) consider({kWg * (q * budget / 4), small, own != 0});
+      for (int q = std::max(0, 4 * (rounds - 1)); q <= 4 * (rounds + 1) && kWg * (q * budget / 4) < tiles; q += rounds > 2 ? 2 : 1)
+        estimate({kWg * (q * budget / 4), small, own != 0});
+  }
+  std::stable_sort(candidates.begin(), candidates.end(), [](const Candidate& a, const Candidate& b) { return a.time < b.time; });
+  AttnPlan best;
+  double best_time = 0.0;
+  for (size_t i = 0; i < candidates.size() && i < 6 && (i == 0 || candidates[i].time < 1.05 * best_time); ++i) {
+    const double time = walk(candidates[i].plan);
+    if (i == 0 || time < 0.999 * best_time) { best_time = time; best = candidates[i].plan; }
   }
   return best;
 }
@@ -1730,6 +1808,16 @@ extern "C" eas_status eas_kernel_norm(const float* x, void* y, const void* gamma
   EAS_TRY(resolve_budget(sm_budget, &budget));
   NormParams np{x, y, static_cast<const bf16*>(gamma), static_cast<const bf16*>(beta), nullptr, rows, d, eps};
   return launch_norm(kind, out_fp32 != 0, np, budget, static_cast<cudaStream_t>(stream));
+}
+
+extern "C" eas_status eas_attention_plan(const int32_t* cu, int32_t n_items, int32_t n_heads, int32_t sm_budget, int32_t* plan) {
+  if (cu == nullptr || plan == nullptr || n_items < 1 || n_items > EAS_MAX_ITEMS || n_heads <= 0 || sm_budget <= 0)
+    return fail(EAS_ERR_INVALID_ARG, "bad arguments");
+  for (int i = 0; i < n_items; ++i)
+    if (cu[i + 1] <= cu[i]) return fail(EAS_ERR_INVALID_ARG, "cu_seqlens is not strictly increasing");
+  const AttnPlan p = attention_plan(cu, n_items, n_heads, sm_budget);
+  plan[0] = p.own_p ? 2 : 3; plan[1] = p.full_tiles; plan[2] = p.small;
+  return EAS_OK;
 }
 
 extern "C" eas_status eas_kernel_attention(const void* qkv, void* out, const int32_t* cu, int32_t n_items, int32_t n_heads,
