@@ -656,6 +656,7 @@ extern "C" int64_t eas_encoder_out_rows(const eas_encoder* enc, const int32_t* c
 // kernel's last CTA to the next one past its wait, 32 images of 577 tokens on 74 SMs: 4.0-4.9 us without the attribute, 2.0-2.3
 // this way, 1.0-1.7 with the early release (on all SMs).  Set by every entry point before its first launch (per host thread).
 static thread_local bool g_overlap_launches = true;
+static thread_local int g_device_sms = 0;      // SMs of the device, set with it
 template <typename Params>
 static eas_status launch_kernel(void (*kern)(Params), int grid, int block, size_t smem, cudaStream_t stream, const Params& params,
                                 int cluster = 1) {
@@ -787,7 +788,12 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
     if (kernel_of(tile) == nullptr)
       return fail(EAS_ERR_UNSUPPORTED, "no %dx%d tile for this GEMM (512 columns: N %% 512 == 0, a plain or GELU epilogue and row-aligned output; 64, 96, 160, 192, 224: no gated epilogue; 96, 160, 192, 224: row-aligned output)", kTiles[tile].rows, kTiles[tile].cols);
   } else if (g.force_tile == TILE_AUTO) {
-    tile = pick_tile(g.M, L.N, kb, g.splits, budget, plain, [&](int t) { return kernel_of(t) != nullptr && (t != TILE_WIDE || k_total >= 2048); });
+    // The wide tile's figures hold at the power cap, where its fewer operand bytes buy clock; on up to three quarters of the SMs
+    // the board stays below it and the pair tiles are faster (M = 9000, N = 8192, K = 8192 on 46 SMs: 1050 us wide, 976 as 256x256;
+    // M = 18464, N = 1024, K = 4096 on 37: 5 %).  GELU in its exposed epilogue costs it everywhere (5120 x 5120, M = 9000: on 46 SMs
+    // 838 us wide, 713 as 256x224; on all, M = 8192, 5 %).
+    const bool wide_pays = k_total >= 2048 && g.act == ACT_NONE && 4 * budget > 3 * g_device_sms;
+    tile = pick_tile(g.M, L.N, kb, g.splits, budget, plain, [&](int t) { return kernel_of(t) != nullptr && (t != TILE_WIDE || wide_pays); });
 #ifdef EAS_GEMM_FORCE_TILE   // calibration builds only: this shape wherever it exists
     if (budget >= 2 && kernel_of(EAS_GEMM_FORCE_TILE) != nullptr) tile = EAS_GEMM_FORCE_TILE;
 #endif
@@ -1230,6 +1236,7 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
     return fail(EAS_ERR_INVALID_ARG, "data / out_embeddings must be 16-byte aligned");
   const int budget = sm_budget == 0 ? e->sm_count : sm_budget;
   g_overlap_launches = budget == e->sm_count;
+  g_device_sms = e->sm_count;
   const eas_arch_config& c = e->cfg;
   const int32_t* cu = in->cu_seqlens_host;
   const int d = c.d_model;
@@ -1768,6 +1775,7 @@ static eas_status resolve_budget(int32_t sm_budget, int* budget) {
   if (sm_budget < 0 || sm_budget > sm_count) return fail(EAS_ERR_INVALID_ARG, "sm_budget %d outside 0..%d", sm_budget, sm_count);
   *budget = sm_budget == 0 ? sm_count : sm_budget;
   g_overlap_launches = *budget == sm_count;
+  g_device_sms = sm_count;
   return EAS_OK;
 }
 
