@@ -171,6 +171,10 @@ eas_status eas_encode_microbatch_static(eas_encoder* enc, const eas_packed_input
 eas_status eas_encoder_status(eas_encoder* enc, void* stream);
 
 /* Number of kernel launches the last eas_encode_microbatch enqueued. */
+/* For tests: every GEMM of the forward pass takes this tile shape (numbered as in eas_kernel_gemm_tile) where it has a kernel of
+ * that shape, and chooses as usual elsewhere.  0 (default): choose.  The results do not depend on it. */
+eas_status eas_encoder_set_gemm_tile(eas_encoder* enc, int32_t tile_shape);
+
 int32_t eas_encoder_last_launch_count(const eas_encoder* enc);
 
 /* Selects the attention kernel: 0 = default (tcgen05, probabilities kept in tensor memory); 1 = register-tile
@@ -285,6 +289,12 @@ eas_status eas_attention_plan(const int32_t* cu_seqlens_host, int32_t n_items, i
 eas_status eas_kernel_attention(const void* qkv, void* out, const int32_t* cu_seqlens_host, int32_t n_items,
                                 int32_t n_heads, int32_t head_dim, int32_t sm_budget, void* stream, int32_t impl,
                                 uint32_t* status_dev);
+
+/* The default attention kernel with the plan fixed (as eas_attention_plan returns it; plan[2] up to plan[0]) instead of chosen by
+ * the host.  The output does not depend on the plan; the tests use this to check exactly that. */
+eas_status eas_kernel_attention_plan(const void* qkv, void* out, const int32_t* cu_seqlens_host, int32_t n_items,
+                                     int32_t n_heads, int32_t head_dim, int32_t sm_budget, void* stream, const int32_t* plan,
+                                     uint32_t* status_dev);
 
 #ifdef __cplusplus
 }

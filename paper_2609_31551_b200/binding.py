@@ -18,7 +18,7 @@ EXPORTED_SYMBOLS = [
     "eas_encode_microbatch", "eas_encode_microbatch_static", "eas_encoder_status", "eas_encoder_last_launch_count", "eas_encoder_set_attention_impl",
     "eas_encoder_set_graph_mode", "eas_encoder_graph_stats", "eas_encoder_enable_timing", "eas_encoder_timing_read", "eas_last_error", "eas_encoder_destroy", "eas_kernel_gemm", "eas_kernel_gemm_tile", "eas_kernel_norm", "eas_kernel_attention",
     "eas_encoder_set_split_k", "eas_encoder_set_norm_fold", "eas_sm_partition_create", "eas_sm_partition_sm_count", "eas_sm_partition_stream", "eas_sm_partition_destroy",
-    "eas_attention_plan",
+    "eas_attention_plan", "eas_kernel_attention_plan", "eas_encoder_set_gemm_tile",
 ]
 
 
@@ -106,6 +106,11 @@ def load_library():
     lib.eas_kernel_attention.restype = C.c_int
     lib.eas_kernel_attention.argtypes = [C.c_void_p, C.c_void_p, C.POINTER(C.c_int32), C.c_int32, C.c_int32, C.c_int32,
                                          C.c_int32, C.c_void_p, C.c_int32, C.c_void_p]
+    lib.eas_kernel_attention_plan.restype = C.c_int
+    lib.eas_kernel_attention_plan.argtypes = [C.c_void_p, C.c_void_p, C.POINTER(C.c_int32), C.c_int32, C.c_int32, C.c_int32,
+                                              C.c_int32, C.c_void_p, C.POINTER(C.c_int32), C.c_void_p]
+    lib.eas_encoder_set_gemm_tile.restype = C.c_int
+    lib.eas_encoder_set_gemm_tile.argtypes = [C.c_void_p, C.c_int32]
     lib.eas_attention_plan.restype = C.c_int
     lib.eas_attention_plan.argtypes = [C.POINTER(C.c_int32), C.c_int32, C.c_int32, C.c_int32, C.POINTER(C.c_int32)]
     lib.eas_sm_partition_create.restype = C.c_int
@@ -263,6 +268,10 @@ class Encoder:
         """eas_encoder_set_norm_fold: the blocks' normalisations inside the GEMMs around them (default off)."""
         _check(self.lib.eas_encoder_set_norm_fold(self.handle, 1 if on else 0))
 
+    def set_gemm_tile(self, tile_shape: int):
+        """eas_encoder_set_gemm_tile (tests): this tile shape for every GEMM that has it; 0 = choose."""
+        _check(self.lib.eas_encoder_set_gemm_tile(self.handle, tile_shape))
+
     def set_graph_mode(self, on: bool):
         """eas_encoder_set_graph_mode: replay captured forward passes for repeated micro-batch shapes.  Needs a
         non-default stream, and the same data / cu_seqlens_dev / out / workspace tensors from call to call."""
@@ -356,14 +365,18 @@ def kernel_norm(x, gamma, beta, kind, eps, out_fp32=False, sm_budget=0, stream=N
     return y
 
 
-def kernel_attention(qkv, cu_seqlens_host, n_heads, head_dim, sm_budget=0, stream=None, impl=0):
+def kernel_attention(qkv, cu_seqlens_host, n_heads, head_dim, sm_budget=0, stream=None, impl=0, plan=None):
+    """eas_kernel_attention (eas_kernel_attention_plan when `plan`, three ints as of attention_plan, is given)."""
     lib = load_library()
     cu = np.ascontiguousarray(cu_seqlens_host, dtype=np.int32)
     T = qkv.shape[0]
     out = torch.empty((T, n_heads * head_dim), dtype=torch.bfloat16, device=qkv.device)
     status = torch.zeros(4, dtype=torch.int32, device=qkv.device)
-    _check(lib.eas_kernel_attention(qkv.data_ptr(), out.data_ptr(), cu.ctypes.data_as(C.POINTER(C.c_int32)), len(cu) - 1,
-                                    n_heads, head_dim, sm_budget, _stream_ptr(stream), impl, status.data_ptr()))
+    args = (qkv.data_ptr(), out.data_ptr(), cu.ctypes.data_as(C.POINTER(C.c_int32)), len(cu) - 1, n_heads, head_dim, sm_budget, _stream_ptr(stream))
+    if plan is not None:
+        _check(lib.eas_kernel_attention_plan(*args, (C.c_int32 * 3)(*plan), status.data_ptr()))
+    else:
+        _check(lib.eas_kernel_attention(*args, impl, status.data_ptr()))
     return out, status
 
 

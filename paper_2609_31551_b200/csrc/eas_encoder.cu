@@ -162,6 +162,7 @@ struct eas_encoder {
   std::vector<Layer> layers;
   int attn_impl = 0;
   int split_k = 0;            // small micro-batches split the K loop of the residual GEMMs (eas_encoder_set_split_k)
+  int gemm_tile = 0;          // tests: this tile shape for every GEMM that has it (eas_encoder_set_gemm_tile)
   int fold = 0;               // 1: the blocks' normalisations are folded into the GEMMs around them (eas_encoder_set_norm_fold)
   int last_launches = 0;
   uint32_t* last_status = nullptr;
@@ -570,6 +571,13 @@ extern "C" eas_status eas_encoder_set_norm_fold(eas_encoder* enc, int32_t on) {
   return EAS_OK;
 }
 
+extern "C" eas_status eas_encoder_set_gemm_tile(eas_encoder* enc, int32_t tile_shape) {
+  if (enc == nullptr) return fail(EAS_ERR_INVALID_ARG, "encoder is null");
+  if (tile_shape < 0 || tile_shape >= TILE_COUNT) return fail(EAS_ERR_INVALID_ARG, "tile_shape %d outside 0..%d", tile_shape, TILE_COUNT - 1);
+  enc->gemm_tile = tile_shape;
+  return EAS_OK;
+}
+
 extern "C" int32_t eas_encoder_last_launch_count(const eas_encoder* enc) { return enc ? enc->last_launches : 0; }
 
 // ------------------------------------------------------------------------------------ workspace plan
@@ -706,7 +714,8 @@ struct GemmCall {
   const float2* rope_cs = nullptr;
   int reverse = 0;             // walk the tiles last to first
   int w_const = 1;             // the weights are constant (set at create time): their loads may start before the stream's earlier work ends
-  int force_tile = TILE_AUTO;  // others: tests
+  int force_tile = TILE_AUTO;  // others: tests; an error where the GEMM has no such kernel
+  int prefer_tile = TILE_AUTO; // others: tests; only where it has one
   int splits = 1;              // split K (see GemmParams::splits); the partial sums of splits 1.. go to `part`
   float* part = nullptr;       // [(splits - 1) * part_rows, N] fp32
   int64_t part_rows = 0;
@@ -737,7 +746,7 @@ struct GemmCall {
 //   M = 577:  (1024, 4096) 17.5 us -> 14.0 as 256x96;  (4096, 1024) 12.3 -> 9.9 as 128x160
 //   M = 1500: (1280, 5120) 25.4 -> 20.1 as 256x128;    (3840, 1280) 17.5 -> 14.4 as 256x160
 //   M = 5000: (1280, 5120) 57.3 -> 49.5 as 256x192
-// 128x96 and 128x192 would win another 0.2 % on average and are left out.
+// 128x96 and 128x192 would be best on a few shapes (0.2 % on average) and are left out.
 template <typename Usable>
 static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bool plain, Usable usable) {
   struct Cost { int tile; double base, per_kb, per_wave, partial; };    // us
@@ -789,14 +798,12 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
       return fail(EAS_ERR_UNSUPPORTED, "no %dx%d tile for this GEMM (512 columns: N %% 512 == 0, a plain or GELU epilogue and row-aligned output; 64, 96, 160, 192, 224: no gated epilogue; 96, 160, 192, 224: row-aligned output)", kTiles[tile].rows, kTiles[tile].cols);
   } else if (g.force_tile == TILE_AUTO) {
     // The wide tile's figures hold at the power cap, where its fewer operand bytes buy clock; on up to three quarters of the SMs
-    // the board stays below it and the pair tiles are faster (M = 9000, N = 8192, K = 8192 on 46 SMs: 1050 us wide, 976 as 256x256;
-    // M = 18464, N = 1024, K = 4096 on 37: 5 %).  GELU in its exposed epilogue costs it everywhere (5120 x 5120, M = 9000: on 46 SMs
+    // the board stays below it and the pair tiles are faster (M = 4616, N = K = 8192 on 46 SMs: 1050 us wide, 976 as 256x256;
+    // M = 18464, N = 1024, K = 4096 on 74: 179 and 164).  GELU in its exposed epilogue costs it everywhere (5120 x 5120, M = 9000: on 46 SMs
     // 838 us wide, 713 as 256x224; on all, M = 8192, 5 %).
     const bool wide_pays = k_total >= 2048 && g.act == ACT_NONE && 4 * budget > 3 * g_device_sms;
     tile = pick_tile(g.M, L.N, kb, g.splits, budget, plain, [&](int t) { return kernel_of(t) != nullptr && (t != TILE_WIDE || wide_pays); });
-#ifdef EAS_GEMM_FORCE_TILE   // calibration builds only: this shape wherever it exists
-    if (budget >= 2 && kernel_of(EAS_GEMM_FORCE_TILE) != nullptr) tile = EAS_GEMM_FORCE_TILE;
-#endif
+    if (g.prefer_tile != TILE_AUTO && kTiles[g.prefer_tile].ctas <= budget && kernel_of(g.prefer_tile) != nullptr) tile = g.prefer_tile;
   }
   const int ctas = kTiles[tile].ctas, tile_n = kTiles[tile].cols;
   const bool deep = is_deep(tile);
@@ -992,8 +999,8 @@ static void attention_item_units(int n, int before, const AttnPlan& plan, int* f
 
 // Units of three tiles use an SM best but are coarse: one clip of 8192 tokens and 16 heads is 342 of them, 2.3 rounds on 148
 // SMs, and one of 1500 tokens and 20 heads is 80.  The plan takes the variant, the cut and the small unit with the shortest
-// estimated time over the CTAs, from the measured time of an 80-key step with one, two and three tiles (relative to three)
-// and 1.5 steps per unit.  Past eight rounds everything is cut into threes.  (Rows do not depend on the plan: it may follow the
+// estimated time over the CTAs, from the time of an 80-key step with one, two and three tiles (relative to three; fitted to kernel
+// times, of which clock stamps of a lone tile differ by 3 %: 0.71 and, for the variant, 0.60) and 1.5 steps per unit.  Past eight rounds everything is cut into threes.  (Rows do not depend on the plan: it may follow the
 // micro-batch and the budget.)
 // The search is host work, once per forward pass.  Every candidate is first estimated as if items of one length dealt their units
 // of one size together (closed form for whole rounds, one difference per run); then at most six of the best are walked unit by
@@ -1307,6 +1314,10 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
   int launches = 0;
   e->last_status = status;
 
+  auto gemm = [&](GemmCall& g) {
+    g.prefer_tile = e->gemm_tile;
+    return launch_gemm(g, budget, stream, status);
+  };
   e->tcls.clear();
   EAS_TRY(mark(e, EAS_KC_PREP, stream));
 
@@ -1346,13 +1357,13 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
     g1.a_rows = pl.padded_rows; g1.M = static_cast<int>(pl.padded_rows); g1.lin = &e->conv1; g1.act = ACT_GELU;
     g1.out = h1_pad; g1.ldo = d; g1.row_map = conv1_map;
     EAS_TRY(mark(e, EAS_KC_GEMM_EMBED, stream));
-    EAS_TRY(launch_gemm(g1, budget, stream, status)); ++launches;
+    EAS_TRY(gemm(g1)); ++launches;
     GemmCall g2;   // conv2 (k=3, stride 2) + GELU + position table -> residual stream
     g2.A = h1_pad; g2.a_run = d; g2.a_row_elems = d; g2.conv_stride = 2; g2.taps = 3;
     g2.a_rows = pl.padded_rows; g2.M = static_cast<int>(pl.embed_rows); g2.lin = &e->conv2; g2.act = ACT_GELU; g2.out_fp32 = 1;
     g2.out = x; g2.ldo = d; g2.row_map = row_map; g2.pos_idx = pos_idx; g2.pos = e->pos;
     EAS_TRY(mark(e, EAS_KC_GEMM_EMBED, stream));
-    EAS_TRY(launch_gemm(g2, budget, stream, status)); ++launches;
+    EAS_TRY(gemm(g2)); ++launches;
   } else {
     // patch embedding: the im2col gather is the GEMM's A producer (no patch matrix in global memory)
     EmbedGemmParams gp{};
@@ -1411,7 +1422,7 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
       if (c.pos == EAS_POS_ROPE_2D) { g.rope_cs = rope; g.rope_stride = T; g.rope_pairs = e->hd / 2; g.rope_ncols = 2 * d; g.head_dim = e->hd; }
       g.reverse = dir; dir ^= 1;
       EAS_TRY(mark(e, EAS_KC_GEMM_QKV, stream));
-      EAS_TRY(launch_gemm(g, budget, stream, status)); ++launches;
+      EAS_TRY(gemm(g)); ++launches;
     }
     EAS_TRY(mark(e, EAS_KC_ATTENTION, stream));
     EAS_TRY(launch_attention(qkv, obuf, cu, n, c.n_heads, e->hd, budget, stream, e->attn_impl, status, attn_plan, dir != 0)); ++launches;
@@ -1424,7 +1435,7 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
       if (fold) { g.fold_stats_out = stats; g.fold_xb = nbuf; g.fold_gamma = L.n2g; g.fold_rows = T; }
       g.reverse = dir; dir ^= 1;
       EAS_TRY(mark(e, EAS_KC_GEMM_PROJ, stream));
-      EAS_TRY(launch_gemm(g, budget, stream, status)); ++launches;
+      EAS_TRY(gemm(g)); ++launches;
     }
     if (!fold) {
       NormParams np{x, nbuf, L.n2g, L.n2b, nullptr, static_cast<int>(T), d, c.norm_eps};
@@ -1441,7 +1452,7 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
       g.out = abuf; g.ldo = c.d_mlp;
       g.reverse = dir; dir ^= 1;
       EAS_TRY(mark(e, EAS_KC_GEMM_FC1, stream));
-      EAS_TRY(launch_gemm(g, budget, stream, status)); ++launches;
+      EAS_TRY(gemm(g)); ++launches;
     }
     {
       GemmCall g;
@@ -1453,7 +1464,7 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
       }
       g.reverse = dir; dir ^= 1;
       EAS_TRY(mark(e, EAS_KC_GEMM_FC2, stream));
-      EAS_TRY(launch_gemm(g, budget, stream, status)); ++launches;
+      EAS_TRY(gemm(g)); ++launches;
     }
   }
 
@@ -1485,12 +1496,12 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
     g1.A = nbuf; g1.a_run = k_in; g1.a_row_elems = k_in; g1.a_rows = rows_in; g1.M = static_cast<int>(rows_in); g1.lin = &e->head1;
     g1.act = ACT_GELU; g1.out = abuf; g1.ldo = c.d_head_hidden;
     EAS_TRY(mark(e, EAS_KC_GEMM_HEAD, stream));
-    EAS_TRY(launch_gemm(g1, budget, stream, status)); ++launches;
+    EAS_TRY(gemm(g1)); ++launches;
     GemmCall g2;
     g2.A = abuf; g2.a_run = c.d_head_hidden; g2.a_row_elems = c.d_head_hidden; g2.a_rows = rows_in; g2.M = static_cast<int>(rows_in); g2.lin = &e->head2;
     g2.out = out_embeddings; g2.ldo = c.d_out; g2.out_fp32 = out_f32 ? 1 : 0;
     EAS_TRY(mark(e, EAS_KC_GEMM_HEAD, stream));
-    EAS_TRY(launch_gemm(g2, budget, stream, status)); ++launches;
+    EAS_TRY(gemm(g2)); ++launches;
   }
   EAS_TRY(mark(e, -1, stream));
   e->last_launches = launches;
@@ -1512,7 +1523,7 @@ static eas_status encode_cached(eas_encoder* e, const eas_packed_inputs* in, voi
   const int n = in->n_items;
   std::vector<int64_t> key;
   key.reserve(8 + 5 * static_cast<size_t>(n) + 1);
-  key.push_back(n); key.push_back(sm_budget); key.push_back(e->attn_impl * 4 + e->split_k * 2 + e->fold);
+  key.push_back(n); key.push_back(sm_budget); key.push_back((e->gemm_tile * 4 + e->attn_impl) * 4 + e->split_k * 2 + e->fold);
   key.push_back(static_cast<int64_t>(reinterpret_cast<uintptr_t>(in->data)));
   key.push_back(static_cast<int64_t>(reinterpret_cast<uintptr_t>(workspace)));
   key.push_back(static_cast<int64_t>(workspace_bytes));
@@ -1828,8 +1839,9 @@ extern "C" eas_status eas_attention_plan(const int32_t* cu, int32_t n_items, int
   return EAS_OK;
 }
 
-extern "C" eas_status eas_kernel_attention(const void* qkv, void* out, const int32_t* cu, int32_t n_items, int32_t n_heads,
-                                           int32_t head_dim, int32_t sm_budget, void* stream, int32_t impl, uint32_t* status_dev) {
+// plan_in: nullptr = the host's own choice
+static eas_status kernel_attention(const void* qkv, void* out, const int32_t* cu, int32_t n_items, int32_t n_heads, int32_t head_dim,
+                                   int32_t sm_budget, void* stream, int32_t impl, const int32_t* plan_in, uint32_t* status_dev) {
   if (qkv == nullptr || out == nullptr || cu == nullptr || status_dev == nullptr) return fail(EAS_ERR_INVALID_ARG, "a required pointer is null");
   if (n_items < 1 || n_items > EAS_MAX_ITEMS || n_heads <= 0) return fail(EAS_ERR_INVALID_ARG, "bad sizes");
   if (head_dim != 64 && head_dim != 80) return fail(EAS_ERR_UNSUPPORTED, "head_dim %d", head_dim);
@@ -1837,8 +1849,27 @@ extern "C" eas_status eas_kernel_attention(const void* qkv, void* out, const int
     if (cu[i + 1] <= cu[i]) return fail(EAS_ERR_INVALID_ARG, "cu_seqlens is not strictly increasing");
   int budget = 0;
   EAS_TRY(resolve_budget(sm_budget, &budget));
+  AttnPlan plan;
+  if (plan_in == nullptr) {
+    plan = attention_plan(cu, n_items, n_heads, budget);
+  } else {
+    if (plan_in[0] < 2 || plan_in[0] > 3 || plan_in[1] < 0 || plan_in[2] < 1 || plan_in[2] > plan_in[0])
+      return fail(EAS_ERR_INVALID_ARG, "attention plan {%d, %d, %d}", plan_in[0], plan_in[1], plan_in[2]);
+    plan.own_p = plan_in[0] == 2; plan.full_tiles = plan_in[1]; plan.small = plan_in[2];
+  }
   return launch_attention(static_cast<const bf16*>(qkv), static_cast<bf16*>(out), cu, n_items, n_heads, head_dim, budget,
-                          static_cast<cudaStream_t>(stream), impl, status_dev, attention_plan(cu, n_items, n_heads, budget));
+                          static_cast<cudaStream_t>(stream), impl, status_dev, plan);
+}
+
+extern "C" eas_status eas_kernel_attention(const void* qkv, void* out, const int32_t* cu, int32_t n_items, int32_t n_heads,
+                                           int32_t head_dim, int32_t sm_budget, void* stream, int32_t impl, uint32_t* status_dev) {
+  return kernel_attention(qkv, out, cu, n_items, n_heads, head_dim, sm_budget, stream, impl, nullptr, status_dev);
+}
+
+extern "C" eas_status eas_kernel_attention_plan(const void* qkv, void* out, const int32_t* cu, int32_t n_items, int32_t n_heads,
+                                                int32_t head_dim, int32_t sm_budget, void* stream, const int32_t* plan, uint32_t* status_dev) {
+  if (plan == nullptr) return fail(EAS_ERR_INVALID_ARG, "a required pointer is null");
+  return kernel_attention(qkv, out, cu, n_items, n_heads, head_dim, sm_budget, stream, 0, plan, status_dev);
 }
 
 #ifdef EAS_GEMM_PROFILE

@@ -62,8 +62,9 @@ constexpr int kFoldGroup = 128;                   // columns per statistics grou
 
 struct alignas(64) GemmParams {
   CUtensorMap tma_a;      // 3-D: {K-run, phase, rows}; box {64, 1, 128}.  Deep kernels: {64, rows, K/64}; box {64, 128, 2}
-  CUtensorMap tma_b;      // 2-D: {K, N}; box {64, 256} (one CTA per tile) or {64, 128} (CTA pair).  Deep: {64, N, K/64}; box {64, rows, 2}
-  CUtensorMap tma_out;    // 2-D over out: box {64 bf16 | 32 fp32, 32 rows}, 128-byte swizzle (valid if use_tma_out)
+  CUtensorMap tma_b;      // 2-D: {K, N}; box {64, weight rows of a CTA: at most 256}.  Deep: {64, N, K/64}; box {64, rows, 2}
+  CUtensorMap tma_out;    // 2-D over out (valid if use_tma_out): box {64 bf16 | 32 fp32, 32 rows}, 128-byte swizzle; {32 bf16, 32 rows},
+                          // 64-byte swizzle, where gemm_out_row says 32
   int use_tma_out;        // 1: epilogue stages 32-row sub-tiles in shared memory and stores them with TMA
   int M, N;               // rows of A walked by tiles; rows of W
   int k_blocks;           // k-steps: K / 64, or ceil(K / 128) for the deep kernels (TMA fills past K with zeros)

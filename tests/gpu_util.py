@@ -52,16 +52,16 @@ def assert_parity(gpu, ref, what=""):
     return rel, mabs
 
 
-MARGIN_LOG = os.environ.get("EAS_PARITY_LOG",
-                            os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "gpurun_out",
-                                         "parity_margins.jsonl"))
+MARGIN_LOG = os.environ.get("EAS_PARITY_LOG")      # a file that collects the margins of a test run; unset: not kept
 
 
 def record_margin(case, profile, seed, rel, mabs, **extra):
     """Appends one line (case, weight profile, input seed, row-relative error, max-abs error) to the margin log, so
     that a test run leaves the measured distance to the tolerances on record.  Never fails a test."""
+    if not MARGIN_LOG:
+        return
     try:
-        os.makedirs(os.path.dirname(MARGIN_LOG), exist_ok=True)
+        os.makedirs(os.path.dirname(os.path.abspath(MARGIN_LOG)), exist_ok=True)
         with open(MARGIN_LOG, "a") as f:
             f.write(json.dumps(dict(case=case, profile=profile, seed=seed, row_rel=rel, max_abs=mabs,
                                     rel_tol=REL_TOL, abs_tol=ABS_TOL, **extra)) + "\n")

@@ -244,3 +244,21 @@ def test_item_is_untouched_by_a_non_finite_neighbour(case):
     rows = np.concatenate([[0], np.cumsum([S.out_tokens_per_item(cfg, s) for s in shapes])])
     assert torch.isnan(got[rows[1]:rows[2]].float()).all()
     assert torch.equal(got[:rows[1]], want[:rows[1]]) and torch.equal(got[rows[2]:], want[rows[2]:])
+
+
+@pytest.mark.parametrize("case", ["c1_2layers", "c2_2layers", "c4_2layers"])
+@pytest.mark.parametrize("split", [False, True])
+def test_every_gemm_tile_shape_gives_the_same_bits_in_the_forward_pass(case, split):
+    """The GEMMs that the single-kernel entry point cannot issue, with their tile shape fixed: convolutions through a row map
+    with a position table (shallow 64- and 128-column tiles), rotary epilogues, and residual GEMMs that split K."""
+    name, over, shapes = CASES[case]
+    cfg = S.get_config(name, **over)
+    w, enc = _make(cfg)
+    enc.set_split_k(split)
+    items = S.make_items(cfg, shapes, seed=2060)
+    _, want = G.run_gpu(enc, cfg, items)
+    for tile in range(1, 13):
+        enc.set_gemm_tile(tile)
+        for budget in (0, 7):
+            _, got = G.run_gpu(enc, cfg, items, sm_budget=budget)
+            assert torch.equal(got, want), (tile, budget)

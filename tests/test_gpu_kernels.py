@@ -273,10 +273,10 @@ def test_attention_ctas_leave_nothing_behind_for_their_successors(hd, impl):
 
 @pytest.mark.parametrize("H", [1, 2, 5, 16])
 def test_attention_dual_head_units(H):
-    """head_dim 64, items with an odd number of 128-row query tiles: their last tiles of two adjacent heads share a
-    unit (with an odd head count the last head's tile stays alone); items with an even count in the same launch keep
-    the ordinary units.  The tcgen05 kernel must agree with the oracle and, bit for bit, with itself at another budget;
-    the register-tile kernel (impl 1) has no such units and serves as a second opinion."""
+    """head_dim 64, items of one to five 128-row query tiles a head in one launch, so that units of two and three tiles span
+    the last tile of one head and the first of the next, with 1 to 16 heads.  The default kernel must agree with the oracle
+    and, bit for bit, with itself at another budget; the register-tile kernel (impl 1), whose units stay inside a head, serves
+    as a second opinion."""
     import paper_2609_31551_b200 as P
     hd, lens = 64, [577, 65, 640, 320, 577, 128, 1]
     rng = np.random.Generator(np.random.PCG64(900 + H))
@@ -302,9 +302,9 @@ def test_attention_dual_head_units(H):
 
 @pytest.mark.parametrize("H", [1, 3])
 def test_attention_head_dim_80_key_tile_edges(H):
-    """head_dim 80 runs on 112-key tiles with one issuer thread per warpgroup: item lengths around the multiples of 112
-    and of 128 (query tiles stay 128 rows), single-tile items whose second warpgroup idles, and few CTAs for many units
-    (long per-CTA unit sequences, look-ahead across unit boundaries)."""
+    """head_dim 80: item lengths around the multiples of 112 and of 128 (query tiles are 128 rows; the last of the 80-key steps
+    holds 1 to 80 keys), single-tile items beside which the other warpgroups idle, and few CTAs for many units (long per-CTA unit
+    sequences, look-ahead across unit boundaries)."""
     import paper_2609_31551_b200 as P
     hd, lens = 80, [112, 113, 224, 225, 336, 1, 127, 128, 129, 257, 640, 1000, 16, 111]
     rng = np.random.Generator(np.random.PCG64(1200 + H))
@@ -455,3 +455,35 @@ def test_gemm_choice_on_a_share_keeps_up_with_the_pair_tile(M, N, K, act, budget
             e1.synchronize()
             best[shape] = min(best[shape], e0.elapsed_time(e1))
     assert best[0] <= 1.08 * best[2], best
+
+
+@pytest.mark.parametrize("hd", [64, 80])
+@pytest.mark.parametrize("H,lens", [(1, [79, 80, 81]), (3, [640, 240, 161, 160, 1]), (5, [577, 400, 129])])
+def test_attention_plans_agree_bit_for_bit(hd, H, lens):
+    """Both variants of the kernel under every kind of cut: all full units, none, and a change from full to small units on an
+    item's border, inside an item and inside a head, with small units of one tile up to a full one's.  Held against the oracle
+    once; the other plans must give the same bits."""
+    import paper_2609_31551_b200 as P
+    rng = np.random.Generator(np.random.PCG64(hd + H))
+    T, d = sum(lens), H * hd
+    qkv = _bf16_exact(rng, (T, 3 * d))
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    q = O._t(qkv)
+    ref = torch.cat([O.attention_one_item(q[a:b, :d].reshape(-1, H, hd), q[a:b, d:2 * d].reshape(-1, H, hd),
+                                          q[a:b, 2 * d:].reshape(-1, H, hd)) for a, b in zip(cu[:-1], cu[1:])])
+    dev, first = _dev(qkv), None
+    tiles = H * sum(-(-S // 128) for S in lens)
+    longest = H * -(-max(lens) // 128)
+    for per_unit in (2, 3):
+        for cut in sorted({0, 1, per_unit, per_unit + 1, longest - 1, longest, longest + 1, tiles - 1, 1 << 30}):
+            for small in range(1, per_unit + 1):
+                for budget in (0, 1, 3):
+                    out, status = P.kernel_attention(dev, cu, H, hd, sm_budget=budget, plan=(per_unit, cut, small))
+                    torch.cuda.synchronize()
+                    assert int(status[0]) == 0
+                    if first is None:
+                        first = out
+                        assert (first.double().cpu() - ref).abs().max() <= 2e-2      # as in test_attention_block_diagonal
+                    assert torch.equal(out, first), (per_unit, cut, small, budget)
+    with pytest.raises(P.EasError):
+        P.kernel_attention(dev, cu, H, hd, plan=(3, 0, 4))

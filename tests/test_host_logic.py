@@ -241,3 +241,12 @@ def test_attention_plan_is_the_best_cut_and_cheap(lib):
         P.attention_plan(cu, 16, 148)
         best_us = min(best_us, (time.perf_counter() - t0) * 1e6)
     assert best_us < 20.0, best_us
+
+
+def test_attention_plan_takes_both_variants_and_a_mixed_cut(lib):
+    """What the host chooses on 148 SMs for the lengths of the workload: which variant a later change of its figures reaches."""
+    import paper_2609_31551_b200 as P
+    assert P.attention_plan([0, 577], 16, 148)[0] == 2
+    assert P.attention_plan(np.arange(33) * 577, 16, 148) == (3, 1 << 30, 1)
+    per_unit, cut, small = P.attention_plan([0, 8192], 16, 148)
+    assert per_unit == 3 and 0 < cut < 1024 and small == 2
