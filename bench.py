@@ -50,7 +50,7 @@ def other_rooflines(cfg, shapes, f, acc, n_prof, peaks):
     if 5 in acc and acc[5][0] > 0:
         t = acc[5][0] / n_prof * 1e-3
         tf = f["attention"] / t / 1e12
-        out.append({"kernel": "attn_tc_kernel", "bound": "tensor", "achieved": tf, "peak": peaks["burst"], "unit": "TFLOP/s",
+        out.append({"kernel": "attn_rr_kernel", "bound": "tensor", "achieved": tf, "peak": peaks["burst"], "unit": "TFLOP/s",
                     "frac": tf / peaks["burst"], "frac_burst": tf / peaks["burst"], "frac_sustained": tf / peaks["sustained"],
                     "launches_per_step": acc[5][1] // n_prof})
     if 3 in acc and acc[3][0] > 0:
