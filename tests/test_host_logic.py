@@ -234,13 +234,18 @@ def test_attention_plan_is_the_best_cut_and_cheap(lib):
         ratios.append(_walk_attention_plan(lens, heads, budget, plan) / best)
     assert max(ratios) <= 1.05 and np.mean(ratios) <= 1.005, (max(ratios), np.mean(ratios))
 
+    def best_of(fn):
+        best = float("inf")
+        for _ in range(200):
+            t0 = time.perf_counter()
+            fn()
+            best = min(best, time.perf_counter() - t0)
+        return best
+
     cu = (np.arange(129) * 64).astype(np.int32)
-    best_us = float("inf")
-    for _ in range(200):
-        t0 = time.perf_counter()
-        P.attention_plan(cu, 16, 148)
-        best_us = min(best_us, (time.perf_counter() - t0) * 1e6)
-    assert best_us < 20.0, best_us
+    unit = best_of(lambda: sum(range(1000)))            # the machine's speed of the moment
+    cost = min(best_of(lambda: P.attention_plan(cu, 16, 148)) / unit for _ in range(3))
+    assert cost < 3.0, cost                             # about 1.5; walking every candidate 3.3 and more
 
 
 def test_attention_plan_takes_both_variants_and_a_mixed_cut(lib):
