@@ -267,7 +267,8 @@ eas_status eas_kernel_gemm(const void* A, const void* W, const void* bias, void*
  * 1 = one CTA per 128x256 tile, 2 = a CTA pair per 256x256 tile, 3 = a CTA pair per 256x512 tile (needs N % 512 == 0,
  * act 0 or 1; EAS_ERR_UNSUPPORTED otherwise), 4 = one CTA per 128x128 tile, 5 = one CTA per 128x64 tile (act 0 or 1),
  * 6, 7 = one CTA per 128x160, 128x224 tile (act 0 or 1), 8..12 = a CTA pair per 256x96, 256x128, 256x160, 256x192, 256x224
- * tile (act 0 or 1, except 256x128).  All shapes accumulate over K in the same order, so their results are bit-identical; the tests use this to check exactly that.
+ * tile (act 0 or 1, except 256x128), 13..17 = a CTA pair per 128x64, 128x96, 128x128, 128x160, 128x224 tile (act 0 or 1 with bf16
+ * output, act 0 with fp32).  All shapes accumulate over K in the same order, so their results are bit-identical; the tests use this to check exactly that.
  * With sm_budget 1 the argument is ignored. */
 eas_status eas_kernel_gemm_tile(const void* A, const void* W, const void* bias, void* out, const float* resid,
                                 int32_t M, int32_t N, int32_t K, int32_t act, int32_t out_fp32, int32_t sm_budget,

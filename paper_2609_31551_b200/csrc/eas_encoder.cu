@@ -99,25 +99,26 @@ static eas_status make_w_tmap_deep(CUtensorMap* m, const void* w, int64_t N, int
   const uint32_t box[3] = {kBK, box_rows, 2};
   return make_tmap(m, w, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
-static eas_status make_a_tmap_deep(CUtensorMap* m, const void* a, int64_t run, int64_t row_elems, int64_t rows) {
+static eas_status make_a_tmap_deep(CUtensorMap* m, const void* a, int64_t run, int64_t row_elems, int64_t rows, uint32_t box_rows) {
   const uint64_t dims[3] = {kBK, static_cast<uint64_t>(rows), static_cast<uint64_t>(run / kBK)};
   const uint64_t strides[2] = {static_cast<uint64_t>(row_elems) * 2, kBK * 2};
-  const uint32_t box[3] = {kBK, kBM, 2};
+  const uint32_t box[3] = {kBK, box_rows, 2};
   return make_tmap(m, a, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 // output [rows, ld] as a store / reduce target: 32-row boxes whose rows are 128 bytes (64 bf16 or 32 fp32)
-// (bf16_cols: 64, or 32 for narrow tiles, whose staging rows are then 64 bytes with the 64-byte swizzle)
-static eas_status make_out_tmap(CUtensorMap* m, const void* out, bool fp32, int64_t cols, int64_t ld, int64_t rows, int bf16_cols = 64) {
+// (box_cols: 64 bf16 or 32 fp32; 32 bf16 for narrow tiles, whose staging rows are then 64 bytes with the 64-byte swizzle; 16 of
+// either, unswizzled, for the odd columns of half-height tiles)
+static eas_status make_out_tmap(CUtensorMap* m, const void* out, bool fp32, int64_t cols, int64_t ld, int64_t rows, int box_cols) {
   PFN_cuTensorMapEncodeTiled_v12000 fn = get_encode_fn();
   if (fn == nullptr) return fail(EAS_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
   const cuuint64_t gdim[2] = {static_cast<cuuint64_t>(cols), static_cast<cuuint64_t>(rows)};
   const cuuint64_t gstr[1] = {static_cast<cuuint64_t>(ld) * (fp32 ? 4 : 2)};
-  const cuuint32_t box[2] = {fp32 ? 32u : static_cast<cuuint32_t>(bf16_cols), 32u};
+  const cuuint32_t box[2] = {static_cast<cuuint32_t>(box_cols), 32u};
   const cuuint32_t es[2] = {1, 1};
   CUresult r = fn(m, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(out),
                   gdim, gstr, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  !fp32 && bf16_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                  box_cols == 16 ? CU_TENSOR_MAP_SWIZZLE_NONE : !fp32 && box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                   CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(EAS_ERR_CUDA, "cuTensorMapEncodeTiled (output) failed with code %d", static_cast<int>(r));
   return EAS_OK;
@@ -323,12 +324,15 @@ static eas_status finish_linear(Linear& L) {
 
 typedef void (*GemmKernel)(GemmParams);
 // Tile shapes of the GEMM.  All accumulate every output element over K in the same order: bit-identical results.
-// N..: one CTA per 128-row tile, P..: a CTA pair per 256-row tile, and the tile's columns (SINGLE, PAIR: 256, WIDE: 512).
+// N..: one CTA per 128-row tile, P..: a CTA pair per 256-row tile, H..: a CTA pair per 128-row tile (half-height: 64 rows a
+// CTA), and the tile's columns (SINGLE, PAIR: 256, WIDE: 512).
 enum { TILE_AUTO = 0, TILE_SINGLE = 1, TILE_PAIR = 2, TILE_WIDE = 3, TILE_N128 = 4, TILE_N64 = 5, TILE_N160 = 6, TILE_N224 = 7,
-       TILE_P96 = 8, TILE_P128 = 9, TILE_P160 = 10, TILE_P192 = 11, TILE_P224 = 12, TILE_COUNT = 13 };
-struct TileShape { int ctas, rows, cols; };
+       TILE_P96 = 8, TILE_P128 = 9, TILE_P160 = 10, TILE_P192 = 11, TILE_P224 = 12,
+       TILE_H64 = 13, TILE_H96 = 14, TILE_H128 = 15, TILE_H160 = 16, TILE_H224 = 17, TILE_COUNT = 18 };
+struct TileShape { int ctas, rows, cols; bool half = false; };
 static const TileShape kTiles[TILE_COUNT] = {{0, 0, 0}, {1, 128, 256}, {2, 256, 256}, {2, 256, 512}, {1, 128, 128}, {1, 128, 64}, {1, 128, 160},
-                                             {1, 128, 224}, {2, 256, 96}, {2, 256, 128}, {2, 256, 160}, {2, 256, 192}, {2, 256, 224}};
+                                             {1, 128, 224}, {2, 256, 96}, {2, 256, 128}, {2, 256, 160}, {2, 256, 192}, {2, 256, 224},
+                                             {2, 128, 64, true}, {2, 128, 96, true}, {2, 128, 128, true}, {2, 128, 160, true}, {2, 128, 224, true}};
 // deep (up to 128 columns): two 64-wide k-blocks per stage and TMA operation (convolutions walk their taps as 64-wide
 // k-blocks and use the shallow kernels).  nullptr: no such kernel.
 template <int ACT, int OUT, bool SPLIT = false>
@@ -349,6 +353,14 @@ static GemmKernel gemm_kernel_of(int tile, bool deep) {
       if (tile == TILE_P160) return gemm_kernel<ACT, OUT, 2, 160>;
       if (tile == TILE_P192) return gemm_kernel<ACT, OUT, 2, 192>;
       if (tile == TILE_P224) return gemm_kernel<ACT, OUT, 2, 224>;
+      if constexpr (!(ACT == ACT_GELU && OUT == OUT_F32)) {
+        if (kTiles[tile].half && !deep) return nullptr;
+        if (tile == TILE_H64) return gemm_kernel<ACT, OUT, 2, 64, 2, false, true>;
+        if (tile == TILE_H96) return gemm_kernel<ACT, OUT, 2, 96, 2, false, true>;
+        if (tile == TILE_H128) return gemm_kernel<ACT, OUT, 2, 128, 2, false, true>;
+        if (tile == TILE_H160) return gemm_kernel<ACT, OUT, 2, 160, 2, false, true>;
+        if (tile == TILE_H224) return gemm_kernel<ACT, OUT, 2, 224, 2, false, true>;
+      }
     }
   }
   return nullptr;
@@ -747,13 +759,25 @@ struct GemmCall {
 //   M = 1500: (1280, 5120) 25.4 -> 20.1 as 256x128;    (3840, 1280) 17.5 -> 14.4 as 256x160
 //   M = 5000: (1280, 5120) 57.3 -> 49.5 as 256x192
 // 128x96 and 128x192 would be best on a few shapes (0.2 % on average) and are left out.
+//
+// Half-height tiles pull 64 rows of A and half the weight rows per SM and k-block, less than any other shape of their width: 112 rows
+// as 128x96 against 176 as 256x96 and 192 as 128x64.  They are for launches of one wave (with more, the wider tiles' fewer operand bytes
+// per output win), fitted to 190 shapes forced with weights that rotate through memory.  On a share of the SMs a pair is set up
+// behind the predecessor (kShareUs more); with fewer than eight k-blocks they pay only while half the SMs suffice (M = 784, N = 768, K = 256: 4.0 us
+// as 128x96, 3.5 as 128x64; M = 196, N = 256: 3.5 and 3.8).  (N, K) on 148 SMs, best other shape -> half-height:
+//   M = 577:  (1024, 4096) 14.5 us as 128x256 ... 14.9 as 256x96 -> 10.7 as 128x96;  (1024, 1024) 6.4 -> 6.1
+//   M = 468:  (1280, 5120) 17.8 -> 12.5;  (1280, 1280) 7.1 -> 6.5;  (3840, 1280) 8.5 -> 8.2 as 128x224
+//   M = 196:  (256, 1024) 5.8 -> 4.5 as 128x64
 template <typename Usable>
 static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bool plain, Usable usable) {
+  constexpr double kShareUs = 1.05;
   struct Cost { int tile; double base, per_kb, per_wave, partial; };    // us
   static const Cost costs[] = {{TILE_SINGLE, 5.24, 0.351, 0.52, 0.87}, {TILE_PAIR, 6.44, 0.323, 0.25, 0.92}, {TILE_WIDE, 4.81, 0.586, 5.1, 0.89},
                                {TILE_N128, 3.91, 0.228, 0.45, 0.95}, {TILE_N64, 3.48, 0.173, 0.20, 1.0}, {TILE_N160, 4.61, 0.265, 0.31, 0.92},
                                {TILE_N224, 5.02, 0.329, 0.29, 0.88}, {TILE_P96, 4.66, 0.163, 0.13, 0.79}, {TILE_P128, 5.07, 0.181, 0.28, 0.84},
-                               {TILE_P160, 5.20, 0.212, 0.48, 0.80}, {TILE_P192, 5.52, 0.250, 0.34, 0.85}, {TILE_P224, 5.98, 0.291, 0.20, 0.84}};
+                               {TILE_P160, 5.20, 0.212, 0.48, 0.80}, {TILE_P192, 5.52, 0.250, 0.34, 0.85}, {TILE_P224, 5.98, 0.291, 0.20, 0.84},
+                               {TILE_H64, 3.19, 0.120, 0.0, 0.69}, {TILE_H96, 3.66, 0.122, 0.0, 0.78}, {TILE_H128, 3.83, 0.132, 0.0, 0.70},
+                               {TILE_H160, 4.27, 0.140, 0.0, 0.86}, {TILE_H224, 4.77, 0.174, 0.0, 0.86}};
   int tile = TILE_SINGLE;
   double best = 0.0;
   for (const Cost& c : costs) {
@@ -761,10 +785,12 @@ static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bo
     if (t.ctas > budget || !usable(c.tile)) continue;
     const int64_t slots = budget / t.ctas;
     const int64_t tiles = ((M + t.rows - 1) / t.rows) * ((N + t.cols - 1) / t.cols) * splits;
+    if (t.half && tiles > (kb < 8 ? slots / 2 : slots)) continue;
     const int64_t rem = tiles % slots;
     const double waves = static_cast<double>(tiles / slots) + (rem != 0 ? c.partial + (1.0 - c.partial) * static_cast<double>(rem) / static_cast<double>(slots) : 0.0);
     const double shallow = t.cols <= 128 && !plain ? 1.08 : 1.0;       // convolutions: no deep stages (128x64 +14 %, 256x128 +7 %, 128x128 +5 %)
-    const double cost = c.base + waves * (kb * c.per_kb * shallow + c.per_wave);
+    double cost = c.base + waves * (kb * c.per_kb * shallow + c.per_wave);
+    if (t.half) cost = 1.02 * (cost + (budget < g_device_sms ? kShareUs : 0.0));      // 2 % in hand: what the fit is off by
     if (best == 0.0 || cost < best) { best = cost; tile = c.tile; }
   }
   return tile;
@@ -782,11 +808,12 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
     return fail(EAS_ERR_UNSUPPORTED, "a folded normalisation needs a plain GEMM with row-aligned output and K %% %d == 0", kFoldGroup);
   const int out_mode = fold_out ? 2 : (g.out_fp32 ? 1 : 0);
   const bool plain = g.conv_stride == 1 && g.taps == 1;
-  auto is_deep = [&](int t) { return plain && kTiles[t].cols <= 128; };
+  auto is_deep = [&](int t) { return plain && (kTiles[t].cols <= 128 || kTiles[t].half); };
   auto kernel_of = [&](int t) -> GemmKernel {       // nullptr: this GEMM has no kernel of that shape
     // wide tiles: the output splits evenly into 512-column blocks; they and the odd widths: TMA-stored epilogue only
     if (t == TILE_WIDE && (!tma_out || L.N % 512 != 0)) return nullptr;
-    if (gemm_alt(kTiles[t].cols) && !tma_out) return nullptr;
+    if ((gemm_alt(kTiles[t].cols) || kTiles[t].half) && !tma_out) return nullptr;
+    if (kTiles[t].half && g.fold_stats != nullptr) return nullptr;      // (its last 16 columns read 32 of the folded constants)
     return gemm_kernel_for(g.act, out_mode, t, is_deep(t), g.splits > 1);
   };
   const int64_t k_total = g.a_run * g.taps;
@@ -795,7 +822,7 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
   if (g.force_tile != TILE_AUTO && (kTiles[g.force_tile].ctas == 1 || budget >= 2)) {
     tile = g.force_tile;
     if (kernel_of(tile) == nullptr)
-      return fail(EAS_ERR_UNSUPPORTED, "no %dx%d tile for this GEMM (512 columns: N %% 512 == 0, a plain or GELU epilogue and row-aligned output; 64, 96, 160, 192, 224: no gated epilogue; 96, 160, 192, 224: row-aligned output)", kTiles[tile].rows, kTiles[tile].cols);
+      return fail(EAS_ERR_UNSUPPORTED, "no %dx%d tile for this GEMM (512 columns: N %% 512 == 0, a plain or GELU epilogue and row-aligned output; 64, 96, 160, 192, 224 and half-height: no gated epilogue; 96, 160, 192, 224 and half-height: row-aligned output of a plain GEMM)", kTiles[tile].rows, kTiles[tile].cols);
   } else if (g.force_tile == TILE_AUTO) {
     // The wide tile's figures hold at the power cap, where its fewer operand bytes buy clock; on up to three quarters of the SMs
     // the board stays below it and the pair tiles are faster (M = 4616, N = K = 8192 on 46 SMs: 1050 us wide, 976 as 256x256;
@@ -808,11 +835,11 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
   const int ctas = kTiles[tile].ctas, tile_n = kTiles[tile].cols;
   const bool deep = is_deep(tile);
   GemmParams p{};
-  if (deep) EAS_TRY(make_a_tmap_deep(&p.tma_a, g.A, g.a_run, g.a_row_elems, g.a_rows));
+  if (deep) EAS_TRY(make_a_tmap_deep(&p.tma_a, g.A, g.a_run, g.a_row_elems, g.a_rows, kTiles[tile].half ? kBM / 2 : kBM));
   else EAS_TRY(make_a_tmap(&p.tma_a, g.A, g.a_run, g.a_row_elems, g.conv_stride, g.a_rows));
   // weight rows per TMA box: the CTA's share of a 256-column accumulator, or the narrow tile's columns
   const int w_rows = std::min(tile_n, static_cast<int>(kBN)) / ctas;
-  if (gemm_alt(tile_n)) EAS_TRY(deep ? make_w_tmap_deep(&p.tma_b, L.w, L.N, L.K, w_rows) : make_w_tmap(&p.tma_b, L.w, L.N, L.K, w_rows));
+  if (gemm_alt(tile_n) || kTiles[tile].half) EAS_TRY(deep ? make_w_tmap_deep(&p.tma_b, L.w, L.N, L.K, w_rows) : make_w_tmap(&p.tma_b, L.w, L.N, L.K, w_rows));
   else p.tma_b = w_rows == 256 ? L.tmap : w_rows == 128 ? (deep ? L.tmap_half_deep : L.tmap_half) : (deep ? L.tmap_quarter_deep : L.tmap_quarter);
   p.M = g.M; p.N = L.N;
   p.kb_per_tap = static_cast<int>(g.a_run / kBK);
@@ -829,9 +856,9 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
     p.splits = g.splits;
     p.kb_per_split = p.k_blocks / g.splits;
     p.part_rows = static_cast<int>(g.part_rows);
-    EAS_TRY(make_out_tmap(&p.tma_part, g.part, true, L.N, L.N, static_cast<int64_t>(g.splits - 1) * g.part_rows));
+    EAS_TRY(make_out_tmap(&p.tma_part, g.part, true, L.N, L.N, static_cast<int64_t>(g.splits - 1) * g.part_rows, 32));
   }
-  p.m_blocks = (g.M + kBM * ctas - 1) / (kBM * ctas);
+  p.m_blocks = (g.M + kTiles[tile].rows - 1) / kTiles[tile].rows;
   p.n_blocks = (L.N + tile_n - 1) / tile_n;
   p.bias = L.b;
   p.out = g.out; p.ldo = g.ldo; p.resid = g.resid;
@@ -845,7 +872,8 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
   p.use_tma_out = tma_out ? 1 : 0;
   if (p.use_tma_out) {
     const int64_t out_cols = g.act == ACT_SWIGLU ? L.N / 2 : L.N;
-    EAS_TRY(make_out_tmap(&p.tma_out, g.out, g.out_fp32 != 0, out_cols, g.ldo, g.M, gemm_out_row(g.act, tile_n)));
+    EAS_TRY(make_out_tmap(&p.tma_out, g.out, g.out_fp32 != 0, out_cols, g.ldo, g.M, g.out_fp32 ? 32 : gemm_out_row(g.act, tile_n, kTiles[tile].half)));
+    if (kTiles[tile].half) EAS_TRY(make_out_tmap(&p.tma_out16, g.out, g.out_fp32 != 0, out_cols, g.ldo, g.M, 16));
   }
   const int tiles = p.m_blocks * p.n_blocks * p.splits;
   GemmKernel kern = kernel_of(tile);

@@ -7,7 +7,8 @@
 //               (TMA reduce-add into the fp32 residual stream); scatter epilogues (row maps) store directly
 //
 // Tile shapes (template arguments CTAS, TN, KD; the launcher picks by estimated time): one CTA per 128 x {64, 128, 160, 224,
-// 256} tile, or a CTA pair (cta_group::2) per 256 x {96, 128, 160, 192, 224, 256, 512} tile.
+// 256} tile, or a CTA pair (cta_group::2) per 256 x {96, 128, 160, 192, 224, 256, 512} or half-height 128 x {64, 96, 128, 160,
+// 224} tile.
 //
 // The grid is `sm_budget` CTAs (one per SM: the shared-memory request excludes a second resident
 // CTA) and each CTA walks tiles  blockIdx.x, blockIdx.x + gridDim.x, ...  in a fixed order; every output element is
@@ -24,7 +25,6 @@ constexpr int kBM = 128, kBN = 256, kBK = 64;
 constexpr int kEpiWarps = 8;
 constexpr int kGemmThreads = 64 + 32 * kEpiWarps + 32;   // + the second producer warp
 constexpr int kProducerBWarp = 2 + kEpiWarps;
-constexpr int kABytes = kBM * kBK * 2;            // 16 KB: 128 rows of A
 // A stage holds this CTA's 128 rows of A (16 KB) and its weight rows (all TN of them, or a pair's half) of one 64-wide
 // k-block; the ring takes 192 KB.
 // TN = 512 ("wide", CTA pairs only): the pair owns a 256x512 tile, i.e. two 256-column accumulators fed by the same
@@ -37,13 +37,22 @@ constexpr int kABytes = kBM * kBK * 2;            // 16 KB: 128 rows of A
 // TN < 256: with few tokens a launch has fewer 256-column tiles than the device has SMs and the K loop of ONE tile is the
 // kernel's time, at the rate one SM pulls operands from L2 (48 KB per 64-wide k-block of a 128x256 tile, 24 KB of a 128x64
 // or 256x128 one): more, narrower tiles shorten that loop and use the idle SMs, and the width that just fills one wave is best.
-template <int CTAS, int TN, int KD = 1> struct GemmCfg {
-  static constexpr int kBBytes = (TN / CTAS) * kBK * 2;            // per 64-wide k-block
+// HALF (half-height, CTA pairs): a pair owns 128 x TN outputs, 64 rows of A a CTA.  UMMA with M = 128 over two CTAs keeps a CTA's 64
+// rows in ALL 128 lanes of its tensor memory: lanes 0..63 hold columns 0 .. TN/2 - 1 of the rows, lanes 64..127 the others (measured:
+// 33 cycles per 128x96x16, 60 per 128x224x16, the rate of the 256-row form).  With one tile a CTA the K loop runs at the rate an
+// SM pulls operands, and no other shape needs fewer of them: M = 577, N = 1024, K = 4096: 128x96 over 110 CTAs 10.7 us (112 rows a
+// k-block and SM), 256x96 over 66 14.9 (176), 128x64 over 80 17.5 (192).
+template <int CTAS, int TN, int KD = 1, bool HALF = false> struct GemmCfg {
+  static_assert(!HALF || (CTAS == 2 && KD == 2), "half-height tiles: CTA pairs, deep stages");
+  static constexpr int kARows = HALF ? 64 : kBM;                   // rows of A per CTA
+  static constexpr int kABytes = kARows * kBK * 2;                 // per 64-wide k-block
+  static constexpr int kBBytes = (TN / CTAS) * kBK * 2;
   static constexpr int kStageBytes = (kABytes + kBBytes) * KD;
   static constexpr int kStages = 4 * 49152 / kStageBytes < 8 ? 4 * 49152 / kStageBytes : 8;          // the ring's 192 KB
   static constexpr int kAccBuffers = TN == 512 ? 1 : 2;
-  static constexpr int kAccCols = TN < kBN ? TN : kBN;             // tensor-memory columns of one accumulator
-  static constexpr int kTmemCols = TN > 128 ? 512 : TN > 64 ? 256 : 128;     // a power of two that holds the accumulators
+  static constexpr int kMmaN = TN < kBN ? TN : kBN;                // columns of one UMMA
+  static constexpr int kAccCols = HALF ? TN / 2 : kMmaN;           // tensor-memory columns of one accumulator
+  static constexpr int kTmemCols = 2 * kAccCols > 256 ? 512 : 2 * kAccCols > 128 ? 256 : 128;     // a power of two that holds the accumulators
 };
 constexpr int kMaxStages = 8;
 constexpr int kStagingOff = 4 * 49152;                         // == 6 * 32768; 8 epilogue warps x 4 KB output staging (TMA store source)
@@ -63,6 +72,7 @@ constexpr int kFoldGroup = 128;                   // columns per statistics grou
 struct alignas(64) GemmParams {
   CUtensorMap tma_a;      // 3-D: {K-run, phase, rows}; box {64, 1, 128}.  Deep kernels: {64, rows, K/64}; box {64, 128, 2}
   CUtensorMap tma_b;      // 2-D: {K, N}; box {64, weight rows of a CTA: at most 256}.  Deep: {64, N, K/64}; box {64, rows, 2}
+  CUtensorMap tma_out16;  // half-height tiles: 2-D over out, box {16 columns, 32 rows}, no swizzle
   CUtensorMap tma_out;    // 2-D over out (valid if use_tma_out): box {64 bf16 | 32 fp32, 32 rows}, 128-byte swizzle; {32 bf16, 32 rows},
                           // 64-byte swizzle, where gemm_out_row says 32
   int use_tma_out;        // 1: epilogue stages 32-row sub-tiles in shared memory and stores them with TMA
@@ -157,36 +167,38 @@ __device__ __noinline__ float2 fold_row_factors(const float2* stats, long long r
 // four-warp groups of the epilogue
 __host__ __device__ constexpr bool gemm_alt(int tn) { return tn % 128 != 0 && tn != 64; }
 // bf16 outputs of an epilogue warp's row: the columns of one output box (64, or 32 where a warp has no more)
-__host__ __device__ constexpr int gemm_out_row(int act, int tn) {
-  if (gemm_alt(tn)) return 32;
+__host__ __device__ constexpr int gemm_out_row(int act, int tn, bool half) {
+  if (half || gemm_alt(tn)) return 32;
   const int per_warp = act == ACT_SWIGLU ? tn / 4 : tn / 2;
   return per_warp >= 64 ? 64 : 32;
 }
 
 // SPLIT: the launch splits K (GemmParams::splits > 1); the ordinary instantiations keep their code free of it.
-template <int ACT, int OUT, int CTAS, int TN, int KD = 1, bool SPLIT = false>
+template <int ACT, int OUT, int CTAS, int TN, int KD = 1, bool SPLIT = false, bool HALF = false>
 __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_constant__ GemmParams p) {
-  constexpr bool kAlt = gemm_alt(TN);
+  constexpr bool kAlt = HALF || gemm_alt(TN);
+  static_assert(!HALF || (TN <= 256 && OUT != OUT_F32_FOLD), "half-height tiles: one accumulator, plain epilogues");
   static_assert(TN % 32 == 0 && TN >= 64 && (TN <= 256 || TN == 512), "tile width");
   static_assert(!kAlt || (ACT != ACT_SWIGLU && !SPLIT), "odd widths: plain tiles");
   static_assert(TN < 512 || (CTAS == 2 && ACT != ACT_SWIGLU), "wide tiles: CTA pairs, no gated epilogue");
   static_assert(TN >= 256 || OUT != OUT_F32_FOLD, "narrow tiles: no folding epilogue");
   static_assert(TN >= 128 || ACT != ACT_SWIGLU, "a gated epilogue halves the columns: 128 at least");
   static_assert(KD == 1 || (KD == 2 && TN <= kBN), "one or two 64-wide k-blocks per stage");
-  using Cfg = GemmCfg<CTAS, TN, KD>;
+  using Cfg = GemmCfg<CTAS, TN, KD, HALF>;
+  constexpr int kARows = Cfg::kARows, kABytes = Cfg::kABytes;
   constexpr int kStages = Cfg::kStages;
   static_assert(kStages <= kMaxStages, "barrier area");
   constexpr int kStageBytes = Cfg::kStageBytes;
   constexpr int kAccBuffers = Cfg::kAccBuffers;
   constexpr int kAccCols = Cfg::kAccCols;
   constexpr int kTmemCols = Cfg::kTmemCols;
-  constexpr int NW = TN / kAccCols;                // accumulators of a tile
-  constexpr int kBRows = kAccCols / CTAS;          // weight rows per CTA and accumulator
+  constexpr int NW = TN / Cfg::kMmaN;              // accumulators of a tile
+  constexpr int kBRows = Cfg::kMmaN / CTAS;         // weight rows per CTA and accumulator
   constexpr int kBAtom = kBRows * kBK * 2;         // bytes of one 64-wide k-block of those rows
   constexpr int kTileN = TN;                       // output columns of a tile
   constexpr int kHalfN = TN / 2;                   // ... of which an epilogue warp's four-warp group takes half
   // bf16 output: columns of one staging row (and of the output map's box): 64, 128-byte swizzle; 32, 64-byte swizzle
-  constexpr int kOutRow = gemm_out_row(ACT, TN);
+  constexpr int kOutRow = gemm_out_row(ACT, TN, HALF);
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   // 1024-byte alignment: the 128-byte swizzle pattern repeats every 8 rows of 128 bytes
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -249,7 +261,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
       const int tile = SPLIT ? work / n_splits : work, split = SPLIT ? work - tile * n_splits : 0;
       int mg, nb;
       tile_coords(p.reverse ? num_tiles - 1 - tile : tile, p.m_blocks, p.n_blocks, mg, nb);
-      const int mb = mg * CTAS + cta_rank;       // this CTA's 128-row block
+      const int row0 = (mg * CTAS + cta_rank) * kARows;       // this CTA's rows
       const int kb0 = split * kb_per_split, kb1 = SPLIT ? min(p.k_blocks, kb0 + kb_per_split) : p.k_blocks;
       // position of a shallow k-block: column kx of the tap that reads phase `phase` of the strided rows, `shift` rows on
       // (running counters: three integer divisions per k-block held every kernel with shallow stages at 0.34 us per k-block;
@@ -278,21 +290,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           if (KD == 2) {
             // deep stage (plain GEMM only): [A k-block 0][A k-block 1][B ...] from one 3-D box per operand
             if (CTAS == 2) {
-              if (do_a) tma_load_3d_pair(sa, &p.tma_a, &full_bar[s], 0, mb * kBM, kb * KD);
+              if (do_a) tma_load_3d_pair(sa, &p.tma_a, &full_bar[s], 0, row0, kb * KD);
               if (do_b) tma_load_3d_pair(sb, &p.tma_b, &full_bar[s], 0, nb * kTileN + cta_rank * kBRows, kb * KD);
             } else {
-              if (do_a) tma_load_3d(sa, &p.tma_a, &full_bar[s], 0, mb * kBM, kb * KD);
+              if (do_a) tma_load_3d(sa, &p.tma_a, &full_bar[s], 0, row0, kb * KD);
               if (do_b) tma_load_3d(sb, &p.tma_b, &full_bar[s], 0, nb * kTileN, kb * KD);
             }
           } else if (CTAS == 2) {
-            if (do_a) tma_load_3d_pair(sa, &p.tma_a, &full_bar[s], kx, phase, mb * kBM + shift);
+            if (do_a) tma_load_3d_pair(sa, &p.tma_a, &full_bar[s], kx, phase, row0 + shift);
             if (do_b) {
 #pragma unroll
               for (int h = 0; h < NW; ++h)
                 tma_load_2d_pair(sb + h * kBAtom, &p.tma_b, &full_bar[s], kb * kBK, nb * kTileN + h * kBN + cta_rank * kBRows);
             }
           } else {
-            if (do_a) tma_load_3d(sa, &p.tma_a, &full_bar[s], kx, phase, mb * kBM + shift);
+            if (do_a) tma_load_3d(sa, &p.tma_a, &full_bar[s], kx, phase, row0 + shift);
             if (do_b) tma_load_2d(sb, &p.tma_b, &full_bar[s], kb * kBK, nb * kTileN);
           }
         }
@@ -316,7 +328,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     // 105 cycles of issue, which bounded the narrow tiles (128x64, M = 577, N = 1024, K = 4096: 18.2 -> 15.1 us; all 128x64
     // shapes -17 %, 128x128 -6 %, 128x256 -3 %, pair and wide tiles -1 %).
     if (cta_rank == 0) {
-      constexpr uint32_t idesc = make_idesc_bf16(kBM * CTAS, kAccCols, 0, 0);
+      constexpr uint32_t idesc = make_idesc_bf16(kARows * CTAS, Cfg::kMmaN, 0, 0);
       uint32_t it = 0, tcount = 0;
       bool ok = true;
       for (int work = first_tile; work < num_work && ok; work += tile_step, ++tcount) {
@@ -383,7 +395,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
       const int tile = SPLIT ? work / n_splits : work, split = SPLIT ? work - tile * n_splits : 0;
       int mg, nb;
       tile_coords(p.reverse ? num_tiles - 1 - tile : tile, p.m_blocks, p.n_blocks, mg, nb);
-      const int mb = mg * CTAS + cta_rank;
+      const int ycoord = (mg * CTAS + cta_rank) * kARows + (HALF ? quarter & 1 : quarter) * 32;      // this warp's first row
+      const int arow = ycoord + lane;                             // row of A (== accumulator row)
       const uint32_t acc = tcount % kAccBuffers;
       const uint32_t acc_ph = (tcount / kAccBuffers) & 1u;
       if (p.use_tma_out) {
@@ -409,14 +422,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         float fold_a = 1.f, fold_b = 0.f;
         if (p.fold_stats != nullptr) {
           const float2 f = fold_row_factors(p.fold_stats, p.fold_rows, p.fold_parts, p.fold_rms, p.fold_eps,
-                                            min(mb * kBM + quarter * 32 + lane, p.M - 1));
+                                            min(arow, p.M - 1));
           fold_a = f.x; fold_b = f.y;
         }
         if (OUT == OUT_F32_FOLD) {
           // the rows this tile updates, towards L2 while the main loop runs (the epilogue reads them with plain loads)
-          const int r = mb * kBM + quarter * 32 + lane;
-          if (r < p.M) {
-            const char* base = reinterpret_cast<const char*>(p.resid + static_cast<long long>(r) * p.ldo + nb * kTileN + half * kHalfN);
+          if (arow < p.M) {
+            const char* base = reinterpret_cast<const char*>(p.resid + static_cast<long long>(arow) * p.ldo + nb * kTileN + half * kHalfN);
 #pragma unroll
             for (int i = 0; i < 4 * NW; ++i)
               if (nb * kTileN + half * kHalfN + i * 32 < p.N) asm volatile("prefetch.global.L2 [%0];" ::"l"(base + i * 128));
@@ -433,13 +445,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         constexpr int kRowBytes = OUT == OUT_BF16 ? kOutRow * 2 : 128;     // 128: 128-byte swizzle; 64: 64-byte swizzle
         uint8_t* srow = stage + lane * kRowBytes;
         const int sw = kRowBytes == 128 ? (lane & 7) : ((lane >> 1) & 3);
-        const int arow = mb * kBM + quarter * 32 + lane;
-        // this warp's chunks of 32 columns: its half of the tile, or every second one
-        const int my_chunks = kAlt ? (TN / 32 + 1 - half) / 2 : kHalfN / 32;
-        auto my_col = [&](int c) { return kAlt ? (half + 2 * c) * 32 : half * kHalfN + c * 32; };
-        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * kAccCols + my_col(0);
+        // this warp's chunks of 32 columns: its half of the tile, or every second one (half-height tiles: of the lane half's
+        // TN / 2 columns; the last chunk has 16 where TN / 2 is no multiple of 32, and what is computed behind them is not stored)
+        constexpr int kLaneCols = HALF ? TN / 2 : TN, kLaneChunks = (kLaneCols + 31) / 32;
+        constexpr bool kNarrow = HALF && kLaneCols % 32 != 0;
+        const int lane_col0 = HALF ? (quarter >> 1) * kLaneCols : 0;
+        const int my_chunks = kAlt ? (kLaneChunks + 1 - half) / 2 : kHalfN / 32;
+        auto my_col = [&](int c) { return kAlt ? lane_col0 + (half + 2 * c) * 32 : half * kHalfN + c * 32; };
+        auto narrow = [&](int c) { return kNarrow && half + 2 * c == kLaneChunks - 1; };
+        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * kAccCols + (my_col(0) - lane_col0);
         constexpr int kChunkStep = kAlt ? 64 : 32;
-        const int ycoord = mb * kBM + quarter * 32;
 
         auto finish_chunk = [&](float (&v)[32], int c) {   // bias, rotary, activation on 32 accumulator columns
           const int col0 = nb * kTileN + my_col(c);
@@ -489,13 +504,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         // where the sub-tiles go: the output (reduce-added into the fp32 residual stream), or, for the bare partial sums
         // of a later split, this split's region of the scratch matrix (plain stores)
         const bool later_split = SPLIT && OUT == OUT_F32 && split > 0;
-        const uint64_t out_map = reinterpret_cast<uint64_t>(later_split ? &p.tma_part : &p.tma_out);
+        const uint64_t wide_map = reinterpret_cast<uint64_t>(later_split ? &p.tma_part : &p.tma_out);
         const int out_y = later_split ? (split - 1) * p.part_rows + ycoord : ycoord;
         const bool out_reduce = OUT == OUT_F32 && p.resid != nullptr && !later_split;
-        auto store_subtile = [&](int x) { // one TMA store / reduce-add of the 32-row staging buffer at column x
+        auto store_subtile = [&](int x, bool cols16 = false) { // one TMA store / reduce-add of the 32-row staging buffer at column x
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
+            const uint64_t out_map = kNarrow && cols16 ? reinterpret_cast<uint64_t>(&p.tma_out16) : wide_map;
             if (out_reduce) {
               // the residual rows keep their place in L2 (evict-last): the normalisation that follows reads them there,
               // and their write-back does not compete with this launch's own traffic (measured: out-projection -5 %)
@@ -595,7 +611,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           const int kChunks = my_chunks;
           uint32_t r[32];
           __syncwarp();
-          tmem_ld_32x32(taddr, r);
+          if (kChunks > 0) tmem_ld_32x32(taddr, r);
 #pragma unroll 1
           for (int c = 0; c < kChunks; ++c) {
             tmem_ld_wait();
@@ -609,10 +625,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
             finish_chunk(v, c);
             const int col0 = nb * kTileN + my_col(c);
             staging_free();
+            if (narrow(c)) {
 #pragma unroll
-            for (int q = 0; q < 8; ++q)
-              *reinterpret_cast<float4*>(srow + ((q ^ sw) << 4)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-            if (col0 < p.N) store_subtile(col0);
+              for (int q = 0; q < 4; ++q)
+                *reinterpret_cast<float4*>(stage + lane * 64 + (q << 4)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            } else {
+#pragma unroll
+              for (int q = 0; q < 8; ++q)
+                *reinterpret_cast<float4*>(srow + ((q ^ sw) << 4)) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            }
+            if (col0 < p.N) store_subtile(col0, narrow(c));
           }
         } else {
 #pragma unroll 1
@@ -650,6 +672,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
             // 64 bf16 columns = one 128-byte staging row (one chunk per round: 32 columns, 64 bytes)
             staging_free();
             GEMM_STAMP(5 + pr * 4);
+            if (narrow(pr)) {
+#pragma unroll
+              for (int q = 0; q < 2; ++q)
+                *reinterpret_cast<uint4*>(stage + lane * 32 + (q << 4)) =
+                    make_uint4(pack_bf16x2(v0[8 * q], v0[8 * q + 1]), pack_bf16x2(v0[8 * q + 2], v0[8 * q + 3]),
+                               pack_bf16x2(v0[8 * q + 4], v0[8 * q + 5]), pack_bf16x2(v0[8 * q + 6], v0[8 * q + 7]));
+            } else
 #pragma unroll
             for (int h2 = 0; h2 < kPerRound; ++h2) {
               float (&v)[32] = h2 ? v1 : v0;
@@ -659,7 +688,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
                     make_uint4(pack_bf16x2(v[8 * q], v[8 * q + 1]), pack_bf16x2(v[8 * q + 2], v[8 * q + 3]),
                                pack_bf16x2(v[8 * q + 4], v[8 * q + 5]), pack_bf16x2(v[8 * q + 6], v[8 * q + 7]));
             }
-            if (col0 < p.N) store_subtile(col0);
+            if (col0 < p.N) store_subtile(col0, narrow(pr));
             GEMM_STAMP(6 + pr * 4);
           }
         }
@@ -675,7 +704,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
       if (!mbar_wait(&acc_full[acc], acc_ph, abort_flag)) { ok = false; break; }
       tc_fence_after_sync();
 
-      const int arow = mb * kBM + quarter * 32 + lane;            // row of A (== accumulator row)
       long long orow = arow;
       bool row_ok = arow < p.M;
       if (row_ok && p.row_map != nullptr) {

@@ -137,6 +137,33 @@ def test_gemm_narrow_tiles_agree_bit_for_bit(M, N, K, act, out_fp32):
             assert torch.equal(run(shape, budget), ref), (shape, budget)
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 32, 64), (63, 96, 64), (65, 64, 192), (129, 160, 320), (300, 256, 1024), (577, 992, 256), (260, 736, 192)])
+@pytest.mark.parametrize("act,out_fp32", [(0, False), (1, False), (0, True)])
+def test_gemm_half_height_tiles_agree_bit_for_bit(M, N, K, act, out_fp32):
+    """A CTA pair per 128 x {64, 96, 128, 160, 224} tile, 64 rows a CTA: edges of rows (a CTA or a 32-row store without
+    rows), columns (chunks of 16 and 32, N not a multiple of the tile) and K (odd numbers of 64-wide k-blocks) give the bits of the
+    128x256 tile, also in the columns behind a stored chunk of 16."""
+    import paper_2609_31551_b200 as P
+    rng = np.random.Generator(np.random.PCG64(M + N + K + act))
+    A, W, b = _dev(_bf16_exact(rng, (M, K))), _dev(_bf16_exact(rng, (N, K), 0.05)), _dev(_bf16_exact(rng, (N,), 0.5))
+    x0 = torch.from_numpy(rng.standard_normal((M, N)).astype(np.float32)).cuda() if out_fp32 else None
+
+    def run(shape, budget):
+        x = x0.clone() if x0 is not None else None
+        out, st = P.kernel_gemm(A, W, b, act=act, out_fp32=out_fp32, resid=x, out=x, sm_budget=budget, tile_shape=shape)
+        torch.cuda.synchronize()
+        assert int(st[0]) == 0
+        return out
+
+    ref = run(1, 0)
+    for shape in range(13, 18):
+        for budget in (0, 2, 5):
+            assert torch.equal(run(shape, budget), ref), (shape, budget)
+    with pytest.raises(P.EasError) as e:
+        P.kernel_gemm(A, W, b, act=2, tile_shape=14)          # no gated epilogue
+    assert e.value.status == 2
+
+
 def test_gemm_wide_tile_is_refused_where_it_does_not_exist():
     import paper_2609_31551_b200 as P
     rng = np.random.Generator(np.random.PCG64(92))
