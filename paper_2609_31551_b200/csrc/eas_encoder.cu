@@ -1214,7 +1214,40 @@ static eas_status launch_attention(const bf16* qkv, bf16* out, const int32_t* cu
   return fail(EAS_ERR_UNSUPPORTED, "head_dim %d", hd);
 }
 
-// Patch embedding: rows R of a patch block and column groups by estimated time (the result does not depend on them).
+// Patch embedding, vectors of up to kErMaxK k-blocks: patches R of a unit and column groups by estimated time (the result does not
+// depend on them): base + blocks * first + (waves - 1) * max(blocks * next, gather), us, each linear in the k-blocks.  Fitted to every (R,
+// groups in 1, 2, 4, all) forced over one image to 32, one clip of 4 to 64 frames, on 148 and 74 SMs.  Time between launch events against
+// embed_gemm_kernel: one 224 x 224 image (d 256) 21.3 -> 14.4 us, 64 of them 54 -> 33; one 336 x 336 image (d 1024) 23.2 -> 19.2, eight
+// 40 -> 33; one 252 x 364 image (d 1280) 25 -> 21, eight at native resolution 156 -> 126; 4, 16 and 64 frames 58 -> 36, 97 -> 75, 367 -> 240.
+// (32 images of 336 x 336, exactly one wave of embed_gemm_kernel's 128-patch units, 85 -> 91.)
+static eas_status launch_embed_resident(EmbedGemmParams& gp, const CUtensorMap& w_half, int budget, cudaStream_t stream) {
+  static OncePerDevice once;
+  if (once.first()) {
+    CUDA_TRY(cudaFuncSetAttribute(embed_resident_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, EmbedResidentCfg<32>::kBytes));
+    CUDA_TRY(cudaFuncSetAttribute(embed_resident_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, EmbedResidentCfg<64>::kBytes));
+    once.settled();
+  }
+  const int n_blocks = gp.N / 128;
+  const double kb = gp.k_pad / 64;
+  int rows = 32, groups = 1;
+  double best = 0.0;
+  const struct { int rows; double base, first, next, gather; } shapes[] = {{32, 14.2 + 0.35 * kb, std::max(0.5, 0.24 * kb - 0.9), 0.45 + 0.265 * kb, 0.75 + 0.565 * kb},
+                                                                           {64, 14.2 + 0.38 * kb, 2.4 + 0.11 * kb, 4.0 + 0.1 * kb, std::max(2.0, 0.9 * kb - 1.6)}};
+  for (const auto& sh : shapes)
+    for (int g = 1; g <= n_blocks; ++g) {
+      const int64_t units = static_cast<int64_t>((gp.n_patches + sh.rows - 1) / sh.rows) * g;
+      const double waves = static_cast<double>((units + budget - 1) / budget), blocks = (n_blocks + g - 1) / g;
+      const double cost = sh.base + blocks * sh.first + (waves - 1.0) * std::max(blocks * sh.next, sh.gather);
+      if (best == 0.0 || cost < best) { best = cost; rows = sh.rows; groups = g; }
+    }
+  gp.tma_w = w_half;
+  gp.col_groups = groups;
+  const int units = (gp.n_patches + rows - 1) / rows * groups;
+  return rows == 32 ? launch_kernel(embed_resident_kernel<32>, std::min(budget, units), kEgThreads, EmbedResidentCfg<32>::kBytes, stream, gp)
+                    : launch_kernel(embed_resident_kernel<64>, std::min(budget, units), kEgThreads, EmbedResidentCfg<64>::kBytes, stream, gp);
+}
+
+// Longer patch vectors: rows R of a patch block and column groups by estimated time (the result does not depend on them).
 // A unit gathers its k-blocks (G) and works off its column blocks (E: mostly the scattered fp32 stores; a later pass over K
 // adds to them), and units of a CTA overlap: G + E + (waves - 1) max(G, E), us.  Fitted to every (R, groups) forced over one
 // image to three 1344 x 1344 ones, one clip of 4 to 64 frames.  Kernel time, one 336 x 336 image (d 1024): 77 us as 5 units of
@@ -1405,11 +1438,14 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
     gp.pairs_ok = (c.patch % 2 == 0 && (reinterpret_cast<uintptr_t>(in->data) & 3) == 0) ? 1 : 0;
     for (int i = 0; i < n && gp.pairs_ok; ++i)
       if ((in->item_offset[i] & 1) != 0 || (in->item_shape[3 * i + 2] & 1) != 0) gp.pairs_ok = 0;
+    gp.chunks_ok = c.patch % 8 == 0 ? 1 : 0;      // (the data starts on a 16-byte boundary: checked above)
+    for (int i = 0; i < n && gp.chunks_ok; ++i)
+      if ((in->item_offset[i] & 7) != 0 || (in->item_shape[3 * i + 2] & 7) != 0) gp.chunks_ok = 0;
     gp.table = e->embed_table;
     gp.status = status;
     gp.items = items;
     EAS_TRY(mark(e, EAS_KC_GEMM_EMBED, stream));
-    EAS_TRY(launch_embed_gemm(gp, budget, stream));
+    EAS_TRY(gp.k_pad <= 64 * kErMaxK ? launch_embed_resident(gp, e->embed.tmap_half, budget, stream) : launch_embed_gemm(gp, budget, stream));
     ++launches;
   }
   if (c.embed_norm) {

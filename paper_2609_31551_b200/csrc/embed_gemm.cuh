@@ -1,4 +1,5 @@
-// Patch embedding as an im2col-fused GEMM for sm_100a:
+// Patch embedding as an im2col-fused GEMM for sm_100a (two kernels: embed_resident_kernel for patch vectors of up to 1216 elements, at
+// the end, and embed_gemm_kernel for longer ones, described here):
 //
 //     x[row(m), :] = patch(m) * W_emb^T + b (+ pos[posrow(m), :])        m = patch index over the micro-batch
 //
@@ -61,6 +62,7 @@ struct EmbedGemmParams {
   int merge_order;         // 0: patches in raster order; 1: merge-group-major (the four patches of a 2x2 group adjacent)
   int col_groups;          // the column blocks are dealt to this many units per patch block
   int pairs_ok;            // 1: patch edge, image widths and item offsets are even, so pixel pairs are 4-byte aligned
+  int chunks_ok;           // 1: patch edge, image widths and item offsets are multiples of 8, so eight elements of a run are 16-byte aligned
   const uint32_t* table;   // [k_pad / 2] where each pixel pair of the patch vector comes from (built once per encoder)
   uint32_t* status;
   ItemTable items;         // aux_start = patch-row prefix per item
@@ -85,6 +87,55 @@ __global__ void embed_table_kernel(uint32_t* table, int k, int k_pad, int patch,
     }
     table[j] = e;
   }
+}
+
+// Where patch m lies: its first pixel in frame-in-patch 0 of channel 0, the elements between channels and between the frames of a
+// clip (an item has fewer than 2^31 elements: checked by the host), and the image width.
+struct EgPatch { const bf16* base; int plane_stride, frame_stride, width; };
+__device__ __forceinline__ EgPatch eg_locate(const EmbedGemmParams& p, int m) {
+  const int item = find_item(p.items.aux_start, p.items.n_items, m);
+  const int local = m - p.items.aux_start[item];
+  const int H = p.items.height[item], W = p.items.width[item];
+  const int gh = H / p.patch, gw = W / p.patch;
+  const int tt = local / (gh * gw);
+  const int rem = local - tt * gh * gw;
+  int r, c;
+  if (p.merge_order) {
+    const int grp = rem >> 2, within = rem & 3;
+    const int hb = grp / (gw >> 1), wb = grp - hb * (gw >> 1);
+    r = 2 * hb + (within >> 1);
+    c = 2 * wb + (within & 1);
+  } else {
+    r = rem / gw;
+    c = rem - r * gw;
+  }
+  EgPatch e;
+  e.width = W;
+  e.plane_stride = H * W;
+  const bool clip = p.tpatch > 1 || p.items.frames[item] > 1;
+  e.frame_stride = clip ? e.plane_stride * p.channels : 0;
+  e.base = p.data + p.items.offset[item] + static_cast<long long>(tt) * p.tpatch * e.frame_stride +
+           static_cast<long long>(r) * p.patch * W + c * p.patch;
+  return e;
+}
+__device__ __forceinline__ int eg_offset(uint32_t e, int plane_stride, int frame_stride, int W) {
+  return static_cast<int>((e >> 16) & 0xFFu) * frame_stride + static_cast<int>(e >> 24) * plane_stride + static_cast<int>((e >> 8) & 0xFFu) * W +
+         static_cast<int>(e & 0xFFu);
+}
+// the pixel pair `pair` of the patch vector, whose table entry is e
+__device__ __forceinline__ uint32_t eg_load_pair(const EmbedGemmParams& p, const bf16* base, int plane_stride, int frame_stride, int W,
+                                                 uint32_t e, int pair) {
+  if (e == kEgPad) return 0u;
+  const bf16* src = base + eg_offset(e, plane_stride, frame_stride, W);
+  if (p.pairs_ok) return *reinterpret_cast<const uint32_t*>(src);
+  // odd geometry (odd patch edge, width or item offset): element loads; the second element of the pair
+  // may belong to the next run
+  const unsigned short lo = *reinterpret_cast<const unsigned short*>(src);
+  int px1 = static_cast<int>(e & 0xFFu) + 1, py1 = static_cast<int>((e >> 8) & 0xFFu), f1 = static_cast<int>((e >> 16) & 0xFFu), ch1 = static_cast<int>(e >> 24);
+  if (px1 == p.patch) { px1 = 0; if (++py1 == p.patch) { py1 = 0; if (++f1 == p.tpatch) { f1 = 0; ++ch1; } } }
+  unsigned short hi = 0;
+  if (2 * pair + 1 < p.k) hi = *reinterpret_cast<const unsigned short*>(base + (f1 * frame_stride + ch1 * plane_stride + py1 * W + px1));
+  return static_cast<uint32_t>(lo) | (static_cast<uint32_t>(hi) << 16);
 }
 
 template <int R>
@@ -207,65 +258,19 @@ __global__ void __launch_bounds__(kEgThreads, 1) embed_gemm_kernel(const __grid_
     bool ok = true;
     for (int unit = blockIdx.x; unit < n_units && ok; unit += gridDim.x) {
       const int m = unit / p.col_groups * R + row;
-      // this patch: first pixel of its top-left corner in frame-in-patch 0 of channel 0, and the strides
-      const bf16* base = p.data;
-      int plane_stride = 0, frame_stride = 0;       // elements between channels, and between frames of a clip (an item
-      int W = 0;                                    // has fewer than 2^31 elements: checked by the host)
       const bool row_ok = m < p.n_patches;
-      if (row_ok) {
-        const int item = find_item(p.items.aux_start, p.items.n_items, m);
-        const int local = m - p.items.aux_start[item];
-        const int H = p.items.height[item];
-        W = p.items.width[item];
-        const int gh = H / p.patch, gw = W / p.patch;
-        const int tt = local / (gh * gw);
-        const int rem = local - tt * gh * gw;
-        int r, c;
-        if (p.merge_order) {
-          const int grp = rem >> 2, within = rem & 3;
-          const int hb = grp / (gw >> 1), wb = grp - hb * (gw >> 1);
-          r = 2 * hb + (within >> 1);
-          c = 2 * wb + (within & 1);
-        } else {
-          r = rem / gw;
-          c = rem - r * gw;
-        }
-        plane_stride = H * W;
-        const bool clip = p.tpatch > 1 || p.items.frames[item] > 1;
-        frame_stride = clip ? plane_stride * p.channels : 0;
-        base = p.data + p.items.offset[item] + static_cast<long long>(tt) * p.tpatch * frame_stride +
-               static_cast<long long>(r) * p.patch * W + c * p.patch;
-      }
+      EgPatch e{p.data, 0, 0, 0};
+      if (row_ok) e = eg_locate(p, m);
       // the pairs of this thread in k-block kb (registers only)
       auto load_block = [&](int kb, uint32_t (&v)[4 * kChunks]) {
         const uint4* tab4 = reinterpret_cast<const uint4*>(p.table + kb * 32 + sub * (4 * kChunks));
 #pragma unroll
         for (int q = 0; q < kChunks; ++q) {
           const uint4 e4 = __ldg(tab4 + q);
-          const uint32_t e[4] = {e4.x, e4.y, e4.z, e4.w};
+          const uint32_t ent[4] = {e4.x, e4.y, e4.z, e4.w};
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            uint32_t val = 0u;
-            if (row_ok && e[j] != kEgPad) {
-              const int ch = static_cast<int>(e[j] >> 24), f = static_cast<int>((e[j] >> 16) & 0xFFu);
-              const int py = static_cast<int>((e[j] >> 8) & 0xFFu), px = static_cast<int>(e[j] & 0xFFu);
-              const bf16* src = base + (f * frame_stride + ch * plane_stride + py * W + px);
-              if (p.pairs_ok) {
-                val = *reinterpret_cast<const uint32_t*>(src);
-              } else {
-                // odd geometry (odd patch edge, width or item offset): element loads; the second element of the pair
-                // may belong to the next run
-                const unsigned short lo = *reinterpret_cast<const unsigned short*>(src);
-                int px1 = px + 1, py1 = py, f1 = f, ch1 = ch;
-                if (px1 == p.patch) { px1 = 0; if (++py1 == p.patch) { py1 = 0; if (++f1 == p.tpatch) { f1 = 0; ++ch1; } } }
-                unsigned short hi = 0;
-                if (2 * (kb * 32 + (sub * kChunks + q) * 4 + j) + 1 < p.k)
-                  hi = *reinterpret_cast<const unsigned short*>(base + (f1 * frame_stride + ch1 * plane_stride + py1 * W + px1));
-                val = static_cast<uint32_t>(lo) | (static_cast<uint32_t>(hi) << 16);
-              }
-            }
-            v[q * 4 + j] = val;
-          }
+          for (int j = 0; j < 4; ++j)
+            v[q * 4 + j] = row_ok ? eg_load_pair(p, e.base, e.plane_stride, e.frame_stride, e.width, ent[j], kb * 32 + (sub * kChunks + q) * 4 + j) : 0u;
         }
       };
       for (int pass = 0; pass < passes && ok; ++pass) {
@@ -370,6 +375,255 @@ __global__ void __launch_bounds__(kEgThreads, 1) embed_gemm_kernel(const __grid_
   if (warp == 1) {
     tc_fence_after_sync();
     tmem_dealloc(tmem_base, 512);
+  }
+  if (threadIdx.x == 0 && *abort_flag) atomicCAS(p.status, DEV_OK, DEV_ERR_WAIT_TIMEOUT);
+}
+
+// ------------------------------------------------------------------------------- vectors that stay resident
+// Patch vectors of up to kErMaxK k-blocks (1216 elements).  The same product with the operands exchanged: the UMMA's 128 rows are output
+// columns (the weight tile) and its columns are R patches.  What bounds embed_gemm_kernel is a unit's chain of latencies with few
+// patches and the second pass over K with longer vectors; here
+//   - a unit (R = 32 or 64 patches, a group of 128-column blocks) is small, so that one image fills the chip;
+//   - the whole patch vector stays in shared memory, 16 KB weight tiles run through a ring of eight or four;
+//   - an epilogue thread owns one output column, so its stores are whole 128-byte lines, and it has loaded the position rows before the
+//     accumulator is complete (one load behind each store cost a column block 8 us);
+//   - where the patches' pixels are (item, row, column, table entries) is worked out before the grid dependency resolves;
+//   - where eight elements of a pixel run lie on a 16-byte boundary (patch edges, widths and offsets that are multiples of 8) they are one load.
+// A vector that embed_gemm_kernel walks in two passes has an accumulator per pass, added in that order: the same bits.
+constexpr int kErMaxK = 19;
+constexpr int kErWBytes = 128 * 64 * 2;                 // 16 KB: 128 weight rows x 64 elements
+template <int R> struct EmbedResidentCfg {
+  static constexpr int kSlot = R * 128;                 // R patch rows x 64 elements
+  static constexpr int kWStages = R == 32 ? 8 : 4;
+  static constexpr int kWOff = kErMaxK * kSlot, kBarOff = kWOff + kWStages * kErWBytes;
+  static constexpr int kBytes = kBarOff + 512 + 1024;   // + barriers + alignment slack
+  static_assert(kBytes <= 232448 && kBytes > 116224, "one CTA per SM");
+  static_assert((2 * kErMaxK + 2 * kWStages + 4) * 8 + 8 <= 512, "barrier area");
+};
+
+template <int R>
+__global__ void __launch_bounds__(kEgThreads, 1) embed_resident_kernel(const __grid_constant__ EmbedGemmParams p) {
+  using Cfg = EmbedResidentCfg<R>;
+  constexpr int kSlot = Cfg::kSlot, kWStages = Cfg::kWStages;
+  extern __shared__ __align__(1024) uint8_t smem_raw_eg[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_eg) + 1023) & ~uintptr_t(1023));
+  uint8_t* wring = smem + Cfg::kWOff;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Cfg::kBarOff);
+  uint64_t* a_full = bars;                              // [kErMaxK] the gather warps have written the slot
+  uint64_t* a_free = a_full + kErMaxK;                  // [kErMaxK] the last UMMA that reads the slot has completed
+  uint64_t* w_full = a_free + kErMaxK;                  // [kWStages]
+  uint64_t* w_empty = w_full + kWStages;                // [kWStages]
+  uint64_t* acc_full = w_empty + kWStages;              // [2]
+  uint64_t* acc_empty = acc_full + 2;                   // [2] 8 epilogue warps
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  volatile uint32_t* abort_flag = tmem_slot + 1;
+
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const int k_blocks = p.k_pad / 64;
+  const int passes = (k_blocks + kEgMaxResident - 1) / kEgMaxResident;          // 1 or 2, dealt as in embed_gemm_kernel
+  const int pass0 = k_blocks / passes + (k_blocks % passes != 0 ? 1 : 0);       // k-blocks of the first
+  const int n_blocks = p.N / 128;
+  const int n_units = (p.n_patches + R - 1) / R * p.col_groups;
+  auto first_col = [&](int group) { return group * n_blocks / p.col_groups; };
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kErMaxK; ++s) { mbar_init(&a_full[s], kEgGatherWarps); mbar_init(&a_free[s], 1); }
+    for (int s = 0; s < kWStages; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], 1); }
+    for (int a = 0; a < 2; ++a) { mbar_init(&acc_full[a], 1); mbar_init(&acc_empty[a], 8); }
+    *abort_flag = 0;
+    mbar_fence_init();
+    tma_prefetch_desc(&p.tma_w);
+  }
+  if (warp == 1) { tmem_alloc(tmem_slot, 256); tmem_relinquish(); }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem_base = *tmem_slot;
+  if (p.early_launch) pdl_launch_dependents();
+
+  if (warp == 0) {
+    // ------------------------------------------------------------------ W producer (constant weights: no wait for earlier work yet)
+    uint32_t it = 0;
+    bool ok = true;
+    for (int unit = blockIdx.x; unit < n_units && ok; unit += gridDim.x)
+      for (int nb = first_col(unit % p.col_groups); nb < first_col(unit % p.col_groups + 1) && ok; ++nb)
+        for (int j = 0; j < k_blocks; ++j, ++it) {
+          const uint32_t s = it % kWStages;
+          if (it == kWStages) pdl_wait();               // the next wait needs the consumer, hence the earlier kernels
+          if (!warp_mbar_wait(&w_empty[s], ((it / kWStages) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+          if (elect_one()) {
+            mbar_expect_tx(&w_full[s], kErWBytes);
+            tma_load_2d(wring + s * kErWBytes, &p.tma_w, &w_full[s], j * 64, nb * 128);
+          }
+          __syncwarp();
+        }
+    if (!ok) {
+      const long long t0 = clock64();
+      while (clock64() - t0 < 4000000) {}               // let loads in flight land before the CTA retires
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ UMMA issuer
+    pdl_wait();
+    constexpr uint32_t idesc = make_idesc_bf16(128, R, 0, 0);
+    uint32_t it = 0, tcount = 0, round = 0;
+    bool ok = true;
+    for (int unit = blockIdx.x; unit < n_units && ok; unit += gridDim.x, ++round) {
+      const int nb0 = first_col(unit % p.col_groups), nb1 = first_col(unit % p.col_groups + 1);
+      for (int nb = nb0; nb < nb1 && ok; ++nb, ++tcount) {
+        const uint32_t acc = tcount & 1u;
+        if (!warp_mbar_wait(&acc_empty[acc], ((tcount >> 1) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
+        for (int j = 0; j < k_blocks; ++j, ++it) {
+          const uint32_t s = it % kWStages;
+          if (nb == nb0 && !warp_mbar_wait(&a_full[j], round & 1u, abort_flag)) { ok = false; break; }
+          if (!warp_mbar_wait(&w_full[s], (it / kWStages) & 1u, abort_flag)) { ok = false; break; }
+          tc_fence_after_sync();
+          if (elect_one()) {
+            const uint64_t wdesc = make_smem_desc(smem_u32(wring + s * kErWBytes), 16, 1024, kSwizzle128B);
+            const uint64_t pdesc = make_smem_desc(smem_u32(smem + j * kSlot), 16, 1024, kSwizzle128B);
+            const uint32_t d = tmem_base + acc * (2 * R) + (j < pass0 ? 0 : R);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) umma_bf16_ss(d, wdesc + 2 * k, pdesc + 2 * k, idesc, (k != 0 || (j != 0 && j != pass0)) ? 1u : 0u);
+            umma_commit(&w_empty[s]);
+            if (nb == nb1 - 1) umma_commit(&a_free[j]);   // the slot's last reader: the gather may refill it
+            if (j == k_blocks - 1) umma_commit(&acc_full[acc]);
+          }
+          __syncwarp();
+        }
+      }
+    }
+    // the last hand-backs are asynchronous arrivals that nothing else waits for: in before the shared memory passes on
+    for (uint32_t e = it; e < it + kWStages && ok; ++e) ok = warp_mbar_wait(&w_empty[e % kWStages], ((e / kWStages) & 1u) ^ 1u, abort_flag);
+    for (int j = 0; j < k_blocks && ok && round > 0; ++j) ok = warp_mbar_wait(&a_free[j], (round - 1) & 1u, abort_flag);
+  } else if (warp < 2 + kEgGatherWarps) {
+    // ------------------------------------------------------------------ gather: kThreadsPerRow threads per patch row
+    constexpr int kThreadsPerRow = 32 * kEgGatherWarps / R, kChunks = 8 / kThreadsPerRow;   // 16-byte chunks per thread and k-block
+    constexpr int kDepth = R == 32 ? 6 : 3;           // k-blocks whose loads are in flight
+    const int t = threadIdx.x - 64;                   // 0..255
+    const int row = t / kThreadsPerRow, sub = t % kThreadsPerRow;
+    const int sw = row & 7;
+    const bf16* base = p.data;                        // first pixel of the patch in frame-in-patch 0 of channel 0, and the strides
+    int plane_stride = 0, frame_stride = 0, W = 0;
+    bool row_ok = false;
+    auto locate = [&](int unit) {
+      const int m = unit / p.col_groups * R + row;
+      row_ok = m < p.n_patches;
+      if (!row_ok) return;
+      const EgPatch e = eg_locate(p, m);
+      base = e.base; plane_stride = e.plane_stride; frame_stride = e.frame_stride; W = e.width;
+    };
+    uint4 ent[kDepth][kChunks];                       // table entries of the next k-blocks
+    auto load_table = [&](int kb, uint4 (&e)[kChunks]) {
+#pragma unroll
+      for (int q = 0; q < kChunks; ++q) e[q] = __ldg(reinterpret_cast<const uint4*>(p.table + kb * 32 + (sub * kChunks + q) * 4));
+    };
+    auto load_pixels = [&](int kb, const uint4 (&e4)[kChunks], uint4 (&v)[kChunks]) {
+#pragma unroll
+      for (int q = 0; q < kChunks; ++q) {
+        if (p.chunks_ok) {                              // a chunk of eight elements lies inside a pixel run, on a 16-byte boundary
+          v[q] = row_ok && e4[q].x != kEgPad ? *reinterpret_cast<const uint4*>(base + eg_offset(e4[q].x, plane_stride, frame_stride, W)) : make_uint4(0u, 0u, 0u, 0u);
+          continue;
+        }
+        const uint32_t e[4] = {e4[q].x, e4[q].y, e4[q].z, e4[q].w};
+        uint32_t o[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          o[j] = row_ok ? eg_load_pair(p, base, plane_stride, frame_stride, W, e[j], kb * 32 + (sub * kChunks + q) * 4 + j) : 0u;
+        v[q] = make_uint4(o[0], o[1], o[2], o[3]);
+      }
+    };
+    if (static_cast<int>(blockIdx.x) < n_units) locate(blockIdx.x);
+#pragma unroll
+    for (int d = 0; d < kDepth; ++d)
+      if (d < k_blocks) load_table(d, ent[d]);
+    pdl_wait();
+    uint32_t round = 0;
+    bool ok = true;
+    for (int unit = blockIdx.x; unit < n_units && ok; unit += gridDim.x, ++round) {
+      if (round != 0) {
+        locate(unit);
+#pragma unroll
+        for (int d = 0; d < kDepth; ++d)
+          if (d < k_blocks) load_table(d, ent[d]);
+      }
+      uint4 buf[kDepth][kChunks];
+#pragma unroll
+      for (int d = 0; d < kDepth; ++d)
+        if (d < k_blocks) {
+          load_pixels(d, ent[d], buf[d]);
+          if (d + kDepth < k_blocks) load_table(d + kDepth, ent[d]);
+        }
+      for (int j0 = 0; j0 < k_blocks && ok; j0 += kDepth) {
+#pragma unroll
+        for (int d = 0; d < kDepth; ++d) {
+          const int j = j0 + d;
+          if (j >= k_blocks) break;
+          if (round != 0 && !warp_mbar_wait(&a_free[j], (round - 1) & 1u, abort_flag)) { ok = false; break; }
+          uint8_t* srow = smem + j * kSlot + row * 128;
+#pragma unroll
+          for (int q = 0; q < kChunks; ++q) *reinterpret_cast<uint4*>(srow + (((sub * kChunks + q) ^ sw) << 4)) = buf[d][q];
+          fence_proxy_async_smem();                   // generic-proxy stores -> visible to the tensor core's operand reads
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&a_full[j]);
+          if (j + kDepth < k_blocks) {
+            load_pixels(j + kDepth, ent[d], buf[d]);
+            if (j + 2 * kDepth < k_blocks) load_table(j + 2 * kDepth, ent[d]);
+          }
+        }
+      }
+    }
+  } else {
+    // ------------------------------------------------------------------ epilogue: a thread per output column, half of the patches a warp
+    const int quarter = warp & 3, half = (warp - 2 - kEgGatherWarps) >> 2;
+    constexpr int kHalf = R / 2;
+    pdl_wait();
+    uint32_t tcount = 0;
+    bool ok = true;
+    for (int unit = blockIdx.x; unit < n_units && ok; unit += gridDim.x) {
+      const int m0 = unit / p.col_groups * R + half * kHalf;
+      int my_row = -1, my_pos = 0;                    // of patch m0 + lane
+      if (lane < kHalf && m0 + lane < p.n_patches) {
+        my_row = p.row_map[m0 + lane];
+        if (p.pos != nullptr) my_pos = p.pos_idx[m0 + lane];
+      }
+      for (int nb = first_col(unit % p.col_groups); nb < first_col(unit % p.col_groups + 1) && ok; ++nb, ++tcount) {
+        const uint32_t acc = tcount & 1u;
+        const int col = nb * 128 + quarter * 32 + lane;
+        const float bias = __bfloat162float(p.bias[col]);
+        bf16 pos[kHalf];                              // all ahead of the stores (and of the accumulator): a load each costs an L2 round trip
+#pragma unroll
+        for (int i = 0; i < kHalf; ++i)
+          if (p.pos != nullptr) pos[i] = p.pos[static_cast<long long>(__shfl_sync(0xffffffffu, my_pos, i)) * p.N + col];
+        if (!warp_mbar_wait(&acc_full[acc], (tcount >> 1) & 1u, abort_flag)) { ok = false; break; }
+        tc_fence_after_sync();
+        const uint32_t d = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + acc * (2 * R) + half * kHalf;
+#pragma unroll
+        for (int c = 0; c < kHalf; c += 16) {
+          uint32_t v0[16], v1[16];
+          __syncwarp();
+          tmem_ld_32x16(d + c, v0);
+          if (passes > 1) tmem_ld_32x16(d + R + c, v1);
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const int orow = __shfl_sync(0xffffffffu, my_row, c + i);
+            float v = __uint_as_float(v0[i]) + bias;
+            if (p.pos != nullptr) v += __bfloat162float(pos[c + i]);
+            if (passes > 1) v = __uint_as_float(v1[i]) + v;
+            if (orow >= 0) p.x[static_cast<long long>(orow) * p.N + col] = v;
+          }
+        }
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_empty[acc]);
+      }
+    }
+  }
+
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after_sync();
+    tmem_dealloc(tmem_base, 256);
   }
   if (threadIdx.x == 0 && *abort_flag) atomicCAS(p.status, DEV_OK, DEV_ERR_WAIT_TIMEOUT);
 }

@@ -191,6 +191,22 @@ def test_fused_patch_embedding_alone(name):
         assert torch.equal(b, dev), budget
 
 
+@pytest.mark.parametrize("name,over,shapes", [("c3", dict(temporal_patch=3), [(6, 56, 84), (3, 28, 28)]), ("c0", dict(patch=32, max_pos=64), [(1, 224, 224), (1, 32, 64)]),
+                                              ("c0", dict(patch=20, max_pos=64), [(1, 100, 60), (1, 20, 20)])])
+def test_patch_embedding_of_other_vector_lengths(name, over, shapes):
+    """Patch vectors of 28, 48 and 19 k-blocks of 64 (the last the longest whose kernel keeps it resident, and padded): embeddings alone against the
+    oracle, and the same bits at budgets of one and a few SMs."""
+    cfg = S.get_config(name, n_layers=0, **over)
+    w, enc = _make(cfg)
+    items = S.make_items(cfg, shapes, seed=4200)
+    ref, _, _ = O.encode_microbatch(cfg, w, items)
+    got, dev = G.run_gpu(enc, cfg, items)
+    G.assert_parity(got, ref, f"{name} patch vector {over}")
+    for budget in (1, 3):
+        _, b = G.run_gpu(enc, cfg, items, sm_budget=budget)
+        assert torch.equal(b, dev), budget
+
+
 @pytest.mark.parametrize("name", ["c0", "c1", "c2", "c3"])
 def test_fused_patch_embedding_same_bits_for_every_block_shape(name):
     """The embedding's patch blocks (32, 64 or 128 rows) and column groups follow the micro-batch size and the budget: an
