@@ -273,8 +273,33 @@ def test_every_gemm_tile_shape_gives_the_same_bits_in_the_forward_pass(case, spl
     enc.set_split_k(split)
     items = S.make_items(cfg, shapes, seed=2060)
     _, want = G.run_gpu(enc, cfg, items)
-    for tile in range(1, 13):
+    for tile in range(1, 18):
         enc.set_gemm_tile(tile)
         for budget in (0, 7):
             _, got = G.run_gpu(enc, cfg, items, sm_budget=budget)
             assert torch.equal(got, want), (tile, budget)
+
+
+@pytest.mark.parametrize("d,hd,shape,budgets", [(128, 64, (392, 504), ()), (512, 64, (280, 336), ()), (896, 64, (196, 252), ()), (1408, 64, (224, 280), ()),
+                                                (1536, 64, (224, 280), ()), (2048, 64, (112, 140), ()), (1280, 80, (112, 140), range(112, 120))])
+def test_rotary_ends_where_the_values_begin_in_every_tile_shape(d, hd, shape, budgets):
+    """Half-height tiles have column chunks that start 16 columns off the others, so one of them can hold the last rotated key columns
+    and the first value columns.  Widths and token counts where the automatic choice is such a tile (on all SMs, or on the given
+    budgets), against the oracle and the bits of the 128x256 tile; and every other shape."""
+    cfg = S.get_config("c2", n_layers=1, d_model=d, n_heads=d // hd, d_mlp=256, d_head_hidden=256, d_out=256)
+    w, enc = _make(cfg, "sharp")
+    items = S.make_items(cfg, [(1,) + shape], seed=2080)
+    ref, _, _ = O.encode_microbatch(cfg, w, items)
+    got, auto = G.run_gpu(enc, cfg, items)
+    enc.set_gemm_tile(1)
+    _, want = G.run_gpu(enc, cfg, items)
+    G.assert_parity(got, ref, f"rotary at d {d}")
+    assert torch.equal(auto, want)
+    for tile in range(2, 18):
+        enc.set_gemm_tile(tile)
+        _, forced = G.run_gpu(enc, cfg, items)
+        assert torch.equal(forced, want), tile
+    enc.set_gemm_tile(0)
+    for budget in budgets:
+        _, share = G.run_gpu(enc, cfg, items, sm_budget=budget)
+        assert torch.equal(share, want), budget
