@@ -1214,12 +1214,31 @@ static eas_status launch_attention(const bf16* qkv, bf16* out, const int32_t* cu
   return fail(EAS_ERR_UNSUPPORTED, "head_dim %d", hd);
 }
 
+static eas_status launch_embed_blocks(EmbedGemmParams& gp, int rows, int groups, int budget, cudaStream_t stream) {
+  static OncePerDevice once;
+  if (once.first()) {
+    CUDA_TRY(cudaFuncSetAttribute(embed_gemm_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgSmemBytes));
+    CUDA_TRY(cudaFuncSetAttribute(embed_gemm_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgSmemBytes));
+    CUDA_TRY(cudaFuncSetAttribute(embed_gemm_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgSmemBytes));
+    once.settled();
+  }
+  gp.col_groups = groups;
+  const int units = (gp.n_patches + rows - 1) / rows * groups;
+  void (*kern)(EmbedGemmParams) = rows == 128 ? embed_gemm_kernel<128> : rows == 64 ? embed_gemm_kernel<64> : embed_gemm_kernel<32>;
+  return launch_kernel(kern, std::min(budget, units), kEgThreads, kEgSmemBytes, stream, gp);
+}
+
 // Patch embedding, vectors of up to kErMaxK k-blocks: patches R of a unit and column groups by estimated time (the result does not
-// depend on them): base + blocks * first + (waves - 1) * max(blocks * next, gather), us, each linear in the k-blocks.  Fitted to every (R,
-// groups in 1, 2, 4, all) forced over one image to 32, one clip of 4 to 64 frames, on 148 and 74 SMs.  Time between launch events against
-// embed_gemm_kernel: one 224 x 224 image (d 256) 21.3 -> 14.4 us, 64 of them 54 -> 33; one 336 x 336 image (d 1024) 23.2 -> 19.2, eight
-// 40 -> 33; one 252 x 364 image (d 1280) 25 -> 21, eight at native resolution 156 -> 126; 4, 16 and 64 frames 58 -> 36, 97 -> 75, 367 -> 240.
-// (32 images of 336 x 336, exactly one wave of embed_gemm_kernel's 128-patch units, 85 -> 91.)
+// depend on them): base + blocks * first + (waves - 1) * max(blocks * next, gather), us, each linear in the k-blocks, `next` at least the
+// time of a block's stores.  Fitted to every (R, groups in 1, 2, 3, 4, 5, all) forced over 76 to 73728 patches, 3 to 19 k-blocks, d 256 to
+// 2048, on 148, 111, 74 and 37 SMs, all forms in turn and L2 overwritten in between: 1.5 % behind the best form on average.
+// Short vectors (up to 7 k-blocks) leave the stores as the bound, and there embed_gemm_kernel with 128 patches and all columns in one
+// unit is the faster one once it fills its waves (d 1024, 4 k-blocks, 18432 patches: 68 and 60 us; 73728: 227 and 195): the third shape.
+// Longer ones are faster resident at every size.  us between launch events against embed_gemm_kernel: one 224 x 224 image (d 256) 24.4 ->
+// 16.4, 64 of them 53 -> 30; one 336 x 336 image (d 1024) 24 -> 18.5, eight 41 -> 35, 32 of them 91 -> 85 and on 74 SMs 144 -> 134; one
+// 252 x 364 image (d 1280) 22.5 -> 20.5, 8 and 16 at native resolution 161 -> 132 and 283 -> 245, eight of 1344 x 1344 on 74 SMs
+// 566 -> 454; 4, 16 and 64 frames 53 -> 35, 98 -> 70, 321 -> 208.  (Constants that overrated a block's time dealt the columns to groups that
+// each gathered the patches again: 16 at native resolution 275 for 215, eight of 1344 x 1344 on 74 SMs 776.)
 static eas_status launch_embed_resident(EmbedGemmParams& gp, const CUtensorMap& w_half, int budget, cudaStream_t stream) {
   static OncePerDevice once;
   if (once.first()) {
@@ -1231,15 +1250,18 @@ static eas_status launch_embed_resident(EmbedGemmParams& gp, const CUtensorMap& 
   const double kb = gp.k_pad / 64;
   int rows = 32, groups = 1;
   double best = 0.0;
-  const struct { int rows; double base, first, next, gather; } shapes[] = {{32, 14.2 + 0.35 * kb, std::max(0.5, 0.24 * kb - 0.9), 0.45 + 0.265 * kb, 0.75 + 0.565 * kb},
-                                                                           {64, 14.2 + 0.38 * kb, 2.4 + 0.11 * kb, 4.0 + 0.1 * kb, std::max(2.0, 0.9 * kb - 1.6)}};
+  const struct { int rows; double base, first, next, gather; } shapes[] = {
+      {32, 12.8 + 0.12 * kb, std::max(0.3, 0.28 * kb - 0.11), std::max(1.85, 0.7 + 0.17 * kb), 2.6 + 0.38 * kb},
+      {64, 14.1 + 0.24 * kb, 1.66 + 0.16 * kb, std::max(3.84, 1.41 + 0.23 * kb), 2.15 + 0.71 * kb},
+      {128, 7.9 + 2.54 * kb, 5.4, 6.4, 4.6 + 2.54 * kb}};
   for (const auto& sh : shapes)
-    for (int g = 1; g <= n_blocks; ++g) {
+    for (int g = 1; g <= (sh.rows < 128 ? n_blocks : kb <= 7 ? 1 : 0); ++g) {
       const int64_t units = static_cast<int64_t>((gp.n_patches + sh.rows - 1) / sh.rows) * g;
       const double waves = static_cast<double>((units + budget - 1) / budget), blocks = (n_blocks + g - 1) / g;
       const double cost = sh.base + blocks * sh.first + (waves - 1.0) * std::max(blocks * sh.next, sh.gather);
       if (best == 0.0 || cost < best) { best = cost; rows = sh.rows; groups = g; }
     }
+  if (rows == 128) return launch_embed_blocks(gp, rows, groups, budget, stream);
   gp.tma_w = w_half;
   gp.col_groups = groups;
   const int units = (gp.n_patches + rows - 1) / rows * groups;
@@ -1249,18 +1271,9 @@ static eas_status launch_embed_resident(EmbedGemmParams& gp, const CUtensorMap& 
 
 // Longer patch vectors: rows R of a patch block and column groups by estimated time (the result does not depend on them).
 // A unit gathers its k-blocks (G) and works off its column blocks (E: mostly the scattered fp32 stores; a later pass over K
-// adds to them), and units of a CTA overlap: G + E + (waves - 1) max(G, E), us.  Fitted to every (R, groups) forced over one
-// image to three 1344 x 1344 ones, one clip of 4 to 64 frames.  Kernel time, one 336 x 336 image (d 1024): 77 us as 5 units of
-// R = 128, 19 as 72 of R = 32; 8 images 72 -> 37; 32 images stay at R = 128, one group (74; 76 with R = 64); one 224 x 224 image
-// (d 256) 41 -> 18; a 16-frame clip 182 -> 117; three 1344 x 1344 images 154 -> 122 (R = 64).
+// adds to them), and units of a CTA overlap: G + E + (waves - 1) max(G, E), us.  Fitted to every (R, groups) forced over vectors of
+// 10 and 19 k-blocks (one image to three 1344 x 1344 ones, one clip of 4 to 64 frames), which embed_resident_kernel has taken over since.
 static eas_status launch_embed_gemm(EmbedGemmParams& gp, int budget, cudaStream_t stream) {
-  static OncePerDevice once;
-  if (once.first()) {
-    CUDA_TRY(cudaFuncSetAttribute(embed_gemm_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgSmemBytes));
-    CUDA_TRY(cudaFuncSetAttribute(embed_gemm_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgSmemBytes));
-    CUDA_TRY(cudaFuncSetAttribute(embed_gemm_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kEgSmemBytes));
-    once.settled();
-  }
   const int k_blocks = gp.k_pad / 64, n_blocks = (gp.N + 255) / 256;
   int rows = 128, groups = 1;
   double best = 0.0;
@@ -1274,10 +1287,7 @@ static eas_status launch_embed_gemm(EmbedGemmParams& gp, int budget, cudaStream_
       const double cost = G + E + (waves - 1.0) * std::max(G, E);
       if (best == 0.0 || cost < best) { best = cost; rows = sh.rows; groups = g; }
     }
-  gp.col_groups = groups;
-  const int units = (gp.n_patches + rows - 1) / rows * groups;
-  void (*kern)(EmbedGemmParams) = rows == 128 ? embed_gemm_kernel<128> : rows == 64 ? embed_gemm_kernel<64> : embed_gemm_kernel<32>;
-  return launch_kernel(kern, std::min(budget, units), kEgThreads, kEgSmemBytes, stream, gp);
+  return launch_embed_blocks(gp, rows, groups, budget, stream);
 }
 
 // ------------------------------------------------------------------------------------ the forward pass

@@ -1,5 +1,5 @@
 // Patch embedding as an im2col-fused GEMM for sm_100a (two kernels: embed_resident_kernel for patch vectors of up to 1216 elements, at
-// the end, and embed_gemm_kernel for longer ones, described here):
+// the end, and embed_gemm_kernel for longer ones and many short ones, described here):
 //
 //     x[row(m), :] = patch(m) * W_emb^T + b (+ pos[posrow(m), :])        m = patch index over the micro-batch
 //

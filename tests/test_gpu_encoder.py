@@ -192,10 +192,13 @@ def test_fused_patch_embedding_alone(name):
 
 
 @pytest.mark.parametrize("name,over,shapes", [("c3", dict(temporal_patch=3), [(6, 56, 84), (3, 28, 28)]), ("c0", dict(patch=32, max_pos=64), [(1, 224, 224), (1, 32, 64)]),
-                                              ("c0", dict(patch=20, max_pos=64), [(1, 100, 60), (1, 20, 20)])])
+                                              ("c0", dict(patch=20, max_pos=64), [(1, 100, 60), (1, 20, 20)]), ("c0", dict(patch=32, max_pos=64), [(1, 256, 256)] * 4),
+                                              ("c0", dict(patch=33, max_pos=64), [(1, 231, 264), (1, 33, 66)]), ("c0", dict(patch=33, max_pos=64), [(1, 264, 264)] * 4),
+                                              ("c0", dict(patch=15, max_pos=64), [(1, 105, 120), (1, 15, 15)]), ("c2", dict(in_channels=1), [(1, 364, 560), (1, 28, 56)])])
 def test_patch_embedding_of_other_vector_lengths(name, over, shapes):
-    """Patch vectors of 28, 48 and 19 k-blocks of 64 (the last the longest whose kernel keeps it resident, and padded): embeddings alone against the
-    oracle, and the same bits at budgets of one and a few SMs."""
+    """Embeddings alone against the oracle, and the same bits at budgets of one and a few SMs.  Patch vectors of 28 and 48 k-blocks of 64; 19 (the
+    longest whose kernel keeps it resident, and padded); 48 with 256 patches (units of 128 on up to three SMs); odd patch edges (pixel pairs
+    that straddle runs) in vectors of 52, in units of 64 and of 128 patches, and of 11; and 4 (units of 128 on few SMs, 32 on all)."""
     cfg = S.get_config(name, n_layers=0, **over)
     w, enc = _make(cfg)
     items = S.make_items(cfg, shapes, seed=4200)
@@ -209,7 +212,7 @@ def test_patch_embedding_of_other_vector_lengths(name, over, shapes):
 
 @pytest.mark.parametrize("name", ["c0", "c1", "c2", "c3"])
 def test_fused_patch_embedding_same_bits_for_every_block_shape(name):
-    """The embedding's patch blocks (32, 64 or 128 rows) and column groups follow the micro-batch size and the budget: an
+    """The embedding's units (32 or 64 patches) and column groups follow the micro-batch size and the budget: an
     item's rows must have the same bits alone, packed, and at budgets that take every shape."""
     cfg = S.get_config(name, n_layers=0)
     w, enc = _make(cfg)
