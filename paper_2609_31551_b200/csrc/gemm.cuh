@@ -25,7 +25,7 @@ constexpr int kBM = 128, kBN = 256, kBK = 64;
 constexpr int kEpiWarps = 8;
 constexpr int kGemmThreads = 64 + 32 * kEpiWarps + 32;   // + the second producer warp
 constexpr int kProducerBWarp = 2 + kEpiWarps;
-// A stage holds this CTA's 128 rows of A (16 KB; half-height tiles: 64) and its weight rows (all TN of them, or a pair's half) of one 64-wide
+// A stage holds this CTA's 128 rows of A (16 KB) and its weight rows (all TN of them, or a pair's half) of one 64-wide
 // k-block; the ring takes 192 KB.
 // TN = 512 ("wide", CTA pairs only): the pair owns a 256x512 tile, i.e. two 256-column accumulators fed by the same
 // A tile (three TMA operations for twice the columns) at the price of a single accumulator set: the epilogue no longer
@@ -70,8 +70,9 @@ enum { OUT_BF16 = 0, OUT_F32 = 1, OUT_F32_FOLD = 2 };
 constexpr int kFoldGroup = 128;                   // columns per statistics group
 
 struct alignas(64) GemmParams {
-  CUtensorMap tma_a;      // 3-D: {K-run, phase, rows}; box {64, 1, 128}.  Deep kernels: {64, rows, K/64}; box {64, 128 or 64, 2}
+  CUtensorMap tma_a;      // 3-D: {K-run, phase, rows}; box {64, 1, 128}.  Deep kernels: {64, rows, K/64}; box {64, 128, 2}
   CUtensorMap tma_b;      // 2-D: {K, N}; box {64, weight rows of a CTA: at most 256}.  Deep: {64, N, K/64}; box {64, rows, 2}
+  CUtensorMap tma_out16;  // half-height tiles: 2-D over out, box {16 columns, 32 rows}, no swizzle
   CUtensorMap tma_out;    // 2-D over out (valid if use_tma_out): box {64 bf16 | 32 fp32, 32 rows}, 128-byte swizzle; {32 bf16, 32 rows},
                           // 64-byte swizzle, where gemm_out_row says 32
   int use_tma_out;        // 1: epilogue stages 32-row sub-tiles in shared memory and stores them with TMA
@@ -79,7 +80,7 @@ struct alignas(64) GemmParams {
   int k_blocks;           // k-steps: K / 64, or ceil(K / 128) for the deep kernels (TMA fills past K with zeros)
   int kb_per_tap;         // k-blocks per convolution tap (== k_blocks for a plain GEMM)
   int conv_stride;        // 1 for a plain GEMM; row stride of a convolution otherwise
-  int m_blocks, n_blocks; // m_blocks counts blocks of 128 rows (one CTA, or a half-height pair) or 256 (CTA pair)
+  int m_blocks, n_blocks; // m_blocks counts 128-row blocks (one CTA per tile) or 256-row blocks (CTA pair)
   int reverse;            // 1: walk the tiles last to first (start with the rows the producer of A wrote last: L2)
   const bf16* bias;       // [N] (for SWIGLU: interleaved gate/up like the W rows)
   void* out;              // bf16 or fp32 [*, ldo]
@@ -102,8 +103,7 @@ struct alignas(64) GemmParams {
   int splits;             // >= 1
   int kb_per_split;
   int part_rows;          // rows of one split's region of the scratch matrix (a multiple of the tile height)
-  CUtensorMap tma_part;   // [(splits - 1) * part_rows, N] fp32, 32-row boxes of 32 columns.  Half-height tiles (never split) whose lane half
-                          // ends in 16 columns: 2-D over out, box {16 columns, 32 rows}, no swizzle
+  CUtensorMap tma_part;   // [(splits - 1) * part_rows, N] fp32, 32-row boxes of 32 columns
   // Folded normalisation.  LayerNorm / RMSNorm followed by a linear layer is  rstd * ((gamma .* x) - mean gamma) W^T + const:
   // the GEMM can run on the rows scaled by gamma only (rounded to bf16: the same single rounding of the operand as
   // with a normalisation kernel) and apply the row's rstd and mean in its epilogue,
@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
-            const uint64_t out_map = kNarrow && cols16 ? reinterpret_cast<uint64_t>(&p.tma_part) : wide_map;
+            const uint64_t out_map = kNarrow && cols16 ? reinterpret_cast<uint64_t>(&p.tma_out16) : wide_map;
             if (out_reduce) {
               // the residual rows keep their place in L2 (evict-last): the normalisation that follows reads them there,
               // and their write-back does not compete with this launch's own traffic (measured: out-projection -5 %)
