@@ -481,17 +481,18 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
             }
           }
           if (p.rope_cs != nullptr && col0 < p.rope_ncols && arow < p.M) {
-            // (the last rotated column ends a chunk of 32, except in half-height tiles, whose second lane half may start 16 columns off)
+            // The last rotated column ends a chunk of 32, except in half-height tiles, whose second lane half may start 16 columns off.
+            // (There by selection: a loop that ends early takes its loads one by one, 5 us of a 468 x 3840 launch.)
             const int turned = kNarrow ? p.rope_ncols - col0 : 32;
             int pi = (col0 % p.head_dim) >> 1;
             const float2* cs = p.rope_cs + arow;
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-              if (2 * j >= turned) break;
               const float2 t = __ldg(cs + pi * p.rope_stride);
               const float x0 = v[2 * j], x1 = v[2 * j + 1];
-              v[2 * j] = x0 * t.x - x1 * t.y;
-              v[2 * j + 1] = x1 * t.x + x0 * t.y;
+              const float y0 = x0 * t.x - x1 * t.y, y1 = x1 * t.x + x0 * t.y;
+              v[2 * j] = !kNarrow || 2 * j < turned ? y0 : x0;
+              v[2 * j + 1] = !kNarrow || 2 * j < turned ? y1 : x1;
               if (++pi == p.rope_pairs) pi = 0;
             }
           }
