@@ -839,7 +839,7 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
   else EAS_TRY(make_a_tmap(&p.tma_a, g.A, g.a_run, g.a_row_elems, g.conv_stride, g.a_rows));
   // weight rows per TMA box: the CTA's share of a 256-column accumulator, or the narrow tile's columns
   const int w_rows = std::min(tile_n, static_cast<int>(kBN)) / ctas;
-  if (gemm_alt(tile_n) || kTiles[tile].half) EAS_TRY(deep ? make_w_tmap_deep(&p.tma_b, L.w, L.N, L.K, w_rows) : make_w_tmap(&p.tma_b, L.w, L.N, L.K, w_rows));
+  if (gemm_alt(tile_n) || w_rows < 64) EAS_TRY(deep ? make_w_tmap_deep(&p.tma_b, L.w, L.N, L.K, w_rows) : make_w_tmap(&p.tma_b, L.w, L.N, L.K, w_rows));
   else p.tma_b = w_rows == 256 ? L.tmap : w_rows == 128 ? (deep ? L.tmap_half_deep : L.tmap_half) : (deep ? L.tmap_quarter_deep : L.tmap_quarter);
   p.M = g.M; p.N = L.N;
   p.kb_per_tap = static_cast<int>(g.a_run / kBK);
@@ -873,7 +873,7 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
   if (p.use_tma_out) {
     const int64_t out_cols = g.act == ACT_SWIGLU ? L.N / 2 : L.N;
     EAS_TRY(make_out_tmap(&p.tma_out, g.out, g.out_fp32 != 0, out_cols, g.ldo, g.M, g.out_fp32 ? 32 : gemm_out_row(g.act, tile_n, kTiles[tile].half)));
-    if (kTiles[tile].half) EAS_TRY(make_out_tmap(&p.tma_out16, g.out, g.out_fp32 != 0, out_cols, g.ldo, g.M, 16));
+    if (kTiles[tile].half && tile_n % 64 != 0) EAS_TRY(make_out_tmap(&p.tma_out16, g.out, g.out_fp32 != 0, out_cols, g.ldo, g.M, 16));
   }
   const int tiles = p.m_blocks * p.n_blocks * p.splits;
   GemmKernel kern = kernel_of(tile);
