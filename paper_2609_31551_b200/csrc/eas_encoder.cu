@@ -346,21 +346,21 @@ static GemmKernel gemm_kernel_of(int tile, bool deep) {
     if (tile == TILE_P128) return deep ? gemm_kernel<ACT, OUT, 2, 128, 2, SPLIT> : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 2, 128, 1>);
     if constexpr (ACT != ACT_SWIGLU)
       if (tile == TILE_N64) return deep ? gemm_kernel<ACT, OUT, 1, 64, 2, SPLIT> : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 1, 64, 1>);
-    if constexpr (ACT != ACT_SWIGLU && !SPLIT) {
-      if (tile == TILE_P96) return deep ? gemm_kernel<ACT, OUT, 2, 96, 2> : nullptr;
-      if (tile == TILE_N160) return gemm_kernel<ACT, OUT, 1, 160>;
-      if (tile == TILE_N224) return gemm_kernel<ACT, OUT, 1, 224>;
-      if (tile == TILE_P160) return gemm_kernel<ACT, OUT, 2, 160>;
-      if (tile == TILE_P192) return gemm_kernel<ACT, OUT, 2, 192>;
-      if (tile == TILE_P224) return gemm_kernel<ACT, OUT, 2, 224>;
-      if constexpr (!(ACT == ACT_GELU && OUT == OUT_F32)) {
-        if (kTiles[tile].half && !deep) return nullptr;
-        if (tile == TILE_H64) return gemm_kernel<ACT, OUT, 2, 64, 2, false, true>;
-        if (tile == TILE_H96) return gemm_kernel<ACT, OUT, 2, 96, 2, false, true>;
-        if (tile == TILE_H128) return gemm_kernel<ACT, OUT, 2, 128, 2, false, true>;
-        if (tile == TILE_H160) return gemm_kernel<ACT, OUT, 2, 160, 2, false, true>;
-        if (tile == TILE_H224) return gemm_kernel<ACT, OUT, 2, 224, 2, false, true>;
-      }
+    if constexpr (ACT != ACT_SWIGLU) {
+      if (tile == TILE_P96) return deep ? gemm_kernel<ACT, OUT, 2, 96, 2, SPLIT> : nullptr;
+      if (tile == TILE_N160) return gemm_kernel<ACT, OUT, 1, 160, 1, SPLIT>;
+      if (tile == TILE_N224) return gemm_kernel<ACT, OUT, 1, 224, 1, SPLIT>;
+      if (tile == TILE_P160) return gemm_kernel<ACT, OUT, 2, 160, 1, SPLIT>;
+      if (tile == TILE_P192) return gemm_kernel<ACT, OUT, 2, 192, 1, SPLIT>;
+      if (tile == TILE_P224) return gemm_kernel<ACT, OUT, 2, 224, 1, SPLIT>;
+    }
+    if constexpr (ACT != ACT_SWIGLU && !SPLIT && !(ACT == ACT_GELU && OUT == OUT_F32)) {
+      if (kTiles[tile].half && !deep) return nullptr;
+      if (tile == TILE_H64) return gemm_kernel<ACT, OUT, 2, 64, 2, false, true>;
+      if (tile == TILE_H96) return gemm_kernel<ACT, OUT, 2, 96, 2, false, true>;
+      if (tile == TILE_H128) return gemm_kernel<ACT, OUT, 2, 128, 2, false, true>;
+      if (tile == TILE_H160) return gemm_kernel<ACT, OUT, 2, 160, 2, false, true>;
+      if (tile == TILE_H224) return gemm_kernel<ACT, OUT, 2, 224, 2, false, true>;
     }
   }
   return nullptr;
@@ -602,16 +602,7 @@ struct Plan {
 };
 }  // namespace
 
-// Split-K factor of a residual GEMM x[M, N] += A[M, K] W^T with few tiles (small micro-batches: the K loop of one tile is
-// the whole kernel, and most SMs have no tile).  A function of the shape and the device only, never of the SM budget, so
-// that results do not depend on the budget; every split is a whole number of 128-wide k-steps, so that they do not
-// depend on the tile shape either.
-static int pick_splits(int64_t M, int64_t N, int64_t K, int sm_count) {
-  const int64_t items = ((M + kBM - 1) / kBM) * ((N + kBN - 1) / kBN);
-  for (int s = 4; s >= 2; s >>= 1)
-    if (items * s <= sm_count && K % (s * 2 * kBK) == 0 && K / s >= 1024) return s;
-  return 1;
-}
+static int pick_splits(int64_t M, int64_t N, int64_t K, int sm_count);
 
 static Plan make_plan(const eas_encoder* e, int64_t T, int n_items) {
   const eas_arch_config& c = e->cfg;
@@ -769,7 +760,7 @@ struct GemmCall {
 //   M = 468:  (1280, 5120) 17.8 -> 12.5;  (1280, 1280) 7.1 -> 6.5;  (3840, 1280) 8.5 -> 8.2 as 128x224
 //   M = 196:  (256, 1024) 5.8 -> 4.5 as 128x64
 template <typename Usable>
-static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bool plain, Usable usable) {
+static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bool plain, Usable usable, double* us = nullptr) {
   constexpr double kShareUs = 1.05;
   struct Cost { int tile; double base, per_kb, per_wave, partial; };    // us
   static const Cost costs[] = {{TILE_SINGLE, 5.24, 0.351, 0.52, 0.87}, {TILE_PAIR, 6.44, 0.323, 0.25, 0.92}, {TILE_WIDE, 4.81, 0.586, 5.1, 0.89},
@@ -793,7 +784,31 @@ static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bo
     if (t.half) cost = 1.02 * (cost + (budget < g_device_sms ? kShareUs : 0.0));      // 2 % in hand: what the fit is off by
     if (best == 0.0 || cost < best) { best = cost; tile = c.tile; }
   }
+  if (us != nullptr) *us = best;
   return tile;
+}
+
+// Split-K factor of a residual GEMM x[M, N] += A[M, K] W^T with few tiles (small micro-batches: the K loop of one tile is
+// the whole kernel, and most SMs have no tile).  A function of the shape and the device only, never of the SM budget, so
+// that results do not depend on the budget; every split is a whole number of 128-wide k-steps, so that they do not
+// depend on the tile shape either.  4 or 2 by estimated time on all SMs, where every further split costs partial sums that the GEMM
+// writes and the normalisation reads (kPartUs; measured 0.4 to 3 us).  A forward pass replayed as a graph, split by 4 and by 2, and whole:
+// one 336 x 336 image 1193, 1181 and 1171 us, 128 tokens 831, 858 and 848, 400 of d 1024 1080, 1070 and 1068; 64 of d 1280 1270,
+// 1356 and 1285, 256 1466, 1520 and 1480, 500 of audio 1681, 1672 and 1644.
+static int pick_splits(int64_t M, int64_t N, int64_t K, int sm_count) {
+  constexpr double kPartUs = 0.75;
+  const int64_t items = ((M + kBM - 1) / kBM) * ((N + kBN - 1) / kBN);
+  int splits = 1;
+  double best = 0.0;
+  for (int s = 4; s >= 2; s >>= 1) {
+    if (items * s > sm_count || K % (s * 2 * kBK) != 0 || K / s < 1024) continue;
+    double us = 0.0;
+    pick_tile(M, N, static_cast<double>(K / kBK) / s, s, sm_count, true,
+              [&](int t) { return !kTiles[t].half && (t != TILE_WIDE || N % 512 == 0) && gemm_kernel_for(ACT_NONE, 1, t, kTiles[t].cols <= 128, true) != nullptr; }, &us);
+    us += kPartUs * s;
+    if (best == 0.0 || us < best) { best = us; splits = s; }
+  }
+  return splits;
 }
 
 static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream, uint32_t* status) {

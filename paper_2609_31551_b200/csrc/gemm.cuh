@@ -180,7 +180,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   constexpr bool kAlt = HALF || gemm_alt(TN);
   static_assert(!HALF || (TN <= 256 && OUT != OUT_F32_FOLD), "half-height tiles: one accumulator, plain epilogues");
   static_assert(TN % 32 == 0 && TN >= 64 && (TN <= 256 || TN == 512), "tile width");
-  static_assert(!kAlt || (ACT != ACT_SWIGLU && !SPLIT), "odd widths: plain tiles");
+  static_assert(!kAlt || ACT != ACT_SWIGLU, "odd widths: no gated epilogue");
+  static_assert(!HALF || !SPLIT, "half-height tiles: one pass over K");
   static_assert(TN < 512 || (CTAS == 2 && ACT != ACT_SWIGLU), "wide tiles: CTA pairs, no gated epilogue");
   static_assert(TN >= 256 || OUT != OUT_F32_FOLD, "narrow tiles: no folding epilogue");
   static_assert(TN >= 128 || ACT != ACT_SWIGLU, "a gated epilogue halves the columns: 128 at least");

@@ -144,6 +144,17 @@ def test_split_k_is_deterministic_budget_independent_and_optional():
     assert torch.equal(packed_on, packed)
 
 
+@pytest.mark.parametrize("name,tokens,rows,splits", [("c1", 89, 256, 4), ("c1", 577, 768, 2), ("c1", 1154, 1280, 2), ("c4", 129, 256, 4), ("c4", 1500, 1536, 2), ("c1", 2308, 0, 1)])
+def test_split_k_factor(name, tokens, rows, splits):
+    """The workspace shows the split factor: s - 1 regions of whole 256-row blocks for the partial sums.  Two where the tiles of two
+    splits fill the SMs, four with few tokens, none past the documented line."""
+    cfg = S.get_config(name, n_layers=2)
+    _, enc = _make(cfg)
+    whole = enc.workspace_bytes(tokens, 1)
+    enc.set_split_k(True)
+    assert enc.workspace_bytes(tokens, 1) - whole == (splits - 1) * rows * cfg["d_model"] * 4
+
+
 @pytest.mark.parametrize("case", ["c1_2layers", "c2_2layers", "c3_2layers", "c4_2layers"])
 def test_split_k_parity_all_families(case):
     """The small cases of every family with split K on (RMSNorm and LayerNorm, SwiGLU and GELU MLPs, d = 1024 and 1280)."""
