@@ -170,11 +170,11 @@ eas_status eas_encode_microbatch_static(eas_encoder* enc, const eas_packed_input
  * EAS_OK, EAS_ERR_DEVICE_TIMEOUT, EAS_ERR_DEVICE_CHECK or EAS_ERR_CUDA. */
 eas_status eas_encoder_status(eas_encoder* enc, void* stream);
 
-/* Number of kernel launches the last eas_encode_microbatch enqueued. */
 /* For tests: every GEMM of the forward pass takes this tile shape (numbered as in eas_kernel_gemm_tile) where it has a kernel of
  * that shape, and chooses as usual elsewhere.  0 (default): choose.  The results do not depend on it. */
 eas_status eas_encoder_set_gemm_tile(eas_encoder* enc, int32_t tile_shape);
 
+/* Number of kernel launches the last eas_encode_microbatch enqueued. */
 int32_t eas_encoder_last_launch_count(const eas_encoder* enc);
 
 /* Selects the attention kernel: 0 = default (tcgen05, probabilities kept in tensor memory); 1 = register-tile
@@ -184,23 +184,25 @@ eas_status eas_encoder_set_attention_impl(eas_encoder* enc, int32_t impl);
 
 /* Split K for small micro-batches (default off; part of the latency path, like the graph mode below).  With few tokens
  * the residual GEMMs of a block (x += o W_proj^T, x += h W_fc2^T) have fewer tiles than the device has SMs, and the K
- * loop of one tile is the whole kernel.  With on = 1, when tiles x s <= SMs and K / s >= 1024 (s = 4 or 2; a function of
+ * loop of one tile is the whole kernel.  With on = 1, when 128x256 tiles x s <= SMs and K / s >= 1024 (s = 4 or 2, by estimated time; a function of
  * the token count, the layer sizes and the device, never of sm_budget), s CTAs share a tile's K range: the first adds its
  * sum and the bias into the residual stream as usual, the others store bare partial sums, and the normalisation kernel
  * that follows adds those to the row in a fixed order before normalising it.  Results stay deterministic and independent
  * of sm_budget, but no longer of what else is in the micro-batch: an item encoded alone (split) and the same item in a
  * large micro-batch (not split) differ in the last bits, which is why the mode is off unless asked for (off: every
  * item's embeddings are bit-identical whatever it is packed with).  eas_encoder_workspace_bytes follows the mode (the
- * partial sums need scratch): set it before sizing the workspace. */
+ * partial sums need scratch): set it before sizing the workspace.  With graph replay 128 tokens of the ViT-L/14-style
+ * encoder take 849 us unsplit and 833 split, 256 tokens 978 and 987, 577 tokens 1175 and 1182, 1154 tokens 1494 and 1515: half-height
+ * tiles, which split launches do not have, have overtaken the split. */
 eas_status eas_encoder_set_split_k(eas_encoder* enc, int32_t on);
 
-/* Folded normalisation (default on).  A block's norm1 / norm2 (Section 2.1: pre-norm transformer blocks) are followed by
+/* Folded normalisation (default off: measured slower than the kernels it saves).  A block's norm1 / norm2 (Section 2.1: pre-norm transformer blocks) are followed by
  * a linear layer, and  LN(x) W^T + b  =  rstd * ((gamma .* x) W^T - mean (gamma W^T)) + (b + beta W^T):  the qkv and
  * MLP-up GEMMs run on the residual rows scaled by gamma only (rounded to bf16) and apply each row's rstd and mean in
- * their epilogue, with two constants per output computed at create time, so no normalisation kernel runs inside a block.  The rows' statistics (mean
+ * their epilogue, with two constants per output computed at create time, so with on = 1 no normalisation kernel runs inside a block.  The rows' statistics (mean
  * and squared deviations per 128 columns, merged in index order: independent of sm_budget and of the tile shape) and
  * their scaled bf16 copy are written by the residual GEMM that produced the rows, in the same pass that adds into the fp32
- * stream.  on = 0 restores one normalisation kernel per norm1 / norm2 (the result differs in rounding only: the
+ * stream.  on = 0 runs one normalisation kernel per norm1 / norm2 (the result differs in rounding only: the
  * normalised values are then rounded to bf16 before the GEMM instead of the scaled ones).  While split K is in effect for a
  * micro-batch its blocks run unfolded.  Both modes stay within the same parity tolerance of the definition. */
 eas_status eas_encoder_set_norm_fold(eas_encoder* enc, int32_t on);
