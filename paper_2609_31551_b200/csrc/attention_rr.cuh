@@ -190,7 +190,8 @@ __global__ void __launch_bounds__(AttnRrSmem<HD, OWN_P>::kThreads, 1) attn_rr_ke
   const uint32_t tmem_base = *tmem_slot;
   if (p.early_launch) pdl_launch_dependents();
   // The parameters that the first unit's decoding reads come from a cold constant cache, some 650 cycles in all: ahead of the grid
-  // dependency's wait they cost nothing (4 x 8192 tokens 1325 -> 1311 us, 8 items of 577 27.8 -> 27.5).  The variant for little work
+  // dependency's wait they cost nothing (the kernel alone, 4 x 8192 tokens 1325 -> 1311 us, 8 items of 577 27.8 -> 27.5; whole calls move
+  // by less than their runs differ).  The variant for little work
   // has its SMs to itself and is ready too late for that (one item of 468 tokens 8.92 -> 9.00).
   if (!OWN_P && attn_unit_at(0) < p.total_units) {
     int cursor = 0;
