@@ -25,6 +25,7 @@ constexpr int kBM = 128, kBN = 256, kBK = 64;
 constexpr int kEpiWarps = 8;
 constexpr int kGemmThreads = 64 + 32 * kEpiWarps + 32;   // + the second producer warp
 constexpr int kProducerBWarp = 2 + kEpiWarps;
+constexpr int kTmemWarp = 2;                             // the first epilogue warp allocates tensor memory and gives it back
 // A stage holds this CTA's 128 rows of A (16 KB; half-height tiles: 64) and its weight rows (all TN of them, or a pair's half) of one 64-wide
 // k-block; the ring takes 192 KB.
 // TN = 512 ("wide", CTA pairs only): the pair owns a 256x512 tile, i.e. two 256-column accumulators fed by the same
@@ -58,7 +59,7 @@ constexpr int kMaxStages = 8;
 constexpr int kStagingOff = 4 * 49152;                         // == 6 * 32768; 8 epilogue warps x 4 KB output staging (TMA store source)
 constexpr int kBiasOff = kStagingOff + kEpiWarps * 4096;       // 2 x 256 fp32 bias values of the current tiles
 constexpr int kBarOff = kBiasOff + 2 * 256 * 4;
-constexpr int kGemmSmemBytes = kBarOff + 192 /*barriers*/ + 832 /*alignment slack*/;
+constexpr int kGemmSmemBytes = kBarOff + 208 /*barriers*/ + 816 /*alignment slack*/;
 static_assert(kGemmSmemBytes <= 232448, "exceeds the 227 KB shared memory of an SM");
 constexpr int kPanelM = 8;                        // m-blocks per rasterisation panel (L2 reuse of W tiles)
 
@@ -211,6 +212,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   uint64_t* acc_empty = bars + 2 * kMaxStages + 2; // [2]        epilogue -> MMA (pair: both CTAs' warps arrive at the leader)
   uint64_t* bias_bar = bars + 2 * kMaxStages + 4;  // [2]        epilogue warps: bias values staged
   uint64_t* bias_free = bars + 2 * kMaxStages + 7; // [1]        wide tiles: every epilogue warp has read the staged bias
+  uint64_t* tmem_free = bars + 2 * kMaxStages + 8; // [1]        every epilogue warp has read its last accumulator
+  uint64_t* peer_free = bars + 2 * kMaxStages + 9; // [1]        ... and so have the other CTA's
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 6);
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
@@ -225,23 +228,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   const int first_tile = blockIdx.x / CTAS;        // both CTAs of a pair walk the same tiles
   const int tile_step = gridDim.x / CTAS;
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(&acc_full[a], 1); mbar_init(&acc_empty[a], kEpiWarps * CTAS); mbar_init(&bias_bar[a], kEpiWarps); }
-    mbar_init(bias_free, kEpiWarps);
-    *abort_flag = 0;
+  if (warp == kProducerBWarp) {                    // one barrier a lane
+    if (lane < 2 * kMaxStages) mbar_init(&bars[lane], 1);
+    else if (lane < 2 * kMaxStages + 2) mbar_init(&acc_full[lane - 2 * kMaxStages], 1);
+    else if (lane < 2 * kMaxStages + 4) mbar_init(&acc_empty[lane - 2 * kMaxStages - 2], kEpiWarps * CTAS);
+    else if (lane < 2 * kMaxStages + 6) mbar_init(&bias_bar[lane - 2 * kMaxStages - 4], kEpiWarps);
+    else if (lane == 22) mbar_init(bias_free, kEpiWarps);
+    else if (lane == 23) mbar_init(tmem_free, kEpiWarps);
+    else if (lane == 24) mbar_init(peer_free, 1);
+    else if (lane == 25) *abort_flag = 0;
     mbar_fence_init();
-    tma_prefetch_desc(&p.tma_a);
-    tma_prefetch_desc(&p.tma_b);
-    if (p.use_tma_out) tma_prefetch_desc(&p.tma_out);
-  }
-  if (warp == 1) {
+  } else if (warp == 0) {
+    if (lane == 0) {
+      tma_prefetch_desc(&p.tma_a);
+      tma_prefetch_desc(&p.tma_b);
+      if (p.use_tma_out) tma_prefetch_desc(&p.tma_out);
+    }
+  } else if (warp == kTmemWarp) {
     if (CTAS == 2) { tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
     else { tmem_alloc(tmem_slot, kTmemCols); tmem_relinquish(); }
   }
   tc_fence_before_sync();
-  __syncthreads();
-  if (CTAS == 2) cluster_sync_all();               // the peer's barriers are initialised before anything signals them
+  // (a pair: the peer's barriers are initialised before anything signals them)
+  if (CTAS == 2) cluster_sync_all(); else __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   if (threadIdx.x == 0) GEMM_TL(1);
@@ -251,6 +260,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   if (!(p.w_const && warp == kProducerBWarp)) pdl_wait();
   if (threadIdx.x == 0) GEMM_TL(2);
 
+  bool ok = true;
   if (warp == 0 || warp == kProducerBWarp) {
     // ------------------------------------------------------------------ producers: warp 0 loads A, the last warp B
     // The two operands have a warp each (128 KB of boxes from one thread: 476 ns a step, from two 396); a whole warp walks the
@@ -258,7 +268,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     // announces the bytes of the whole stage.
     const bool do_a = warp == 0, do_b = warp != 0;
     uint32_t it = 0;
-    bool ok = true;
     for (int work = first_tile; work < num_work && ok; work += tile_step) {
       const int tile = SPLIT ? work / n_splits : work, split = SPLIT ? work - tile * n_splits : 0;
       int mg, nb;
@@ -317,6 +326,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         }
       }
     }
+    // The stages' last hand-backs are asynchronous arrivals that nothing else waits for (from the leader's UMMAs in both CTAs of a
+    // pair): they have to be in before the CTA's shared memory passes to another one.  (Never used stages pass at once.)
+    if (do_a)
+      for (uint32_t e = it; e < it + kStages && ok; ++e) ok = warp_mbar_wait(&empty_bar[e % kStages], ((e / kStages) & 1u) ^ 1u, abort_flag);
     if (!ok) {
       // give loads already in flight a bounded chance to land before the CTA retires
       for (int s = 0; s < kStages; ++s) {
@@ -332,7 +345,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     if (cta_rank == 0) {
       constexpr uint32_t idesc = make_idesc_bf16(kARows * CTAS, Cfg::kMmaN, 0, 0);
       uint32_t it = 0, tcount = 0;
-      bool ok = true;
       for (int work = first_tile; work < num_work && ok; work += tile_step, ++tcount) {
         const uint32_t acc = tcount % kAccBuffers;
         const uint32_t acc_ph = (tcount / kAccBuffers) & 1u;
@@ -383,14 +395,18 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     const int quarter = warp & 3;               // TMEM lane quarter this warp may read
     const int half = ew >> 2;                   // which 128 accumulator columns
     uint32_t tcount = 0;
-    bool ok = true;
-    auto release_accumulator = [&](uint32_t acc) {   // this warp has read its part of the accumulator
+    // This warp has read its part of the accumulator.  Nobody waits for the last ones: no remote arrival may be under way to a
+    // CTA that retires.
+    auto release_accumulator = [&](uint32_t acc, int work) {
       tc_fence_before_sync();
       GEMM_STAMP(12);
       __syncwarp();
       GEMM_STAMP(13);
       if (lane == 0) {
-        if (CTAS == 2) mbar_arrive_cluster_relaxed(&acc_empty[acc], 0); else mbar_arrive(&acc_empty[acc]);
+        if (work + kAccBuffers * tile_step < num_work) {
+          if (CTAS == 2) mbar_arrive_cluster_relaxed(&acc_empty[acc], 0); else mbar_arrive(&acc_empty[acc]);
+        }
+        if (work + tile_step >= num_work) mbar_arrive(tmem_free);
       }
     };
     for (int work = first_tile; work < num_work && ok; work += tile_step, ++tcount) {
@@ -408,7 +424,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         // With two accumulator buffers the other buffer's bias_bar (eight arrivals) lies between two uses of a bias slot
         // and orders them.  A wide tile has ONE slot: nobody may overwrite it before all eight warps have finished
         // reading the previous tile's values (each arrives at bias_free after its last chunk).
-        if (kAccBuffers == 1 && tcount > 0 && !mbar_wait(bias_free, (tcount - 1) & 1u, abort_flag)) { ok = false; break; }
+        if (kAccBuffers == 1 && tcount > 0 && !warp_mbar_wait(bias_free, (tcount - 1) & 1u, abort_flag)) { ok = false; break; }
         {
 #pragma unroll
           for (int h = 0; h < NW; ++h) {
@@ -437,10 +453,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           }
         }
         GEMM_STAMP(0);
-        if (!mbar_wait(&acc_full[acc], acc_ph, abort_flag)) { ok = false; break; }
+        if (!warp_mbar_wait(&acc_full[acc], acc_ph, abort_flag)) { ok = false; break; }
         GEMM_STAMP(1);
         if (tcount == 0 && ew == 0 && lane == 0) GEMM_TL(4);
-        if (!mbar_wait(&bias_bar[acc], acc_ph, abort_flag)) { ok = false; break; }
+        if (!warp_mbar_wait(&bias_bar[acc], acc_ph, abort_flag)) { ok = false; break; }
         tc_fence_after_sync();
         GEMM_STAMP(2);
         uint8_t* stage = smem + kStagingOff + ew * 4096;
@@ -699,7 +715,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           }
         }
         }
-        release_accumulator(acc);
+        release_accumulator(acc, work);
         if (kAccBuffers == 1 && lane == 0) mbar_arrive(bias_free);   // this warp's reads of the staged bias are done (after the __syncwarp above)
         GEMM_STAMP(11);
         if (tcount == 0 && ew == 0 && lane == 0) GEMM_TL(5);
@@ -707,7 +723,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
       }
 
       if (kAlt) { ok = false; break; }                            // (these widths have TMA-stored outputs only: the launcher)
-      if (!mbar_wait(&acc_full[acc], acc_ph, abort_flag)) { ok = false; break; }
+      if (!warp_mbar_wait(&acc_full[acc], acc_ph, abort_flag)) { ok = false; break; }
       tc_fence_after_sync();
 
       long long orow = arow;
@@ -814,7 +830,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         }
       }
       // all TMEM reads of this warp are complete (wait::ld above): hand the accumulator back
-      release_accumulator(acc);
+      release_accumulator(acc, work);
+    }
+    // Tensor memory goes back as soon as all warps (a pair: of both CTAs) have read their last accumulator, beside the last stores.
+    // The other CTA's arrival is the last that anything sends to this one.
+    if (warp == kTmemWarp && ok) {
+      ok = warp_mbar_wait(tmem_free, 0, abort_flag);
+      if (CTAS == 2 && ok) {
+        if (lane == 0) mbar_arrive_cluster_relaxed(peer_free, static_cast<uint32_t>(cta_rank ^ 1));
+        __syncwarp();
+        ok = warp_mbar_wait(peer_free, 0, abort_flag);
+      }
+      if (ok) {
+        tc_fence_after_sync();
+        if (CTAS == 2) tmem_dealloc_pair(tmem_base, kTmemCols); else tmem_dealloc(tmem_base, kTmemCols);
+      }
     }
     // bulk stores still READING the staging buffer must finish before the CTA's shared memory is released; that they are
     // performed is the grid's completion, which the next kernel waits for: the tear-down overlaps it (one 252 x 364 image: 2304 -> 2214 us a pass, with the norm rows
@@ -823,15 +853,22 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     if (ew == 0 && lane == 0) GEMM_TL(6);
   }
 
-  tc_fence_before_sync();
-  __syncthreads();
-  if (CTAS == 2) cluster_sync_all();               // no CTA of the pair retires while the other may still signal it
-  if (warp == 1) {
+  // The warps retire one by one.  A barrier of the pair here costs 0.6 us a launch, tensor memory given back behind the last store
+  // 0.15 (a chain of launches that each load and store 32 KB a CTA, 148 CTAs: 3.4 us with both, 2.6 without); whole calls, with the one
+  // barrier at set-up: one 224 x 224 image 75.7 -> 71.0 us, one 336 x 336 image 1253 -> 1223, one of 252 x 364 1941 -> 1874.  Only
+  // after a wait that ran out does everybody who is still there meet (a cluster barrier does not count threads that have
+  // retired), so that tensor memory is given back when nobody uses it any more.
+  if (!ok) {
+    __syncwarp();
+    tc_fence_before_sync();
+    cluster_sync_all();
     tc_fence_after_sync();
-    if (CTAS == 2) tmem_dealloc_pair(tmem_base, kTmemCols); else tmem_dealloc(tmem_base, kTmemCols);
+    if (warp == kTmemWarp) {
+      if (CTAS == 2) tmem_dealloc_pair(tmem_base, kTmemCols); else tmem_dealloc(tmem_base, kTmemCols);
+    }
+    if (lane == 0) atomicCAS(p.status, DEV_OK, DEV_ERR_WAIT_TIMEOUT);
   }
-  if (threadIdx.x == 0) GEMM_TL(7);
-  if (threadIdx.x == 0 && *abort_flag) atomicCAS(p.status, DEV_OK, DEV_ERR_WAIT_TIMEOUT);
+  if (threadIdx.x == 64) GEMM_TL(7);
 }
 
 }  // namespace eas
