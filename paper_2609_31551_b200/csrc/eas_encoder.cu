@@ -875,6 +875,7 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
   }
   p.m_blocks = (g.M + kTiles[tile].rows - 1) / kTiles[tile].rows;
   p.n_blocks = (L.N + tile_n - 1) / tile_n;
+  tile_magic(p.m_blocks, p.n_blocks, &p.panel_magic, &p.rest_magic);
   p.bias = L.b;
   p.out = g.out; p.ldo = g.ldo; p.resid = g.resid;
   p.row_map = g.row_map; p.pos_idx = g.pos_idx; p.pos = g.pos;

@@ -59,7 +59,7 @@ constexpr int kMaxStages = 8;
 constexpr int kStagingOff = 4 * 49152;                         // == 6 * 32768; 8 epilogue warps x 4 KB output staging (TMA store source)
 constexpr int kBiasOff = kStagingOff + kEpiWarps * 4096;       // 2 x 256 fp32 bias values of the current tiles
 constexpr int kBarOff = kBiasOff + 2 * 256 * 4;
-constexpr int kGemmSmemBytes = kBarOff + 208 /*barriers*/ + 816 /*alignment slack*/;
+constexpr int kGemmSmemBytes = kBarOff + 264 /*barriers*/ + 760 /*alignment slack*/;
 static_assert(kGemmSmemBytes <= 232448, "exceeds the 227 KB shared memory of an SM");
 constexpr int kPanelM = 8;                        // m-blocks per rasterisation panel (L2 reuse of W tiles)
 
@@ -84,6 +84,8 @@ struct alignas(64) GemmParams {
   int conv_stride;        // 1 for a plain GEMM; row stride of a convolution otherwise
   int m_blocks, n_blocks; // m_blocks counts blocks of 128 rows (one CTA, or a half-height pair) or 256 (CTA pair)
   int reverse;            // 1: walk the tiles last to first (start with the rows the producer of A wrote last: L2)
+  uint32_t panel_magic;   // see tile_coords
+  uint32_t rest_magic;
   const bf16* bias;       // [N] (for SWIGLU: interleaved gate/up like the W rows)
   void* out;              // bf16 or fp32 [*, ldo]
   long long ldo;          // leading dimension of out (elements)
@@ -139,13 +141,23 @@ __device__ __forceinline__ unsigned long long gemm_globaltimer() { unsigned long
 #define GEMM_TL(k) do { } while (0)
 #endif
 
-__device__ __forceinline__ void tile_coords(int tile, int m_blocks, int n_blocks, int& mb, int& nb) {
-  const int per_panel = kPanelM * n_blocks;
-  const int panel = tile / per_panel;
+// Tile -> row block, column block: panels of kPanelM row blocks x all column blocks, the last panel with what is left.  Both divisions
+// are multiplications by ceil(2^32 / divisor), exact while tile * divisor < 2^32 (the host passes 0 otherwise; a panel of one row
+// block divides by nothing).
+__device__ __forceinline__ void tile_coords(int tile, const GemmParams& p, int& mb, int& nb) {
+  const int per_panel = kPanelM * p.n_blocks;
+  const int panel = p.panel_magic != 0 ? static_cast<int>(__umulhi(static_cast<uint32_t>(tile), p.panel_magic)) : tile / per_panel;
   const int within = tile - panel * per_panel;
-  const int rows_here = min(kPanelM, m_blocks - panel * kPanelM);
-  nb = within / rows_here;
+  const int rows_here = min(kPanelM, p.m_blocks - panel * kPanelM);
+  nb = rows_here == kPanelM ? within / kPanelM : p.rest_magic != 0 ? static_cast<int>(__umulhi(static_cast<uint32_t>(within), p.rest_magic)) : within;
   mb = panel * kPanelM + (within - nb * rows_here);
+}
+// the host's side: (panel_magic, rest_magic)
+inline void tile_magic(int64_t m_blocks, int64_t n_blocks, uint32_t* panel, uint32_t* rest) {
+  const uint64_t per_panel = static_cast<uint64_t>(kPanelM * n_blocks), left = static_cast<uint64_t>(m_blocks % kPanelM);
+  const uint64_t two32 = 1ull << 32;
+  *panel = static_cast<uint64_t>(m_blocks * n_blocks) * per_panel < two32 ? static_cast<uint32_t>((two32 + per_panel - 1) / per_panel) : 0u;
+  *rest = left > 1 ? static_cast<uint32_t>((two32 + left - 1) / left) : 0u;
 }
 
 // Folded normalisation: a row's factor and offset (rstd, -rstd * mean) from its group statistics, merged in index
@@ -209,17 +221,43 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   uint64_t* full_bar = bars;                       // [kStages]  TMA -> MMA (pair: the leader's copy collects both CTAs' bytes)
   uint64_t* empty_bar = bars + kMaxStages;         // [kStages]  MMA -> TMA (pair: signalled in both CTAs)
   uint64_t* acc_full = bars + 2 * kMaxStages;      // [2]        MMA -> epilogue (pair: signalled in both CTAs)
-  uint64_t* acc_empty = bars + 2 * kMaxStages + 2; // [2]        epilogue -> MMA (pair: both CTAs' warps arrive at the leader)
-  uint64_t* bias_bar = bars + 2 * kMaxStages + 4;  // [2]        epilogue warps: bias values staged
-  uint64_t* bias_free = bars + 2 * kMaxStages + 7; // [1]        wide tiles: every epilogue warp has read the staged bias
-  uint64_t* tmem_free = bars + 2 * kMaxStages + 8; // [1]        every epilogue warp has read its last accumulator
-  uint64_t* peer_free = bars + 2 * kMaxStages + 9; // [1]        ... and so have the other CTA's
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxStages + 6);
+  uint64_t* peer_free = acc_full + 2;              // [1]        the other CTA's epilogue warps have read their last accumulator
+  uint64_t* tmem_ready = peer_free + 1;            // [1]        tensor memory is allocated (a pair: in both CTAs)
+  uint64_t* acc_empty = tmem_ready + 1;            // [2]        epilogue -> MMA (pair: both CTAs' warps arrive at the leader)
+  uint64_t* bias_bar = acc_empty + 2;              // [2]        epilogue warps: bias values staged
+  uint64_t* bias_free = bias_bar + 2;              // [1]        wide tiles: every epilogue warp has read the staged bias
+  uint64_t* tmem_free = bias_free + 1;             // [1]        every epilogue warp has read its last accumulator
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 32);
   volatile uint32_t* abort_flag = tmem_slot + 1;
 
   const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);    // uniform: see elect_one
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) GEMM_TL(0);
+  // A launch of one wave waits for the first load of its last CTA, which starts when the predecessor's last CTA retires.  From a CTA's
+  // start to its first load: 3400 cycles with the barriers initialised one by one (1150 to that point), a releasing arrival at the
+  // pair's barrier (370) and the first tile's coordinates and parameters behind the waits (700); 1400 to 1800 in this form.  Whole
+  // calls: one 224 x 224 image 71.0 -> 67.1 us, one 336 x 336 image 1223 -> 1180, one of 252 x 364 1874 -> 1820, 30 s of audio 3111 -> 3085.
+  if (warp == kProducerBWarp) {                    // a barrier a lane (those behind the last are never used)
+    const int i = lane - 2 * kMaxStages - 3;       // 0: tmem_ready, 1, 2: acc_empty, then one arrival per epilogue warp
+    mbar_init(&bars[lane], i < 0 ? 1u : i == 0 ? static_cast<uint32_t>(CTAS) : i <= 2 ? static_cast<uint32_t>(kEpiWarps * CTAS) : static_cast<uint32_t>(kEpiWarps));
+    mbar_fence_init();
+  } else if (warp == 0) {
+    if (lane == 0) {
+      *abort_flag = 0;
+      __threadfence_block();
+      tma_prefetch_desc(&p.tma_a);
+      tma_prefetch_desc(&p.tma_b);
+      if (p.use_tma_out) tma_prefetch_desc(&p.tma_out);
+    }
+  }
+  // Tensor memory is allocated beside the barrier: the producers start without it.  (A pair: the peer's barriers are initialised
+  // before anything signals them.)
+  if (CTAS == 2) { __syncwarp(); cluster_arrive_relaxed(); } else __syncthreads();
+  if (warp == kTmemWarp) {
+    if (CTAS == 2) { tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
+    else { tmem_alloc(tmem_slot, kTmemCols); tmem_relinquish(); }
+    tc_fence_before_sync();
+  }
   const int num_tiles = p.m_blocks * p.n_blocks;
   const int n_splits = SPLIT ? p.splits : 1;
   const int kb_per_split = SPLIT ? p.kb_per_split : p.k_blocks;
@@ -227,72 +265,54 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   const int cta_rank = CTAS == 2 ? static_cast<int>(cluster_ctarank()) : 0;
   const int first_tile = blockIdx.x / CTAS;        // both CTAs of a pair walk the same tiles
   const int tile_step = gridDim.x / CTAS;
-
-  if (warp == kProducerBWarp) {                    // one barrier a lane
-    if (lane < 2 * kMaxStages) mbar_init(&bars[lane], 1);
-    else if (lane < 2 * kMaxStages + 2) mbar_init(&acc_full[lane - 2 * kMaxStages], 1);
-    else if (lane < 2 * kMaxStages + 4) mbar_init(&acc_empty[lane - 2 * kMaxStages - 2], kEpiWarps * CTAS);
-    else if (lane < 2 * kMaxStages + 6) mbar_init(&bias_bar[lane - 2 * kMaxStages - 4], kEpiWarps);
-    else if (lane == 22) mbar_init(bias_free, kEpiWarps);
-    else if (lane == 23) mbar_init(tmem_free, kEpiWarps);
-    else if (lane == 24) mbar_init(peer_free, 1);
-    else if (lane == 25) *abort_flag = 0;
-    mbar_fence_init();
-  } else if (warp == 0) {
-    if (lane == 0) {
-      tma_prefetch_desc(&p.tma_a);
-      tma_prefetch_desc(&p.tma_b);
-      if (p.use_tma_out) tma_prefetch_desc(&p.tma_out);
-    }
-  } else if (warp == kTmemWarp) {
-    if (CTAS == 2) { tmem_alloc_pair(tmem_slot, kTmemCols); tmem_relinquish_pair(); }
-    else { tmem_alloc(tmem_slot, kTmemCols); tmem_relinquish(); }
-  }
-  tc_fence_before_sync();
-  // (a pair: the peer's barriers are initialised before anything signals them)
-  if (CTAS == 2) cluster_sync_all(); else __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem_base = *tmem_slot;
-  if (threadIdx.x == 0) GEMM_TL(1);
-  if (p.early_launch) pdl_launch_dependents();   // the next kernel may set itself up while this one runs
-  // everything before this kernel in the stream is complete and visible; the W producer of a GEMM on constant
-  // weights goes ahead and fills the ring's W halves meanwhile (the stages complete once A has arrived too)
-  if (!(p.w_const && warp == kProducerBWarp)) pdl_wait();
-  if (threadIdx.x == 0) GEMM_TL(2);
-
+  // What the producers' first loads are made of, ahead of the waits: behind them it was 700 cycles, most of it cold parameters.
+  int mg0, nb0;                                    // the first tile
+  tile_coords(p.reverse ? num_tiles - 1 - (SPLIT ? first_tile / n_splits : first_tile) : (SPLIT ? first_tile / n_splits : first_tile), p, mg0, nb0);
+  const int k_blocks = p.k_blocks, kb_per_tap = p.kb_per_tap, conv_stride = p.conv_stride, w_const = p.w_const, early_launch = p.early_launch;
+  asm volatile("" ::"r"(mg0), "r"(nb0), "r"(k_blocks), "r"(kb_per_tap), "r"(conv_stride), "r"(w_const), "r"(early_launch), "r"(num_work), "r"(kb_per_split));
   bool ok = true;
+  // Each role passes the waits in its own code, so that the instructions behind them are fetched meanwhile.
+  auto enter = [&](bool dependent) {
+    if (CTAS == 2) cluster_wait();
+    if (early_launch) pdl_launch_dependents();   // the next kernel may set itself up while this one runs
+    if (dependent) pdl_wait();                   // everything before this kernel in the stream is complete and visible
+  };
+
   if (warp == 0 || warp == kProducerBWarp) {
     // ------------------------------------------------------------------ producers: warp 0 loads A, the last warp B
     // The two operands have a warp each (128 KB of boxes from one thread: 476 ns a step, from two 396); a whole warp walks the
     // tiles and one elected lane issues, as in the UMMA warp (1 to 3 % at large M against a lone diverged thread).  The A warp
     // announces the bytes of the whole stage.
     const bool do_a = warp == 0, do_b = warp != 0;
+    // the W producer of a GEMM on constant weights goes ahead and fills the ring's W halves while the rest of the CTA waits for the
+    // stream's earlier work (the stages complete once A has arrived too)
+    enter(!(w_const && do_b));
     uint32_t it = 0;
+    int mg = mg0, nb = nb0;
     for (int work = first_tile; work < num_work && ok; work += tile_step) {
       const int tile = SPLIT ? work / n_splits : work, split = SPLIT ? work - tile * n_splits : 0;
-      int mg, nb;
-      tile_coords(p.reverse ? num_tiles - 1 - tile : tile, p.m_blocks, p.n_blocks, mg, nb);
+      if (work != first_tile) tile_coords(p.reverse ? num_tiles - 1 - tile : tile, p, mg, nb);
       const int row0 = (mg * CTAS + cta_rank) * kARows;       // this CTA's rows
-      const int kb0 = split * kb_per_split, kb1 = SPLIT ? min(p.k_blocks, kb0 + kb_per_split) : p.k_blocks;
+      const int kb0 = split * kb_per_split, kb1 = SPLIT ? min(k_blocks, kb0 + kb_per_split) : k_blocks;
       // position of a shallow k-block: column kx of the tap that reads phase `phase` of the strided rows, `shift` rows on
       // (running counters: three integer divisions per k-block held every kernel with shallow stages at 0.34 us per k-block;
       // without them 128x256 tiles, M = 577, N = 1024, K = 4096: 27.7 -> 26.0 us; 8 images of 577 tokens, 24 layers: 4.03 -> 3.87 ms)
       int kx = 0, phase = 0, shift = 0;
-      if (KD == 1) {
-        const int tap = kb0 / p.kb_per_tap;
-        kx = (kb0 - tap * p.kb_per_tap) * kBK;
-        phase = tap % p.conv_stride;
-        shift = tap / p.conv_stride;
+      if (KD == 1 && SPLIT) {
+        const int tap = kb0 / kb_per_tap;
+        kx = (kb0 - tap * kb_per_tap) * kBK;
+        phase = tap % conv_stride;
+        shift = tap / conv_stride;
       }
-      const int run = p.kb_per_tap * kBK;
+      const int run = kb_per_tap * kBK;
       for (int kb = kb0; kb < kb1; ++kb, ++it) {
         const int s = it % kStages;
         const uint32_t ph = (it / kStages) & 1u;
         // The W producer of constant weights skipped the grid-dependency wait above and has filled every stage once;
         // its next wait needs the consumer, which needs A, which needs the earlier kernels: join the dependency first,
         // so that the bounded wait below never runs while a predecessor is still working.
-        if (do_b && p.w_const && it == kStages) pdl_wait();
-        if (!warp_mbar_wait(&empty_bar[s], ph ^ 1u, abort_flag)) { ok = false; break; }
+        if (do_b && w_const && it == kStages) pdl_wait();
+        if (it >= kStages && !warp_mbar_wait(&empty_bar[s], ph ^ 1u, abort_flag)) { ok = false; break; }
         uint8_t* sa = smem + s * kStageBytes;
         uint8_t* sb = sa + kABytes * KD;
         if (elect_one()) {
@@ -322,7 +342,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         __syncwarp();
         if ((kx += kBK) == run) {
           kx = 0;
-          if (++phase == p.conv_stride) { phase = 0; ++shift; }
+          if (++phase == conv_stride) { phase = 0; ++shift; }
         }
       }
     }
@@ -342,7 +362,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     // The whole warp walks the tiles and one elected lane issues (see elect_one): with a lone diverged thread a UMMA cost about
     // 105 cycles of issue, which bounded the narrow tiles (128x64, M = 577, N = 1024, K = 4096: 18.2 -> 15.1 us; all 128x64
     // shapes -17 %, 128x128 -6 %, 128x256 -3 %, pair and wide tiles -1 %).
+    enter(true);
     if (cta_rank == 0) {
+      ok = warp_mbar_wait(tmem_ready, 0, abort_flag);
+      tc_fence_after_sync();
+      const uint32_t tmem_base = *tmem_slot;
       constexpr uint32_t idesc = make_idesc_bf16(kARows * CTAS, Cfg::kMmaN, 0, 0);
       uint32_t it = 0, tcount = 0;
       for (int work = first_tile; work < num_work && ok; work += tile_step, ++tcount) {
@@ -394,6 +418,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     const int ew = warp - 2;                    // 0..7
     const int quarter = warp & 3;               // TMEM lane quarter this warp may read
     const int half = ew >> 2;                   // which 128 accumulator columns
+    enter(true);
+    if (warp == kTmemWarp) {
+      if (lane < CTAS) mbar_arrive_cluster(tmem_ready, lane);
+      __syncwarp();
+    }
+    ok = warp_mbar_wait(tmem_ready, 0, abort_flag);
+    tc_fence_after_sync();
+    const uint32_t tmem_base = *tmem_slot;
     uint32_t tcount = 0;
     // This warp has read its part of the accumulator.  Nobody waits for the last ones: no remote arrival may be under way to a
     // CTA that retires.
@@ -412,7 +444,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     for (int work = first_tile; work < num_work && ok; work += tile_step, ++tcount) {
       const int tile = SPLIT ? work / n_splits : work, split = SPLIT ? work - tile * n_splits : 0;
       int mg, nb;
-      tile_coords(p.reverse ? num_tiles - 1 - tile : tile, p.m_blocks, p.n_blocks, mg, nb);
+      tile_coords(p.reverse ? num_tiles - 1 - tile : tile, p, mg, nb);
       const int ycoord = (mg * CTAS + cta_rank) * kARows + (HALF ? quarter & 1 : quarter) * 32;      // this warp's first row
       const int arow = ycoord + lane;                             // row of A (== accumulator row)
       const uint32_t acc = tcount % kAccBuffers;
@@ -864,7 +896,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     cluster_sync_all();
     tc_fence_after_sync();
     if (warp == kTmemWarp) {
-      if (CTAS == 2) tmem_dealloc_pair(tmem_base, kTmemCols); else tmem_dealloc(tmem_base, kTmemCols);
+      if (CTAS == 2) tmem_dealloc_pair(*tmem_slot, kTmemCols); else tmem_dealloc(*tmem_slot, kTmemCols);
     }
     if (lane == 0) atomicCAS(p.status, DEV_OK, DEV_ERR_WAIT_TIMEOUT);
   }

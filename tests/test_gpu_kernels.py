@@ -164,6 +164,26 @@ def test_gemm_half_height_tiles_agree_bit_for_bit(M, N, K, act, out_fp32):
     assert e.value.status == 2
 
 
+@pytest.mark.parametrize("left", range(1, 9))
+def test_gemm_walks_every_tile_of_every_panel(left):
+    """Tiles are walked in panels of eight row blocks and a last one of `left`; launches of different shapes follow one another
+    without a host wait, so that one's tensor memory and barriers pass to the next while its CTAs retire one by one."""
+    import paper_2609_31551_b200 as P
+    rng = np.random.Generator(np.random.PCG64(40 + left))
+    M, N, K = 128 * (8 + left) - 5, 320, 128
+    A, W, b = _bf16_exact(rng, (M, K)), _bf16_exact(rng, (N, K), 0.05), _bf16_exact(rng, (N,), 0.5)
+    y = O.linear(O._t(A), O._t(W), O._t(b))
+    dA, dW, db = _dev(A), _dev(W), _dev(b)
+    runs = [(shape, budget) for budget in (148, 4, 2) for shape in (5, 14, 1, 2, 8)]
+    outs = [P.kernel_gemm(dA, dW, db, sm_budget=budget, tile_shape=shape) for shape, budget in runs]
+    torch.cuda.synchronize()
+    tol = 2.0 ** -8 * y.abs() + 1e-5                 # one rounding to bf16; sums of 128 products in fp32
+    for (shape, budget), (out, status) in zip(runs, outs):
+        assert int(status[0]) == 0, (shape, budget)
+        assert torch.equal(out, outs[0][0]), (shape, budget)
+    assert not ((outs[0][0].double().cpu() - y).abs() > tol).any()
+
+
 def test_gemm_wide_tile_is_refused_where_it_does_not_exist():
     import paper_2609_31551_b200 as P
     rng = np.random.Generator(np.random.PCG64(92))
