@@ -48,6 +48,7 @@ namespace eas {
 
 constexpr int kTcTile = 128;            // query rows per tile
 constexpr float kRescaleThreshold = 8.0f;
+constexpr uint32_t kWarmPiece = 16384;
 
 struct AttnRrParams {
   CUtensorMap map_q_lo;   // qkv [T, 3d], box {64 columns, 128 rows}, 128-byte swizzle
@@ -65,6 +66,9 @@ struct AttnRrParams {
   // an item's units: item_full of them with kWg query tiles, the others with small_tiles (<= kWg): see attention_plan
   int item_full[128];
   int small_tiles;
+  // Constant memory that later launches read (weights), towards L2 beside this one: each CTA asks for its share
+  const uint8_t* warm[4];
+  uint32_t warm_bytes[4];
   uint32_t* status;
   int early_launch;       // see pdl_launch_dependents
 };
@@ -214,11 +218,18 @@ __global__ void __launch_bounds__(AttnRrSmem<HD, OWN_P>::kThreads, 1) attn_rr_ke
       uint32_t g = 0, round = 0;
       bool ok = true;
       int cursor = 0;
+      auto warm_up = [&]() {
+#pragma unroll 1
+        for (int r = 0; r < 4; ++r)
+          for (uint32_t off = blockIdx.x * kWarmPiece; off < p.warm_bytes[r]; off += gridDim.x * kWarmPiece)
+            l2_prefetch(p.warm[r] + off, min(kWarmPiece, p.warm_bytes[r] - off));
+      };
       for (int unit = unit_at(0); unit < p.total_units && ok; unit = unit_at(++round)) {
         const RrUnit u = decode(unit, cursor);
         for (int j = 0; j < u.n_kv && ok; ++j)
           for (int st = 0; st < u.n_streams; ++st, ++g) {
             const int s = g % NST;
+            if (g == NST) warm_up();
             if (!mbar_wait(&kv_empty[s], ((g / NST) & 1u) ^ 1u, abort_flag)) { ok = false; break; }
             const int x = (u.head0 + st) * HD, y = u.row0 + j * KEYS;
             mbar_expect_tx(&k_full[s], L::kKTxBytes);
@@ -229,6 +240,7 @@ __global__ void __launch_bounds__(AttnRrSmem<HD, OWN_P>::kThreads, 1) attn_rr_ke
             if (HI) tma_load_2d(v_tile(s) + L::kAtomBytes, &p.map_k_lo, &v_full[s], 2 * p.d_model + x + 64, y);
           }
       }
+      if (g <= NST) warm_up();
       // The last hand-backs of the stages are asynchronous arrivals (UMMA commits) that nothing else waits for: they have to be
       // in before the CTA's shared memory passes to another one.  (Never used stages pass at once.)
       for (uint32_t e = g; e < g + NST && ok; ++e) ok = mbar_wait(&kv_empty[e % NST], ((e / NST) & 1u) ^ 1u, abort_flag);
