@@ -287,7 +287,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
     // the W producer of a GEMM on constant weights goes ahead and fills the ring's W halves while the rest of the CTA waits for the
     // stream's earlier work (the stages complete once A has arrived too)
     enter(!(w_const && do_b));
-    uint32_t it = 0;
+    uint32_t it = 0, s = 0, ph = 1;                 // stages filled; the ring's position and the parity of its hand-back
+    uint32_t ready = 1;                             // this stage has been handed back (tested beside the loads of the stage before)
+    const CUtensorMap* map = do_a ? &p.tma_a : &p.tma_b;
     int mg = mg0, nb = nb0;
     for (int work = first_tile; work < num_work && ok; work += tile_step) {
       const int tile = SPLIT ? work / n_splits : work, split = SPLIT ? work - tile * n_splits : 0;
@@ -305,14 +307,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         shift = tap / conv_stride;
       }
       const int run = kb_per_tap * kBK;
+      const int row_deep = do_a ? row0 : nb * kTileN + cta_rank * kBRows;      // first row of a deep stage's box
       for (int kb = kb0; kb < kb1; ++kb, ++it) {
-        const int s = it % kStages;
-        const uint32_t ph = (it / kStages) & 1u;
         // The W producer of constant weights skipped the grid-dependency wait above and has filled every stage once;
         // its next wait needs the consumer, which needs A, which needs the earlier kernels: join the dependency first,
         // so that the bounded wait below never runs while a predecessor is still working.
         if (do_b && w_const && it == kStages) pdl_wait();
-        if (it >= kStages && !warp_mbar_wait(&empty_bar[s], ph ^ 1u, abort_flag)) { ok = false; break; }
+        if (!warp_mbar_wait_tested(ready, &empty_bar[s], ph, abort_flag)) { ok = false; break; }
+        const uint32_t s_next = s + 1 == kStages ? 0u : s + 1, ph_next = s + 1 == kStages ? ph ^ 1u : ph;
         uint8_t* sa = smem + s * kStageBytes;
         uint8_t* sb = sa + kABytes * KD;
         if (elect_one()) {
@@ -320,13 +322,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           if (do_a && cta_rank == 0) mbar_expect_tx(&full_bar[s], CTAS * kStageBytes);
           if (KD == 2) {
             // deep stage (plain GEMM only): [A k-block 0][A k-block 1][B ...] from one 3-D box per operand
-            if (CTAS == 2) {
-              if (do_a) tma_load_3d_pair(sa, &p.tma_a, &full_bar[s], 0, row0, kb * KD);
-              if (do_b) tma_load_3d_pair(sb, &p.tma_b, &full_bar[s], 0, nb * kTileN + cta_rank * kBRows, kb * KD);
-            } else {
-              if (do_a) tma_load_3d(sa, &p.tma_a, &full_bar[s], 0, row0, kb * KD);
-              if (do_b) tma_load_3d(sb, &p.tma_b, &full_bar[s], 0, nb * kTileN, kb * KD);
-            }
+            if (CTAS == 2) tma_load_3d_pair(do_a ? sa : sb, map, &full_bar[s], 0, row_deep, kb * KD);
+            else tma_load_3d(do_a ? sa : sb, map, &full_bar[s], 0, row_deep, kb * KD);
           } else if (CTAS == 2) {
             if (do_a) tma_load_3d_pair(sa, &p.tma_a, &full_bar[s], kx, phase, row0 + shift);
             if (do_b) {
@@ -340,7 +337,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
           }
         }
         __syncwarp();
-        if ((kx += kBK) == run) {
+        s = s_next;
+        ph = ph_next;
+        ready = mbar_test_wait(&empty_bar[s], ph);
+        if (KD == 1 && (kx += kBK) == run) {
           kx = 0;
           if (++phase == conv_stride) { phase = 0; ++shift; }
         }
@@ -368,28 +368,33 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
       tc_fence_after_sync();
       const uint32_t tmem_base = *tmem_slot;
       constexpr uint32_t idesc = make_idesc_bf16(kARows * CTAS, Cfg::kMmaN, 0, 0);
-      uint32_t it = 0, tcount = 0;
+      uint32_t tcount = 0;
+      // The ring's position and phase as running values, the next stage's barrier tested beside this stage's UMMAs (and by the producers
+      // beside their loads): what a step costs the issuing warp apart from its UMMAs, 185 cycles before, bounds tiles of up to 128
+      // columns.  M = 577, weights in L2: (1024, 4096) as half-height 128x96 9.29 -> 8.75 us, (1024, 1024) 4.98 -> 4.75, M = 468,
+      // (1280, 5120) 10.72 -> 10.02; (4096, 1024) as 128x160 8.79 -> 8.53.
+      uint32_t s = 0, ph = 0, ready = mbar_test_wait(&full_bar[0], 0);
+      const uint64_t adesc0 = make_smem_desc(smem_u32(smem), 16, 1024, kSwizzle128B);
       for (int work = first_tile; work < num_work && ok; work += tile_step, ++tcount) {
         const uint32_t acc = tcount % kAccBuffers;
         const uint32_t acc_ph = (tcount / kAccBuffers) & 1u;
-        if (!warp_mbar_wait(&acc_empty[acc], acc_ph ^ 1u, abort_flag)) { ok = false; break; }
+        if (tcount >= kAccBuffers && !warp_mbar_wait(&acc_empty[acc], acc_ph ^ 1u, abort_flag)) { ok = false; break; }
         tc_fence_after_sync();
         const uint32_t tmem_d = tmem_base + acc * kAccCols;
         const int split = SPLIT ? work % n_splits : 0;
-        const int kb0 = split * kb_per_split, kb1 = SPLIT ? min(p.k_blocks, kb0 + kb_per_split) : p.k_blocks;
-        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-          const int s = it % kStages;
-          const uint32_t ph = (it / kStages) & 1u;
-          if (!warp_mbar_wait(&full_bar[s], ph, abort_flag)) { ok = false; break; }
+        const int kb0 = split * kb_per_split, kb1 = SPLIT ? min(k_blocks, kb0 + kb_per_split) : k_blocks;
+        for (int kb = kb0; kb < kb1; ++kb) {
+          if (!warp_mbar_wait_tested(ready, &full_bar[s], ph, abort_flag)) { ok = false; break; }
           if (tcount == 0 && kb == kb0 && lane == 0) GEMM_TL(3);
           tc_fence_after_sync();
-          const uint32_t a_addr = smem_u32(smem + s * kStageBytes);
-          const uint32_t b_addr = a_addr + kABytes * KD;
+          const uint32_t s_next = s + 1 == kStages ? 0u : s + 1, ph_next = s + 1 == kStages ? ph ^ 1u : ph;
+          ready = mbar_test_wait(&full_bar[s_next], ph_next);
+          const uint64_t a_desc = adesc0 + s * (kStageBytes >> 4);
           if (elect_one()) {
 #pragma unroll
             for (int a = 0; a < KD; ++a) {         // the 64-wide k-blocks of the stage: one swizzle-atom block each
-              const uint64_t adesc = make_smem_desc(a_addr + a * kABytes, 16, 1024, kSwizzle128B);
-              const uint64_t bdesc = make_smem_desc(b_addr + a * kBAtom, 16, 1024, kSwizzle128B);
+              const uint64_t adesc = a_desc + a * (kABytes >> 4);
+              const uint64_t bdesc = a_desc + ((kABytes * KD + a * kBAtom) >> 4);
 #pragma unroll
               for (int k = 0; k < kBK / 16; ++k) {
                 // advancing 16 bf16 = 32 bytes along K inside the swizzle atom: +2 in the (>>4) address field
@@ -410,6 +415,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
             }
           }
           __syncwarp();
+          s = s_next;
+          ph = ph_next;
         }
       }
     }
