@@ -93,16 +93,16 @@ static eas_status make_a_tmap(CUtensorMap* m, const void* a, int64_t run, int64_
 // "Deep" maps: the same matrices seen as {64 columns, rows, K/64 blocks}, so that ONE box {64, rows, 2} brings two
 // 64-wide k-blocks, each landing as its own swizzle-atom block [rows x 128 bytes] (see GemmCfg).  A k-block index
 // past K/64 is filled with zeros.
-static eas_status make_w_tmap_deep(CUtensorMap* m, const void* w, int64_t N, int64_t K, uint32_t box_rows) {
+static eas_status make_w_tmap_deep(CUtensorMap* m, const void* w, int64_t N, int64_t K, uint32_t box_rows, uint32_t depth = 2) {
   const uint64_t dims[3] = {kBK, static_cast<uint64_t>(N), static_cast<uint64_t>(K / kBK)};
   const uint64_t strides[2] = {static_cast<uint64_t>(K) * 2, kBK * 2};
-  const uint32_t box[3] = {kBK, box_rows, 2};
+  const uint32_t box[3] = {kBK, box_rows, depth};
   return make_tmap(m, w, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
-static eas_status make_a_tmap_deep(CUtensorMap* m, const void* a, int64_t run, int64_t row_elems, int64_t rows, uint32_t box_rows) {
+static eas_status make_a_tmap_deep(CUtensorMap* m, const void* a, int64_t run, int64_t row_elems, int64_t rows, uint32_t box_rows, uint32_t depth = 2) {
   const uint64_t dims[3] = {kBK, static_cast<uint64_t>(rows), static_cast<uint64_t>(run / kBK)};
   const uint64_t strides[2] = {static_cast<uint64_t>(row_elems) * 2, kBK * 2};
-  const uint32_t box[3] = {kBK, box_rows, 2};
+  const uint32_t box[3] = {kBK, box_rows, depth};
   return make_tmap(m, a, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
@@ -356,7 +356,7 @@ static GemmKernel gemm_kernel_of(int tile, bool deep) {
     }
     if constexpr (ACT != ACT_SWIGLU && !SPLIT && !(ACT == ACT_GELU && OUT == OUT_F32)) {
       if (kTiles[tile].half && !deep) return nullptr;
-      if (tile == TILE_H64) return gemm_kernel<ACT, OUT, 2, 64, 2, false, true>;
+      if (tile == TILE_H64) return gemm_kernel<ACT, OUT, 2, 64, 4, false, true>;
       if (tile == TILE_H96) return gemm_kernel<ACT, OUT, 2, 96, 2, false, true>;
       if (tile == TILE_H128) return gemm_kernel<ACT, OUT, 2, 128, 2, false, true>;
       if (tile == TILE_H160) return gemm_kernel<ACT, OUT, 2, 160, 2, false, true>;
@@ -753,22 +753,25 @@ struct GemmCall {
 //
 // Half-height tiles pull 64 rows of A and half the weight rows per SM and k-block, less than any other shape of their width: 112 rows
 // as 128x96 against 176 as 256x96 and 192 as 128x64.  They are for launches of one wave (with more, the wider tiles' fewer operand bytes
-// per output win), fitted to 190 shapes forced with weights that rotate through memory.  On a share of the SMs a pair is set up
-// behind the predecessor (kShareUs more); with fewer than eight k-blocks they pay only while half the SMs suffice (M = 784, N = 768, K = 256: 4.0 us
-// as 128x96, 3.5 as 128x64; M = 196, N = 256: 3.5 and 3.8).  (N, K) on 148 SMs, best other shape -> half-height:
-//   M = 577:  (1024, 4096) 14.5 us as 128x256 ... 14.9 as 256x96 -> 10.7 as 128x96;  (1024, 1024) 6.4 -> 6.1
-//   M = 468:  (1280, 5120) 17.8 -> 12.5;  (1280, 1280) 7.1 -> 6.5;  (3840, 1280) 8.5 -> 8.2 as 128x224
-//   M = 196:  (256, 1024) 5.8 -> 4.5 as 128x64
+// per output win), fitted to 230 shapes of up to 2048 rows on 148 and 74 SMs with the weights in L2, where the attention launch puts
+// them.  On a share of the SMs a pair is set up behind the predecessor (kShareUs more); with fewer than eight k-blocks only the two
+// narrowest pay, and while half the SMs suffice (M = 784, N = 1024, K = 256: 3.9 us as 128x64, 4.8 as half-height 128x224).  Over those
+// shapes the choice is 0.5 % behind the best tile on average; with the figures of the kernels before their set-up and loops were shortened it
+// was 1.5 %, and up to 19 % on 74 SMs (M = 196, N = K = 256: 4.3 us as 128x64, 3.6 as half-height 128x64; M = 108, (3840, 1280): 6.6 and 5.6 as
+// 128x128).  (N, K) on 148 SMs, best other shape -> half-height:
+//   M = 577:  (1024, 4096) 14.5 us as 128x256 ... 14.9 as 256x96 -> 10.7 as 128x96 (8.8 now);  (1024, 1024) 6.4 -> 6.1 (4.8)
+//   M = 468:  (1280, 5120) 17.8 -> 12.5 (10.0);  (1280, 1280) 7.1 -> 6.5 (5.1);  (3840, 1280) 8.5 -> 8.2 as 128x224 (6.5)
+//   M = 196:  (256, 1024) 5.8 -> 4.5 as 128x64 (3.5)
 template <typename Usable>
 static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bool plain, Usable usable, double* us = nullptr) {
-  constexpr double kShareUs = 1.05;
+  constexpr double kShareUs = 0.63;
   struct Cost { int tile; double base, per_kb, per_wave, partial; };    // us
   static const Cost costs[] = {{TILE_SINGLE, 5.24, 0.351, 0.52, 0.87}, {TILE_PAIR, 6.44, 0.323, 0.25, 0.92}, {TILE_WIDE, 4.81, 0.586, 5.1, 0.89},
                                {TILE_N128, 3.91, 0.228, 0.45, 0.95}, {TILE_N64, 3.48, 0.173, 0.20, 1.0}, {TILE_N160, 4.61, 0.265, 0.31, 0.92},
                                {TILE_N224, 5.02, 0.329, 0.29, 0.88}, {TILE_P96, 4.66, 0.163, 0.13, 0.79}, {TILE_P128, 5.07, 0.181, 0.28, 0.84},
                                {TILE_P160, 5.20, 0.212, 0.48, 0.80}, {TILE_P192, 5.52, 0.250, 0.34, 0.85}, {TILE_P224, 5.98, 0.291, 0.20, 0.84},
-                               {TILE_H64, 3.19, 0.120, 0.0, 0.69}, {TILE_H96, 3.66, 0.122, 0.0, 0.78}, {TILE_H128, 3.83, 0.132, 0.0, 0.70},
-                               {TILE_H160, 4.27, 0.140, 0.0, 0.86}, {TILE_H224, 4.77, 0.174, 0.0, 0.86}};
+                               {TILE_H64, 1.29, 0.088, 1.16, 0.80}, {TILE_H96, 1.29, 0.100, 1.36, 0.70}, {TILE_H128, 1.46, 0.108, 2.24, 0.60},
+                               {TILE_H160, 1.32, 0.113, 2.39, 0.83}, {TILE_H224, 1.59, 0.143, 2.73, 0.70}};
   int tile = TILE_SINGLE;
   double best = 0.0;
   for (const Cost& c : costs) {
@@ -776,12 +779,12 @@ static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bo
     if (t.ctas > budget || !usable(c.tile)) continue;
     const int64_t slots = budget / t.ctas;
     const int64_t tiles = ((M + t.rows - 1) / t.rows) * ((N + t.cols - 1) / t.cols) * splits;
-    if (t.half && tiles > (kb < 8 ? slots / 2 : slots)) continue;
+    if (t.half && (tiles > (kb < 8 ? slots / 2 : slots) || (kb < 8 && t.cols > 96))) continue;
     const int64_t rem = tiles % slots;
     const double waves = static_cast<double>(tiles / slots) + (rem != 0 ? c.partial + (1.0 - c.partial) * static_cast<double>(rem) / static_cast<double>(slots) : 0.0);
     const double shallow = t.cols <= 128 && !plain ? 1.08 : 1.0;       // convolutions: no deep stages (128x64 +14 %, 256x128 +7 %, 128x128 +5 %)
     double cost = c.base + waves * (kb * c.per_kb * shallow + c.per_wave);
-    if (t.half) cost = 1.02 * (cost + (budget < g_device_sms ? kShareUs : 0.0));      // 2 % in hand: what the fit is off by
+    if (t.half && budget < g_device_sms) cost += kShareUs;
     if (best == 0.0 || cost < best) { best = cost; tile = c.tile; }
   }
   if (us != nullptr) *us = best;
@@ -849,16 +852,17 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
   }
   const int ctas = kTiles[tile].ctas, tile_n = kTiles[tile].cols;
   const bool deep = is_deep(tile);
+  const int depth = tile == TILE_H64 ? 4 : deep ? 2 : 1;      // 64-wide k-blocks of a stage
   GemmParams p{};
-  if (deep) EAS_TRY(make_a_tmap_deep(&p.tma_a, g.A, g.a_run, g.a_row_elems, g.a_rows, kTiles[tile].half ? kBM / 2 : kBM));
+  if (deep) EAS_TRY(make_a_tmap_deep(&p.tma_a, g.A, g.a_run, g.a_row_elems, g.a_rows, kTiles[tile].half ? kBM / 2 : kBM, depth));
   else EAS_TRY(make_a_tmap(&p.tma_a, g.A, g.a_run, g.a_row_elems, g.conv_stride, g.a_rows));
   // weight rows per TMA box: the CTA's share of a 256-column accumulator, or the narrow tile's columns
   const int w_rows = std::min(tile_n, static_cast<int>(kBN)) / ctas;
-  if (gemm_alt(tile_n) || w_rows < 64) EAS_TRY(deep ? make_w_tmap_deep(&p.tma_b, L.w, L.N, L.K, w_rows) : make_w_tmap(&p.tma_b, L.w, L.N, L.K, w_rows));
+  if (gemm_alt(tile_n) || w_rows < 64) EAS_TRY(deep ? make_w_tmap_deep(&p.tma_b, L.w, L.N, L.K, w_rows, depth) : make_w_tmap(&p.tma_b, L.w, L.N, L.K, w_rows));
   else p.tma_b = w_rows == 256 ? L.tmap : w_rows == 128 ? (deep ? L.tmap_half_deep : L.tmap_half) : (deep ? L.tmap_quarter_deep : L.tmap_quarter);
   p.M = g.M; p.N = L.N;
   p.kb_per_tap = static_cast<int>(g.a_run / kBK);
-  p.k_blocks = deep ? (p.kb_per_tap + 1) / 2 : p.kb_per_tap * g.taps;
+  p.k_blocks = deep ? (p.kb_per_tap + depth - 1) / depth : p.kb_per_tap * g.taps;
   p.conv_stride = g.conv_stride;
   p.reverse = g.reverse;
   p.w_const = g.w_const;

@@ -34,7 +34,8 @@ constexpr int kTmemWarp = 2;                             // the first epilogue w
 // KD = 2 ("deep", TN <= 128): a stage holds TWO 64-wide k-blocks of each operand, fetched by ONE TMA operation per operand
 // (a 3-D box {64 columns, rows, 2 k-blocks}, which lands as two consecutive swizzle-atom blocks): a step of a ring costs
 // some 0.16 us whatever its bytes, which is what bounds small tiles (deep against shallow: 128x64 -12 %, 256x96 -6 to -14 %,
-// 256x128 -7 % at K = 1024, 128x128 -5 %).  Wider tiles are no faster with it.
+// 256x128 -7 % at K = 1024, 128x128 -5 %).  Wider tiles are no faster with it.  KD = 4, half-height 128x64 tiles: four (M = 300, N = 1024,
+// K = 4096: 7.9 -> 7.1 us, M = 196, N = 256, K = 1024: 3.7 -> 3.5); 128x96 would have a ring of three stages, 8.75 -> 9.2 us.
 // TN < 256: with few tokens a launch has fewer 256-column tiles than the device has SMs and the K loop of ONE tile is the
 // kernel's time, at the rate one SM pulls operands from L2 (48 KB per 64-wide k-block of a 128x256 tile, 24 KB of a 128x64
 // or 256x128 one): more, narrower tiles shorten that loop and use the idle SMs, and the width that just fills one wave is best.
@@ -44,7 +45,7 @@ constexpr int kTmemWarp = 2;                             // the first epilogue w
 // SM pulls operands, and no other shape needs fewer of them: M = 577, N = 1024, K = 4096: 128x96 over 110 CTAs 10.7 us (112 rows a
 // k-block and SM), 256x96 over 66 14.9 (176), 128x64 over 80 17.5 (192).
 template <int CTAS, int TN, int KD = 1, bool HALF = false> struct GemmCfg {
-  static_assert(!HALF || (CTAS == 2 && KD == 2), "half-height tiles: CTA pairs, deep stages");
+  static_assert(!HALF || (CTAS == 2 && KD >= 2), "half-height tiles: CTA pairs, deep stages");
   static constexpr int kARows = HALF ? 64 : kBM;                   // rows of A per CTA
   static constexpr int kABytes = kARows * kBK * 2;                 // per 64-wide k-block
   static constexpr int kBBytes = (TN / CTAS) * kBK * 2;
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   static_assert(TN < 512 || (CTAS == 2 && ACT != ACT_SWIGLU), "wide tiles: CTA pairs, no gated epilogue");
   static_assert(TN >= 256 || OUT != OUT_F32_FOLD, "narrow tiles: no folding epilogue");
   static_assert(TN >= 128 || ACT != ACT_SWIGLU, "a gated epilogue halves the columns: 128 at least");
-  static_assert(KD == 1 || (KD == 2 && TN <= kBN), "one or two 64-wide k-blocks per stage");
+  static_assert(KD == 1 || ((KD == 2 || KD == 4) && TN <= kBN), "one, two or four 64-wide k-blocks per stage");
   using Cfg = GemmCfg<CTAS, TN, KD, HALF>;
   constexpr int kARows = Cfg::kARows, kABytes = Cfg::kABytes;
   constexpr int kStages = Cfg::kStages;
@@ -320,7 +321,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
         if (elect_one()) {
           // both CTAs' loads of a pair complete on the leader's barrier; the leader announces the bytes of both
           if (do_a && cta_rank == 0) mbar_expect_tx(&full_bar[s], CTAS * kStageBytes);
-          if (KD == 2) {
+          if (KD >= 2) {
             // deep stage (plain GEMM only): [A k-block 0][A k-block 1][B ...] from one 3-D box per operand
             if (CTAS == 2) tma_load_3d_pair(do_a ? sa : sb, map, &full_bar[s], 0, row_deep, kb * KD);
             else tma_load_3d(do_a ? sa : sb, map, &full_bar[s], 0, row_deep, kb * KD);
