@@ -3,7 +3,7 @@
 //   warp 0, 10  TMA producers, one thread per operand (A tiles in warp 0, W tiles in warp 10) into a shared-memory ring
 //   warp 1      UMMA issuer: tcgen05.mma (128x256x16, or 256x256x16 for a CTA pair), fp32 accumulators in TMEM, two
 //               accumulator buffers (2 x 256 columns) so that the epilogue of tile i overlaps the main loop of tile i+1
-//   warps 2..9  epilogue: tcgen05.ld -> bias / activation / rotary -> swizzled shared-memory staging -> TMA store
+//   warps 2..9  epilogue (warp 2 also allocates tensor memory and gives it back): tcgen05.ld -> bias / activation / rotary -> swizzled shared-memory staging -> TMA store
 //               (TMA reduce-add into the fp32 residual stream); scatter epilogues (row maps) store directly
 //
 // Tile shapes (template arguments CTAS, TN, KD; the launcher picks by estimated time): one CTA per 128 x {64, 128, 160, 224,
@@ -43,7 +43,7 @@ constexpr int kTmemWarp = 2;                             // the first epilogue w
 // rows in ALL 128 lanes of its tensor memory: lanes 0..63 hold columns 0 .. TN/2 - 1 of the rows, lanes 64..127 the others (measured:
 // 33 cycles per 128x96x16, 60 per 128x224x16, the rate of the 256-row form).  With one tile a CTA the K loop runs at the rate an
 // SM pulls operands, and no other shape needs fewer of them: M = 577, N = 1024, K = 4096: 128x96 over 110 CTAs 10.7 us (112 rows a
-// k-block and SM), 256x96 over 66 14.9 (176), 128x64 over 80 17.5 (192).
+// k-block and SM; 9.4 with the present set-up and loops, 8.8 with the weights in L2), 256x96 over 66 14.9 (176), 128x64 over 80 17.5 (192).
 template <int CTAS, int TN, int KD = 1, bool HALF = false> struct GemmCfg {
   static_assert(!HALF || (CTAS == 2 && KD >= 2), "half-height tiles: CTA pairs, deep stages");
   static constexpr int kARows = HALF ? 64 : kBM;                   // rows of A per CTA
