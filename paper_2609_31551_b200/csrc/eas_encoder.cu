@@ -1179,8 +1179,11 @@ static AttnPlan attention_plan(const int32_t* cu, int n_items, int H, int budget
 // GEMM of one wave otherwise waits for its first weights (1.1 us from HBM instead of 0.7).  Up to kWarmTokens, where the GEMMs are
 // such launches, and kWarmBytes a block, what one attention launch of 8 us brings in without holding up its neighbours.  Whole calls,
 // us: one 336 x 336 image (24 MB a block, all four) 1184 -> 1167, 30 s of audio (39 MB) 3092 -> 3055 with 13 to 16 MB, 3067 with 29 and
-// 3071 with all, one 252 x 364 image (52 MB) 1814 -> 1781 with 26 MB, 1828 with 42 and 1847 with all; 2308 tokens +-0.
-constexpr int64_t kWarmTokens = 2048;
+// 3071 with all, one 252 x 364 image (52 MB) 1814 -> 1781 with 26 MB, 1828 with 42 and 1847 with all; 2308 tokens +-0.  Below
+// kWarmFewTokens the whole block is bound by its weights' way from HBM and what is asked for delays what comes first: only the block's
+// last weights.  64 tokens of d 1024: none 833, the last 813, all 903; of d 1280, gated: 1370, 1338, MLP-up (26 MB) 1479; 50 of audio:
+// 1284, 1256, both of the MLP 1334; with 200 and 256 tokens both or all are the better ones (1310, 1282, 1273; 970, 956, 946).
+constexpr int64_t kWarmTokens = 2048, kWarmFewTokens = 160;
 constexpr uint64_t kWarmBytes = 28u << 20;
 struct WarmList {
   const bf16* w[4] = {};
@@ -1546,7 +1549,9 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
     }
     EAS_TRY(mark(e, EAS_KC_ATTENTION, stream));
     WarmList warm;
-    if (T <= kWarmTokens) {
+    if (T < kWarmFewTokens) {
+      warm.add(L.fc2);
+    } else if (T <= kWarmTokens) {
       warm.add(L.fc1);
       warm.add(L.fc2);
       if (li + 1 < c.n_layers) warm.add(e->layers[li + 1].qkv);
