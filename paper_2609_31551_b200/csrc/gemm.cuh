@@ -895,16 +895,25 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
 
   // The warps retire one by one.  A barrier of the pair here costs 0.6 us a launch, tensor memory given back behind the last store
   // 0.15 (a chain of launches that each load and store 32 KB a CTA, 148 CTAs: 3.4 us with both, 2.6 without); whole calls, with the one
-  // barrier at set-up: one 224 x 224 image 75.7 -> 71.0 us, one 336 x 336 image 1253 -> 1223, one of 252 x 364 1941 -> 1874.  Only
-  // after a wait that ran out does everybody who is still there meet (a cluster barrier does not count threads that have
-  // retired), so that tensor memory is given back when nobody uses it any more.
+  // barrier at set-up: one 224 x 224 image 75.7 -> 71.0 us, one 336 x 336 image 1253 -> 1223, one of 252 x 364 1941 -> 1874.
+  // After a wait that ran out everybody who is still there meets (a cluster barrier does not count threads that have retired), so that
+  // neither CTA of a pair retires while the other may still signal it and a single CTA's tensor memory goes back when nobody uses it any
+  // more.  A pair's goes back BEFORE that: its deallocation may wait for the other CTA's, whose warp may have given up while this one's
+  // was already under way, so nobody who owes one may stand at the barrier.  Who still uses the memory then is waited for by time: the other
+  // roles leave at their next wait, and without this warp's arrivals the issuer has two more tiles at most.
   if (!ok) {
     __syncwarp();
     tc_fence_before_sync();
+    if (CTAS == 2 && warp == kTmemWarp) {
+      const long long t0 = clock64();
+      while (clock64() - t0 < kWaitCycleLimit / 8) {}
+      tc_fence_after_sync();
+      tmem_dealloc_pair(*tmem_slot, kTmemCols);
+    }
     cluster_sync_all();
-    tc_fence_after_sync();
-    if (warp == kTmemWarp) {
-      if (CTAS == 2) tmem_dealloc_pair(*tmem_slot, kTmemCols); else tmem_dealloc(*tmem_slot, kTmemCols);
+    if (CTAS == 1 && warp == kTmemWarp) {
+      tc_fence_after_sync();
+      tmem_dealloc(*tmem_slot, kTmemCols);
     }
     if (lane == 0) atomicCAS(p.status, DEV_OK, DEV_ERR_WAIT_TIMEOUT);
   }
