@@ -276,6 +276,13 @@ eas_status eas_kernel_gemm_tile(const void* A, const void* W, const void* bias, 
                                 int32_t M, int32_t N, int32_t K, int32_t act, int32_t out_fp32, int32_t sm_budget,
                                 void* stream, uint32_t* status_dev, int32_t tile_shape);
 
+/* For tests of the bounded waits: the same launch with loads of the weights that bring half of what each stage waits for.  Nothing is
+ * read or written out of range and every load ends; the kernel's waits run out after about a second, it raises the status word to 1,
+ * gives tensor memory back and returns.  `out` is not written. */
+eas_status eas_kernel_gemm_starved(const void* A, const void* W, const void* bias, void* out, const float* resid,
+                                   int32_t M, int32_t N, int32_t K, int32_t act, int32_t out_fp32, int32_t sm_budget,
+                                   void* stream, uint32_t* status_dev, int32_t tile_shape);
+
 /* y[rows,d] = norm(x[rows,d]): kind 0 LayerNorm (gamma, beta), 1 RMSNorm (gamma), 2 plain cast.  x device fp32;
  * gamma/beta device bf16; y device bf16 (out_fp32 = 0) or fp32.  d % 128 == 0, d <= 2048. */
 eas_status eas_kernel_norm(const float* x, void* y, const void* gamma, const void* beta, int32_t rows, int32_t d,

@@ -16,7 +16,7 @@ STATUS_NAMES = {0: "EAS_OK", 1: "EAS_ERR_INVALID_ARG", 2: "EAS_ERR_UNSUPPORTED",
 EXPORTED_SYMBOLS = [
     "eas_encoder_create", "eas_encoder_weight_arena_bytes", "eas_encoder_workspace_bytes", "eas_encoder_out_rows",
     "eas_encode_microbatch", "eas_encode_microbatch_static", "eas_encoder_status", "eas_encoder_last_launch_count", "eas_encoder_set_attention_impl",
-    "eas_encoder_set_graph_mode", "eas_encoder_graph_stats", "eas_encoder_enable_timing", "eas_encoder_timing_read", "eas_last_error", "eas_encoder_destroy", "eas_kernel_gemm", "eas_kernel_gemm_tile", "eas_kernel_norm", "eas_kernel_attention",
+    "eas_encoder_set_graph_mode", "eas_encoder_graph_stats", "eas_encoder_enable_timing", "eas_encoder_timing_read", "eas_last_error", "eas_encoder_destroy", "eas_kernel_gemm", "eas_kernel_gemm_tile", "eas_kernel_gemm_starved", "eas_kernel_norm", "eas_kernel_attention",
     "eas_encoder_set_split_k", "eas_encoder_set_norm_fold", "eas_sm_partition_create", "eas_sm_partition_sm_count", "eas_sm_partition_stream", "eas_sm_partition_destroy",
     "eas_attention_plan", "eas_kernel_attention_plan", "eas_encoder_set_gemm_tile",
 ]
@@ -100,6 +100,8 @@ def load_library():
                                     C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_void_p, C.c_void_p]
     lib.eas_kernel_gemm_tile.restype = C.c_int
     lib.eas_kernel_gemm_tile.argtypes = lib.eas_kernel_gemm.argtypes + [C.c_int32]
+    lib.eas_kernel_gemm_starved.restype = C.c_int
+    lib.eas_kernel_gemm_starved.argtypes = lib.eas_kernel_gemm_tile.argtypes
     lib.eas_kernel_norm.restype = C.c_int
     lib.eas_kernel_norm.argtypes = [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int32, C.c_int32, C.c_int32,
                                     C.c_float, C.c_int32, C.c_int32, C.c_void_p]
@@ -335,9 +337,10 @@ class SmPartition:
 
 
 def kernel_gemm(A, W, bias, act=0, out_fp32=False, resid=None, sm_budget=0, stream=None, out=None, status=None,
-                tile_shape=0):
+                tile_shape=0, starved=False):
     """eas_kernel_gemm (eas_kernel_gemm_tile when tile_shape != 0) on device tensors.  Returns (out, device status
-    word).  `status` (device int32, zeroed by the caller) can be passed in so that a call allocates nothing."""
+    word).  `status` (device int32, zeroed by the caller) can be passed in so that a call allocates nothing.
+    `starved`: eas_kernel_gemm_starved, whose waits run out."""
     lib = load_library()
     M, K = A.shape
     N = W.shape[0]
@@ -348,7 +351,9 @@ def kernel_gemm(A, W, bias, act=0, out_fp32=False, resid=None, sm_budget=0, stre
     args = (A.data_ptr(), W.data_ptr(), bias.data_ptr(), out.data_ptr(),
             resid.data_ptr() if resid is not None else None, M, N, K, act, int(out_fp32), sm_budget,
             _stream_ptr(stream), status.data_ptr())
-    if tile_shape:
+    if starved:
+        _check(lib.eas_kernel_gemm_starved(*args, tile_shape))
+    elif tile_shape:
         _check(lib.eas_kernel_gemm_tile(*args, tile_shape))
     else:
         _check(lib.eas_kernel_gemm(*args))

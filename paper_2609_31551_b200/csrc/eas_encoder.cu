@@ -719,6 +719,7 @@ struct GemmCall {
   int w_const = 1;             // the weights are constant (set at create time): their loads may start before the stream's earlier work ends
   int force_tile = TILE_AUTO;  // others: tests; an error where the GEMM has no such kernel
   int prefer_tile = TILE_AUTO; // others: tests; only where it has one
+  bool starved = false;        // tests: every stage gets half its weight rows, so that the waits for it run out
   int splits = 1;              // split K (see GemmParams::splits); the partial sums of splits 1.. go to `part`
   float* part = nullptr;       // [(splits - 1) * part_rows, N] fp32
   int64_t part_rows = 0;
@@ -860,6 +861,7 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
   const int w_rows = std::min(tile_n, static_cast<int>(kBN)) / ctas;
   if (gemm_alt(tile_n) || w_rows < 64) EAS_TRY(deep ? make_w_tmap_deep(&p.tma_b, L.w, L.N, L.K, w_rows, depth) : make_w_tmap(&p.tma_b, L.w, L.N, L.K, w_rows));
   else p.tma_b = w_rows == 256 ? L.tmap : w_rows == 128 ? (deep ? L.tmap_half_deep : L.tmap_half) : (deep ? L.tmap_quarter_deep : L.tmap_quarter);
+  if (g.starved) EAS_TRY(deep ? make_w_tmap_deep(&p.tma_b, L.w, L.N, L.K, w_rows / 2, depth) : make_w_tmap(&p.tma_b, L.w, L.N, L.K, w_rows / 2));
   p.M = g.M; p.N = L.N;
   p.kb_per_tap = static_cast<int>(g.a_run / kBK);
   p.k_blocks = deep ? (p.kb_per_tap + depth - 1) / depth : p.kb_per_tap * g.taps;
@@ -1922,15 +1924,9 @@ static eas_status resolve_budget(int32_t sm_budget, int* budget) {
   return EAS_OK;
 }
 
-extern "C" eas_status eas_kernel_gemm(const void* A, const void* W, const void* bias, void* out, const float* resid,
-                                      int32_t M, int32_t N, int32_t K, int32_t act, int32_t out_fp32, int32_t sm_budget,
-                                      void* stream, uint32_t* status_dev) {
-  return eas_kernel_gemm_tile(A, W, bias, out, resid, M, N, K, act, out_fp32, sm_budget, stream, status_dev, 0);
-}
-
-extern "C" eas_status eas_kernel_gemm_tile(const void* A, const void* W, const void* bias, void* out, const float* resid,
-                                           int32_t M, int32_t N, int32_t K, int32_t act, int32_t out_fp32, int32_t sm_budget,
-                                           void* stream, uint32_t* status_dev, int32_t tile_shape) {
+static eas_status kernel_gemm(const void* A, const void* W, const void* bias, void* out, const float* resid, int32_t M, int32_t N, int32_t K,
+                              int32_t act, int32_t out_fp32, int32_t sm_budget, void* stream, uint32_t* status_dev, int32_t tile_shape,
+                              bool starved) {
   if (tile_shape < 0 || tile_shape >= TILE_COUNT) return fail(EAS_ERR_INVALID_ARG, "tile_shape %d outside 0..%d", tile_shape, TILE_COUNT - 1);
   if (A == nullptr || W == nullptr || bias == nullptr || out == nullptr || status_dev == nullptr)
     return fail(EAS_ERR_INVALID_ARG, "a required pointer is null");
@@ -1947,7 +1943,26 @@ extern "C" eas_status eas_kernel_gemm_tile(const void* A, const void* W, const v
   g.out = out; g.ldo = act == ACT_SWIGLU ? N / 2 : N; g.resid = out_fp32 ? resid : nullptr;
   g.w_const = 0;             // W is the caller's tensor: work earlier in the stream may have produced it
   g.force_tile = budget >= 2 ? tile_shape : 0;
+  g.starved = starved;
   return launch_gemm(g, budget, static_cast<cudaStream_t>(stream), status_dev);
+}
+
+extern "C" eas_status eas_kernel_gemm(const void* A, const void* W, const void* bias, void* out, const float* resid,
+                                      int32_t M, int32_t N, int32_t K, int32_t act, int32_t out_fp32, int32_t sm_budget,
+                                      void* stream, uint32_t* status_dev) {
+  return kernel_gemm(A, W, bias, out, resid, M, N, K, act, out_fp32, sm_budget, stream, status_dev, 0, false);
+}
+
+extern "C" eas_status eas_kernel_gemm_tile(const void* A, const void* W, const void* bias, void* out, const float* resid,
+                                           int32_t M, int32_t N, int32_t K, int32_t act, int32_t out_fp32, int32_t sm_budget,
+                                           void* stream, uint32_t* status_dev, int32_t tile_shape) {
+  return kernel_gemm(A, W, bias, out, resid, M, N, K, act, out_fp32, sm_budget, stream, status_dev, tile_shape, false);
+}
+
+extern "C" eas_status eas_kernel_gemm_starved(const void* A, const void* W, const void* bias, void* out, const float* resid,
+                                              int32_t M, int32_t N, int32_t K, int32_t act, int32_t out_fp32, int32_t sm_budget,
+                                              void* stream, uint32_t* status_dev, int32_t tile_shape) {
+  return kernel_gemm(A, W, bias, out, resid, M, N, K, act, out_fp32, sm_budget, stream, status_dev, tile_shape, true);
 }
 
 extern "C" eas_status eas_kernel_norm(const float* x, void* y, const void* gamma, const void* beta, int32_t rows, int32_t d,

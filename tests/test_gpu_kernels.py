@@ -184,6 +184,30 @@ def test_gemm_walks_every_tile_of_every_panel(left):
     assert not ((outs[0][0].double().cpu() - y).abs() > tol).any()
 
 
+@pytest.mark.parametrize("shape", [2, 1, 3, 5, 9, 13, 14, 17])
+def test_gemm_reports_waits_that_run_out(shape):
+    """A launch whose stages never fill up (its loads bring half of what they announce): every wait runs out after a second, the status
+    word says so, nothing is stored, and tensor memory is back: launches on all SMs that take all of it give the same bits as before."""
+    import paper_2609_31551_b200 as P
+    rng = np.random.Generator(np.random.PCG64(70 + shape))
+    M, N, K = 300, 512, 1024
+    A, W, b = _dev(_bf16_exact(rng, (M, K))), _dev(_bf16_exact(rng, (N, K), 0.05)), _dev(_bf16_exact(rng, (N,), 0.5))
+    big = _dev(_bf16_exact(rng, (128 * 148, K)))
+    before = [P.kernel_gemm(big, W, b, tile_shape=t)[0] for t in (1, 2, 3)]
+    mark = torch.full((M, N), 7.0, dtype=torch.bfloat16, device="cuda")
+    out = mark.clone()
+    torch.cuda.synchronize()
+    _, status = P.kernel_gemm(A, W, b, out=out, sm_budget=6, tile_shape=shape, starved=True)
+    torch.cuda.synchronize()
+    assert int(status[0]) == 1
+    assert torch.equal(out, mark)
+    for t, ref in zip((1, 2, 3), before):
+        got, status = P.kernel_gemm(big, W, b, tile_shape=t)
+        torch.cuda.synchronize()
+        assert int(status[0]) == 0
+        assert torch.equal(got, ref), t
+
+
 def test_gemm_wide_tile_is_refused_where_it_does_not_exist():
     import paper_2609_31551_b200 as P
     rng = np.random.Generator(np.random.PCG64(92))
