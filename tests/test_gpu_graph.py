@@ -180,3 +180,40 @@ def test_graph_replay_with_split_k_is_bit_identical():
     enc.encode_microbatch_static(data, shapes, offsets, cu, cu_dev, out)
     enc.status()
     assert torch.equal(out, ref)
+
+
+def test_passes_that_follow_one_another_directly_are_those_a_host_wait_apart():
+    """Two micro-batches of different sizes in turn through ONE workspace, replayed without a host wait between them.  The weight loads of a
+    GEMM do not wait for the launch before it, its activations do: what was read too early would be the other micro-batch's."""
+    import paper_2609_31551_b200 as P
+    cfg = S.get_config("c0")
+    enc = P.Encoder(cfg, P.weights_to_device(S.make_weights(cfg)))
+    calls, rows = [], 0
+    for seed, n in ((31, 3), (32, 2)):
+        shapes = [(1, 224, 224)] * n
+        items = S.make_items(cfg, shapes, seed=seed)
+        data, offsets = P.pack_items(items)
+        cu = G.cu_seqlens_of(cfg, items)
+        calls.append((data, shapes, offsets, cu, torch.from_numpy(cu).cuda()))
+        rows = max(rows, enc.workspace_bytes(int(cu[-1]), n))
+    ws = torch.empty(rows + 1024, dtype=torch.uint8, device="cuda")
+    refs = []
+    for data, shapes, offsets, cu, cu_dev in calls:
+        refs.append(enc.encode_microbatch(data, shapes, offsets, cu, cu_seqlens_dev=cu_dev, workspace=ws))
+        enc.status()
+    side = torch.cuda.Stream()
+    for graph in (False, True):
+        enc.set_graph_mode(graph)
+        outs = [torch.full_like(r, float("nan")) for r in refs]
+        kept = []
+        torch.cuda.synchronize()
+        with torch.cuda.stream(side):
+            for i in range(24):
+                data, shapes, offsets, cu, cu_dev = calls[i % 2]
+                enc.encode_microbatch(data, shapes, offsets, cu, cu_seqlens_dev=cu_dev, workspace=ws, out=outs[i % 2], stream=side)
+                if i % 6 == 5:
+                    kept += [o.clone() for o in outs]
+        enc.status(side)
+        for i, o in enumerate(kept):
+            assert torch.equal(o, refs[i % 2]), (graph, i)
+    enc.set_graph_mode(False)

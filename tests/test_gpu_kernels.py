@@ -184,6 +184,47 @@ def test_gemm_walks_every_tile_of_every_panel(left):
     assert not ((outs[0][0].double().cpu() - y).abs() > tol).any()
 
 
+@pytest.mark.parametrize("budget", [0, 74, 6])
+def test_gemm_launches_that_follow_one_another_directly(budget):
+    """A chain in which each launch reads what the one before wrote, captured so that nothing stands between two launches: a CTA's shared
+    and tensor memory pass to the next launch's while others of its own launch still work.  Tile shapes alternate between single CTAs,
+    pairs, wide and half-height ones; outputs are NaN before each replay and have to be the bits of launches a host wait apart."""
+    import paper_2609_31551_b200 as P
+    rng = np.random.Generator(np.random.PCG64(60 + budget))
+    M, N, K = 128 * 9 + 5, 512, 512
+    shapes = (2, 1, 3, 14, 5, 17, 3, 8, 13, 2, 16, 4, 15, 6, 3, 1, 13, 9)
+    A, b = _dev(_bf16_exact(rng, (M, K))), _dev(_bf16_exact(rng, (N,), 0.5))
+    W = [_dev(_bf16_exact(rng, (N, K), 0.04)) for _ in range(3)]
+    refs, x = [], A
+    for i, shape in enumerate(shapes):
+        x, status = P.kernel_gemm(x, W[i % 3], b, sm_budget=budget, tile_shape=shape)
+        torch.cuda.synchronize()
+        assert int(status[0]) == 0
+        refs.append(x)
+    assert torch.isfinite(refs[-1].float()).all()
+    outs = [torch.empty_like(r) for r in refs]
+    status = torch.zeros(4, dtype=torch.int32, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def chain():
+        for i, shape in enumerate(shapes):
+            P.kernel_gemm(A if i == 0 else outs[i - 1], W[i % 3], b, sm_budget=budget, tile_shape=shape, out=outs[i], status=status, stream=side)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        chain()
+    for go in [chain] + [graph.replay] * 8:
+        with torch.cuda.stream(side):
+            for o in outs:
+                o.fill_(float("nan"))
+            go()
+        torch.cuda.synchronize()
+        assert int(status[0]) == 0
+        for i, (o, r) in enumerate(zip(outs, refs)):
+            assert torch.equal(o, r), (i, shapes[i])
+
+
 @pytest.mark.parametrize("shape", [2, 1, 3, 5, 9, 13, 14, 17])
 def test_gemm_reports_waits_that_run_out(shape):
     """A launch whose stages never fill up (its loads bring half of what they announce): every wait runs out after a second, the status
