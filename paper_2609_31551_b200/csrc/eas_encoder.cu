@@ -1178,14 +1178,21 @@ static AttnPlan attention_plan(const int32_t* cu, int n_items, int H, int budget
 }
 
 // Weights of the GEMMs to come, brought towards L2 by an attention launch (AttnRrParams::warm), whose own work leaves HBM idle: a
-// GEMM of one wave otherwise waits for its first weights (1.1 us from HBM instead of 0.7).  Up to kWarmTokens, where the GEMMs are
-// such launches, and kWarmBytes a block, what one attention launch of 8 us brings in without holding up its neighbours.  Whole calls,
-// us: one 336 x 336 image (24 MB a block, all four) 1184 -> 1167, 30 s of audio (39 MB) 3092 -> 3055 with 13 to 16 MB, 3067 with 29 and
-// 3071 with all, one 252 x 364 image (52 MB) 1814 -> 1781 with 26 MB, 1828 with 42 and 1847 with all; 2308 tokens +-0.  Below
-// kWarmFewTokens the whole block is bound by its weights' way from HBM and what is asked for delays what comes first: only the block's
+// GEMM of one wave otherwise waits for its first weights (1.1 us from HBM instead of 0.7).  By tokens, up to kWarmTokens: beyond, launches
+// of several waves hide their first loads and nothing is gained (2308 tokens +-0).  In the order MLP-up, MLP-down, next qkv, out-projection, each that still fits into
+// kWarmBytes: all four of d 1024 (25 MB), both of the MLP of audio (26), MLP-up alone where it is gated (26; there the out-projection
+// misses the limit by 0.1 MB).  Whole calls on all SMs without and with it, us: 256 tokens of d 1024 968 and 945, 577 1170 and 1152, 1154
+// 1501 and 1488, 1731 1738 and 1730; d 1280, gated: 256 1505 and 1490, 468 1812 and 1778, 1024 2525 and 2506; audio: 500 1646 and 1631, 1500
+// 2882 and 2857 (with 13 to 16 MB 0.4 % less than with 26 when it was built; all 39 MB as much as 29).  All 52 MB of a gated block held up the
+// neighbours: 468 tokens 1814 without, 1847.
+// Below kWarmFewTokens the whole block is bound by its weights' way from HBM and what is asked for delays what comes first: only the block's
 // last weights.  64 tokens of d 1024: none 833, the last 813, all 903; of d 1280, gated: 1370, 1338, MLP-up (26 MB) 1479; 50 of audio:
 // 1284, 1256, both of the MLP 1334; with 200 and 256 tokens both or all are the better ones (1310, 1282, 1273; 970, 956, 946).
-constexpr int64_t kWarmTokens = 2048, kWarmFewTokens = 160;
+// On a share of the SMs up to kWarmShareTokens.  Alone, 577 tokens gain 3 to 4 % there (74 SMs 1556 -> 1490), 1024 to 1936 of either d 0 to 1.4 %
+// (d 1280 costs 0.5 to 1.1 % at 64 tokens and, on 37 SMs, 468).  Beside a worker on the other SMs the reads come out of its bandwidth too:
+// 577 tokens on 74 and 110 SMs 1.96 -> 1.98 and 1.48 -> 1.44 ms, the worker 890 -> 871 and 534 -> 521 TFLOP/s; 1154 tokens 2.78 -> 2.80 and
+// 1.97 -> 2.00 ms, 812 -> 801 and 494 -> 480; 1731 3.59 -> 3.60 and 2.45 -> 2.44 ms, 837 -> 822 and 494 -> 485.
+constexpr int64_t kWarmTokens = 2048, kWarmShareTokens = 1024, kWarmFewTokens = 160;
 constexpr uint64_t kWarmBytes = 28u << 20;
 struct WarmList {
   const bf16* w[4] = {};
@@ -1553,7 +1560,7 @@ static eas_status encode_impl(eas_encoder* e, const eas_packed_inputs* in, void*
     WarmList warm;
     if (T < kWarmFewTokens) {
       warm.add(L.fc2);
-    } else if (T <= kWarmTokens) {
+    } else if (T <= (budget < g_device_sms ? kWarmShareTokens : kWarmTokens)) {
       warm.add(L.fc1);
       warm.add(L.fc2);
       if (li + 1 < c.n_layers) warm.add(e->layers[li + 1].qkv);
