@@ -743,9 +743,12 @@ struct GemmCall {
 // where a last wave that fills a fraction f of the slots counts `partial` + (1 - partial) * f (fewer SMs share the path to L2).
 // Fitted to 1600 measurements on B200: every shape forced over the encoder's GEMMs, 100 <= M <= 18464 tokens, d 256, 1024 and
 // 1280, on 37, 74, 111 and 148 SMs, then adjusted for the choice alone, where runs of 0.25 s back to back at the power cap
-// (large M) count too.  The choice is on average 0.15 % and at most 6 % slower than the best shape (0.3 % on shapes left out
-// of the fit).  What the widths are for: a launch takes whole waves of tiles, so the width that just fills the SMs wins, and
-// a pair pulls half the weight bytes per SM that two single tiles pull, at 100 to 145 GB/s per SM the bound of every tile below
+// (large M) count too.  Those are the times of kernels with a longer set-up and ring step (a launch of one wave now takes 0.1 to 2.2 us less
+// than its row says), so the choice is no longer that close: over 480 GEMMs a share (d 256, 1024, 1280, 65 to 4616 rows, weights in L2 and from
+// memory) it is 2.4, 1.9, 1.6 and 1.5 % slower than the best shape on 37, 74, 111 and 148 SMs on average and up to 20 % on 111 and 148
+// (d 1280 MLP-up at 577 rows: 12.7 us as 128x224, 10.6 as two waves of half-height 128x128; 27 % on 37).  What the widths are for: a launch takes whole
+// waves of tiles, so the width that just fills the SMs wins, and a pair pulls half the weight bytes per SM that two single tiles pull, at 100
+// to 145 GB/s per SM the bound of every tile below
 // 192 columns.  (N, K) on 148 SMs, the best of 128x64, 128x128, 128x256, 256x256, 256x512 -> now:
 //   M = 577:  (1024, 4096) 17.5 us -> 14.0 as 256x96;  (4096, 1024) 12.3 -> 9.9 as 128x160
 //   M = 1500: (1280, 5120) 25.4 -> 20.1 as 256x128;    (3840, 1280) 17.5 -> 14.4 as 256x160
@@ -754,25 +757,27 @@ struct GemmCall {
 //
 // Half-height tiles pull 64 rows of A and half the weight rows per SM and k-block, less than any other shape of their width: 112 rows
 // as 128x96 against 176 as 256x96 and 192 as 128x64.  They are for launches of one wave (with more, the wider tiles' fewer operand bytes
-// per output win), fitted to 230 shapes of up to 2048 rows on 148 and 74 SMs with the weights in L2, where the attention launch puts
-// them.  On a share of the SMs a pair is set up behind the predecessor (kShareUs more); with fewer than eight k-blocks only the two
-// narrowest pay, and while half the SMs suffice (M = 784, N = 1024, K = 256: 3.9 us as 128x64, 4.8 as half-height 128x224).  Over those
-// shapes the choice is 0.5 % behind the best tile on average; with the figures of the kernels before their set-up and loops were shortened it
-// was 1.5 %, and up to 19 % on 74 SMs (M = 196, N = K = 256: 4.3 us as 128x64, 3.6 as half-height 128x64; M = 108, (3840, 1280): 6.6 and 5.6 as
+// per output win).  Their slopes are near least squares over 1152 present launches on the four shares; their bases stand 0.6 us above that, on the
+// scale of the rows above, chosen on half of those launches for the choice.  (With bases of present kernels beside older rows they won too often:
+// 18 of 288 launches on all SMs were up to 6 % slower than as chosen before and none faster, on shares 16 of 864 up to 12 % slower and 160
+// faster.  Now none is more than 1.5 % slower, also in the other half, and 173 of the 1152 are faster.  M = 1500, (1024, 1024): 6.7 us as
+// half-height 128x224, 6.4 as 256x96; whole calls, 1443 tokens of d 1024 1607 -> 1582 us, 1154 on 111 SMs 1697 -> 1666, 257 945 -> 934.)  On a share of the SMs a pair is set
+// up behind the predecessor (kShareUs more); with fewer than eight k-blocks they pay while half the SMs suffice and up to 128 columns
+// (M = 784, N = 1024, K = 256: 3.9 us as 128x64, 4.8 as half-height 128x224; M = 577, (768, 256): 3.3 as 128x64, 3.1 as half-height
 // 128x128).  (N, K) on 148 SMs, best other shape -> half-height:
 //   M = 577:  (1024, 4096) 14.5 us as 128x256 ... 14.9 as 256x96 -> 10.7 as 128x96 (8.8 now);  (1024, 1024) 6.4 -> 6.1 (4.8)
 //   M = 468:  (1280, 5120) 17.8 -> 12.5 (10.0);  (1280, 1280) 7.1 -> 6.5 (5.1);  (3840, 1280) 8.5 -> 8.2 as 128x224 (6.5)
 //   M = 196:  (256, 1024) 5.8 -> 4.5 as 128x64 (3.5)
 template <typename Usable>
 static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bool plain, Usable usable, double* us = nullptr) {
-  constexpr double kShareUs = 0.63;
+  constexpr double kShareUs = 0.20;
   struct Cost { int tile; double base, per_kb, per_wave, partial; };    // us
   static const Cost costs[] = {{TILE_SINGLE, 5.24, 0.351, 0.52, 0.87}, {TILE_PAIR, 6.44, 0.323, 0.25, 0.92}, {TILE_WIDE, 4.81, 0.586, 5.1, 0.89},
                                {TILE_N128, 3.91, 0.228, 0.45, 0.95}, {TILE_N64, 3.48, 0.173, 0.20, 1.0}, {TILE_N160, 4.61, 0.265, 0.31, 0.92},
                                {TILE_N224, 5.02, 0.329, 0.29, 0.88}, {TILE_P96, 4.66, 0.163, 0.13, 0.79}, {TILE_P128, 5.07, 0.181, 0.28, 0.84},
                                {TILE_P160, 5.20, 0.212, 0.48, 0.80}, {TILE_P192, 5.52, 0.250, 0.34, 0.85}, {TILE_P224, 5.98, 0.291, 0.20, 0.84},
-                               {TILE_H64, 1.29, 0.088, 1.16, 0.80}, {TILE_H96, 1.29, 0.100, 1.36, 0.70}, {TILE_H128, 1.46, 0.108, 2.24, 0.60},
-                               {TILE_H160, 1.32, 0.113, 2.39, 0.83}, {TILE_H224, 1.59, 0.143, 2.73, 0.70}};
+                               {TILE_H64, 2.29, 0.076, 1.41, 0.75}, {TILE_H96, 1.55, 0.094, 2.29, 0.90}, {TILE_H128, 3.23, 0.106, 0.61, 0.75},
+                               {TILE_H160, 2.17, 0.100, 2.78, 0.85}, {TILE_H224, 2.21, 0.158, 3.04, 0.93}};
   int tile = TILE_SINGLE;
   double best = 0.0;
   for (const Cost& c : costs) {
