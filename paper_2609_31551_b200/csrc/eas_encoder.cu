@@ -90,16 +90,16 @@ static eas_status make_a_tmap(CUtensorMap* m, const void* a, int64_t run, int64_
   return make_tmap(m, a, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-// "Deep" maps: the same matrices seen as {64 columns, rows, K/64 blocks}, so that ONE box {64, rows, 2} brings two
-// 64-wide k-blocks, each landing as its own swizzle-atom block [rows x 128 bytes] (see GemmCfg).  A k-block index
+// "Deep" maps: the same matrices seen as {64 columns, rows, K/64 blocks}, so that ONE box {64, rows, depth} brings two or four
+// 64-wide k-blocks, each landing as its own swizzle-atom block [rows x 128 bytes] (see GemmCfg and TileShape).  A k-block index
 // past K/64 is filled with zeros.
-static eas_status make_w_tmap_deep(CUtensorMap* m, const void* w, int64_t N, int64_t K, uint32_t box_rows, uint32_t depth = 2) {
+static eas_status make_w_tmap_deep(CUtensorMap* m, const void* w, int64_t N, int64_t K, uint32_t box_rows, uint32_t depth) {
   const uint64_t dims[3] = {kBK, static_cast<uint64_t>(N), static_cast<uint64_t>(K / kBK)};
   const uint64_t strides[2] = {static_cast<uint64_t>(K) * 2, kBK * 2};
   const uint32_t box[3] = {kBK, box_rows, depth};
   return make_tmap(m, w, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
-static eas_status make_a_tmap_deep(CUtensorMap* m, const void* a, int64_t run, int64_t row_elems, int64_t rows, uint32_t box_rows, uint32_t depth = 2) {
+static eas_status make_a_tmap_deep(CUtensorMap* m, const void* a, int64_t run, int64_t row_elems, int64_t rows, uint32_t box_rows, uint32_t depth) {
   const uint64_t dims[3] = {kBK, static_cast<uint64_t>(rows), static_cast<uint64_t>(run / kBK)};
   const uint64_t strides[2] = {static_cast<uint64_t>(row_elems) * 2, kBK * 2};
   const uint32_t box[3] = {kBK, box_rows, depth};
@@ -318,8 +318,8 @@ static eas_status finish_linear(Linear& L) {
   EAS_TRY(make_w_tmap(&L.tmap, L.w, L.N, L.K, kBN));
   EAS_TRY(make_w_tmap(&L.tmap_half, L.w, L.N, L.K, kBN / 2));
   EAS_TRY(make_w_tmap(&L.tmap_quarter, L.w, L.N, L.K, kBN / 4));
-  EAS_TRY(make_w_tmap_deep(&L.tmap_quarter_deep, L.w, L.N, L.K, kBN / 4));
-  return make_w_tmap_deep(&L.tmap_half_deep, L.w, L.N, L.K, kBN / 2);
+  EAS_TRY(make_w_tmap_deep(&L.tmap_quarter_deep, L.w, L.N, L.K, kBN / 4, 2));
+  return make_w_tmap_deep(&L.tmap_half_deep, L.w, L.N, L.K, kBN / 2, 2);
 }
 
 typedef void (*GemmKernel)(GemmParams);
@@ -329,12 +329,17 @@ typedef void (*GemmKernel)(GemmParams);
 enum { TILE_AUTO = 0, TILE_SINGLE = 1, TILE_PAIR = 2, TILE_WIDE = 3, TILE_N128 = 4, TILE_N64 = 5, TILE_N160 = 6, TILE_N224 = 7,
        TILE_P96 = 8, TILE_P128 = 9, TILE_P160 = 10, TILE_P192 = 11, TILE_P224 = 12,
        TILE_H64 = 13, TILE_H96 = 14, TILE_H128 = 15, TILE_H160 = 16, TILE_H224 = 17, TILE_COUNT = 18 };
-struct TileShape { int ctas, rows, cols; bool half = false; };
-static const TileShape kTiles[TILE_COUNT] = {{0, 0, 0}, {1, 128, 256}, {2, 256, 256}, {2, 256, 512}, {1, 128, 128}, {1, 128, 64}, {1, 128, 160},
-                                             {1, 128, 224}, {2, 256, 96}, {2, 256, 128}, {2, 256, 160}, {2, 256, 192}, {2, 256, 224},
-                                             {2, 128, 64, true}, {2, 128, 96, true}, {2, 128, 128, true}, {2, 128, 160, true}, {2, 128, 224, true}};
-// deep (up to 128 columns): two 64-wide k-blocks per stage and TMA operation (convolutions walk their taps as 64-wide
-// k-blocks and use the shallow kernels).  nullptr: no such kernel.
+// depth: 64-wide k-blocks of a stage and TMA operation of a plain GEMM (more than one: the "deep" kernels; convolutions walk their taps as
+// 64-wide k-blocks and use the shallow ones).  Kernels, tensor maps and k-steps all take it from here.
+struct TileShape { int ctas, rows, cols, depth = 1; bool half = false; };
+static constexpr TileShape kTiles[TILE_COUNT] = {{0, 0, 0}, {1, 128, 256}, {2, 256, 256}, {2, 256, 512}, {1, 128, 128, 2}, {1, 128, 64, 2}, {1, 128, 160},
+                                                 {1, 128, 224}, {2, 256, 96, 2}, {2, 256, 128, 2}, {2, 256, 160}, {2, 256, 192}, {2, 256, 224},
+                                                 {2, 128, 64, 4, true}, {2, 128, 96, 2, true}, {2, 128, 128, 2, true}, {2, 128, 160, 2, true}, {2, 128, 224, 2, true}};
+template <int ACT, int OUT, int TILE, bool SPLIT = false>
+static constexpr GemmKernel deep_kernel() {
+  return gemm_kernel<ACT, OUT, kTiles[TILE].ctas, kTiles[TILE].cols, kTiles[TILE].depth, SPLIT, kTiles[TILE].half>;
+}
+// nullptr: no such kernel
 template <int ACT, int OUT, bool SPLIT = false>
 static GemmKernel gemm_kernel_of(int tile, bool deep) {
   if (tile == TILE_SINGLE) return gemm_kernel<ACT, OUT, 1, 256, 1, SPLIT>;
@@ -342,12 +347,12 @@ static GemmKernel gemm_kernel_of(int tile, bool deep) {
   if constexpr (ACT != ACT_SWIGLU && !(ACT == ACT_GELU && OUT == OUT_F32))
     if (tile == TILE_WIDE) return gemm_kernel<ACT, OUT, 2, 512, 1, SPLIT>;
   if constexpr (OUT != OUT_F32_FOLD) {
-    if (tile == TILE_N128) return deep ? gemm_kernel<ACT, OUT, 1, 128, 2, SPLIT> : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 1, 128, 1>);
-    if (tile == TILE_P128) return deep ? gemm_kernel<ACT, OUT, 2, 128, 2, SPLIT> : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 2, 128, 1>);
+    if (tile == TILE_N128) return deep ? deep_kernel<ACT, OUT, TILE_N128, SPLIT>() : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 1, 128, 1>);
+    if (tile == TILE_P128) return deep ? deep_kernel<ACT, OUT, TILE_P128, SPLIT>() : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 2, 128, 1>);
     if constexpr (ACT != ACT_SWIGLU)
-      if (tile == TILE_N64) return deep ? gemm_kernel<ACT, OUT, 1, 64, 2, SPLIT> : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 1, 64, 1>);
+      if (tile == TILE_N64) return deep ? deep_kernel<ACT, OUT, TILE_N64, SPLIT>() : (SPLIT ? nullptr : gemm_kernel<ACT, OUT, 1, 64, 1>);
     if constexpr (ACT != ACT_SWIGLU) {
-      if (tile == TILE_P96) return deep ? gemm_kernel<ACT, OUT, 2, 96, 2, SPLIT> : nullptr;
+      if (tile == TILE_P96) return deep ? deep_kernel<ACT, OUT, TILE_P96, SPLIT>() : nullptr;
       if (tile == TILE_N160) return gemm_kernel<ACT, OUT, 1, 160, 1, SPLIT>;
       if (tile == TILE_N224) return gemm_kernel<ACT, OUT, 1, 224, 1, SPLIT>;
       if (tile == TILE_P160) return gemm_kernel<ACT, OUT, 2, 160, 1, SPLIT>;
@@ -356,11 +361,11 @@ static GemmKernel gemm_kernel_of(int tile, bool deep) {
     }
     if constexpr (ACT != ACT_SWIGLU && !SPLIT && !(ACT == ACT_GELU && OUT == OUT_F32)) {
       if (kTiles[tile].half && !deep) return nullptr;
-      if (tile == TILE_H64) return gemm_kernel<ACT, OUT, 2, 64, 4, false, true>;
-      if (tile == TILE_H96) return gemm_kernel<ACT, OUT, 2, 96, 2, false, true>;
-      if (tile == TILE_H128) return gemm_kernel<ACT, OUT, 2, 128, 2, false, true>;
-      if (tile == TILE_H160) return gemm_kernel<ACT, OUT, 2, 160, 2, false, true>;
-      if (tile == TILE_H224) return gemm_kernel<ACT, OUT, 2, 224, 2, false, true>;
+      if (tile == TILE_H64) return deep_kernel<ACT, OUT, TILE_H64>();
+      if (tile == TILE_H96) return deep_kernel<ACT, OUT, TILE_H96>();
+      if (tile == TILE_H128) return deep_kernel<ACT, OUT, TILE_H128>();
+      if (tile == TILE_H160) return deep_kernel<ACT, OUT, TILE_H160>();
+      if (tile == TILE_H224) return deep_kernel<ACT, OUT, TILE_H224>();
     }
   }
   return nullptr;
@@ -813,7 +818,7 @@ static int pick_splits(int64_t M, int64_t N, int64_t K, int sm_count) {
     if (items * s > sm_count || K % (s * 2 * kBK) != 0 || K / s < 1024) continue;
     double us = 0.0;
     pick_tile(M, N, static_cast<double>(K / kBK) / s, s, sm_count, true,
-              [&](int t) { return !kTiles[t].half && (t != TILE_WIDE || N % 512 == 0) && gemm_kernel_for(ACT_NONE, 1, t, kTiles[t].cols <= 128, true) != nullptr; }, &us);
+              [&](int t) { return !kTiles[t].half && (t != TILE_WIDE || N % 512 == 0) && gemm_kernel_for(ACT_NONE, 1, t, kTiles[t].depth > 1, true) != nullptr; }, &us);
     us += kPartUs * s;
     if (best == 0.0 || us < best) { best = us; splits = s; }
   }
@@ -832,7 +837,7 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
     return fail(EAS_ERR_UNSUPPORTED, "a folded normalisation needs a plain GEMM with row-aligned output and K %% %d == 0", kFoldGroup);
   const int out_mode = fold_out ? 2 : (g.out_fp32 ? 1 : 0);
   const bool plain = g.conv_stride == 1 && g.taps == 1;
-  auto is_deep = [&](int t) { return plain && (kTiles[t].cols <= 128 || kTiles[t].half); };
+  auto is_deep = [&](int t) { return plain && kTiles[t].depth > 1; };
   auto kernel_of = [&](int t) -> GemmKernel {       // nullptr: this GEMM has no kernel of that shape
     // wide tiles: the output splits evenly into 512-column blocks; they and the odd widths: TMA-stored epilogue only
     if (t == TILE_WIDE && (!tma_out || L.N % 512 != 0)) return nullptr;
@@ -858,13 +863,13 @@ static eas_status launch_gemm(const GemmCall& g, int budget, cudaStream_t stream
   }
   const int ctas = kTiles[tile].ctas, tile_n = kTiles[tile].cols;
   const bool deep = is_deep(tile);
-  const int depth = tile == TILE_H64 ? 4 : deep ? 2 : 1;      // 64-wide k-blocks of a stage
+  const int depth = deep ? kTiles[tile].depth : 1;
   GemmParams p{};
   if (deep) EAS_TRY(make_a_tmap_deep(&p.tma_a, g.A, g.a_run, g.a_row_elems, g.a_rows, kTiles[tile].half ? kBM / 2 : kBM, depth));
   else EAS_TRY(make_a_tmap(&p.tma_a, g.A, g.a_run, g.a_row_elems, g.conv_stride, g.a_rows));
   // weight rows per TMA box: the CTA's share of a 256-column accumulator, or the narrow tile's columns
   const int w_rows = std::min(tile_n, static_cast<int>(kBN)) / ctas;
-  if (gemm_alt(tile_n) || w_rows < 64) EAS_TRY(deep ? make_w_tmap_deep(&p.tma_b, L.w, L.N, L.K, w_rows, depth) : make_w_tmap(&p.tma_b, L.w, L.N, L.K, w_rows));
+  if (gemm_alt(tile_n) || w_rows < 64 || depth > 2) EAS_TRY(deep ? make_w_tmap_deep(&p.tma_b, L.w, L.N, L.K, w_rows, depth) : make_w_tmap(&p.tma_b, L.w, L.N, L.K, w_rows));
   else p.tma_b = w_rows == 256 ? L.tmap : w_rows == 128 ? (deep ? L.tmap_half_deep : L.tmap_half) : (deep ? L.tmap_quarter_deep : L.tmap_quarter);
   if (g.starved) EAS_TRY(deep ? make_w_tmap_deep(&p.tma_b, L.w, L.N, L.K, w_rows / 2, depth) : make_w_tmap(&p.tma_b, L.w, L.N, L.K, w_rows / 2));
   p.M = g.M; p.N = L.N;

@@ -31,11 +31,12 @@ constexpr int kTmemWarp = 2;                             // the first epilogue w
 // TN = 512 ("wide", CTA pairs only): the pair owns a 256x512 tile, i.e. two 256-column accumulators fed by the same
 // A tile (three TMA operations for twice the columns) at the price of a single accumulator set: the epilogue no longer
 // overlaps the next main loop, so it pays for large K only.
-// KD = 2 ("deep", TN <= 128): a stage holds TWO 64-wide k-blocks of each operand, fetched by ONE TMA operation per operand
-// (a 3-D box {64 columns, rows, 2 k-blocks}, which lands as two consecutive swizzle-atom blocks): a step of a ring costs
-// some 0.16 us whatever its bytes, which is what bounds small tiles (deep against shallow: 128x64 -12 %, 256x96 -6 to -14 %,
-// 256x128 -7 % at K = 1024, 128x128 -5 %).  Wider tiles are no faster with it.  KD = 4, half-height 128x64 tiles: four (M = 300, N = 1024,
-// K = 4096: 7.9 -> 7.1 us, M = 196, N = 256, K = 1024: 3.7 -> 3.5); 128x96 would have a ring of three stages, 8.75 -> 9.2 us.
+// KD = 2 ("deep": tiles of up to 128 columns and all half-height ones): a stage holds TWO 64-wide k-blocks of each operand, fetched by ONE TMA
+// operation per operand (a 3-D box {64 columns, rows, 2 k-blocks}, which lands as two consecutive swizzle-atom blocks): a step of a ring costs
+// its issuer time whatever its bytes, which is what bounds small tiles (deep against shallow, when a step cost some 0.16 us: 128x64 -12 %,
+// 256x96 -6 to -14 %, 256x128 -7 % at K = 1024, 128x128 -5 %; since then barriers are tested a step ahead, see the issuer).  Wider tiles were no faster
+// with it.  KD = 4, half-height 128x64 tiles: four (M = 300, N = 1024, K = 4096: 7.9 -> 7.1 us, M = 196, N = 256, K = 1024: 3.7 -> 3.5); 128x96 would
+// have a ring of three stages, 8.75 -> 9.2 us.
 // TN < 256: with few tokens a launch has fewer 256-column tiles than the device has SMs and the K loop of ONE tile is the
 // kernel's time, at the rate one SM pulls operands from L2 (48 KB per 64-wide k-block of a 128x256 tile, 24 KB of a 128x64
 // or 256x128 one): more, narrower tiles shorten that loop and use the idle SMs, and the width that just fills one wave is best.
@@ -72,15 +73,15 @@ enum { OUT_BF16 = 0, OUT_F32 = 1, OUT_F32_FOLD = 2 };
 constexpr int kFoldGroup = 128;                   // columns per statistics group
 
 struct alignas(64) GemmParams {
-  CUtensorMap tma_a;      // 3-D: {K-run, phase, rows}; box {64, 1, 128}.  Deep kernels: {64, rows, K/64}; box {64, 128 or 64, 2}
-  CUtensorMap tma_b;      // 2-D: {K, N}; box {64, weight rows of a CTA: at most 256}.  Deep: {64, N, K/64}; box {64, rows, 2}
+  CUtensorMap tma_a;      // 3-D: {K-run, phase, rows}; box {64, 1, 128}.  Deep kernels: {64, rows, K/64}; box {64, 128 or 64, KD}
+  CUtensorMap tma_b;      // 2-D: {K, N}; box {64, weight rows of a CTA: at most 256}.  Deep: {64, N, K/64}; box {64, rows, KD}
   CUtensorMap tma_out16;  // half-height tiles whose lane half ends in 16 columns: 2-D over out, box {16 columns, 32 rows}, no swizzle
                           // (sharing tma_part's place, which only split launches use, made calls of one image 0.2 to 0.5 % slower)
   CUtensorMap tma_out;    // 2-D over out (valid if use_tma_out): box {64 bf16 | 32 fp32, 32 rows}, 128-byte swizzle; {32 bf16, 32 rows},
                           // 64-byte swizzle, where gemm_out_row says 32
   int use_tma_out;        // 1: epilogue stages 32-row sub-tiles in shared memory and stores them with TMA
   int M, N;               // rows of A walked by tiles; rows of W
-  int k_blocks;           // k-steps: K / 64, or ceil(K / 128) for the deep kernels (TMA fills past K with zeros)
+  int k_blocks;           // k-steps: ceil(K / (64 KD)) (TMA fills past K with zeros)
   int kb_per_tap;         // k-blocks per convolution tap (== k_blocks for a plain GEMM)
   int conv_stride;        // 1 for a plain GEMM; row stride of a convolution otherwise
   int m_blocks, n_blocks; // m_blocks counts blocks of 128 rows (one CTA, or a half-height pair) or 256 (CTA pair)
