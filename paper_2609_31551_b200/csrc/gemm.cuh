@@ -135,7 +135,8 @@ struct alignas(64) GemmParams {
 // phase timestamps of epilogue warp 0 of CTA 0 (profiling builds only): [tile][k]
 __device__ unsigned long long g_gemm_dbg[32 * 16];
 #define GEMM_STAMP(k) do { if (blockIdx.x == 0 && ew == 0 && lane == 0 && tcount < 32) g_gemm_dbg[tcount * 16 + (k)] = clock64(); } while (0)
-// one-off timeline of CTA 0 in nanoseconds (row 31 of the same array)
+// one-off timeline of CTA 0 in nanoseconds (row 31 of the same array): 0 start, 1 tensor memory allocated and the set-up barrier passed, 2 past
+// the grid dependency, 3 first stage there, 4 first accumulator complete, 5 handed back, 6 last stores read, 7 the warp's end (1, 2, 4-7: warp 2)
 __device__ __forceinline__ unsigned long long gemm_globaltimer() { unsigned long long t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t; }
 #define GEMM_TL(k) do { if (blockIdx.x == 0) g_gemm_dbg[31 * 16 + (k)] = gemm_globaltimer(); } while (0)
 #else
@@ -276,8 +277,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) gemm_kernel(const __grid_cons
   // Each role passes the waits in its own code, so that the instructions behind them are fetched meanwhile.
   auto enter = [&](bool dependent) {
     if (CTAS == 2) cluster_wait();
+    if (threadIdx.x == 64) GEMM_TL(1);
     if (early_launch) pdl_launch_dependents();   // the next kernel may set itself up while this one runs
     if (dependent) pdl_wait();                   // everything before this kernel in the stream is complete and visible
+    if (threadIdx.x == 64) GEMM_TL(2);
   };
 
   if (warp == 0 || warp == kProducerBWarp) {
