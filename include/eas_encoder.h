@@ -191,8 +191,8 @@ eas_status eas_encoder_set_attention_impl(eas_encoder* enc, int32_t impl);
  * of sm_budget, but no longer of what else is in the micro-batch: an item encoded alone (split) and the same item in a
  * large micro-batch (not split) differ in the last bits, which is why the mode is off unless asked for (off: every
  * item's embeddings are bit-identical whatever it is packed with).  eas_encoder_workspace_bytes follows the mode (the
- * partial sums need scratch): set it before sizing the workspace.  With graph replay 128 tokens of the ViT-L/14-style
- * encoder take 849 us unsplit and 833 split, 256 tokens 978 and 987, 577 tokens 1175 and 1182, 1154 tokens 1494 and 1515: half-height
+ * partial sums need scratch): set it before sizing the workspace.  With graph replay 122 tokens of the ViT-L/14-style
+ * encoder take 774 us unsplit and 792 split, 256 tokens 833 and 849, 577 tokens 1103 and 1108, 1154 tokens 1442 and 1452: half-height
  * tiles, which split launches do not have, have overtaken the split. */
 eas_status eas_encoder_set_split_k(eas_encoder* enc, int32_t on);
 

@@ -808,7 +808,9 @@ static int pick_tile(int64_t M, int64_t N, double kb, int splits, int budget, bo
 // depend on the tile shape either.  4 or 2 by estimated time on all SMs, where every further split costs partial sums that the GEMM
 // writes and the normalisation reads (kPartUs; measured 0.4 to 3 us).  A forward pass replayed as a graph, split by 4 and by 2, and whole:
 // one 336 x 336 image 1193, 1181 and 1171 us, 128 tokens 831, 858 and 848, 400 of d 1024 1080, 1070 and 1068; 64 of d 1280 1270,
-// 1356 and 1285, 256 1466, 1520 and 1480, 500 of audio 1681, 1672 and 1644.
+// 1356 and 1285, 256 1466, 1520 and 1480, 500 of audio 1681, 1672 and 1644.  (Since the unsplit kernels' set-up and ring steps were shortened
+// whole is the fastest of all of them: split and whole, one 336 x 336 image 1108 and 1103, 122 tokens 792 and 774, 64 of d 1280 1264 and
+// 1243, 50 of audio 1190 and 1127.)
 static int pick_splits(int64_t M, int64_t N, int64_t K, int sm_count) {
   constexpr double kPartUs = 0.75;
   const int64_t items = ((M + kBM - 1) / kBM) * ((N + kBN - 1) / kBN);
